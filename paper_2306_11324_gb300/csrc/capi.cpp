@@ -360,6 +360,7 @@ igabem_problem *problem_plan(igabem_geom *geom, const igabem_options *opt) {
     total += 13 * ((gst * sizeof(double) + 255) & ~size_t(255));
     total += bytes_of(S.phi1) + bytes_of(S.dphi1) + bytes_of(S.ext1) + bytes_of(S.gx) + bytes_of(S.gw);
     total += bytes_of(std::vector<float>(S.phi1.size())) + bytes_of(std::vector<float>((size_t)nq));
+    total += CIS_N * 2 * sizeof(double);
     total += 3 * 256 + 5 * nrule * sizeof(double);
     for (const Rule4 *r : {&S.r_id, &S.r_edge, &S.r_vert}) total += (r->share.size() + 255) & ~size_t(255);
     total += bytes_of(S.touch) + bytes_of(S.touch_blk) + bytes_of(S.sing) + bytes_of(S.x2g) + bytes_of(S.g2x_ptr) +
@@ -451,6 +452,15 @@ void problem_materialize(igabem_problem *P, cudaStream_t st) {
     for (int q = 0; q < nq; ++q) gwq[q] = (float)(S.gw[q / S.ng] * S.gw[q % S.ng] * S.h * S.h);
     d.phi1f = upload(A, phi1f, st);
     d.gwqf = upload(A, gwq, st);
+    std::vector<double> cis(2 * CIS_N);
+    for (int k = 0; k < CIS_N; ++k) {  // every entry from an angle in the first eighth of the circle
+      const int n4 = CIS_N / 4, o = k / n4, j = k % n4, jj = std::min(j, n4 - j);
+      double c = std::cos(2 * M_PI * jj / CIS_N), v = std::sin(2 * M_PI * jj / CIS_N);
+      if (j > n4 - j) std::swap(c, v);
+      cis[2 * k] = o == 0 ? c : o == 1 ? -v : o == 2 ? -c : v;
+      cis[2 * k + 1] = o == 0 ? v : o == 1 ? c : o == 2 ? -v : -c;
+    }
+    d.cis = upload(A, cis, st);
     IGA_CUDA(cudaStreamSynchronize(st));  // the host vectors above go out of scope
   }
   for (int k = 0; k < 3; ++k) {

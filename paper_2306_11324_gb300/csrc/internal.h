@@ -245,6 +245,8 @@ class Phase {
 };
 void note_launch();
 
+constexpr int CIS_N = 1024;  // entries of the table of exp(2 pi i k / N) (16 KB)
+
 // device copies of the set-up and the working buffers of a problem
 struct DeviceProblem {
   Profiler *prof = nullptr;
@@ -254,6 +256,7 @@ struct DeviceProblem {
   double *ebez;
   double *gpx, *gpn, *gpa, *gfs, *gft;    // Gauss-point geometry: [3][E*ng*ng] or [E*ng*ng]
   double *phi1, *dphi1, *ext1, *gx, *gw;
+  double *cis;                              // exp(2 pi i k / CIS_N): [CIS_N] complex (FP64 kernel phases)
   float *phi1f, *gwqf;  // FP32 copies: B-spline values at the Gauss points, gw[q1] gw[q2] h^2 per point
   double *rule[3];                          // singular rules (5 arrays each, SoA)
   unsigned char *share[3];                  // their sharing tables (Rule4::share)

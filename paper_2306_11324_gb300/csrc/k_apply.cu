@@ -290,76 +290,6 @@ __global__ void __launch_bounds__(256) k_l2l_sep(Dims D, int l, const double *__
   }
 }
 
-// M2L on level l: yhat[t][a][cr] = sum_{s in far(t)} sum_b S_ts(a, b) xhat[s][b][cr], with the kernel
-// samples between the Chebyshev nodes generated on the fly:
-//   soft: S = a_y G'(r)/r (x-y).n~_x - i eta a_x a_y G      (pull-back of K' - i eta V)
-//   hard: channel 0: S = a_x G'(r)/r (y-x).n~_y  (pull-back of K);  channels 1..6: S = G.
-constexpr int M2L_BT = 16;   // source nodes per tile
-constexpr int M2L_MO = 4;    // outputs per thread
-
-__global__ void k_m2l(Dims D, int ncl, const int *__restrict__ far_ptr, const int *__restrict__ far_src,
-                      const double *__restrict__ nodes, const double2 *__restrict__ xhat,
-                      double2 *__restrict__ yhat, int crc) {
-  extern __shared__ double2 smem[];
-  const int t = blockIdx.x;
-  const int cr0 = blockIdx.y * crc, ncr = min(crc, D.CR - cr0);
-  if (ncr <= 0) return;
-  const int ntypes = D.hard ? 2 : 1;
-  double2 *S = smem;                                   // [ntypes][Q][BT]
-  double2 *Xs = S + ntypes * D.Q * M2L_BT;             // [BT][crc]
-  const long NQ = (long)ncl * D.Q;
-  double2 acc[M2L_MO];
-  for (int k = 0; k < M2L_MO; ++k) acc[k] = cmk(0, 0);
-  const int nout = D.Q * ncr;
-  for (int k = far_ptr[t]; k < far_ptr[t + 1]; ++k) {
-    const int s = far_src[k];
-    for (int b0 = 0; b0 < D.Q; b0 += M2L_BT) {
-      const int nbt = min(M2L_BT, D.Q - b0);
-      for (int i = threadIdx.x; i < D.Q * nbt; i += blockDim.x) {
-        int a = i / nbt, bb = i % nbt;
-        long ia = (long)t * D.Q + a, ib = (long)s * D.Q + b0 + bb;
-        double x[3] = {nodes[ia], nodes[NQ + ia], nodes[2 * NQ + ia]};
-        double y[3] = {nodes[ib], nodes[NQ + ib], nodes[2 * NQ + ib]};
-        double d[3] = {x[0] - y[0], x[1] - y[1], x[2] - y[2]};
-        double r = sqrt(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]);
-        KernelVals kv = helmholtz(D.kappa, r);
-        double ax = nodes[6 * NQ + ia], ay = nodes[6 * NQ + ib];
-        if (!D.hard) {
-          double dn = d[0] * nodes[3 * NQ + ia] + d[1] * nodes[4 * NQ + ia] + d[2] * nodes[5 * NQ + ia];
-          double2 kp = cscale(kv.dGr, ay * dn), v = cscale(kv.G, ax * ay);
-          S[a * M2L_BT + bb] = cmk(kp.x + D.eta * v.y, kp.y - D.eta * v.x);
-        } else {
-          double dn = -(d[0] * nodes[3 * NQ + ib] + d[1] * nodes[4 * NQ + ib] + d[2] * nodes[5 * NQ + ib]);
-          S[a * M2L_BT + bb] = cscale(kv.dGr, ax * dn);
-          S[D.Q * M2L_BT + a * M2L_BT + bb] = kv.G;
-        }
-      }
-      for (int i = threadIdx.x; i < nbt * ncr; i += blockDim.x) {
-        int bb = i / ncr, c = i % ncr;
-        Xs[bb * crc + c] = xhat[((long)s * D.Q + b0 + bb) * D.CR + cr0 + c];
-      }
-      __syncthreads();
-      for (int k2 = 0; k2 < M2L_MO; ++k2) {
-        int o = threadIdx.x + k2 * blockDim.x;
-        if (o >= nout) break;
-        int a = o / ncr, c = o % ncr;
-        int type = (D.hard && (cr0 + c) / D.R >= 1) ? 1 : 0;
-        const double2 *Sr = S + type * D.Q * M2L_BT + a * M2L_BT;
-        double2 v = acc[k2];
-        for (int bb = 0; bb < nbt; ++bb) v = cadd(v, cmul(Sr[bb], Xs[bb * crc + c]));
-        acc[k2] = v;
-      }
-      __syncthreads();
-    }
-  }
-  for (int k2 = 0; k2 < M2L_MO; ++k2) {
-    int o = threadIdx.x + k2 * blockDim.x;
-    if (o >= nout) break;
-    int a = o / ncr, c = o % ncr;
-    yhat[((long)t * D.Q + a) * D.CR + cr0 + c] = acc[k2];
-  }
-}
-
 // L2P, step 1: channel values at the Gauss points, g[e][q][cr] = sum_a L_a(q) yhat_leaf[a][cr]
 __global__ void k_l2p_eval(Dims D, Tables T, const double2 *__restrict__ yhat, double2 *__restrict__ g) {
   const int nlL = 1 << D.L, e1 = 1 << D.b;
@@ -830,22 +760,10 @@ void launch_matvec(const DeviceProblem &d, const HostSetup &S, const igabem_opti
         for (int l = S.lmin; l <= S.L; ++l)
           to_f32(d.xhat[l], d.xhat32[l], (long)S.lev[l].n * S.lev[l].q * S.lev[l].q * D.CR, st);
     }
-    if (m2l_rows_supported(S, o, R)) {
+    {
       Phase ph(d.prof, IGABEM_PH_M2L, st);
       if (tc) launch_m2l_tc(d, S, o, R, st);
       else launch_m2l_rows(d, S, o, R, f32, st);
-    } else {
-      Phase ph(d.prof, IGABEM_PH_M2L, st);
-      for (int l = S.lmin; l <= S.L; ++l) {
-        const Dims Dl = level_dims(l);
-        int crc = std::max(1, std::min(D.CR, (M2L_MO * 256) / Dl.Q));
-        int ntypes = D.hard ? 2 : 1;
-        size_t smem = (size_t)(ntypes * Dl.Q * M2L_BT + M2L_BT * crc) * sizeof(double2);
-        IGA_CUDA(set_max_dynamic_smem(k_m2l, smem));
-        dim3 grid(S.lev[l].n, (D.CR + crc - 1) / crc);
-        k_m2l<<<grid, 256, smem, st>>>(Dl, S.lev[l].n, d.far_ptr[l], d.far_src[l], d.nodes[l], X(l), Y(l), crc);
-        note_launch();
-      }
     }
     {
       Phase ph(d.prof, IGABEM_PH_L2L, st);

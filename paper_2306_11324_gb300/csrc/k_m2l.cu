@@ -1,13 +1,7 @@
-// M2L: couplings of admissible cluster pairs (Sec. 4.4) with the kernel samples between the
-// Chebyshev nodes generated on the fly, FP64 and FP32.
-//
-// Layout: one thread block per target cluster (all levels in one launch), its warps share the
-// target's interaction list; lane l owns target nodes a0 + l and a0 + l + 32 of a chunk of 64 target
-// nodes (levels with q*q > 64 take several chunks, each streaming the interaction list again) and
-// generates their rows of the coupling block in registers while streaming the source nodes of one pair
-// from shared memory (broadcast reads).  Accumulation is blocked: q source nodes per partial sum, q
-// partial sums per pair, then the pairs; the warps are reduced through shared memory at the end of a
-// chunk.  Each level has its own q (level-adaptive interpolation).
+// M2L: couplings of admissible cluster pairs (Sec. 4.4), FP64 and FP32: kernel samples between the
+// Chebyshev nodes generated on the fly (k_m2l_fly; k_m2l_gemm for many columns), or coupling blocks stored
+// at set-up (k_m2l_stored).  All levels go in one launch, each with its own q (level-adaptive
+// interpolation), one block (or a cluster of blocks) per target cluster.
 //
 // FP32 phase split: the sample phase kappa r is formed as kappa |D| (D = c_t - c_s, the distance of
 // the two cluster centres, taken in FP64 once per pair and reduced mod 2 pi) plus kappa (r - |D|),
@@ -15,6 +9,8 @@
 // delta = (x_a - c_t) - (y_b - c_s).  The FP32 error of the phase is then of the order of the
 // cluster size times the unit roundoff instead of kappa r times it, and the factor
 // exp(i kappa |D|) multiplies the pair's partial sums once.
+#include <cooperative_groups.h>
+
 #include <algorithm>
 #include <type_traits>
 
@@ -51,181 +47,243 @@ struct M2LArgs {
   int CR, R;
   double kappa, eta;
   bool hard;
+  const double2 *cis;    // exp(2 pi i k / CIS_N), k < CIS_N
+  int rows_most;         // P Q of the level that uses most of a block's threads (k_m2l_fly)
 };
 
-// per-source-node data in shared memory
-template <class T> struct SrcNode {
-  T dy[3], ny[3], ay, Ddy, Dny, pad;
-};
+// ---- FP64 arithmetic of the coupling samples -------------------------------------------------------
+// The FP64 pipe is what bounds the FP64 product (a warp instruction of it holds a quarter of an SM for
+// about 76 cycles; integer, FP32 and shared-memory instructions hide behind it), so these helpers count
+// FP64 instructions: 1/sqrt in 5 and exp(i phi) in 9 + 4 (a complex product with the table entry).
 
-// Kernel sample(s) between target node (x, n~x, ax) and source node (y, n~y, ay).
-//   soft: ks = a_y G'(r)/r (x-y).n~x - i eta a_x a_y G                       (K' - i eta V)
-//   hard: kk = a_x G'(r)/r (y-x).n~y (K),  g = G (the six W channels)
-// e = (cos, sin) of the phase carried by the sample; for FP32 the pair factor exp(i kappa |D|) is
-// applied by the caller.
-template <class T, int NCR, bool HARD>
-__global__ void __launch_bounds__(32 * M2L_WARPS) k_m2l_rows(M2LArgs A, int cr0) {
-  extern __shared__ __align__(16) unsigned char smraw[];
+// 1/sqrt(x), x a positive normal number: the single-precision estimate of the scaled argument (exponent
+// handled by integer instructions), one step of Householder's third-order iteration (relative error of
+// the estimate 2^-22, cubed).
+__device__ inline double rsqrt64(double x) {
+  const int hi = __double2hiint(x), lo = __double2loint(x);
+  const int k = ((hi >> 20) - 1023) >> 1;           // x = m 4^k, m in [1, 4)
+  const int hm = hi - (k << 21);
+  float f;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(f) : "f"(__uint_as_float((unsigned)(hm - (896 << 20)) << 3 | (unsigned)lo >> 29)));
+  const unsigned fb = __float_as_uint(f);
+  const double y = __hiloint2double((int)(fb >> 3) + (896 << 20) - (k << 20), (int)(fb << 29));
+  const double e = fma(-(x * y), y, 1.0);
+  return fma(y, e * fma(e, 0.375, 0.5), y);
+}
+
+// Table-driven exp(i kappa r) (Tang's method): kappa r = 2 pi (k + u) / CIS_N, |u| <= 1/2, so
+// exp(i kappa r) = table[k] (1 + m1 + i s) with m1 + i s = exp(2 pi i u / CIS_N) - 1 by its series.  c0 + c1 is
+// kappa CIS_N / (2 pi) in two doubles, so that u is correct to the rounding of r.
+struct Phase64 {
+  double2 E;
+  double m1, s;
+};
+__device__ inline Phase64 phase64(const double2 *__restrict__ tab, double r, double c0, double c1) {
+  constexpr double M = 6755399441055744.0;          // 1.5 2^52: adding it rounds to an integer
+  constexpr double T1 = TWO_PI / CIS_N;
+  const double tm = fma(r, c0, M);
+  const int k = __double2loint(tm) & (CIS_N - 1);
+  double u = fma(r, c0, M - tm);
+  u = fma(r, c1, u);
+  const double u2 = u * u;
+  Phase64 p;
+  p.s = u * fma(u2, fma(u2, T1 * T1 * T1 * T1 * T1 / 120.0, -T1 * T1 * T1 / 6.0), T1);
+  p.m1 = u2 * fma(u2, T1 * T1 * T1 * T1 / 24.0, -T1 * T1 / 2.0);
+  p.E = tab[k];
+  return p;
+}
+// p (1 + m1 + i s)
+__device__ inline C2<double> phase_mul(double px, double py, const Phase64 &f) {
+  return c2(fma(-py, f.s, fma(px, f.m1, px)), fma(px, f.s, fma(py, f.m1, py)));
+}
+
+// Per-source-node data in shared memory: position (FP32: its offset from the cluster centre), the
+// Jacobian (soft; FP64: / (4 pi)) or the normal (hard), and in FP32 the products with D = c_t - c_s.
+template <class T, bool HARD> struct FlyNode;
+template <> struct __align__(16) FlyNode<double, false> { double y[3], a; };
+template <> struct __align__(16) FlyNode<double, true> { double y[3], n[3]; };
+template <> struct __align__(16) FlyNode<float, false> { float y[3], Dy, a, pad[3]; };
+template <> struct __align__(16) FlyNode<float, true> { float y[3], Dy, n[3], Dn; };
+
+// M2L with the samples generated on the fly.  A thread owns one target node of one pair: the Q nodes of P
+// pairs (P = 256 / Q) lie side by side in a block's 256 threads (Q = 49: 245 of them at work; one warp
+// per pair with two rows a lane used 49 of 64).  It generates its row of the pair's coupling block in
+// registers, reading the source nodes from shared memory, and multiplies it into NC columns: for
+// sound-hard one sample gives K and G, which serve the columns of all seven channels.  Sums: the pair's in
+// registers, then over the thread's pairs, then over the P threads of a node and over the blocks
+// of a cluster, in that fixed order (FP64).  A target's interaction list is split over a cluster of
+// gridDim.y blocks, which add their sums through distributed shared memory, where a level has too few
+// targets to fill the device.  Measured on GB300, FP64 products (before: one warp per pair, 72 FP64
+// instructions a sample and CUDA's sincos, or for several columns the tile of k_m2l_gemm mostly padding): 6936
+// unknowns, one column, 175 M samples 32.2 -> 17.1 ms; 150 unknowns, 8 M samples 2.20 -> 1.08 ms; sound-hard,
+// 1736 unknowns, 3 columns of 7 channels 41 -> 4 ms.
+template <class T, int NC, bool HARD>
+__global__ void __launch_bounds__(256) k_m2l_fly(const __grid_constant__ M2LArgs A) {
+  extern __shared__ __align__(16) unsigned char smf[];
   constexpr bool F32 = std::is_same<T, float>::value;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  // locate the level of this block
+  using Node = FlyNode<T, HARD>;
+  const int tid = threadIdx.x, nsplit = gridDim.y, rank = blockIdx.y, cr0 = blockIdx.z * NC;
   int li = 0;
   while (li + 1 < A.nlev && (int)blockIdx.x >= A.lev[li + 1].first) ++li;
   const M2LLevel &L = A.lev[li];
-  const int t = blockIdx.x - L.first;
-  const int Q = L.Q, q = L.q, QS = A.QS;
+  const int t = blockIdx.x - L.first, Q = L.Q, P = 256 / Q, slot = tid / Q, a = tid - slot * Q;
   const long NQ = (long)L.n * Q;
-  const int ncr = min(NCR, A.CR - cr0);
-  // shared memory: per warp QS source nodes + QS x NCR source coefficients; then the reduction area
-  SrcNode<T> *src = reinterpret_cast<SrcNode<T> *>(smraw) + warp * QS;
-  C2<T> *xs = reinterpret_cast<C2<T> *>(reinterpret_cast<SrcNode<T> *>(smraw) + M2L_WARPS * QS) + warp * QS * NCR;
-  double2 *red = reinterpret_cast<double2 *>(smraw);
+  const int ncr = min(NC, A.CR - cr0);
+  double2 *tab = reinterpret_cast<double2 *>(smf);                       // FP64: the table of phase64
+  Node *src = reinterpret_cast<Node *>(smf + (F32 ? 0 : CIS_N * sizeof(double2)));  // [P Q]
+  C2<T> *xs = reinterpret_cast<C2<T> *>(src + A.rows_most);              // [P Q][NC]
+  C2<T> *red = xs;
+  if constexpr (!F32)
+    for (int i = tid; i < CIS_N; i += 256) tab[i] = A.cis[i];
+  const double c0 = A.kappa * (CIS_N / TWO_PI);
+  // the rest of kappa CIS_N / (2 pi): CIS_N / (2 pi) = CH + CL to twice the precision
+  constexpr double CH = CIS_N / TWO_PI, CL = -CIS_N * 9.839338337591243e-18;
+  const double c1 = fma(A.kappa, CL, fma(A.kappa, CH, -c0));
   const T kappa = (T)A.kappa, eta = (T)A.eta;
-  const T inv4pi = (T)(0.25 / IGA_PI);
-  for (int a0 = 0; a0 < Q; a0 += 64) {
-    // target rows of this lane in the chunk
-    T tx[2][3], tn[2][3], ta[2];
-    bool valid[2];
-    for (int k = 0; k < 2; ++k) {
-      int a = a0 + lane + 32 * k;
-      valid[k] = a < Q;
-      long ia = (long)t * Q + (valid[k] ? a : 0);
-      for (int c = 0; c < 3; ++c) {
-        tx[k][c] = F32 ? (T)L.nodes32[c * NQ + ia] : (T)L.nodes[c * NQ + ia];
-        tn[k][c] = F32 ? (T)L.nodes32[(3 + c) * NQ + ia] : (T)L.nodes[(3 + c) * NQ + ia];
-      }
-      ta[k] = F32 ? (T)L.nodes32[6 * NQ + ia] : (T)L.nodes[6 * NQ + ia];
+  const bool on = slot < P;
+  T tx[3] = {0, 0, 0}, tn[3] = {0, 0, 0}, ta = 0;
+  if (on) {
+    const long ia = (long)t * Q + a;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      tx[c] = F32 ? (T)L.nodes32[c * NQ + ia] : (T)L.nodes[c * NQ + ia];
+      if (!HARD) tn[c] = F32 ? (T)L.nodes32[(3 + c) * NQ + ia] : (T)L.nodes[(3 + c) * NQ + ia];
     }
-    C2<T> tot[2][NCR];
-    for (int k = 0; k < 2; ++k)
-      for (int c = 0; c < NCR; ++c) tot[k][c] = c2((T)0, (T)0);
-    for (int kk = L.far_ptr[t] + warp; kk < L.far_ptr[t + 1]; kk += M2L_WARPS) {
-      const int s = L.far_src[kk];
-      // pair constants (FP32 path): D = c_t - c_s, |D|, |D|^2 and exp(i kappa |D|), from the set-up
-      T D[3] = {0, 0, 0}, Dn = 0, D2 = 0;
-      C2<T> e0 = c2((T)1, (T)0);
-      if constexpr (F32) {
-        const float4 p0 = reinterpret_cast<const float4 *>(L.pc)[2 * kk];
-        const float4 p1 = reinterpret_cast<const float4 *>(L.pc)[2 * kk + 1];
-        D[0] = p0.x; D[1] = p0.y; D[2] = p0.z; Dn = p0.w;
-        D2 = p1.x;
-        e0 = c2(p1.y, p1.z);
-      }
-      // stage the source nodes and coefficients of this pair
-      __syncwarp();
-      for (int b = lane; b < Q; b += 32) {
-        long ib = (long)s * Q + b;
-        SrcNode<T> sn;
-        for (int c = 0; c < 3; ++c) {
-          sn.dy[c] = F32 ? (T)L.nodes32[c * NQ + ib] : (T)L.nodes[c * NQ + ib];
-          sn.ny[c] = F32 ? (T)L.nodes32[(3 + c) * NQ + ib] : (T)L.nodes[(3 + c) * NQ + ib];
-        }
-        sn.ay = F32 ? (T)L.nodes32[6 * NQ + ib] : (T)L.nodes[6 * NQ + ib];
-        sn.Ddy = D[0] * sn.dy[0] + D[1] * sn.dy[1] + D[2] * sn.dy[2];
-        sn.Dny = D[0] * sn.ny[0] + D[1] * sn.ny[1] + D[2] * sn.ny[2];
-        src[b] = sn;
-        for (int c = 0; c < ncr; ++c) {
-          if constexpr (F32) {
-            const float2 v = L.xhat32[ib * A.CR + cr0 + c];
-            xs[b * NCR + c] = c2((T)v.x, (T)v.y);
-          } else {
-            const double2 v = L.xhat[ib * A.CR + cr0 + c];
-            xs[b * NCR + c] = c2((T)v.x, (T)v.y);
-          }
-        }
-      }
-      __syncwarp();
-      for (int k = 0; k < 2; ++k) {
-        if (!valid[k]) continue;
-        const T Ddx = D[0] * tx[k][0] + D[1] * tx[k][1] + D[2] * tx[k][2];
-        const T Dnx = D[0] * tn[k][0] + D[1] * tn[k][1] + D[2] * tn[k][2];
-        C2<T> acc[NCR];
-        for (int c = 0; c < NCR; ++c) acc[c] = c2((T)0, (T)0);
-        for (int b1 = 0; b1 < q; ++b1) {
-          C2<T> part[NCR];
-          for (int c = 0; c < NCR; ++c) part[c] = c2((T)0, (T)0);
-          for (int b2 = 0; b2 < q; ++b2) {
-            const int b = b1 * q + b2;
-            const SrcNode<T> &y = src[b];
-            T d0 = tx[k][0] - y.dy[0], d1 = tx[k][1] - y.dy[1], d2 = tx[k][2] - y.dy[2];
-            T r2, ir, r, cph, sph;
-            T dn_x, dn_y;  // (x-y).n~x and (x-y).n~y
-            if constexpr (F32) {
-              // delta = d; x - y = D + delta
-              T Dd = Ddx - y.Ddy;
-              T dd = d0 * d0 + d1 * d1 + d2 * d2;
-              T num = (T)2 * Dd + dd;
-              r2 = D2 + num;
-              ir = rsqrtf((float)r2);
-              r = r2 * ir;
-              T del = __fdividef((float)num, (float)(r + Dn));
-              T ph = kappa * del;
-              T kq = rintf((float)(ph * (T)0.15915494309189535));
-              ph = fmaf(-(float)kq, 6.28318548202514648f, (float)ph);
-              ph = fmaf(-(float)kq, -1.7484556e-07f, (float)ph);
-              float sf, cf;
-              __sincosf((float)ph, &sf, &cf);
-              cph = cf;
-              sph = sf;
-              dn_x = Dnx + d0 * tn[k][0] + d1 * tn[k][1] + d2 * tn[k][2];
-              dn_y = y.Dny + d0 * y.ny[0] + d1 * y.ny[1] + d2 * y.ny[2];
-            } else {
-              r2 = d0 * d0 + d1 * d1 + d2 * d2;
-              ir = rsqrt((double)r2);
-              r = r2 * ir;
-              double sd, cd;
-              sincos(A.kappa * (double)r, &sd, &cd);
-              cph = cd;
-              sph = sd;
-              dn_x = d0 * tn[k][0] + d1 * tn[k][1] + d2 * tn[k][2];
-              dn_y = d0 * y.ny[0] + d1 * y.ny[1] + d2 * y.ny[2];
-            }
-            const T f = ir * inv4pi;
-            const T kr = kappa * r;
-            const T g2 = f * ir * ir;
-            // G = e f;  G'(r)/r = e (-1 + i kappa r) f / r^2
-            const C2<T> G = c2(cph * f, sph * f);
-            const C2<T> dG = c2((-cph - sph * kr) * g2, (-sph + cph * kr) * g2);
-            if (!HARD) {
-              const T w1 = y.ay * dn_x, w2 = ta[k] * y.ay * eta;
-              // ks = dG w1 - i eta a_x a_y G
-              const C2<T> ks = c2(dG.x * w1 + G.y * w2, dG.y * w1 - G.x * w2);
-              for (int c = 0; c < NCR; ++c) part[c] = fma2(ks, xs[b * NCR + c], part[c]);
-            } else {
-              const T w1 = -ta[k] * dn_y;  // a_x (y-x).n~y
-              const C2<T> kk2 = c2(dG.x * w1, dG.y * w1);
-              for (int c = 0; c < NCR; ++c) {
-                const int ch = (cr0 + c) / A.R;
-                part[c] = fma2(ch == 0 ? kk2 : G, xs[b * NCR + c], part[c]);
-              }
-            }
-          }
-          for (int c = 0; c < NCR; ++c) acc[c] = add(acc[c], part[c]);
-        }
-        for (int c = 0; c < NCR; ++c) tot[k][c] = fma2(e0, acc[c], tot[k][c]);
-      }
-    }
-    // reduce over the warps (the staging area is reused)
-    __syncthreads();
-    for (int k = 0; k < 2; ++k)
-      for (int c = 0; c < NCR; ++c) {
-        int a = lane + 32 * k;
-        red[(warp * 64 + a) * NCR + c] = make_double2((double)tot[k][c].x, (double)tot[k][c].y);
-      }
-    __syncthreads();
-    const int na = min(64, Q - a0);
-    for (int o = threadIdx.x; o < na * ncr; o += blockDim.x) {
-      int a = o / ncr, c = o % ncr;
-      double2 sum = make_double2(0, 0);
-      for (int w = 0; w < M2L_WARPS; ++w) {
-        double2 v = red[(w * 64 + a) * NCR + c];
-        sum.x += v.x;
-        sum.y += v.y;
-      }
-      L.yhat[((long)t * Q + a0 + a) * A.CR + cr0 + c] = sum;
-    }
-    __syncthreads();  // the reduction area is the staging area of the next chunk
+    ta = F32 ? (T)L.nodes32[6 * NQ + ia] : (T)L.nodes[6 * NQ + ia];
+    if (!HARD) ta *= eta;
   }
+  C2<T> tot[NC];
+#pragma unroll
+  for (int c = 0; c < NC; ++c) tot[c] = c2((T)0, (T)0);
+  const int k0 = L.far_ptr[t], np = L.far_ptr[t + 1] - k0;
+  for (int p0 = rank * P; p0 < np; p0 += nsplit * P) {
+    const bool work = on && p0 + slot < np;
+    const int kk = k0 + p0 + slot;
+    T D[3] = {0, 0, 0}, Dn = 0, D2 = 0;
+    C2<T> e0 = c2((T)1, (T)0);
+    __syncthreads();  // the previous pairs' nodes and columns are read
+    if (work) {
+      if constexpr (F32) {
+        const float4 q0 = reinterpret_cast<const float4 *>(L.pc)[2 * (long)kk];
+        const float4 q1 = reinterpret_cast<const float4 *>(L.pc)[2 * (long)kk + 1];
+        D[0] = q0.x; D[1] = q0.y; D[2] = q0.z; Dn = q0.w;
+        D2 = q1.x;
+        e0 = c2(q1.y, q1.z);
+      }
+      // the thread stages the source node with its own index
+      const long ib = (long)L.far_src[kk] * Q + a;
+      Node sn;
+      T nn[3];
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        sn.y[c] = F32 ? (T)L.nodes32[c * NQ + ib] : (T)L.nodes[c * NQ + ib];
+        if (HARD) nn[c] = F32 ? (T)L.nodes32[(3 + c) * NQ + ib] : (T)L.nodes[(3 + c) * NQ + ib];
+      }
+      if constexpr (HARD) {
+#pragma unroll
+        for (int c = 0; c < 3; ++c) sn.n[c] = nn[c];
+        if constexpr (F32) sn.Dn = D[0] * nn[0] + D[1] * nn[1] + D[2] * nn[2];
+      } else {
+        sn.a = F32 ? (T)L.nodes32[6 * NQ + ib] : (T)(L.nodes[6 * NQ + ib] * (0.25 / IGA_PI));
+      }
+      if constexpr (F32) sn.Dy = D[0] * sn.y[0] + D[1] * sn.y[1] + D[2] * sn.y[2];
+      src[tid] = sn;
+#pragma unroll
+      for (int c = 0; c < NC; ++c) {
+        C2<T> v = c2((T)0, (T)0);
+        if (c < ncr) {
+          if constexpr (F32) {
+            const float2 w = L.xhat32[ib * A.CR + cr0 + c];
+            v = c2((T)w.x, (T)w.y);
+          } else {
+            const double2 w = L.xhat[ib * A.CR + cr0 + c];
+            v = c2((T)w.x, (T)w.y);
+          }
+        }
+        xs[tid * NC + c] = v;
+      }
+    }
+    __syncthreads();
+    if (!work) continue;
+    C2<T> part[NC];
+#pragma unroll
+    for (int c = 0; c < NC; ++c) part[c] = c2((T)0, (T)0);
+    const Node *sp = src + slot * Q;
+    const C2<T> *xp = xs + slot * Q * NC;
+    const T Ddx = D[0] * tx[0] + D[1] * tx[1] + D[2] * tx[2];
+    const T Dnx = D[0] * tn[0] + D[1] * tn[1] + D[2] * tn[2];
+    for (int b = 0; b < Q; ++b) {
+      const Node y = sp[b];
+      const T d0 = tx[0] - y.y[0], d1 = tx[1] - y.y[1], d2 = tx[2] - y.y[2];
+      C2<T> S0, S1 = c2((T)0, (T)0);  // soft: S0; hard: S0 = K, S1 = G
+      if constexpr (F32) {
+        const T num = (T)2 * (Ddx - y.Dy) + (d0 * d0 + d1 * d1 + d2 * d2);
+        const T r2 = D2 + num, ir = rsqrtf(r2), r = r2 * ir;
+        T ph = kappa * __fdividef(num, r + Dn);
+        const T kq = rintf(ph * 0.15915494309189535f);
+        ph = fmaf(-kq, 6.28318548202514648f, ph);
+        ph = fmaf(-kq, -1.7484556e-07f, ph);
+        T sph, cph;
+        __sincosf(ph, &sph, &cph);
+        const T f = ir * (T)(0.25 / IGA_PI), kr = kappa * r, g2 = f * ir * ir;
+        const C2<T> G = c2(cph * f, sph * f);
+        const C2<T> dG = c2((-cph - sph * kr) * g2, (-sph + cph * kr) * g2);
+        if constexpr (!HARD) {
+          const T w1 = y.a * (Dnx + d0 * tn[0] + d1 * tn[1] + d2 * tn[2]), w2 = ta * y.a;
+          S0 = c2(dG.x * w1 + G.y * w2, dG.y * w1 - G.x * w2);
+        } else {
+          const T w1 = -ta * (y.Dn + d0 * y.n[0] + d1 * y.n[1] + d2 * y.n[2]);
+          S0 = c2(dG.x * w1, dG.y * w1);
+          S1 = G;
+        }
+      } else {
+        const double r2 = d0 * d0 + d1 * d1 + d2 * d2, ir = rsqrt64(r2);
+        const Phase64 ph = phase64(tab, r2 * ir, c0, c1);
+        if constexpr (!HARD) {
+          // exp(i kappa r) (A + i B), with w = a_y / (4 pi r): A = -w (d.n)/r^2, B = kappa w (d.n)/r - eta a_x w
+          const double w = y.a * ir, gw = (d0 * tn[0] + d1 * tn[1] + d2 * tn[2]) * ir * w;
+          const double Ar = -gw * ir, Br = fma(kappa, gw, -(ta * w));
+          S0 = phase_mul(ph.E.x * Ar - ph.E.y * Br, ph.E.x * Br + ph.E.y * Ar, ph);
+        } else {
+          // G = exp(i kappa r) / (4 pi r); K = G (A + i B), w = -a_x (d.n_y) / r: A = -w / r, B = kappa w
+          const double f = ir * (0.25 / IGA_PI);
+          S1 = phase_mul(ph.E.x * f, ph.E.y * f, ph);
+          const double w = -ta * (d0 * y.n[0] + d1 * y.n[1] + d2 * y.n[2]) * ir, Ar = -w * ir, Br = kappa * w;
+          S0 = c2(S1.x * Ar - S1.y * Br, S1.x * Br + S1.y * Ar);
+        }
+      }
+#pragma unroll
+      for (int c = 0; c < NC; ++c) {
+        const bool k = !HARD || cr0 + c < A.R;  // the first R columns are channel 0
+        part[c] = fma2(k ? S0 : S1, xp[b * NC + c], part[c]);
+      }
+    }
+#pragma unroll
+    for (int c = 0; c < NC; ++c) tot[c] = F32 ? fma2(e0, part[c], tot[c]) : add(tot[c], part[c]);
+  }
+  // sums over the P threads of a node and the blocks of the cluster
+  __syncthreads();
+  if (on)
+#pragma unroll
+    for (int c = 0; c < NC; ++c) red[tid * NC + c] = tot[c];
+  cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
+  if (nsplit > 1) cl.sync();
+  else __syncthreads();
+  const int per = (Q * ncr + nsplit - 1) / nsplit, o1 = min(Q * ncr, (rank + 1) * per);
+  for (int o = rank * per + tid; o < o1; o += 256) {
+    const int aa = o / ncr, c = o - aa * ncr;
+    double2 sum = make_double2(0, 0);
+    for (int z = 0; z < nsplit; ++z) {
+      const C2<T> *rz = nsplit > 1 ? cl.map_shared_rank(red, z) : red;
+      for (int p = 0; p < P; ++p) {
+        const C2<T> v = rz[(p * Q + aa) * NC + c];
+        sum.x += (double)v.x;
+        sum.y += (double)v.y;
+      }
+    }
+    L.yhat[((long)t * Q + aa) * A.CR + cr0 + c] = sum;
+  }
+  if (nsplit > 1) cl.sync();  // no block leaves while another reads its shared memory
 }
 
 // ---- stored coupling blocks (m2l_stored): the same kernel samples (node_sample, the samples of the
@@ -553,23 +611,49 @@ __global__ void k_pair_consts(const int *__restrict__ far_ptr, const int *__rest
   o[7] = (float)exp2(12.0 - ceil(log2(bound)));
 }
 
-// shared memory of the row kernel: per warp QS source nodes and their NCR coefficients (or the
-// reduction area)
-size_t rows_smem(int QS, int ncr, bool fp32) {
-  const size_t node = fp32 ? sizeof(SrcNode<float>) : sizeof(SrcNode<double>);
-  const size_t coef = fp32 ? sizeof(C2<float>) : sizeof(C2<double>);
-  return std::max((size_t)M2L_WARPS * QS * node + (size_t)M2L_WARPS * QS * ncr * coef,
-                  (size_t)M2L_WARPS * 64 * ncr * sizeof(double2));
+template <class T, int NC, bool HARD>
+void launch_fly(const M2LArgs &A, int nblocks, int nsplit, cudaStream_t st) {
+  const size_t smem = (std::is_same<T, float>::value ? 0 : CIS_N * sizeof(double2)) +
+                      (size_t)A.rows_most * (sizeof(FlyNode<T, HARD>) + NC * sizeof(C2<T>));
+  auto kfn = k_m2l_fly<T, NC, HARD>;
+  IGA_CUDA(set_max_dynamic_smem(kfn, smem));
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(nblocks, nsplit, (A.CR + NC - 1) / NC);
+  cfg.blockDim = dim3(256);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = 1;
+  at.val.clusterDim.y = nsplit;
+  at.val.clusterDim.z = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  IGA_CUDA(cudaLaunchKernelEx(&cfg, kfn, A));
+  note_launch();
 }
 
-template <class T, int NCR, bool HARD>
-void launch_rows(const M2LArgs &A, int nblocks, cudaStream_t st) {
-  const size_t smem = rows_smem(A.QS, NCR, std::is_same<T, float>::value);
-  auto kfn = k_m2l_rows<T, NCR, HARD>;
-  IGA_CUDA(set_max_dynamic_smem(kfn, smem));
-  for (int cr0 = 0; cr0 < A.CR; cr0 += NCR) {
-    kfn<<<nblocks, 32 * M2L_WARPS, smem, st>>>(A, cr0);
-    note_launch();
+// All columns, in passes of at most 24 (the FP64 accumulators of 24 columns fill the registers; each pass
+// generates the samples again), the passes as even as the kernel's column counts allow.
+template <class T>
+void launch_fly_all(const M2LArgs &A, int nblocks, int nsplit, cudaStream_t st) {
+  const int passes = (A.CR + 23) / 24, w = (A.CR + passes - 1) / passes;
+  if (A.hard) {
+    if (w > 16) launch_fly<T, 24, true>(A, nblocks, nsplit, st);
+    else if (w > 8) launch_fly<T, 16, true>(A, nblocks, nsplit, st);
+    else launch_fly<T, 8, true>(A, nblocks, nsplit, st);
+  } else if (w > 16) {
+    launch_fly<T, 24, false>(A, nblocks, nsplit, st);
+  } else if (w > 8) {
+    launch_fly<T, 16, false>(A, nblocks, nsplit, st);
+  } else if (w > 4) {
+    launch_fly<T, 8, false>(A, nblocks, nsplit, st);
+  } else if (w > 2) {
+    launch_fly<T, 4, false>(A, nblocks, nsplit, st);
+  } else if (w == 2) {
+    launch_fly<T, 2, false>(A, nblocks, nsplit, st);
+  } else {
+    launch_fly<T, 1, false>(A, nblocks, nsplit, st);
   }
 }
 
@@ -599,21 +683,6 @@ void launch_stored_typed(const M2LArgs &A, int nblocks, cudaStream_t st) {
   else if (A.CR == 2) launch_stored<T, 2, false>(A, nblocks, st);
   else if (A.CR < 8) launch_stored<T, 4, false>(A, nblocks, st);
   else launch_stored<T, 8, false>(A, nblocks, st);
-}
-
-template <class T>
-void launch_typed(const M2LArgs &A, int nblocks, cudaStream_t st) {
-  if (A.hard) {
-    launch_rows<T, 7, true>(A, nblocks, st);
-  } else if (A.CR == 1) {
-    launch_rows<T, 1, false>(A, nblocks, st);
-  } else if (A.CR == 2) {
-    launch_rows<T, 2, false>(A, nblocks, st);
-  } else if (A.CR < 8 || !std::is_same<T, float>::value) {
-    launch_rows<T, 4, false>(A, nblocks, st);
-  } else {
-    launch_rows<T, 8, false>(A, nblocks, st);
-  }
 }
 
 }  // namespace
@@ -664,17 +733,6 @@ void launch_m2l_fill(const DeviceProblem &d, const HostSetup &S, const igabem_op
   IGA_CUDA(cudaGetLastError());
 }
 
-bool m2l_rows_supported(const HostSetup &S, const igabem_options &o, int R) {
-  if (S.L - S.lmin + 1 > 16) return false;
-  int QS = 0;
-  for (int l = S.lmin; l <= S.L; ++l) QS = std::max(QS, S.lev[l].q * S.lev[l].q);
-  if (R > 1 && QS <= 64) return true;  // the multi-column kernel
-  const bool fp32 = o.precision != IGABEM_FP64;
-  const int CR = (S.hard ? 7 : 1) * R;
-  const int ncr = S.hard ? 7 : (CR == 1 ? 1 : CR == 2 ? 2 : (CR < 8 || !fp32) ? 4 : 8);
-  return rows_smem(QS, ncr, fp32) <= (size_t)max_optin_smem();
-}
-
 void launch_m2l_rows(const DeviceProblem &d, const HostSetup &S, const igabem_options &o, int R,
                      bool fp32, cudaStream_t st) {
   M2LArgs A;
@@ -684,7 +742,10 @@ void launch_m2l_rows(const DeviceProblem &d, const HostSetup &S, const igabem_op
   A.kappa = o.kappa;
   A.eta = o.eta_cfie;
   A.hard = S.hard;
+  A.cis = reinterpret_cast<const double2 *>(d.cis);
   A.nlev = 0;
+  A.rows_most = 0;
+  if (S.L - S.lmin + 1 > 16) fail(IGABEM_EINVAL, "more than 16 cluster levels with admissible pairs");
   int nblocks = 0;
   for (int l = S.lmin; l <= S.L; ++l) {
     M2LLevel &L = A.lev[A.nlev++];
@@ -702,19 +763,23 @@ void launch_m2l_rows(const DeviceProblem &d, const HostSetup &S, const igabem_op
     L.q = S.lev[l].q;
     L.Q = L.q * L.q;
     A.QS = std::max(A.QS, L.Q);
+    A.rows_most = std::max(A.rows_most, 256 / L.Q * L.Q);
     nblocks += S.lev[l].n;
   }
+  // column chunk of the multi-column kernel: the largest divisor of R not above 64 (chunks never straddle two
+  // channels)
+  int Wc = 1;
+  for (int w = std::min(R, 64); w >= 1; --w)
+    if (R % w == 0) {
+      Wc = w;
+      break;
+    }
   if (A.nlev > 0 && A.lev[0].stored) {  // stored coupling blocks: stream them
     if (fp32) launch_stored_typed<float>(A, nblocks, st);
     else launch_stored_typed<double>(A, nblocks, st);
-  } else if (R > 1 && A.QS <= 64) {
-    // column chunk: the largest divisor of R not above 64 (chunks never straddle two channels)
-    int Wc = 1;
-    for (int w = std::min(R, 64); w >= 1; --w)
-      if (R % w == 0) {
-        Wc = w;
-        break;
-      }
+  } else if (Wc >= 48 && A.QS <= 64) {
+    // Its tile has room for 64 columns: below 48 the padding costs more than k_m2l_fly's regenerated samples
+    // (FP64 operations per sample and 7 x 5 columns: 7 (72 + 256) here, 2 x 43 + 140 there).
     const size_t tsz = fp32 ? sizeof(float) : sizeof(double);
     size_t smem = (size_t)A.QS * A.QS * 2 * tsz + (size_t)A.QS * Wc * 2 * tsz + (size_t)A.QS * 16 * tsz;
     dim3 grid(nblocks, A.CR / Wc);
@@ -726,10 +791,15 @@ void launch_m2l_rows(const DeviceProblem &d, const HostSetup &S, const igabem_op
       k_m2l_gemm<double><<<grid, 256, smem, st>>>(A, Wc);
     }
     note_launch();
-  } else if (fp32) {
-    launch_typed<float>(A, nblocks, st);
   } else {
-    launch_typed<double>(A, nblocks, st);
+    // split the interaction lists over clusters of blocks while the device is not filled several times and
+    // every block keeps pairs for all its threads
+    const int P = std::max(1, 256 / S.lev[S.L].q / S.lev[S.L].q);
+    const long mean = S.n_far / std::max(1, nblocks);
+    int nsplit = 1;
+    while (nsplit < 8 && (long)nblocks * nsplit < 8 * 152 && 2L * nsplit * P <= mean + P) nsplit *= 2;
+    if (fp32) launch_fly_all<float>(A, nblocks, nsplit, st);
+    else launch_fly_all<double>(A, nblocks, nsplit, st);
   }
   IGA_CUDA(cudaGetLastError());
 }

@@ -9,7 +9,6 @@ namespace igabem {
 void launch_gauss_geometry(const DeviceProblem &d, const HostSetup &S, cudaStream_t st);
 void launch_node_geometry(const DeviceProblem &d, const HostSetup &S, cudaStream_t st);
 void launch_pair_consts(const DeviceProblem &d, const HostSetup &S, double kappa, double eta, cudaStream_t st);
-bool m2l_rows_supported(const HostSetup &S, const igabem_options &o, int R);
 // stored M2L coupling blocks (m2l_stored): complex entries of level l, and their generation at set-up
 size_t m2l_stored_entries(const HostSetup &S, int l);
 void launch_m2l_fill(const DeviceProblem &d, const HostSetup &S, const igabem_options &o, cudaStream_t st);
