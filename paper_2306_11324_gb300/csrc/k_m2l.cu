@@ -24,7 +24,6 @@ namespace igabem {
 namespace {
 
 constexpr int M2L_WARPS = 8;
-constexpr double TWO_PI = 6.283185307179586476925286766559;
 
 struct M2LLevel {
   const int *far_ptr, *far_src;
@@ -50,52 +49,6 @@ struct M2LArgs {
   const double2 *cis;    // exp(2 pi i k / CIS_N), k < CIS_N
   int rows_most;         // P Q of the level that uses most of a block's threads (k_m2l_fly)
 };
-
-// ---- FP64 arithmetic of the coupling samples -------------------------------------------------------
-// The FP64 pipe is what bounds the FP64 product (a warp instruction of it holds a quarter of an SM for
-// about 76 cycles; integer, FP32 and shared-memory instructions hide behind it), so these helpers count
-// FP64 instructions: 1/sqrt in 5 and exp(i phi) in 9 + 4 (a complex product with the table entry).
-
-// 1/sqrt(x), x a positive normal number: the single-precision estimate of the scaled argument (exponent
-// handled by integer instructions), one step of Householder's third-order iteration (relative error of
-// the estimate 2^-22, cubed).
-__device__ inline double rsqrt64(double x) {
-  const int hi = __double2hiint(x), lo = __double2loint(x);
-  const int k = ((hi >> 20) - 1023) >> 1;           // x = m 4^k, m in [1, 4)
-  const int hm = hi - (k << 21);
-  float f;
-  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(f) : "f"(__uint_as_float((unsigned)(hm - (896 << 20)) << 3 | (unsigned)lo >> 29)));
-  const unsigned fb = __float_as_uint(f);
-  const double y = __hiloint2double((int)(fb >> 3) + (896 << 20) - (k << 20), (int)(fb << 29));
-  const double e = fma(-(x * y), y, 1.0);
-  return fma(y, e * fma(e, 0.375, 0.5), y);
-}
-
-// Table-driven exp(i kappa r) (Tang's method): kappa r = 2 pi (k + u) / CIS_N, |u| <= 1/2, so
-// exp(i kappa r) = table[k] (1 + m1 + i s) with m1 + i s = exp(2 pi i u / CIS_N) - 1 by its series.  c0 + c1 is
-// kappa CIS_N / (2 pi) in two doubles, so that u is correct to the rounding of r.
-struct Phase64 {
-  double2 E;
-  double m1, s;
-};
-__device__ inline Phase64 phase64(const double2 *__restrict__ tab, double r, double c0, double c1) {
-  constexpr double M = 6755399441055744.0;          // 1.5 2^52: adding it rounds to an integer
-  constexpr double T1 = TWO_PI / CIS_N;
-  const double tm = fma(r, c0, M);
-  const int k = __double2loint(tm) & (CIS_N - 1);
-  double u = fma(r, c0, M - tm);
-  u = fma(r, c1, u);
-  const double u2 = u * u;
-  Phase64 p;
-  p.s = u * fma(u2, fma(u2, T1 * T1 * T1 * T1 * T1 / 120.0, -T1 * T1 * T1 / 6.0), T1);
-  p.m1 = u2 * fma(u2, T1 * T1 * T1 * T1 / 24.0, -T1 * T1 / 2.0);
-  p.E = tab[k];
-  return p;
-}
-// p (1 + m1 + i s)
-__device__ inline C2<double> phase_mul(double px, double py, const Phase64 &f) {
-  return c2(fma(-py, f.s, fma(px, f.m1, px)), fma(px, f.s, fma(py, f.m1, py)));
-}
 
 // Per-source-node data in shared memory: position (FP32: its offset from the cluster centre), the
 // Jacobian (soft; FP64: / (4 pi)) or the normal (hard), and in FP32 the products with D = c_t - c_s.
@@ -135,10 +88,8 @@ __global__ void __launch_bounds__(256) k_m2l_fly(const __grid_constant__ M2LArgs
   C2<T> *red = xs;
   if constexpr (!F32)
     for (int i = tid; i < CIS_N; i += 256) tab[i] = A.cis[i];
-  const double c0 = A.kappa * (CIS_N / TWO_PI);
-  // the rest of kappa CIS_N / (2 pi): CIS_N / (2 pi) = CH + CL to twice the precision
-  constexpr double CH = CIS_N / TWO_PI, CL = -CIS_N * 9.839338337591243e-18;
-  const double c1 = fma(A.kappa, CL, fma(A.kappa, CH, -c0));
+  double c0, c1;
+  phase64_scale(A.kappa, c0, c1);
   const T kappa = (T)A.kappa, eta = (T)A.eta;
   const bool on = slot < P;
   T tx[3] = {0, 0, 0}, tn[3] = {0, 0, 0}, ta = 0;

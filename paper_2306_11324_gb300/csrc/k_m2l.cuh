@@ -4,6 +4,7 @@
 
 #include <type_traits>
 
+#include "internal.h"
 #include "k_common.cuh"
 
 namespace igabem {
@@ -18,6 +19,59 @@ template <class T> __device__ inline C2<T> mul(C2<T> a, C2<T> b) {
 }
 template <class T> __device__ inline C2<T> fma2(C2<T> a, C2<T> b, C2<T> acc) {  // acc + a b
   return {acc.x + a.x * b.x - a.y * b.y, acc.y + a.x * b.y + a.y * b.x};
+}
+
+constexpr double TWO_PI = 6.283185307179586476925286766559;
+
+// ---- FP64 arithmetic of the kernel samples -------------------------------------------------------
+// The FP64 pipe is what bounds the FP64 product (a warp instruction of it holds a quarter of an SM for
+// about 76 cycles; integer, FP32 and shared-memory instructions hide behind it), so these helpers count
+// FP64 instructions: 1/sqrt in 5 and exp(i phi) in 9 + 4 (a complex product with the table entry).
+
+// 1/sqrt(x), x a positive normal number: the single-precision estimate of the scaled argument (exponent
+// handled by integer instructions), one step of Householder's third-order iteration (relative error of
+// the estimate 2^-22, cubed).
+__device__ inline double rsqrt64(double x) {
+  const int hi = __double2hiint(x), lo = __double2loint(x);
+  const int k = ((hi >> 20) - 1023) >> 1;           // x = m 4^k, m in [1, 4)
+  const int hm = hi - (k << 21);
+  float f;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(f) : "f"(__uint_as_float((unsigned)(hm - (896 << 20)) << 3 | (unsigned)lo >> 29)));
+  const unsigned fb = __float_as_uint(f);
+  const double y = __hiloint2double((int)(fb >> 3) + (896 << 20) - (k << 20), (int)(fb << 29));
+  const double e = fma(-(x * y), y, 1.0);
+  return fma(y, e * fma(e, 0.375, 0.5), y);
+}
+
+// Table-driven exp(i kappa r) (Tang's method): kappa r = 2 pi (k + u) / CIS_N, |u| <= 1/2, so
+// exp(i kappa r) = table[k] (1 + m1 + i s) with m1 + i s = exp(2 pi i u / CIS_N) - 1 by its series.  c0 + c1 is
+// kappa CIS_N / (2 pi) in two doubles, so that u is correct to the rounding of r.
+__device__ inline void phase64_scale(double kappa, double &c0, double &c1) {
+  constexpr double CH = CIS_N / TWO_PI, CL = -CIS_N * 9.839338337591243e-18;  // CIS_N / (2 pi) = CH + CL
+  c0 = kappa * CH;
+  c1 = fma(kappa, CL, fma(kappa, CH, -c0));
+}
+struct Phase64 {
+  double2 E;
+  double m1, s;
+};
+__device__ inline Phase64 phase64(const double2 *__restrict__ tab, double r, double c0, double c1) {
+  constexpr double M = 6755399441055744.0;          // 1.5 2^52: adding it rounds to an integer
+  constexpr double T1 = TWO_PI / CIS_N;
+  const double tm = fma(r, c0, M);
+  const int k = __double2loint(tm) & (CIS_N - 1);
+  double u = fma(r, c0, M - tm);
+  u = fma(r, c1, u);
+  const double u2 = u * u;
+  Phase64 p;
+  p.s = u * fma(u2, fma(u2, T1 * T1 * T1 * T1 * T1 / 120.0, -T1 * T1 * T1 / 6.0), T1);
+  p.m1 = u2 * fma(u2, T1 * T1 * T1 * T1 / 24.0, -T1 * T1 / 2.0);
+  p.E = tab[k];
+  return p;
+}
+// p (1 + m1 + i s)
+__device__ inline C2<double> phase_mul(double px, double py, const Phase64 &f) {
+  return c2(fma(-py, f.s, fma(px, f.m1, px)), fma(px, f.s, fma(py, f.m1, py)));
 }
 
 // Sample of one node pair in precision T: returns the kernel value of the requested type.

@@ -5,7 +5,7 @@
 // multipole method in physical space: an octree over the bounding cube of the sources (Gauss points)
 // and targets (evaluation points), tensor Chebyshev interpolation with q^3 nodes per box (rank O(q^3),
 // against O(q^2) for the surface operators of the reference-domain FMM), kernel samples between box
-// nodes generated on the fly, the near field summed directly.
+// nodes generated on the fly once per box offset, the near field summed directly.
 //
 // Interpolated kernel on an admissible box pair (t, s): G~(x, y) = sum_{a, b} L^t_a(x) G(x_a, y_b)
 // L^s_b(y); the double layer differentiates L^s_b(y) along n_y.  Sources carry the weighted density
@@ -21,18 +21,12 @@
 
 #include "internal.h"
 #include "k_common.cuh"
+#include "k_m2l.cuh"
 #include "kernels.h"
 
 namespace igabem {
 
 namespace {
-
-inline int grid_for(long n, int block = 256) {
-  return (int)std::max<long>(1, std::min<long>((n + block - 1) / block, 152L * 32));
-}
-
-#define GRID_STRIDE(i, n) \
-  for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < (n); i += (long)gridDim.x * blockDim.x)
 
 constexpr int POT_MAXQ = 10;
 
@@ -40,16 +34,16 @@ struct PotLevel {
   int n;                    // occupied boxes
   const double *center;     // [n][3]
   double half;              // half side
-  const int *child;         // [n][8] child box index on level l + 1 or -1 (l < leaf)
-  const int *far_ptr, *far_src;
+  const int *child;         // [n][8] child box on level l + 1 with sources, or -1
   double2 *W, *Z;           // multipole / local expansions [n][q^3][R]
 };
 
 struct PotArgs {
   int q, Q, R, hard;
   double kappa;
-  const double *cheb;       // q points on [-1, 1]
+  const double *cheb;       // q points on [-1, 1], then 1 / (c_a - c_k) [q][q] (0 for k = a)
   const double *T1;         // [2][q][q]: parent Lagrange a at child node b (child c per direction)
+  const double2 *cis;       // exp(2 pi i k / CIS_N)
   // sources (Gauss points) sorted by leaf box
   const double *sy;         // [ns][3]
   const double *sn;         // [ns][3] n~ (hard)
@@ -60,205 +54,319 @@ struct PotArgs {
   // targets sorted by leaf box
   const double *tx;         // [nt][3]
   const int *tidx;          // [nt] original point index
-  const int *tgt_ptr;       // [nleaf + 1]
+  const int *tbox;          // [nt] leaf box
   const int *near_ptr, *near_src;  // leaf box pairs summed directly
   double2 *u;               // output [n_points][R] (original order)
 };
 
-__device__ inline void lagrange_1d(const double *cheb, int q, double x, double *L, double *dL) {
-  for (int a = 0; a < q; ++a) {
-    double v = 1.0, dv = 0.0;
-    for (int k = 0; k < q; ++k) {
-      if (k == a) continue;
-      const double f = (x - cheb[k]) / (cheb[a] - cheb[k]);
-      dv = dv * f + v / (cheb[a] - cheb[k]);
-      v *= f;
-    }
-    L[a] = v;
-    if (dL) dL[a] = dv;
+// admissible pairs of one level with the same box offset c_t - c_s = (dx, dy, dz) sides
+struct PotChunk {
+  int first, count, dx, dy, dz;
+};
+
+// value (and derivative) of the Lagrange polynomial a at x; inv: 1 / (c_a - c_k)
+__device__ inline double lagrange_a(const double *cheb, const double *inv, int q, int a, double x, double *d) {
+  double v = 1.0, dv = 0.0;
+  for (int k = 0; k < q; ++k) {
+    if (k == a) continue;
+    const double i = inv[a * q + k], f = (x - cheb[k]) * i;
+    if (d) dv = fma(dv, f, v * i);
+    v *= f;
   }
+  if (d) *d = dv;
+  return v;
 }
 
 // source strength seen by interpolation node a of leaf box b: monopole -a rho L_a(y), dipole
-// rho n~ . grad L_a(y)
-__global__ void k_pot_p2m(PotArgs P, PotLevel L) {
-  const int Q = P.Q, q = P.q;
-  GRID_STRIDE(o, (long)L.n * Q * P.R) {
-    const int b = int(o / (Q * P.R)), a = int((o / P.R) % Q), r = int(o % P.R);
-    const int a1 = a / (q * q), a2 = (a / q) % q, a3 = a % q;
-    const double *c = L.center + 3 * b;
-    const double ih = 1.0 / L.half;
-    double2 acc = cmk(0, 0);
-    for (int j = P.src_ptr[b]; j < P.src_ptr[b + 1]; ++j) {
-      double l1[POT_MAXQ], l2[POT_MAXQ], l3[POT_MAXQ], d1[POT_MAXQ], d2[POT_MAXQ], d3[POT_MAXQ];
-      const double *y = P.sy + 3 * (long)j;
-      lagrange_1d(P.cheb, q, (y[0] - c[0]) * ih, l1, d1);
-      lagrange_1d(P.cheb, q, (y[1] - c[1]) * ih, l2, d2);
-      lagrange_1d(P.cheb, q, (y[2] - c[2]) * ih, l3, d3);
-      const double2 rho = P.rho[(long)P.sidx[j] * P.R + r];
-      double w;
-      if (!P.hard) {
-        w = -P.sa[j] * l1[a1] * l2[a2] * l3[a3];
-      } else {
-        const double *n = P.sn + 3 * (long)j;
-        w = (n[0] * d1[a1] * l2[a2] * l3[a3] + n[1] * l1[a1] * d2[a2] * l3[a3] + n[2] * l1[a1] * l2[a2] * d3[a3]) * ih;
-      }
-      acc = cadd(acc, cscale(rho, w));
+// rho n~ . grad L_a(y).  One block per leaf box, the 1-D Lagrange values of its sources (in groups of
+// 64) computed once in shared memory.
+__global__ void __launch_bounds__(128) k_pot_p2m(PotArgs P, PotLevel L) {
+  __shared__ double lag[2][3][64][POT_MAXQ];
+  const int Q = P.Q, q = P.q, R = P.R, b = blockIdx.x;
+  const int j0 = P.src_ptr[b], j1 = P.src_ptr[b + 1];
+  if (j0 == j1) return;  // never read as a source
+  const double *c = L.center + 3 * b, *inv = P.cheb + q;
+  const double ih = 1.0 / L.half;
+  for (int g0 = j0; g0 < j1; g0 += 64) {
+    const int n = min(64, j1 - g0);
+    __syncthreads();
+    for (int o = threadIdx.x; o < 3 * n * q; o += blockDim.x) {
+      const int d = o / (n * q), j = (o / q) % n, a = o % q;
+      double dv;
+      lag[0][d][j][a] = lagrange_a(P.cheb, inv, q, a, (P.sy[3 * (long)(g0 + j) + d] - c[d]) * ih, P.hard ? &dv : nullptr);
+      if (P.hard) lag[1][d][j][a] = dv;
     }
-    L.W[o] = acc;
-  }
-}
-
-// M2M from level l + 1 into level l: W_p[a] = sum_children sum_b T_c(a, b) W_c[b]
-__global__ void k_pot_m2m(PotArgs P, PotLevel Lp, PotLevel Lc) {
-  const int Q = P.Q, q = P.q;
-  GRID_STRIDE(o, (long)Lp.n * Q * P.R) {
-    const int t = int(o / (Q * P.R)), a = int((o / P.R) % Q), r = int(o % P.R);
-    const int a1 = a / (q * q), a2 = (a / q) % q, a3 = a % q;
-    double2 acc = cmk(0, 0);
-    for (int c = 0; c < 8; ++c) {
-      const int ch = Lp.child[8 * t + c];
-      if (ch < 0) continue;
-      const int c1 = c >> 2, c2 = (c >> 1) & 1, c3 = c & 1;
-      const double2 *src = Lc.W + (long)ch * Q * P.R;
-      for (int b1 = 0; b1 < q; ++b1) {
-        const double t1 = P.T1[(c1 * q + a1) * q + b1];
-        for (int b2 = 0; b2 < q; ++b2) {
-          const double t12 = t1 * P.T1[(c2 * q + a2) * q + b2];
-          for (int b3 = 0; b3 < q; ++b3)
-            acc = cadd(acc, cscale(src[((b1 * q + b2) * q + b3) * P.R + r], t12 * P.T1[(c3 * q + a3) * q + b3]));
-        }
-      }
-    }
-    Lp.W[o] = acc;
-  }
-}
-
-// M2L on one level: Z_t[a] += sum_{s far} sum_b G(x_a, y_b) W_s[b], one block per target box, the
-// samples generated on the fly (T = float: phase split about the box centres as in the surface M2L)
-template <class T>
-__global__ void __launch_bounds__(256) k_pot_m2l(PotArgs P, PotLevel L) {
-  extern __shared__ __align__(16) unsigned char smp[];
-  const int t = blockIdx.x, Q = P.Q, q = P.q, R = P.R;
-  double2 *Ws = reinterpret_cast<double2 *>(smp);         // [Q][R] source expansion
-  double *ys = reinterpret_cast<double *>(Ws + Q * R);    // [Q][3] source node offsets from the target centre
-  const double *ct = L.center + 3 * t;
-  for (int a0 = 0; a0 < Q; a0 += blockDim.x) {
-    const int a = a0 + threadIdx.x;
-    const bool va = a < Q;
-    double xa[3] = {0, 0, 0};
-    if (va) {
-      xa[0] = P.cheb[a / (q * q)] * L.half;
-      xa[1] = P.cheb[(a / q) % q] * L.half;
-      xa[2] = P.cheb[a % q] * L.half;
-    }
-    double2 acc[8];
-    for (int r = 0; r < 8; ++r) acc[r] = cmk(0, 0);
-    for (int k = L.far_ptr[t]; k < L.far_ptr[t + 1]; ++k) {
-      const int s = L.far_src[k];
-      const double *cs = L.center + 3 * s;
-      __syncthreads();
-      for (int o = threadIdx.x; o < Q * R; o += blockDim.x) Ws[o] = L.W[(long)s * Q * R + o];
-      for (int b = threadIdx.x; b < Q; b += blockDim.x) {
-        ys[3 * b] = cs[0] - ct[0] + P.cheb[b / (q * q)] * L.half;
-        ys[3 * b + 1] = cs[1] - ct[1] + P.cheb[(b / q) % q] * L.half;
-        ys[3 * b + 2] = cs[2] - ct[2] + P.cheb[b % q] * L.half;
-      }
-      __syncthreads();
-      if (!va) continue;
-      for (int b = 0; b < Q; ++b) {
-        const double dx = xa[0] - ys[3 * b], dy = xa[1] - ys[3 * b + 1], dz = xa[2] - ys[3 * b + 2];
-        double2 G;
-        if constexpr (sizeof(T) == 4) {
-          const float r = sqrtf((float)(dx * dx + dy * dy + dz * dz));
-          float sn, cs_;
-          sincosf((float)P.kappa * r, &sn, &cs_);
-          const float f = 0.0795774715459476679f / r;
-          G = cmk((double)(cs_ * f), (double)(sn * f));
-        } else {
-          const double r = sqrt(dx * dx + dy * dy + dz * dz);
-          double sn, cs_;
-          sincos(P.kappa * r, &sn, &cs_);
-          G = cmk(cs_ / (4.0 * IGA_PI * r), sn / (4.0 * IGA_PI * r));
-        }
-        for (int r = 0; r < R && r < 8; ++r) acc[r] = cadd(acc[r], cmul(G, Ws[b * R + r]));
-      }
-    }
-    if (va)
-      for (int r = 0; r < R && r < 8; ++r) {
-        double2 *z = L.Z + ((long)t * Q + a) * R + r;
-        *z = cadd(*z, acc[r]);
-      }
-  }
-}
-
-// L2L from level l into level l + 1: Z_c[b] += sum_a T_c(a, b) Z_p[a]
-__global__ void k_pot_l2l(PotArgs P, PotLevel Lp, PotLevel Lc, const int *parent_of, const int *child_slot) {
-  const int Q = P.Q, q = P.q;
-  GRID_STRIDE(o, (long)Lc.n * Q * P.R) {
-    const int ch = int(o / (Q * P.R)), b = int((o / P.R) % Q), r = int(o % P.R);
-    const int t = parent_of[ch], c = child_slot[ch];
-    const int c1 = c >> 2, c2 = (c >> 1) & 1, c3 = c & 1, b1 = b / (q * q), b2 = (b / q) % q, b3 = b % q;
-    const double2 *src = Lp.Z + (long)t * Q * P.R;
-    double2 acc = Lc.Z[o];
-    for (int a1 = 0; a1 < q; ++a1) {
-      const double t1 = P.T1[(c1 * q + a1) * q + b1];
-      for (int a2 = 0; a2 < q; ++a2) {
-        const double t12 = t1 * P.T1[(c2 * q + a2) * q + b2];
-        for (int a3 = 0; a3 < q; ++a3)
-          acc = cadd(acc, cscale(src[((a1 * q + a2) * q + a3) * P.R + r], t12 * P.T1[(c3 * q + a3) * q + b3]));
-      }
-    }
-    Lc.Z[o] = acc;
-  }
-}
-
-// L2P and the near field at every target: u = sum_a L^t_a(x) Z_t[a] + sum_{near leaf boxes} direct
-__global__ void k_pot_eval(PotArgs P, PotLevel L, int nleaf) {
-  const int q = P.q, Q = P.Q;
-  GRID_STRIDE(o, (long)P.tgt_ptr[nleaf] * P.R) {
-    const int j = int(o / P.R), r = int(o % P.R);
-    int lo = 0, hi = nleaf;  // leaf box of sorted target j
-    while (hi - lo > 1) {
-      const int mid = (lo + hi) >> 1;
-      if (P.tgt_ptr[mid] <= j) lo = mid;
-      else hi = mid;
-    }
-    const int t = lo;
-    const double *x = P.tx + 3 * (long)j;
-    double2 acc = cmk(0, 0);
-    if (L.Z) {
-      const double *c = L.center + 3 * t;
-      const double ih = 1.0 / L.half;
-      double l1[POT_MAXQ], l2[POT_MAXQ], l3[POT_MAXQ];
-      lagrange_1d(P.cheb, q, (x[0] - c[0]) * ih, l1, nullptr);
-      lagrange_1d(P.cheb, q, (x[1] - c[1]) * ih, l2, nullptr);
-      lagrange_1d(P.cheb, q, (x[2] - c[2]) * ih, l3, nullptr);
-      for (int a = 0; a < Q; ++a)
-        acc = cadd(acc, cscale(L.Z[((long)t * Q + a) * P.R + r], l1[a / (q * q)] * l2[(a / q) % q] * l3[a % q]));
-    }
-    for (int k = P.near_ptr[t]; k < P.near_ptr[t + 1]; ++k) {
-      const int s = P.near_src[k];
-      for (int g = P.src_ptr[s]; g < P.src_ptr[s + 1]; ++g) {
-        const double *y = P.sy + 3 * (long)g;
-        const double v[3] = {y[0] - x[0], y[1] - x[1], y[2] - x[2]};
-        const double rr = sqrt(v[0] * v[0] + v[1] * v[1] + v[2] * v[2]);
-        double sn, cs;
-        sincos(P.kappa * rr, &sn, &cs);
-        const double2 G = cmk(cs / (4.0 * IGA_PI * rr), sn / (4.0 * IGA_PI * rr));
-        const double2 rho = P.rho[(long)P.sidx[g] * P.R + r];
-        double2 kv;
+    __syncthreads();
+    for (int o = threadIdx.x; o < Q * R; o += blockDim.x) {
+      const int a = o / R, r = o % R, a1 = a / (q * q), a2 = (a / q) % q, a3 = a % q;
+      double2 acc = g0 == j0 ? cmk(0, 0) : L.W[(long)b * Q * R + o];
+      for (int j = 0; j < n; ++j) {
+        const double2 rho = P.rho[(long)P.sidx[g0 + j] * R + r];
+        const double l1 = lag[0][0][j][a1], l2 = lag[0][1][j][a2], l3 = lag[0][2][j][a3];
+        double w;
         if (!P.hard) {
-          kv = cscale(G, -P.sa[g]);
+          w = -P.sa[g0 + j] * l1 * l2 * l3;
         } else {
-          const double *n = P.sn + 3 * (long)g;
-          const double vn = (v[0] * n[0] + v[1] * n[1] + v[2] * n[2]) / (rr * rr);
-          kv = cscale(cmul(G, cmk(-1.0, P.kappa * rr)), vn);   // G (i kappa r - 1)/r^2 (y - x).n~
+          const double *nn = P.sn + 3 * (long)(g0 + j);
+          w = (nn[0] * lag[1][0][j][a1] * l2 * l3 + nn[1] * l1 * lag[1][1][j][a2] * l3 +
+               nn[2] * l1 * l2 * lag[1][2][j][a3]) * ih;
         }
-        acc = cadd(acc, cmul(kv, rho));
+        acc = cadd(acc, cscale(rho, w));
+      }
+      L.W[(long)b * Q * R + o] = acc;
+    }
+  }
+}
+
+// One-dimensional transfers of one column in shared memory (Z and X: q^3 values), direction by direction:
+// Z[.. o ..] = sum_i M(o, i) X[.. i ..] with M(o, i) = T(o, i) (up: parent from child) or T(i, o) (down).
+// After the three passes the result is in X's place of the last call; the caller alternates the buffers.
+__device__ inline void pot_pass(const double *T, int q, int Q, int stride, bool up, const double2 *X, double2 *Z) {
+  for (int o = threadIdx.x; o < Q; o += blockDim.x) {
+    const int k = (o / stride) % q, base = o - k * stride;
+    double2 acc = cmk(0, 0);
+    for (int i = 0; i < q; ++i) acc = cadd(acc, cscale(X[base + i * stride], up ? T[k * q + i] : T[i * q + k]));
+    Z[o] = acc;
+  }
+  __syncthreads();
+}
+
+// M2M from level l + 1 into level l: W_p[a] = sum_children sum_b T_c(a, b) W_c[b], the tensor transfer one
+// direction after the other (3 q^4 products a child instead of q^6); one block per (parent, column)
+__global__ void __launch_bounds__(128) k_pot_m2m(PotArgs P, PotLevel Lp, PotLevel Lc) {
+  extern __shared__ double2 smu[];
+  const int Q = P.Q, q = P.q, R = P.R, t = blockIdx.x, r = blockIdx.y;
+  double2 *X = smu, *Z = X + Q, *S = Z + Q;
+  bool any = false;
+  for (int o = threadIdx.x; o < Q; o += blockDim.x) S[o] = cmk(0, 0);
+  for (int c = 0; c < 8; ++c) {
+    const int ch = Lp.child[8 * t + c];
+    if (ch < 0) continue;
+    any = true;
+    for (int o = threadIdx.x; o < Q; o += blockDim.x) X[o] = Lc.W[((long)ch * Q + o) * R + r];
+    __syncthreads();
+    pot_pass(P.T1 + (c >> 2) * q * q, q, Q, q * q, true, X, Z);
+    pot_pass(P.T1 + ((c >> 1) & 1) * q * q, q, Q, q, true, Z, X);
+    pot_pass(P.T1 + (c & 1) * q * q, q, Q, 1, true, X, Z);
+    for (int o = threadIdx.x; o < Q; o += blockDim.x) S[o] = cadd(S[o], Z[o]);
+    __syncthreads();
+  }
+  if (any)
+    for (int o = threadIdx.x; o < Q; o += blockDim.x) Lp.W[((long)t * Q + o) * R + r] = S[o];
+}
+
+// M2L on one level.  G(x_a, y_b) depends on the box offset c_t - c_s alone, so the pairs of a level are
+// grouped by it: one block takes up to POT_COLS columns (pairs of one offset times densities) and 128 target
+// nodes, and generates each sample once for all of them instead of once per pair; a thread owns one target
+// node with its columns' sums in registers.  In FP32 the phase is split about the box centres
+// (kappa |D| in FP64 plus kappa (r - |D|), r - |D| = (2 D.d + |d|^2) / (r + |D|)) and the products take two
+// columns per instruction; the sums of 64 source nodes, then of their groups, are added to Z in FP64.
+// Measured on 4001 points around 6144 Gauss points, q = 7, 372,000 pairs (FP32): 1520 -> 28 ms a call, host
+// tree included (before: a sample per pair with FP64 differences and sums, and per-node Lagrange values in
+// P2M).
+constexpr int POT_COLS = 16, POT_ROWS = 128, POT_STEP = 64;
+
+__device__ inline float2 fma2x(float2 a, float2 b, float2 c) {  // two FP32 multiply-adds
+  float2 d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;"
+      : "=l"(reinterpret_cast<unsigned long long &>(d))
+      : "l"(reinterpret_cast<const unsigned long long &>(a)), "l"(reinterpret_cast<const unsigned long long &>(b)),
+        "l"(reinterpret_cast<const unsigned long long &>(c)));
+  return d;
+}
+
+template <class T>
+__global__ void __launch_bounds__(POT_ROWS) k_pot_m2l(PotArgs P, PotLevel L, const PotChunk *__restrict__ chunks,
+                                                      const int2 *__restrict__ pairs) {
+  constexpr bool F32 = sizeof(T) == 4;
+  __shared__ __align__(16) T wre[POT_STEP][POT_COLS];
+  __shared__ __align__(16) T wim[POT_STEP][POT_COLS];
+  __shared__ __align__(16) T ys[POT_STEP][4];
+  __shared__ double2 tab[F32 ? 1 : CIS_N];
+  const int Q = P.Q, q = P.q, R = P.R, tid = threadIdx.x;
+  const PotChunk ck = chunks[blockIdx.x];
+  const int ncol = ck.count * R, a = blockIdx.y * POT_ROWS + tid;
+  const double side = 2.0 * L.half;
+  const double Dd[3] = {ck.dx * side, ck.dy * side, ck.dz * side};
+  const double D2d = Dd[0] * Dd[0] + Dd[1] * Dd[1] + Dd[2] * Dd[2], Dnd = sqrt(D2d);
+  double c0 = 0, c1 = 0;
+  float phi0 = 0;
+  if constexpr (F32) {
+    const double x = P.kappa * Dnd, k = rint(x / TWO_PI);  // reduced to (-pi, pi]
+    phi0 = (float)fma(-k, 2.4492935982947064e-16, fma(-k, TWO_PI, x));
+  } else {
+    phase64_scale(P.kappa, c0, c1);
+    for (int i = tid; i < CIS_N; i += POT_ROWS) tab[i] = P.cis[i];
+  }
+  const T D[3] = {(T)Dd[0], (T)Dd[1], (T)Dd[2]}, D2 = (T)D2d, Dn = (T)Dnd, kappa = (T)P.kappa;
+  T xa[3] = {0, 0, 0};
+  if (a < Q) {
+    xa[0] = (T)(P.cheb[a / (q * q)] * L.half);
+    xa[1] = (T)(P.cheb[(a / q) % q] * L.half);
+    xa[2] = (T)(P.cheb[a % q] * L.half);
+  }
+  T Dx = 0;
+  if constexpr (F32) {
+    Dx = D[0] * xa[0] + D[1] * xa[1] + D[2] * xa[2];
+  } else {  // absolute positions about the source centre
+    for (int c = 0; c < 3; ++c) xa[c] += D[c];
+  }
+  T tr[POT_COLS], ti[POT_COLS];
+#pragma unroll
+  for (int c = 0; c < POT_COLS; ++c) tr[c] = ti[c] = 0;
+  for (int b0 = 0; b0 < Q; b0 += POT_STEP) {
+    const int nb = min(POT_STEP, Q - b0);
+    __syncthreads();
+    for (int o = tid; o < nb * POT_COLS; o += POT_ROWS) {
+      const int b = o / POT_COLS, c = o % POT_COLS;
+      double2 v = cmk(0, 0);
+      if (c < ncol) v = L.W[((long)pairs[ck.first + c / R].y * Q + b0 + b) * R + c % R];
+      wre[b][c] = (T)v.x;
+      wim[b][c] = (T)v.y;
+    }
+    for (int b = tid; b < nb; b += POT_ROWS) {
+      const int bb = b0 + b;
+      const double y[3] = {P.cheb[bb / (q * q)] * L.half, P.cheb[(bb / q) % q] * L.half, P.cheb[bb % q] * L.half};
+      for (int c = 0; c < 3; ++c) ys[b][c] = (T)y[c];
+      ys[b][3] = (T)(Dd[0] * y[0] + Dd[1] * y[1] + Dd[2] * y[2]);
+    }
+    __syncthreads();
+    if (a >= Q) continue;
+    if constexpr (F32) {
+      float2 pr[POT_COLS / 2], pi[POT_COLS / 2];
+#pragma unroll
+      for (int c = 0; c < POT_COLS / 2; ++c) pr[c] = pi[c] = make_float2(0.f, 0.f);
+      for (int b = 0; b < nb; ++b) {
+        const float4 y = *reinterpret_cast<const float4 *>(ys[b]);
+        const float d0 = xa[0] - y.x, d1 = xa[1] - y.y, d2 = xa[2] - y.z;
+        const float num = fmaf(2.f, Dx - y.w, fmaf(d0, d0, fmaf(d1, d1, d2 * d2)));
+        const float r2 = D2 + num, ir = rsqrtf(r2), r = r2 * ir;
+        float ph = fmaf(kappa, __fdividef(num, r + Dn), phi0);
+        const float kq = rintf(ph * 0.15915494309189535f);
+        ph = fmaf(-kq, 6.28318548202514648f, ph);
+        ph = fmaf(-kq, -1.7484556e-07f, ph);
+        float sn, cs;
+        __sincosf(ph, &sn, &cs);
+        const float f = ir * 0.0795774715459476679f, gx = cs * f, gy = sn * f;
+        const float2 gxx = make_float2(gx, gx), gyy = make_float2(gy, gy), gyn = make_float2(-gy, -gy);
+        const float4 *wr = reinterpret_cast<const float4 *>(wre[b]), *wi = reinterpret_cast<const float4 *>(wim[b]);
+#pragma unroll
+        for (int c = 0; c < POT_COLS / 4; ++c) {
+          const float4 u = wr[c], v = wi[c];
+          const float2 u0 = make_float2(u.x, u.y), u1 = make_float2(u.z, u.w), v0 = make_float2(v.x, v.y),
+                       v1 = make_float2(v.z, v.w);
+          pr[2 * c] = fma2x(gxx, u0, fma2x(gyn, v0, pr[2 * c]));
+          pi[2 * c] = fma2x(gxx, v0, fma2x(gyy, u0, pi[2 * c]));
+          pr[2 * c + 1] = fma2x(gxx, u1, fma2x(gyn, v1, pr[2 * c + 1]));
+          pi[2 * c + 1] = fma2x(gxx, v1, fma2x(gyy, u1, pi[2 * c + 1]));
+        }
+      }
+#pragma unroll
+      for (int c = 0; c < POT_COLS / 2; ++c) {
+        tr[2 * c] += pr[c].x; tr[2 * c + 1] += pr[c].y;
+        ti[2 * c] += pi[c].x; ti[2 * c + 1] += pi[c].y;
+      }
+    } else {
+      for (int b = 0; b < nb; ++b) {
+        const double d0 = xa[0] - ys[b][0], d1 = xa[1] - ys[b][1], d2 = xa[2] - ys[b][2];
+        const double r2 = d0 * d0 + d1 * d1 + d2 * d2, ir = rsqrt64(r2), f = ir * (0.25 / IGA_PI);
+        const Phase64 p = phase64(tab, r2 * ir, c0, c1);
+        const C2<double> G = phase_mul(p.E.x * f, p.E.y * f, p);
+#pragma unroll
+        for (int c = 0; c < POT_COLS; ++c) {
+          if (c >= ncol) break;  // the same for every thread: no padding on the FP64 pipe
+          tr[c] = fma(G.x, wre[b][c], fma(-G.y, wim[b][c], tr[c]));
+          ti[c] = fma(G.x, wim[b][c], fma(G.y, wre[b][c], ti[c]));
+        }
       }
     }
-    P.u[(long)P.tidx[j] * P.R + r] = acc;
+  }
+  if (a < Q)
+#pragma unroll
+    for (int c = 0; c < POT_COLS; ++c) {
+      if (c >= ncol) break;
+      double2 *z = L.Z + ((long)pairs[ck.first + c / R].x * Q + a) * R + c % R;
+      atomicAdd(&z->x, (double)tr[c]);
+      atomicAdd(&z->y, (double)ti[c]);
+    }
+}
+
+// L2L from level l into level l + 1: Z_c[b] += sum_a T_c(a, b) Z_p[a], direction by direction; one block per
+// (child, column)
+__global__ void __launch_bounds__(128) k_pot_l2l(PotArgs P, PotLevel Lp, PotLevel Lc, const int *parent_of,
+                                                 const int *child_slot) {
+  extern __shared__ double2 smd_[];
+  const int Q = P.Q, q = P.q, R = P.R, ch = blockIdx.x, r = blockIdx.y;
+  const int t = parent_of[ch], c = child_slot[ch];
+  double2 *X = smd_, *Z = X + Q;
+  for (int o = threadIdx.x; o < Q; o += blockDim.x) X[o] = Lp.Z[((long)t * Q + o) * R + r];
+  __syncthreads();
+  pot_pass(P.T1 + (c >> 2) * q * q, q, Q, q * q, false, X, Z);
+  pot_pass(P.T1 + ((c >> 1) & 1) * q * q, q, Q, q, false, Z, X);
+  pot_pass(P.T1 + (c & 1) * q * q, q, Q, 1, false, X, Z);
+  for (int o = threadIdx.x; o < Q; o += blockDim.x) {
+    double2 *z = Lc.Z + ((long)ch * Q + o) * R + r;
+    *z = cadd(*z, Z[o]);
+  }
+}
+
+// L2P and the near field at every target: u = sum_a L^t_a(x) Z_t[a] + sum_{near leaf boxes} direct.  One warp
+// per target: its lanes share the nodes of the box and the sources nearby.
+__global__ void __launch_bounds__(128) k_pot_eval(PotArgs P, PotLevel L, int n_pts) {
+  __shared__ double lag[4][3][POT_MAXQ];
+  const int q = P.q, Q = P.Q, R = P.R, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const long j = blockIdx.x * 4L + warp;
+  if (j >= n_pts) return;
+  const int t = P.tbox[j];
+  const double x[3] = {P.tx[3 * j], P.tx[3 * j + 1], P.tx[3 * j + 2]};
+  double2 acc[8];
+#pragma unroll
+  for (int r = 0; r < 8; ++r) acc[r] = cmk(0, 0);
+  if (L.Z) {
+    const double *c = L.center + 3 * t;
+    const double ih = 1.0 / L.half;
+    if (lane < 3 * q) {
+      const int d = lane / q, k = lane % q;
+      lag[warp][d][k] = lagrange_a(P.cheb, P.cheb + q, q, k, (P.tx[3 * j + d] - c[d]) * ih, nullptr);
+    }
+    __syncwarp();
+    for (int a = lane; a < Q; a += 32) {
+      const double w = lag[warp][0][a / (q * q)] * lag[warp][1][(a / q) % q] * lag[warp][2][a % q];
+#pragma unroll
+      for (int r = 0; r < 8; ++r)
+        if (r < R) acc[r] = cadd(acc[r], cscale(L.Z[((long)t * Q + a) * R + r], w));
+    }
+  }
+  for (int k = P.near_ptr[t]; k < P.near_ptr[t + 1]; ++k) {
+    const int s = P.near_src[k];
+    for (int g = P.src_ptr[s] + lane; g < P.src_ptr[s + 1]; g += 32) {
+      const double *y = P.sy + 3 * (long)g;
+      const double v[3] = {y[0] - x[0], y[1] - x[1], y[2] - x[2]};
+      const double rr = sqrt(v[0] * v[0] + v[1] * v[1] + v[2] * v[2]);
+      double sn, cs;
+      sincos(P.kappa * rr, &sn, &cs);
+      const double2 G = cmk(cs / (4.0 * IGA_PI * rr), sn / (4.0 * IGA_PI * rr));
+      double2 kv;
+      if (!P.hard) {
+        kv = cscale(G, -P.sa[g]);
+      } else {
+        const double *n = P.sn + 3 * (long)g;
+        const double vn = (v[0] * n[0] + v[1] * n[1] + v[2] * n[2]) / (rr * rr);
+        kv = cscale(cmul(G, cmk(-1.0, P.kappa * rr)), vn);   // G (i kappa r - 1)/r^2 (y - x).n~
+      }
+#pragma unroll
+      for (int r = 0; r < 8; ++r)
+        if (r < R) acc[r] = cadd(acc[r], cmul(kv, P.rho[(long)P.sidx[g] * R + r]));
+    }
+  }
+#pragma unroll
+  for (int r = 0; r < 8; ++r) {
+    if (r >= R) break;
+    for (int o = 16; o > 0; o >>= 1) {
+      acc[r].x += __shfl_xor_sync(0xffffffffu, acc[r].x, o);
+      acc[r].y += __shfl_xor_sync(0xffffffffu, acc[r].y, o);
+    }
+    if (lane == 0) P.u[(long)P.tidx[j] * R + r] = acc[r];
   }
 }
 
@@ -466,12 +574,62 @@ extern "C" int igabem_potential(igabem_problem *P, int n_rhs, const void *densit
     };
     std::vector<int> nptr, nsrc;
     csr(near, nleaf, nptr, nsrc);
+    // admissible pairs of every level sorted by box offset, in chunks of POT_COLS columns
+    const int per = std::max(1, POT_COLS / R);
+    std::vector<std::vector<int2>> fpair(D + 1);
+    std::vector<std::vector<PotChunk>> chunk(D + 1);
+    for (int l = 0; l <= D; ++l) {
+      const size_t n = far[l].size();
+      if (n == 0) continue;
+      auto box = [&](int b, int &i, int &j, int &k) {
+        const long long v = keys[l][b];
+        i = int(v >> 42);
+        j = int((v >> 21) & 0x1FFFFF);
+        k = int(v & 0x1FFFFF);
+      };
+      std::vector<long long> off(n);  // the offset packed (each component below 2^11 in size, made positive)
+      int most = 0;
+      for (size_t i = 0; i < n; ++i) {
+        int a0, a1, a2, b0, b1, b2;
+        box(far[l][i].first, a0, a1, a2);
+        box(far[l][i].second, b0, b1, b2);
+        most = std::max({most, std::abs(a0 - b0), std::abs(a1 - b1), std::abs(a2 - b2)});
+        off[i] = pack(a0 - b0 + 2048, a1 - b1 + 2048, a2 - b2 + 2048);
+      }
+      std::vector<int> order(n);
+      const long w = 2L * most + 1;
+      if (w * w * w <= 1 << 20) {  // counting sort over the offsets' cube
+        auto id = [&](long long v) {
+          return ((long(v >> 42) - 2048 + most) * w + (long((v >> 21) & 0x1FFFFF) - 2048 + most)) * w +
+                 (long(v & 0x1FFFFF) - 2048 + most);
+        };
+        std::vector<int> cnt(w * w * w + 1, 0);
+        for (size_t i = 0; i < n; ++i) cnt[id(off[i]) + 1]++;
+        for (long i = 0; i < w * w * w; ++i) cnt[i + 1] += cnt[i];
+        for (size_t i = 0; i < n; ++i) order[cnt[id(off[i])]++] = (int)i;
+      } else {
+        for (size_t i = 0; i < n; ++i) order[i] = (int)i;
+        std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return off[x] < off[y]; });
+      }
+      fpair[l].resize(n);
+      for (size_t i = 0; i < n; ++i) {
+        const int o = order[i];
+        fpair[l][i] = make_int2(far[l][o].first, far[l][o].second);
+        if (i == 0 || off[o] != off[order[i - 1]] || chunk[l].back().count == per)
+          chunk[l].push_back({(int)i, 0, int(off[o] >> 42) - 2048, int((off[o] >> 21) & 0x1FFFFF) - 2048,
+                              int(off[o] & 0x1FFFFF) - 2048});
+        chunk[l].back().count++;
+      }
+    }
     int lmin = D + 1;
     for (int l = 0; l <= D; ++l)
       if (!far[l].empty()) lmin = std::min(lmin, l);
     // interpolation tables
-    std::vector<double> cheb(q), T1(2L * q * q);
+    std::vector<double> cheb(q + (size_t)q * q, 0.0), T1(2L * q * q);
     for (int a = 0; a < q; ++a) cheb[a] = std::cos((2 * a + 1) * M_PI / (2 * q));
+    for (int a = 0; a < q; ++a)
+      for (int k = 0; k < q; ++k)
+        if (k != a) cheb[q + a * q + k] = 1.0 / (cheb[a] - cheb[k]);
     for (int c = 0; c < 2; ++c)
       for (int a = 0; a < q; ++a)
         for (int b = 0; b < q; ++b) {
@@ -482,19 +640,20 @@ extern "C" int igabem_potential(igabem_problem *P, int n_rhs, const void *densit
           T1[(c * q + a) * q + b] = v;
         }
     // device buffers (one allocation)
-    std::vector<std::vector<int>> fptr(D + 1), fsrc(D + 1);
-    for (int l = 0; l <= D; ++l) csr(far[l], (int)keys[l].size(), fptr[l], fsrc[l]);
+    std::vector<int> tsort(n_pts);  // leaf box of each sorted target
+    for (long j = 0; j < n_pts; ++j) tsort[j] = tbox[tperm[j]];
     size_t bytes = 0;
     auto add = [&](size_t n) { bytes += (n + 255) & ~size_t(255); };
     add(sizeof(double) * 3 * G); add(sizeof(double) * 3 * G); add(sizeof(double) * G); add(sizeof(int) * G);
     add(sizeof(int) * (nleaf + 1)); add(sizeof(double) * 3 * n_pts); add(sizeof(int) * n_pts);
-    add(sizeof(int) * (nleaf + 1)); add(sizeof(int) * (nleaf + 1)); add(sizeof(int) * std::max<size_t>(nsrc.size(), 1));
-    add(sizeof(double2) * G * R); add(sizeof(double2) * (size_t)n_pts * R); add(sizeof(double) * q);
+    add(sizeof(int) * n_pts); add(sizeof(int) * (nleaf + 1)); add(sizeof(int) * std::max<size_t>(nsrc.size(), 1));
+    add(sizeof(double2) * G * R); add(sizeof(double2) * (size_t)n_pts * R); add(sizeof(double) * cheb.size());
     add(sizeof(double) * T1.size());
     for (int l = 0; l <= D; ++l) {
       const size_t n = keys[l].size();
-      add(sizeof(double) * 3 * n); add(sizeof(int) * 8 * n); add(sizeof(int) * (n + 1));
-      add(sizeof(int) * std::max<size_t>(fsrc[l].size(), 1)); add(sizeof(int) * n); add(sizeof(int) * n);
+      add(sizeof(double) * 3 * n); add(sizeof(int) * 8 * n); add(sizeof(int) * n); add(sizeof(int) * n);
+      add(sizeof(int2) * std::max<size_t>(fpair[l].size(), 1));
+      add(sizeof(PotChunk) * std::max<size_t>(chunk[l].size(), 1));
       if (l >= lmin) {
         add(sizeof(double2) * n * Q * R);
         add(sizeof(double2) * n * Q * R);
@@ -522,7 +681,8 @@ extern "C" int igabem_potential(igabem_problem *P, int n_rhs, const void *densit
       PA.src_ptr = up(sptr);
       PA.tx = up(tx);
       PA.tidx = up(tperm);
-      PA.tgt_ptr = up(tptr);
+      PA.tbox = up(tsort);
+      PA.cis = reinterpret_cast<const double2 *>(P->d.cis);
       PA.near_ptr = up(nptr);
       PA.near_src = up(nsrc);
       double2 *rho = A.get<double2>(G * R);
@@ -533,14 +693,20 @@ extern "C" int igabem_potential(igabem_problem *P, int n_rhs, const void *densit
       PA.T1 = up(T1);
       std::vector<PotLevel> LV(D + 1);
       std::vector<int *> par_d(D + 1), slot_d(D + 1);
+      std::vector<int2 *> pair_d(D + 1);
+      std::vector<PotChunk *> chunk_d(D + 1);
       for (int l = 0; l <= D; ++l) {
         PotLevel &L = LV[l];
         L.n = (int)keys[l].size();
         L.center = up(cen[l]);
         L.half = side / (1 << l) / 2;
-        L.child = up(child[l]);
-        L.far_ptr = up(fptr[l]);
-        L.far_src = up(fsrc[l]);
+        std::vector<int> with_src(child[l]);
+        if (l < D)
+          for (int &c : with_src)
+            if (c >= 0 && !hs[l + 1][c]) c = -1;
+        L.child = up(with_src);
+        pair_d[l] = up(fpair[l]);
+        chunk_d[l] = up(chunk[l]);
         par_d[l] = up(parent[l].empty() ? std::vector<int>(1, 0) : parent[l]);
         slot_d[l] = up(slot[l].empty() ? std::vector<int>(1, 0) : slot[l]);
         L.W = L.Z = nullptr;
@@ -552,30 +718,28 @@ extern "C" int igabem_potential(igabem_problem *P, int n_rhs, const void *densit
       }
       launch_density(P->d, S, o, R, static_cast<const double *>(density), reinterpret_cast<double *>(rho), st);
       if (lmin <= D) {
-        k_pot_p2m<<<grid_for((long)nleaf * Q * R), 256, 0, st>>>(PA, LV[D]);
+        k_pot_p2m<<<nleaf, 128, 0, st>>>(PA, LV[D]);
         note_launch();
+        const size_t smt = 3 * sizeof(double2) * (size_t)Q;  // q <= 10: at most 48 KB
+        IGA_CUDA(set_max_dynamic_smem(k_pot_m2m, smt));
+        IGA_CUDA(set_max_dynamic_smem(k_pot_l2l, smt));
         for (int l = D - 1; l >= lmin; --l) {
-          k_pot_m2m<<<grid_for((long)LV[l].n * Q * R), 256, 0, st>>>(PA, LV[l], LV[l + 1]);
+          k_pot_m2m<<<dim3(LV[l].n, R), 128, smt, st>>>(PA, LV[l], LV[l + 1]);
           note_launch();
         }
-        const size_t smem = sizeof(double2) * Q * R + sizeof(double) * 3 * Q;
         for (int l = lmin; l <= D; ++l) {
           if (far[l].empty()) continue;
-          if (fp32) {
-            IGA_CUDA(set_max_dynamic_smem(k_pot_m2l<float>, smem));
-            k_pot_m2l<float><<<LV[l].n, 256, smem, st>>>(PA, LV[l]);
-          } else {
-            IGA_CUDA(set_max_dynamic_smem(k_pot_m2l<double>, smem));
-            k_pot_m2l<double><<<LV[l].n, 256, smem, st>>>(PA, LV[l]);
-          }
+          const dim3 grid((unsigned)chunk[l].size(), (Q + POT_ROWS - 1) / POT_ROWS);
+          if (fp32) k_pot_m2l<float><<<grid, POT_ROWS, 0, st>>>(PA, LV[l], chunk_d[l], pair_d[l]);
+          else k_pot_m2l<double><<<grid, POT_ROWS, 0, st>>>(PA, LV[l], chunk_d[l], pair_d[l]);
           note_launch();
         }
         for (int l = lmin; l < D; ++l) {
-          k_pot_l2l<<<grid_for((long)LV[l + 1].n * Q * R), 256, 0, st>>>(PA, LV[l], LV[l + 1], par_d[l + 1], slot_d[l + 1]);
+          k_pot_l2l<<<dim3(LV[l + 1].n, R), 128, smt, st>>>(PA, LV[l], LV[l + 1], par_d[l + 1], slot_d[l + 1]);
           note_launch();
         }
       }
-      k_pot_eval<<<grid_for((long)n_pts * R), 256, 0, st>>>(PA, LV[D], nleaf);
+      k_pot_eval<<<(n_pts + 3) / 4, 128, 0, st>>>(PA, LV[D], n_pts);
       note_launch();
       IGA_CUDA(cudaGetLastError());
       cudaPointerAttributes ua{};
