@@ -295,7 +295,7 @@ void check_status(igabem_problem *P) {
   IGA_CUDA(cudaMemcpy(&v, P->d.status, sizeof(int), cudaMemcpyDeviceToHost));
   if (v) {
     IGA_CUDA(cudaMemset(P->d.status, 0, sizeof(int)));
-    fail(IGABEM_ETIMEOUT, "a tensor-core M2L wait timed out; the result is incomplete");
+    fail(IGABEM_ETIMEOUT, "a bounded device wait timed out; the result is incomplete");
   }
 }
 

@@ -1,6 +1,6 @@
 // M2L: couplings of admissible cluster pairs (Sec. 4.4), FP64 and FP32: kernel samples between the
-// Chebyshev nodes generated on the fly (k_m2l_fly; k_m2l_gemm for many columns), or coupling blocks stored
-// at set-up (k_m2l_stored).  All levels go in one launch, each with its own q (level-adaptive
+// Chebyshev nodes generated on the fly (k_m2l_fly; k_m2l_gemm for many columns); the blocks stored at
+// set-up (m2l_stored) are generated here and applied in k_stream.cu.  All levels go in one launch, each with its own q (level-adaptive
 // interpolation), one block (or a cluster of blocks) per target cluster.
 //
 // FP32 phase split: the sample phase kappa r is formed as kappa |D| (D = c_t - c_s, the distance of
@@ -23,7 +23,6 @@ namespace igabem {
 
 namespace {
 
-constexpr int M2L_WARPS = 8;
 
 struct M2LLevel {
   const int *far_ptr, *far_src;
@@ -32,7 +31,6 @@ struct M2LLevel {
   const float *pc;       // FP32 pair constants [n_far][8]: D, |D|, |D|^2, cos, sin of kappa|D| (FP32 path)
   const double2 *xhat;
   const float2 *xhat32;  // FP32 copy of xhat (the FP32 kernels read it)
-  const void *stored;    // stored coupling blocks of the level (m2l_stored) or nullptr
   double2 *yhat;
   int n;                 // clusters on the level
   int first;             // first block index of the level in the flattened grid
@@ -277,146 +275,6 @@ __global__ void __launch_bounds__(256) k_m2l_fill(M2LLevel L, bool hard, double 
   }
 }
 
-// cp.async of one coupling-block entry (8 or 16 bytes) into shared memory; src_bytes = 0 fills zeros
-template <int BYTES>
-__device__ inline void cp_async_zfill(void *dst, const void *src, int src_bytes) {
-  const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
-  asm volatile("cp.async.ca.shared.global [%0], [%1], %2, %3;\n" ::"r"(d), "l"(src), "n"(BYTES), "r"(src_bytes)
-               : "memory");
-}
-__device__ inline void cp_async_commit_group() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-template <int N>
-__device__ inline void cp_async_wait_group() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
-
-// M2L from the stored blocks: one block per target cluster, warps over the interaction list, lane rows
-// a0 + lane and a0 + lane + 32.  The stored rows stream through a per-warp ring of D shared-memory
-// slots filled by asynchronous copies (row b + D - 1 is requested while row b is used), so that each
-// warp keeps D rows of the block in flight instead of one load per lane.
-template <class T, int NCR, bool HARD, int D>
-__global__ void __launch_bounds__(32 * M2L_WARPS) k_m2l_stored(M2LArgs A, int cr0) {
-  extern __shared__ __align__(16) unsigned char smst[];
-  constexpr bool F32 = std::is_same<T, float>::value;
-  constexpr int ntype = HARD ? 2 : 1, ES = sizeof(C2<T>);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  int li = 0;
-  while (li + 1 < A.nlev && (int)blockIdx.x >= A.lev[li + 1].first) ++li;
-  const M2LLevel &L = A.lev[li];
-  const int t = blockIdx.x - L.first;
-  const int Q = L.Q, q = L.q, QS = A.QS;
-  const int ncr = min(NCR, A.CR - cr0);
-  C2<T> *xs = reinterpret_cast<C2<T> *>(smst) + warp * QS * NCR;
-  C2<T> *ring = reinterpret_cast<C2<T> *>(smst) + M2L_WARPS * QS * NCR + warp * D * ntype * 64;
-  double2 *red = reinterpret_cast<double2 *>(smst);
-  const C2<T> *Sall = reinterpret_cast<const C2<T> *>(L.stored);
-  const C2<T> zero = c2((T)0, (T)0);
-  for (int a0 = 0; a0 < Q; a0 += 64) {
-    C2<T> tot0[NCR], tot1[NCR];
-    for (int c = 0; c < NCR; ++c) tot0[c] = tot1[c] = zero;
-    for (int kk = L.far_ptr[t] + warp; kk < L.far_ptr[t + 1]; kk += M2L_WARPS) {
-      const int s = L.far_src[kk];
-      const C2<T> *Sk = Sall + (long)kk * ntype * Q * Q;
-      // rows 0 .. D - 2 of the block requested before x_s is staged
-      auto issue = [&](int b) {
-        C2<T> *slot = ring + (b % D) * ntype * 64;
-#pragma unroll
-        for (int ty = 0; ty < ntype; ++ty) {
-          const C2<T> *src = Sk + ((long)ty * Q + b) * Q;
-#pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            const int col = a0 + lane + 32 * h;
-            const bool ok = col < Q;
-            cp_async_zfill<ES>(slot + ty * 64 + lane + 32 * h, ok ? src + col : src, ok ? ES : 0);
-          }
-        }
-      };
-      __syncwarp();  // the previous pair's reads of the ring and of x_s are done
-#pragma unroll
-      for (int i = 0; i < D - 1; ++i) {
-        if (i < Q) issue(i);
-        cp_async_commit_group();
-      }
-      for (int b = lane; b < Q; b += 32) {
-        const long ib = (long)s * Q + b;
-        for (int c = 0; c < ncr; ++c) {
-          if constexpr (F32) {
-            const float2 v = L.xhat32[ib * A.CR + cr0 + c];
-            xs[b * NCR + c] = c2((T)v.x, (T)v.y);
-          } else {
-            const double2 v = L.xhat[ib * A.CR + cr0 + c];
-            xs[b * NCR + c] = c2((T)v.x, (T)v.y);
-          }
-        }
-      }
-      for (int b1 = 0; b1 < q; ++b1) {
-        C2<T> p0[NCR], p1[NCR];
-        for (int c = 0; c < NCR; ++c) p0[c] = p1[c] = zero;
-        for (int b2 = 0; b2 < q; ++b2) {
-          const int b = b1 * q + b2;
-          cp_async_wait_group<D - 2>();  // row b has landed (this lane's copies)
-          __syncwarp();                  // ... and every lane's
-          const C2<T> *slot = ring + (b % D) * ntype * 64;
-          const C2<T> s0a = slot[lane], s0b = slot[lane + 32];
-          // the staged x_s values of row b (broadcast to the warp), two columns per 16-byte load in FP32
-          C2<T> xv[NCR];
-          if constexpr (F32 && NCR % 2 == 0) {
-            const float4 *xp = reinterpret_cast<const float4 *>(xs + b * NCR);
-#pragma unroll
-            for (int c = 0; c < NCR / 2; ++c) {
-              const float4 v = xp[c];
-              xv[2 * c] = c2((T)v.x, (T)v.y);
-              xv[2 * c + 1] = c2((T)v.z, (T)v.w);
-            }
-          } else {
-#pragma unroll
-            for (int c = 0; c < NCR; ++c) xv[c] = xs[b * NCR + c];
-          }
-          if (!HARD) {
-#pragma unroll
-            for (int c = 0; c < NCR; ++c) {
-              p0[c] = fma2(s0a, xv[c], p0[c]);
-              p1[c] = fma2(s0b, xv[c], p1[c]);
-            }
-          } else {
-            const C2<T> s1a = slot[64 + lane], s1b = slot[64 + lane + 32];
-#pragma unroll
-            for (int c = 0; c < NCR; ++c) {
-              const bool k0 = (cr0 + c) / A.R == 0;
-              p0[c] = fma2(k0 ? s0a : s1a, xv[c], p0[c]);
-              p1[c] = fma2(k0 ? s0b : s1b, xv[c], p1[c]);
-            }
-          }
-          // the slot of row b - 1 is free (every lane passed this iteration's __syncwarp)
-          if (b + D - 1 < Q) issue(b + D - 1);
-          cp_async_commit_group();
-        }
-        for (int c = 0; c < NCR; ++c) {
-          tot0[c] = add(tot0[c], p0[c]);
-          tot1[c] = add(tot1[c], p1[c]);
-        }
-      }
-      cp_async_wait_group<0>();
-    }
-    __syncthreads();
-    for (int c = 0; c < NCR; ++c) {
-      red[(warp * 64 + lane) * NCR + c] = make_double2((double)tot0[c].x, (double)tot0[c].y);
-      red[(warp * 64 + lane + 32) * NCR + c] = make_double2((double)tot1[c].x, (double)tot1[c].y);
-    }
-    __syncthreads();
-    const int na = min(64, Q - a0);
-    for (int o = threadIdx.x; o < na * ncr; o += blockDim.x) {
-      const int a = o / ncr, c = o % ncr;
-      double2 sum = make_double2(0, 0);
-      for (int w = 0; w < M2L_WARPS; ++w) {
-        const double2 v = red[(w * 64 + a) * NCR + c];
-        sum.x += v.x;
-        sum.y += v.y;
-      }
-      L.yhat[((long)t * Q + a0 + a) * A.CR + cr0 + c] = sum;
-    }
-    __syncthreads();
-  }
-}
-
 // Multi-column M2L: per target cluster and column chunk, every coupling block S_ts (q^2 x q^2) is
 // generated once into shared memory and applied to the chunk's columns of xhat_s with a register
 // tiled product (4 x 4 complex outputs per thread).  A chunk lies within one channel, so one kernel
@@ -608,34 +466,6 @@ void launch_fly_all(const M2LArgs &A, int nblocks, int nsplit, cudaStream_t st) 
   }
 }
 
-template <class T, int NCR, bool HARD, int D>
-size_t stored_smem(const M2LArgs &A) {
-  const size_t pts = (size_t)M2L_WARPS * (A.QS * NCR + D * (HARD ? 2 : 1) * 64) * sizeof(C2<T>);
-  return std::max(pts, (size_t)M2L_WARPS * 64 * NCR * sizeof(double2));
-}
-
-template <class T, int NCR, bool HARD>
-void launch_stored(const M2LArgs &A, int nblocks, cudaStream_t st) {
-  // eight rows in flight per warp where the shared memory allows, else three
-  const bool deep = stored_smem<T, NCR, HARD, 8>(A) <= 200 * 1024;
-  const size_t smem = deep ? stored_smem<T, NCR, HARD, 8>(A) : stored_smem<T, NCR, HARD, 3>(A);
-  auto kfn = deep ? k_m2l_stored<T, NCR, HARD, 8> : k_m2l_stored<T, NCR, HARD, 3>;
-  IGA_CUDA(set_max_dynamic_smem(kfn, smem));
-  for (int cr0 = 0; cr0 < A.CR; cr0 += NCR) {
-    kfn<<<nblocks, 32 * M2L_WARPS, smem, st>>>(A, cr0);
-    note_launch();
-  }
-}
-
-template <class T>
-void launch_stored_typed(const M2LArgs &A, int nblocks, cudaStream_t st) {
-  if (A.hard) launch_stored<T, 7, true>(A, nblocks, st);
-  else if (A.CR == 1) launch_stored<T, 1, false>(A, nblocks, st);
-  else if (A.CR == 2) launch_stored<T, 2, false>(A, nblocks, st);
-  else if (A.CR < 8) launch_stored<T, 4, false>(A, nblocks, st);
-  else launch_stored<T, 8, false>(A, nblocks, st);
-}
-
 }  // namespace
 
 void launch_pair_consts(const DeviceProblem &d, const HostSetup &S, double kappa, double eta, cudaStream_t st) {
@@ -686,6 +516,10 @@ void launch_m2l_fill(const DeviceProblem &d, const HostSetup &S, const igabem_op
 
 void launch_m2l_rows(const DeviceProblem &d, const HostSetup &S, const igabem_options &o, int R,
                      bool fp32, cudaStream_t st) {
+  if (!d.m2ls.empty() && d.m2ls[S.lmin]) {  // stored coupling blocks
+    launch_stream_m2l(d, S, R, fp32, st);
+    return;
+  }
   M2LArgs A;
   A.QS = 0;
   A.R = R;
@@ -707,7 +541,6 @@ void launch_m2l_rows(const DeviceProblem &d, const HostSetup &S, const igabem_op
     L.pc = d.pairc[l];
     L.xhat = reinterpret_cast<const double2 *>(d.xhat[l]);
     L.xhat32 = d.xhat32.empty() ? nullptr : d.xhat32[l];
-    L.stored = d.m2ls.empty() ? nullptr : d.m2ls[l];
     L.yhat = reinterpret_cast<double2 *>(d.yhat[l]);
     L.n = S.lev[l].n;
     L.first = nblocks;
@@ -725,10 +558,7 @@ void launch_m2l_rows(const DeviceProblem &d, const HostSetup &S, const igabem_op
       Wc = w;
       break;
     }
-  if (A.nlev > 0 && A.lev[0].stored) {  // stored coupling blocks: stream them
-    if (fp32) launch_stored_typed<float>(A, nblocks, st);
-    else launch_stored_typed<double>(A, nblocks, st);
-  } else if (Wc >= 48 && A.QS <= 64) {
+  if (Wc >= 48 && A.QS <= 64) {
     // Its tile has room for 64 columns: below 48 the padding costs more than k_m2l_fly's regenerated samples
     // (FP64 operations per sample and 7 x 5 columns: 7 (72 + 256) here, 2 x 43 + 140 there).
     const size_t tsz = fp32 ? sizeof(float) : sizeof(double);

@@ -39,6 +39,7 @@
 #include <cstdint>
 
 #include "internal.h"
+#include "k_async.cuh"
 #include "k_m2l.cuh"
 #include "kernels.h"
 
@@ -53,7 +54,6 @@ constexpr int TC_NS = 64;                                  // columns of a slice
 constexpr int TC_MAX_SLOTS = 8;
 constexpr int TC_GROUP = 4;                                // slices per CTA (256 accumulator columns)
 constexpr int TC_NBUF = 3;                                 // B buffers (two copies in flight)
-constexpr unsigned long long TC_WAIT_NS = 2000000000ull;   // bound of one mbarrier wait: 2 s
 
 struct TCLevel {
   const int *far_ptr, *far_src;
@@ -80,8 +80,6 @@ struct TCArgs {
   float kappa, eta;
   int *status;
 };
-
-__device__ inline uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
 // two FP32 values as FP16 hi parts (rounded to nearest) and FP16 lo parts (the rounded remainders),
 // each pair packed in one 32-bit word (first value in the low half)
@@ -116,42 +114,6 @@ __device__ inline void mma_f16(uint32_t d, uint64_t a, uint64_t b, uint32_t ides
 __device__ inline void mma_commit(uint32_t bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
                : "memory");
-}
-
-__device__ inline unsigned long long global_ns() {
-  unsigned long long t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
-}
-
-// wait for the completion of the phase with the given parity; false after limit_ns
-__device__ inline bool mbar_wait(uint32_t bar, uint32_t parity, unsigned long long limit_ns = TC_WAIT_NS) {
-  unsigned long long t0 = 0;
-  for (unsigned it = 0;; ++it) {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}\n"
-        : "=r"(ok)
-        : "r"(bar), "r"(parity)
-        : "memory");
-    if (ok) return true;
-    if ((it & 15) == 0) {
-      const unsigned long long t = global_ns();
-      if (t0 == 0) t0 = t;
-      else if (t - t0 > limit_ns) return false;
-    }
-  }
-}
-
-__device__ inline void bulk_load(uint32_t dst, const void *src, uint32_t bytes, uint32_t bar) {
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
-               "l"(src), "r"(bytes), "r"(bar)
-               : "memory");
-}
-
-__device__ inline void mbar_expect(uint32_t bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
 }
 
 // Constants of one pair for the generation of its coupling block.

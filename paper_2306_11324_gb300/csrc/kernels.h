@@ -14,6 +14,10 @@ size_t m2l_stored_entries(const HostSetup &S, int l);
 void launch_m2l_fill(const DeviceProblem &d, const HostSetup &S, const igabem_options &o, cudaStream_t st);
 void launch_m2l_rows(const DeviceProblem &d, const HostSetup &S, const igabem_options &o, int R,
                      bool fp32, cudaStream_t st);
+// products with stored blocks (k_stream.cu): the near field (nL <= 256), the stored M2L
+bool stream_near_supported(const HostSetup &S);
+void launch_stream_near(const DeviceProblem &d, const HostSetup &S, int R, cudaStream_t st);
+void launch_stream_m2l(const DeviceProblem &d, const HostSetup &S, int R, bool fp32, cudaStream_t st);
 // tensor-core M2L for R right-hand sides (k_m2l_tc.cu); yhat from xhat through d.tc_bimg
 bool m2l_tc_supported(const HostSetup &S, int R);
 size_t m2l_tc_image_bytes(const HostSetup &S, int l, int R);

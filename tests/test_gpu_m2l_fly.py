@@ -21,7 +21,7 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("precision,tol", [(B.FP64, 1e-13), (B.MIXED_FP32, 2e-6)])
 @pytest.mark.parametrize("q,m,b,columns", [(2, 3, 1, (1, 5)), (5, 3, 1, (2, 3)), (7, 3, 1, (1, 3, 4, 7, 26)),
                                            (8, 3, 1, (1, 25, 48)), (11, 3, 1, (1, 6)), (12, 3, 1, (3,)),
-                                           (13, 2, 0, (1, 2)), (7, 5, 2, (1, 4))])
+                                           (16, 2, 0, (1, 2)), (7, 5, 2, (1, 4))])
 def test_on_the_fly_equals_stored_blocks(hard, precision, tol, q, m, b, columns):
     kw = dict(level_m=m, degree_p=1 if b == 0 else 2, kappa=5.0, eta_cfie=0.7, bc=int(hard), cheb_q=q, leaf_offset=b,
               precision=precision)
