@@ -1055,6 +1055,10 @@ void launch_near_field(const DeviceProblem &d, const HostSetup &S, const igabem_
     IGA_CUDA(cudaGetLastError());
   }
   Phase ph(d.prof, IGABEM_PH_SETUP_SINGULAR, st);
+  if (sing_tensor_supported(S)) {
+    launch_sing_tensor(d, S, o, st);
+    return;
+  }
   SingArgs SA;
   SA.A = A;
   SA.sing = d.sing;

@@ -29,6 +29,10 @@ size_t near_table_bytes(const HostSetup &S, const igabem_options &o);
 void launch_near_field(const DeviceProblem &d, const HostSetup &S, const igabem_options &o,
                        cudaStream_t st);
 
+// touching pairs in tensor form (k_singular.cu): gauss_singular = 5 and p <= 3
+bool sing_tensor_supported(const HostSetup &S);
+void launch_sing_tensor(const DeviceProblem &d, const HostSetup &S, const igabem_options &o, cudaStream_t st);
+
 // leaf kernels (k_leaf.cu)
 bool leaf_kernels_supported(const HostSetup &S);
 void launch_near_spmv(const DeviceProblem &d, const HostSetup &S, const igabem_options &o, int R,
