@@ -214,7 +214,7 @@ void ensure_work(igabem_problem *P, int R, bool with_gmres) {
   W.gq = W.arena.get<double>((size_t)S.E * nq * C * R * 2);
   W.xin = W.arena.get<double>(S.N * R * 2);
   W.yout = W.arena.get<double>(S.N * R * 2);
-  W.red = W.arena.get<double>((size_t)34 * 304 * R * 2 + 512);
+  W.red = W.arena.get<double>((size_t)std::max(34, W.gmres_m + 2) * 304 * R * 2 + 512);
   W.xhat.assign(S.L + 1, nullptr);
   W.yhat.assign(S.L + 1, nullptr);
   for (int l = S.lmin; l <= S.L; ++l) {
@@ -908,15 +908,14 @@ int solve_impl(igabem_problem *P, int n_rhs, const double *dirs, int kind, void 
     // one Arnoldi step on the device: w = A V_j (A M^-1 V_j with the preconditioner), two CGS passes,
     // the Givens update and V_{j+1}; the finished flags are copied to page-locked host memory
     auto iteration = [&] {
-      {
+      if (pc) {
         Phase ph(&P->prof, IGABEM_PH_KRYLOV, st);
-        launch_copy_vj(G, W.vj, N, st);
-        if (pc) launch_precond(P->d, S, P->opt, R, W.vj, W.t, st);
+        launch_precond(P->d, S, P->opt, R, W.vj, W.t, st);
       }
       matvec_dev(P, R, pc ? W.t : W.vj, W.w);
       {
         Phase ph(&P->prof, IGABEM_PH_KRYLOV, st);
-        launch_gm_iteration_tail(G, W.red, N, st);
+        launch_gm_iteration_tail(G, W.red, N, W.vj, st);
       }
       IGA_CUDA(cudaMemcpyAsync(W.hflags, G.flags, 2 * sizeof(int), cudaMemcpyDeviceToHost, st));
     };
@@ -984,7 +983,7 @@ int solve_impl(igabem_problem *P, int n_rhs, const double *dirs, int kind, void 
       {
         Phase ph(&P->prof, IGABEM_PH_KRYLOV, st);
         launch_gm_init(G, W.beta, W.active, st);
-        launch_scale(W.r, G.s, W.V, N, R, st);  // V_0 = r / beta
+        launch_scale(W.r, G.s, W.V, W.vj, N, R, st);  // V_0 = r / beta
       }
       W.hflags[0] = W.hflags[1] = 0;
       for (int j = 0; j < m; ++j) {

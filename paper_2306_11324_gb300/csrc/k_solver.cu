@@ -238,36 +238,73 @@ __global__ void __launch_bounds__(256) k_farfield32(RhsArgs A, const double2 *__
 // ----------------------------------------------------------------------------------------------
 // GMRES vector kernels; vectors are [N][R] complex, V_i = V + i N R
 
-constexpr int RED_BLOCKS = 304;
+constexpr int RED_BLOCKS = 304;  // most chunks of a reduction over the vectors
+constexpr int DOT_V = 4;         // basis vectors a block multiplies into (w is read once for them)
 
-// partial sums over chunks: red[(i*G + g)*R + r] = sum_{n in chunk g} conj(V_i[n][r]) w[n][r]
-__global__ void k_multidot_partial(const double2 *__restrict__ V, const double2 *__restrict__ w,
-                                   long N, int R, double2 *__restrict__ red) {
-  extern __shared__ double2 sh[];
-  const int i = blockIdx.y, g = blockIdx.x, G = gridDim.x;
-  const int nthr = (blockDim.x / R) * R;  // threads used: a multiple of R
-  const double2 *Vi = V + (size_t)i * N * R;
-  long chunk = (N + G - 1) / G, n0 = g * chunk, n1 = min(N, n0 + chunk);
-  double2 acc = cmk(0, 0);
-  if (threadIdx.x < nthr) {
-    for (long idx = n0 * R + threadIdx.x; idx < n1 * R; idx += nthr) acc = cadd(acc, cconjmul(Vi[idx], w[idx]));
-  }
-  sh[threadIdx.x] = acc;
+// threads of a reduction block in use: a multiple of R, so that a thread keeps its column
+__device__ inline int red_threads(int R) { return ((int)blockDim.x / R) * R; }
+
+// sum over the threads of a column (thread t has column t % R), for each of n values: the threads t < R get the sums.
+// A tree in shared memory ([n][blockDim]); nthr = red_threads(R).
+template <int n>
+__device__ inline void red_columns(double2 (&v)[n], double2 *sh, int R, int nthr) {
+  const int t = threadIdx.x;
+#pragma unroll
+  for (int k = 0; k < n; ++k) sh[k * blockDim.x + t] = v[k];
   __syncthreads();
-  if (threadIdx.x < R) {
-    double2 s = cmk(0, 0);
-    for (int t = threadIdx.x; t < nthr; t += R) s = cadd(s, sh[t]);
-    red[((size_t)i * G + g) * R + threadIdx.x] = s;
+  int rows = nthr / R;  // threads per column left
+  while (rows > 1) {
+    const int half = (rows + 1) / 2;
+    if (t < (rows - half) * R)
+#pragma unroll
+      for (int k = 0; k < n; ++k) sh[k * blockDim.x + t] = cadd(sh[k * blockDim.x + t], sh[k * blockDim.x + t + half * R]);
+    __syncthreads();
+    rows = half;
   }
+  if (t < R)
+#pragma unroll
+    for (int k = 0; k < n; ++k) v[k] = sh[k * blockDim.x + t];
 }
 
-__global__ void k_multidot_final(const double2 *__restrict__ red, int nv, int G, int R, double2 *__restrict__ h) {
-  int o = blockIdx.x * blockDim.x + threadIdx.x;
-  if (o >= nv * R) return;
-  int i = o / R, r = o % R;
+// partial sums over chunk blockIdx.x: red[(i G + g) R + r] = sum_n conj(V_i[n][r]) w[n][r] for i <= j (j = *jdev; 0
+// without it), DOT_V vectors per block
+__global__ void __launch_bounds__(1024) k_dot_partial(const double2 *__restrict__ V, const int *__restrict__ jdev,
+                                                      const double2 *__restrict__ w, long N, int R,
+                                                      double2 *__restrict__ red) {
+  extern __shared__ double2 shd[];
+  const int j = jdev ? *jdev : 0, i0 = blockIdx.y * DOT_V, g = blockIdx.x, G = gridDim.x;
+  if (i0 > j) return;
+  const int nthr = red_threads(R), nv = min(DOT_V, j + 1 - i0);
+  const long chunk = (N + G - 1) / G, n0 = g * chunk, n1 = min(N, n0 + chunk), NR = N * R;
+  const double2 *Vi = V + (size_t)i0 * NR;
+  double2 acc[DOT_V];
+#pragma unroll
+  for (int k = 0; k < DOT_V; ++k) acc[k] = cmk(0, 0);
+  if ((int)threadIdx.x < nthr)
+    for (long idx = n0 * R + threadIdx.x; idx < n1 * R; idx += nthr) {
+      const double2 x = w[idx];
+#pragma unroll
+      for (int k = 0; k < DOT_V; ++k)
+        if (k < nv) acc[k] = cadd(acc[k], cconjmul(Vi[k * NR + idx], x));
+    }
+  red_columns(acc, shd, R, nthr);
+  if ((int)threadIdx.x < R)
+    for (int k = 0; k < nv; ++k) red[((size_t)(i0 + k) * G + g) * R + threadIdx.x] = acc[k];
+}
+
+// h[i][r] for i <= j from the partial sums of G chunks, one warp each
+__global__ void k_dot_final(const double2 *__restrict__ red, const int *__restrict__ jdev, int G, int R,
+                            double2 *__restrict__ h) {
+  const int o = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31, j = jdev ? *jdev : 0;
+  if (o >= (j + 1) * R) return;
+  const int i = o / R, r = o - i * R;
   double2 s = cmk(0, 0);
-  for (int g = 0; g < G; ++g) s = cadd(s, red[((size_t)i * G + g) * R + r]);
-  h[o] = s;
+  for (int g = lane; g < G; g += 32) s = cadd(s, red[((size_t)i * G + g) * R + r]);
+  for (int k = 16; k > 0; k >>= 1) {
+    s.x += __shfl_xor_sync(0xffffffffu, s.x, k);
+    s.y += __shfl_xor_sync(0xffffffffu, s.y, k);
+  }
+  if (lane == 0) h[o] = s;
 }
 
 __global__ void k_multiaxpy(const double2 *__restrict__ V, int nv, const double2 *__restrict__ h,
@@ -275,6 +312,7 @@ __global__ void k_multiaxpy(const double2 *__restrict__ V, int nv, const double2
   GRID_STRIDE(o, N * R) {
     int r = int(o % R);
     double2 acc = w[o];
+#pragma unroll 4
     for (int i = 0; i < nv; ++i) {
       double2 t = cmul(V[(size_t)i * N * R + o], h[i * R + r]);
       acc = cmk(acc.x + sign * t.x, acc.y + sign * t.y);
@@ -283,8 +321,13 @@ __global__ void k_multiaxpy(const double2 *__restrict__ V, int nv, const double2
   }
 }
 
-__global__ void k_scale(const double2 *__restrict__ w, const double *__restrict__ s, double2 *dst, long N, int R) {
-  GRID_STRIDE(o, N * R) dst[o] = cscale(w[o], s[o % R]);
+__global__ void k_scale(const double2 *__restrict__ w, const double *__restrict__ s, double2 *dst, double2 *dst2, long N,
+                        int R) {
+  GRID_STRIDE(o, N * R) {
+    const double2 v = cscale(w[o], s[o % R]);
+    dst[o] = v;
+    dst2[o] = v;
+  }
 }
 
 __global__ void k_sub(const double *__restrict__ b, const double *__restrict__ y, double *__restrict__ r, long n) {
@@ -297,66 +340,43 @@ __global__ void k_sqrt_re(const double2 *__restrict__ h, double *__restrict__ nr
 }
 
 // ---- device-side GMRES iteration: the Arnoldi index j lives on the device, so one captured graph
-// serves every iteration of a cycle (the kernels read j; grids are sized for the whole cycle) ----
+// serves every iteration of a cycle (the kernels read j; grids are sized for the whole cycle).  On small systems the
+// launches and the serial parts are what an iteration costs, so each reduction is a tree, the second
+// Gram-Schmidt update also forms the partial sums of the norm, and V_{j+1} is written together with the copy
+// that the next product reads.  Measured, one column, 1944 unknowns: 0.42 ms an iteration with serial
+// sums and 13 launches beside the product. ----
 
-// partial sums of h[i][r] = sum_n conj(V_i[n][r]) w[n][r] for i <= j (blocks of i > j return)
-__global__ void k_multidot_partial_dev(const double2 *__restrict__ V, const int *__restrict__ jdev,
-                                       const double2 *__restrict__ w, long N, int R, double2 *__restrict__ red) {
+// w[n][r] -= sum_{i <= j} V_i[n][r] h[i][r]; with nrm2 != nullptr also the chunks' sums of |w|^2 (same layout as the
+// partial sums of one vector)
+__global__ void __launch_bounds__(1024) k_orth_update(const double2 *__restrict__ V, const int *__restrict__ jdev,
+                                                      const double2 *__restrict__ h, double2 *__restrict__ w, long N,
+                                                      int R, double2 *__restrict__ nrm2) {
   extern __shared__ double2 shd[];
-  const int i = blockIdx.y, g = blockIdx.x, G = gridDim.x;
-  if (i > *jdev) return;
-  const int nthr = (blockDim.x / R) * R;
-  const double2 *Vi = V + (size_t)i * N * R;
-  long chunk = (N + G - 1) / G, n0 = g * chunk, n1 = min(N, n0 + chunk);
-  double2 acc = cmk(0, 0);
-  if (threadIdx.x < nthr) {
-    for (long idx = n0 * R + threadIdx.x; idx < n1 * R; idx += nthr) acc = cadd(acc, cconjmul(Vi[idx], w[idx]));
-  }
-  shd[threadIdx.x] = acc;
-  __syncthreads();
-  if (threadIdx.x < R) {
-    double2 sum = cmk(0, 0);
-    for (int t = threadIdx.x; t < nthr; t += R) sum = cadd(sum, shd[t]);
-    red[((size_t)i * G + g) * R + threadIdx.x] = sum;
-  }
+  const int nv = *jdev + 1, g = blockIdx.x, G = gridDim.x, nthr = red_threads(R), r = threadIdx.x % R;
+  const long chunk = (N + G - 1) / G, n0 = g * chunk, n1 = min(N, n0 + chunk), NR = N * R;
+  double2 sum[1] = {cmk(0, 0)};
+  if ((int)threadIdx.x < nthr)
+    for (long idx = n0 * R + threadIdx.x; idx < n1 * R; idx += nthr) {
+      double2 acc = w[idx];
+#pragma unroll 4
+      for (int i = 0; i < nv; ++i) acc = csub(acc, cmul(V[(size_t)i * NR + idx], h[i * R + r]));
+      w[idx] = acc;
+      sum[0].x = fma(acc.x, acc.x, fma(acc.y, acc.y, sum[0].x));
+    }
+  if (!nrm2) return;
+  red_columns(sum, shd, R, nthr);
+  if ((int)threadIdx.x < R) nrm2[(size_t)g * R + threadIdx.x] = sum[0];
 }
 
-// h[i][r] for i <= j (zero above j), from the partial sums
-__global__ void k_multidot_final_dev(const double2 *__restrict__ red, const int *__restrict__ jdev, int nmax, int G,
-                                     int R, double2 *__restrict__ h) {
-  int o = blockIdx.x * blockDim.x + threadIdx.x;
-  if (o >= nmax * R) return;
-  int i = o / R, r = o % R;
-  double2 sum = cmk(0, 0);
-  if (i <= *jdev)
-    for (int g = 0; g < G; ++g) sum = cadd(sum, red[((size_t)i * G + g) * R + r]);
-  h[o] = sum;
-}
-
-// w[n][r] -= sum_{i <= j} V_i[n][r] h[i][r]
-__global__ void k_multiaxpy_dev(const double2 *__restrict__ V, const int *__restrict__ jdev,
-                                const double2 *__restrict__ h, double2 *__restrict__ w, long N, int R) {
-  const int nv = *jdev + 1;
-  GRID_STRIDE(o, N * R) {
-    int r = int(o % R);
-    double2 acc = w[o];
-    for (int i = 0; i < nv; ++i) acc = csub(acc, cmul(V[(size_t)i * N * R + o], h[i * R + r]));
-    w[o] = acc;
-  }
-}
-
-// dst = V_j
-__global__ void k_copy_vj(const double2 *__restrict__ V, const int *__restrict__ jdev, double2 *__restrict__ dst,
-                          long NR) {
-  const double2 *src = V + (size_t)(*jdev) * NR;
-  GRID_STRIDE(o, NR) dst[o] = src[o];
-}
-
-// V_{j} = s w for the (already advanced) index j
+// V_{j} = s w for the (already advanced) index j, and its copy vj
 __global__ void k_scale_vj(const double2 *__restrict__ w, const double *__restrict__ s, double2 *__restrict__ V,
-                           const int *__restrict__ jdev, long N, int R) {
+                           const int *__restrict__ jdev, long N, int R, double2 *__restrict__ vj) {
   double2 *dst = V + (size_t)(*jdev) * N * R;
-  GRID_STRIDE(o, N * R) dst[o] = cscale(w[o], s[o % R]);
+  GRID_STRIDE(o, N * R) {
+    const double2 v = cscale(w[o], s[o % R]);
+    dst[o] = v;
+    vj[o] = v;
+  }
 }
 
 // cycle start: H, rotations and g cleared, g_0 = beta for the active columns, s = 1 / beta, j = 0
@@ -380,48 +400,71 @@ __global__ void k_gm_init(GmDev G, const double *__restrict__ beta, const int *_
   }
 }
 
-// Arnoldi column j of every active right-hand side: h = hA + hB (the two Gram-Schmidt passes), the
-// new column of H rotated by the previous Givens rotations, the new rotation, g updated, the
+// Arnoldi column j of every active right-hand side: h = hA + hB (the two Gram-Schmidt passes), the norm from its G
+// partial sums nrm2, the new column of H rotated by the previous Givens rotations, the new rotation, g updated, the
 // convergence test |g_{j+1}| <= tol ||b||; s = 1 / h_{j+1,j} for the next basis vector (0 for finished
-// columns); then j advances.  One block; flags[0] = every column finished, flags[1] = non-finite met.
-__global__ void k_gm_arnoldi(GmDev G) {
-  const int R = G.R, m = G.m, j = *G.j;
+// columns); then j advances.  One block, a warp per column: its lanes load 32 entries and rotations at a time,
+// lane 0 runs the recurrence over them.  flags[0] = every column finished, flags[1] = non-finite met.
+constexpr int ARN_WARPS = 16;
+
+__global__ void __launch_bounds__(32 * ARN_WARPS) k_gm_arnoldi(GmDev G, const double2 *__restrict__ nrm2, int chunks) {
+  __shared__ double2 hs[ARN_WARPS][32], cv[ARN_WARPS][32], sv[ARN_WARPS][32];
   __shared__ int all_done, bad;
+  const int R = G.R, m = G.m, j = *G.j, wp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
     all_done = 1;
     bad = 0;
   }
   __syncthreads();
-  for (int r = threadIdx.x; r < R; r += blockDim.x) {
+  for (int r = wp; r < R; r += ARN_WARPS) {
     if (G.done[r]) {
-      G.s[r] = 0.0;
+      if (lane == 0) G.s[r] = 0.0;
       continue;
     }
-    const double hn = G.nrm[r];
+    double n2 = 0.0;
+    for (int g = lane; g < chunks; g += 32) n2 += nrm2[(size_t)g * R + r].x;
+    for (int k = 16; k > 0; k >>= 1) n2 += __shfl_xor_sync(0xffffffffu, n2, k);
+    const double hn = sqrt(fmax(n2, 0.0));
     double2 *Hc = G.H + (size_t)r;  // H[i][jj][r] at ((i * m) + jj) * R + r
-    for (int i = 0; i <= j; ++i) Hc[((size_t)i * m + j) * R] = cadd(G.hA[i * R + r], G.hB[i * R + r]);
-    Hc[((size_t)(j + 1) * m + j) * R] = cmk(hn, 0);
-    for (int i = 0; i < j; ++i) {
-      const double2 c = G.cs[i * R + r], sv = G.sn[i * R + r];
-      const double2 a = Hc[((size_t)i * m + j) * R], b = Hc[((size_t)(i + 1) * m + j) * R];
-      // [c, s; -conj(s), conj(c)] (a, b)
-      Hc[((size_t)i * m + j) * R] = cadd(cmul(c, a), cmul(sv, b));
-      Hc[((size_t)(i + 1) * m + j) * R] = cadd(cmul(cmk(-sv.x, sv.y), a), cmul(cmk(c.x, -c.y), b));
+    double2 a = cmk(0, 0);          // lane 0: the entry that the next rotation (or the new one) starts from
+    for (int i0 = 0; i0 <= j; i0 += 32) {
+      const int i = i0 + lane, n = min(32, j + 1 - i0);
+      __syncwarp();
+      if (i <= j) hs[wp][lane] = cadd(G.hA[i * R + r], G.hB[i * R + r]);
+      if (i < j) {
+        cv[wp][lane] = G.cs[i * R + r];
+        sv[wp][lane] = G.sn[i * R + r];
+      }
+      __syncwarp();
+      if (lane == 0) {
+        // entry i0 + k and the rotation of rows i0 + k - 1, i0 + k: the last entry of the previous 32 is in a
+        if (i0 == 0) a = hs[wp][0];
+        for (int k = i0 == 0 ? 1 : 0; k < n; ++k) {
+          // rotation i0 + k - 1 (of the previous 32 for k = 0): [c, s; -conj(s), conj(c)] (a, b)
+          const double2 c = k ? cv[wp][k - 1] : G.cs[(i0 - 1) * R + r], q = k ? sv[wp][k - 1] : G.sn[(i0 - 1) * R + r];
+          const double2 b = hs[wp][k], t = cadd(cmul(c, a), cmul(q, b));
+          a = cadd(cmul(cmk(-q.x, q.y), a), cmul(cmk(c.x, -c.y), b));
+          if (k) hs[wp][k - 1] = t;
+          else Hc[((size_t)(i0 - 1) * m + j) * R] = t;
+        }
+      }
+      __syncwarp();
+      if (lane < n - 1) Hc[((size_t)i * m + j) * R] = hs[wp][lane];
     }
-    const double2 a = Hc[((size_t)j * m + j) * R], b = Hc[((size_t)(j + 1) * m + j) * R];
-    const double den = sqrt(a.x * a.x + a.y * a.y + b.x * b.x + b.y * b.y);
+    if (lane) continue;
+    const double den = sqrt(a.x * a.x + a.y * a.y + hn * hn);
     const double2 c = den > 0 ? cmk(a.x / den, -a.y / den) : cmk(1, 0);
-    const double2 sv = den > 0 ? cmk(b.x / den, -b.y / den) : cmk(0, 0);
+    const double2 q = den > 0 ? cmk(hn / den, 0.0) : cmk(0, 0);
     G.cs[j * R + r] = c;
-    G.sn[j * R + r] = sv;
+    G.sn[j * R + r] = q;
     Hc[((size_t)j * m + j) * R] = cmk(den, 0);
     Hc[((size_t)(j + 1) * m + j) * R] = cmk(0, 0);
     const double2 gj = G.g[j * R + r];
-    G.g[(j + 1) * R + r] = cmul(cmk(-sv.x, sv.y), gj);
+    const double2 gn = cmul(cmk(-q.x, q.y), gj);
+    G.g[(j + 1) * R + r] = gn;
     G.g[j * R + r] = cmul(c, gj);
     G.k[r] = j + 1;
     const int its = ++G.its[r];
-    const double2 gn = G.g[(j + 1) * R + r];
     const double res = sqrt(gn.x * gn.x + gn.y * gn.y);
     if (!isfinite(res) || !isfinite(hn)) atomicExch(&bad, 1);
     const bool done = res <= G.tol * G.bn[r] || its >= G.maxit || hn == 0.0 || j + 1 >= m;
@@ -513,50 +556,49 @@ void launch_farfield(const DeviceProblem &d, const HostSetup &S, const igabem_op
   IGA_CUDA(cudaGetLastError());
 }
 
-void launch_multidot(const double *V, int nv, const double *w, long N, int R, double *red,
-                     double *h, cudaStream_t st) {
-  int threads = std::max(R, (256 / R) * R);
-  dim3 grid(RED_BLOCKS, nv);
-  k_multidot_partial<<<grid, threads, threads * sizeof(double2), st>>>(
-      reinterpret_cast<const double2 *>(V), reinterpret_cast<const double2 *>(w), N, R,
+namespace {
+// threads of the reduction kernels (whole columns; at least a warp's worth of columns per thread row) and chunks of the
+// vectors: 8 elements a thread on small vectors, so that few partial sums are left
+int dot_threads(int R) { return std::max(R, (256 / R) * R); }
+int dot_chunks(long N, int R) { return (int)std::max<long>(1, std::min<long>(RED_BLOCKS, N * R / 2048)); }
+
+void launch_dot(const double *V, const int *jdev, int most, const double *w, long N, int R, double *red, double2 *h,
+                cudaStream_t st) {
+  const int threads = dot_threads(R), G = dot_chunks(N, R);
+  const size_t smem = sizeof(double2) * DOT_V * threads;
+  IGA_CUDA(set_max_dynamic_smem(k_dot_partial, smem));
+  k_dot_partial<<<dim3(G, (most + DOT_V - 1) / DOT_V), threads, smem, st>>>(
+      reinterpret_cast<const double2 *>(V), jdev, reinterpret_cast<const double2 *>(w), N, R,
       reinterpret_cast<double2 *>(red));
   note_launch();
-  k_multidot_final<<<(nv * R + 255) / 256, 256, 0, st>>>(reinterpret_cast<const double2 *>(red), nv,
-                                                         RED_BLOCKS, R, reinterpret_cast<double2 *>(h));
+  k_dot_final<<<(most * R * 32 + 255) / 256, 256, 0, st>>>(reinterpret_cast<const double2 *>(red), jdev, G, R, h);
   note_launch();
   IGA_CUDA(cudaGetLastError());
 }
+}  // namespace
 
-void launch_gm_iteration_tail(const GmDev &G, double *red, long N, cudaStream_t st) {
+void launch_gm_iteration_tail(const GmDev &G, double *red, long N, double *vj, cudaStream_t st) {
   // two classical Gram-Schmidt passes against V_0..V_j, the norm, the Arnoldi update, the next basis vector
-  const int R = G.R, threads = std::max(R, (256 / R) * R);
+  const int R = G.R, threads = dot_threads(R), chunks = dot_chunks(N, R);
   for (int pass = 0; pass < 2; ++pass) {
     double2 *h = pass ? G.hB : G.hA;
-    dim3 grid(RED_BLOCKS, G.m + 1);
-    k_multidot_partial_dev<<<grid, threads, threads * sizeof(double2), st>>>(
-        reinterpret_cast<const double2 *>(G.V), G.j, reinterpret_cast<const double2 *>(G.w), N, R,
-        reinterpret_cast<double2 *>(red));
+    launch_dot(G.V, G.j, G.m + 1, G.w, N, R, red, h, st);
+    // the update on finer chunks than the sums, up to the sums' scratch
+    const int blocks = (int)std::max<long>(chunks, std::min<long>(RED_BLOCKS, (N * R + threads - 1) / threads));
+    k_orth_update<<<blocks, threads, threads * sizeof(double2), st>>>(reinterpret_cast<const double2 *>(G.V), G.j, h,
+                                                                      reinterpret_cast<double2 *>(G.w), N, R,
+                                                                      pass ? reinterpret_cast<double2 *>(red) : nullptr);
     note_launch();
-    k_multidot_final_dev<<<((G.m + 1) * R + 255) / 256, 256, 0, st>>>(reinterpret_cast<const double2 *>(red), G.j,
-                                                                     G.m + 1, RED_BLOCKS, R, h);
-    note_launch();
-    k_multiaxpy_dev<<<grid_for(N * R), 256, 0, st>>>(reinterpret_cast<const double2 *>(G.V), G.j, h,
-                                                      reinterpret_cast<double2 *>(G.w), N, R);
-    note_launch();
+    if (pass) {
+      k_gm_arnoldi<<<1, 32 * ARN_WARPS, 0, st>>>(G, reinterpret_cast<const double2 *>(red), blocks);
+      note_launch();
+    }
   }
-  launch_norms(G.w, N, R, red, G.nrm, st);
-  k_gm_arnoldi<<<1, 1024, 0, st>>>(G);
-  note_launch();
   k_scale_vj<<<grid_for(N * R), 256, 0, st>>>(reinterpret_cast<const double2 *>(G.w), G.s,
-                                               reinterpret_cast<double2 *>(G.V), G.j, N, R);
+                                               reinterpret_cast<double2 *>(G.V), G.j, N, R,
+                                               reinterpret_cast<double2 *>(vj));
   note_launch();
   IGA_CUDA(cudaGetLastError());
-}
-
-void launch_copy_vj(const GmDev &G, double *dst, long N, cudaStream_t st) {
-  k_copy_vj<<<grid_for(N * G.R), 256, 0, st>>>(reinterpret_cast<const double2 *>(G.V), G.j,
-                                                 reinterpret_cast<double2 *>(dst), N * G.R);
-  note_launch();
 }
 
 void launch_gm_init(const GmDev &G, const double *beta, const int *active, cudaStream_t st) {
@@ -569,13 +611,6 @@ void launch_gm_solve(const GmDev &G, cudaStream_t st) {
   note_launch();
 }
 
-void launch_multiaxpy(const double *V, int nv, const double *h, double *w, long N, int R, cudaStream_t st) {
-  k_multiaxpy<<<grid_for(N * R), 256, 0, st>>>(reinterpret_cast<const double2 *>(V), nv,
-                                                reinterpret_cast<const double2 *>(h),
-                                                reinterpret_cast<double2 *>(w), N, R, -1.0);
-  note_launch();
-}
-
 void launch_update(const double *V, int nv, const double *y, double *x, long N, int R, cudaStream_t st) {
   k_multiaxpy<<<grid_for(N * R), 256, 0, st>>>(reinterpret_cast<const double2 *>(V), nv,
                                                 reinterpret_cast<const double2 *>(y),
@@ -584,15 +619,15 @@ void launch_update(const double *V, int nv, const double *y, double *x, long N, 
 }
 
 void launch_norms(const double *w, long N, int R, double *red, double *nrm, cudaStream_t st) {
-  double *h = red + (size_t)2 * RED_BLOCKS * R * 2;  // past the partial sums of one vector
-  launch_multidot(w, 1, w, N, R, red, h, st);
-  k_sqrt_re<<<(R + 255) / 256, 256, 0, st>>>(reinterpret_cast<const double2 *>(h), nrm, R);
+  double2 *h = reinterpret_cast<double2 *>(red) + (size_t)RED_BLOCKS * R;  // past the partial sums of one vector
+  launch_dot(w, nullptr, 1, w, N, R, red, h, st);
+  k_sqrt_re<<<(R + 255) / 256, 256, 0, st>>>(h, nrm, R);
   note_launch();
 }
 
-void launch_scale(const double *w, const double *s, double *dst, long N, int R, cudaStream_t st) {
-  k_scale<<<grid_for(N * R), 256, 0, st>>>(reinterpret_cast<const double2 *>(w), s,
-                                            reinterpret_cast<double2 *>(dst), N, R);
+void launch_scale(const double *w, const double *s, double *dst, double *dst2, long N, int R, cudaStream_t st) {
+  k_scale<<<grid_for(N * R), 256, 0, st>>>(reinterpret_cast<const double2 *>(w), s, reinterpret_cast<double2 *>(dst),
+                                            reinterpret_cast<double2 *>(dst2), N, R);
   note_launch();
 }
 

@@ -68,19 +68,13 @@ void launch_farfield(const DeviceProblem &d, const HostSetup &S, const igabem_op
                      cudaStream_t st);
 
 // GMRES vector kernels (k_solver.cu); vectors [N][R] complex, per-column results [.][R]
-// h[i][r] = sum_n conj(V_i[n][r]) w[n][r] for i < nv (V_i = V + i*N*R)
-void launch_multidot(const double *V, int nv, const double *w, long N, int R, double *red,
-                     double *h, cudaStream_t st);
-// w[n][r] -= sum_i V_i[n][r] h[i][r]
-void launch_multiaxpy(const double *V, int nv, const double *h, double *w, long N, int R,
-                      cudaStream_t st);
 // x[n][r] += sum_i V_i[n][r] y[i][r]
 void launch_update(const double *V, int nv, const double *y, double *x, long N, int R,
                    cudaStream_t st);
 // nrm[r] = ||w[:, r]||_2
 void launch_norms(const double *w, long N, int R, double *red, double *nrm, cudaStream_t st);
-// w[n][r] *= s[r] (real), dst may equal w
-void launch_scale(const double *w, const double *s, double *dst, long N, int R, cudaStream_t st);
+// dst[n][r] = dst2[n][r] = w[n][r] s[r] (real)
+void launch_scale(const double *w, const double *s, double *dst, double *dst2, long N, int R, cudaStream_t st);
 // r = b - y
 void launch_sub(const double *b, const double *y, double *r, long n, cudaStream_t st);
 
@@ -101,10 +95,8 @@ struct GmDev {
   double *V, *w;              // basis [(m+1)][N][R] and the new vector [N][R]
 };
 // after the matrix-vector product w = A V_j: two CGS passes, the norm, the Arnoldi / Givens update
-// (k_gm_arnoldi), V_{j+1} = w / h_{j+1,j}; j advances on the device
-void launch_gm_iteration_tail(const GmDev &G, double *red, long N, cudaStream_t st);
-// dst = V_j (j read on the device)
-void launch_copy_vj(const GmDev &G, double *dst, long N, cudaStream_t st);
+// (k_gm_arnoldi), V_{j+1} = w / h_{j+1,j}, copied to vj; j advances on the device
+void launch_gm_iteration_tail(const GmDev &G, double *red, long N, double *vj, cudaStream_t st);
 // cycle start from beta [R] and the active flags [R] (device)
 void launch_gm_init(const GmDev &G, const double *beta, const int *active, cudaStream_t st);
 // y = H^-1 g per column
