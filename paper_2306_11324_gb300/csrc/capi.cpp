@@ -154,6 +154,7 @@ struct ProblemWork {
   int R = 0;
   int gmres_m = 0;
   Arena arena;
+  Arena ff;                          // far-field directions (and a host caller's result), grown as needed
   double *xX, *yleaf, *gq, *xin, *yout, *red;
   std::vector<void *> xhat, yhat;
   std::vector<uint8_t *> tc_bimg;
@@ -169,6 +170,7 @@ struct ProblemWork {
   IterGraph graph;
   ~ProblemWork() {
     graph.release();
+    ff.release();
     if (hflags) cudaFreeHost(hflags);
   }
 };
@@ -1060,16 +1062,16 @@ int igabem_farfield(igabem_problem *P, int n_rhs, const void *density, int n_dir
     bool dd = is_device_ptr(density), du = is_device_ptr(uinf);
     const double *dens = dd ? static_cast<const double *>(density) : W.xin;
     if (!dd) IGA_CUDA(cudaMemcpyAsync(W.xin, density, db, cudaMemcpyHostToDevice, st));
-    // directions and the result need their own device space
-    double *dx = nullptr, *du_ = nullptr;
-    IGA_CUDA(cudaMallocAsync(&dx, 3 * sizeof(double) * n_dir, st));
-    IGA_CUDA(cudaMallocAsync(&du_, 2 * sizeof(double) * n_dir * n_rhs, st));
+    // the directions (and, for a host result, the pattern) in a buffer kept with the problem
+    const size_t xb = (3 * sizeof(double) * (size_t)n_dir + 255) & ~size_t(255);
+    const size_t need = xb + (du ? 0 : 2 * sizeof(double) * (size_t)n_dir * n_rhs);
+    if (W.ff.cap < need) W.ff.reserve(need);
+    double *dx = reinterpret_cast<double *>(W.ff.base);
+    double *du_ = du ? static_cast<double *>(uinf) : reinterpret_cast<double *>(W.ff.base + xb);
     IGA_CUDA(cudaMemcpyAsync(dx, xhat, 3 * sizeof(double) * n_dir, cudaMemcpyHostToDevice, st));
     launch_farfield(P->d, P->S, P->opt, n_rhs, dens, n_dir, dx, du_, P->d.gq, st);
-    IGA_CUDA(cudaMemcpyAsync(uinf, du_, 2 * sizeof(double) * n_dir * n_rhs,
-                             du ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, st));
-    IGA_CUDA(cudaFreeAsync(dx, st));
-    IGA_CUDA(cudaFreeAsync(du_, st));
+    if (!du)
+      IGA_CUDA(cudaMemcpyAsync(uinf, du_, 2 * sizeof(double) * n_dir * n_rhs, cudaMemcpyDeviceToHost, st));
     IGA_CUDA(cudaStreamSynchronize(st));
     P->prof.flush();
   });

@@ -443,14 +443,15 @@ void launch_fly(const M2LArgs &A, int nblocks, int nsplit, cudaStream_t st) {
 }
 
 // All columns, in passes of at most 24 (the FP64 accumulators of 24 columns fill the registers; each pass
-// generates the samples again), the passes as even as the kernel's column counts allow.
+// generates the samples again), sound-hard 21 (three columns of seven channels), the passes as even as the kernel's
+// column counts allow.
 template <class T>
 void launch_fly_all(const M2LArgs &A, int nblocks, int nsplit, cudaStream_t st) {
-  const int passes = (A.CR + 23) / 24, w = (A.CR + passes - 1) / passes;
+  const int most = A.hard ? 21 : 24, passes = (A.CR + most - 1) / most, w = (A.CR + passes - 1) / passes;
   if (A.hard) {
-    if (w > 16) launch_fly<T, 24, true>(A, nblocks, nsplit, st);
-    else if (w > 8) launch_fly<T, 16, true>(A, nblocks, nsplit, st);
-    else launch_fly<T, 8, true>(A, nblocks, nsplit, st);
+    if (w > 14) launch_fly<T, 21, true>(A, nblocks, nsplit, st);
+    else if (w > 7) launch_fly<T, 14, true>(A, nblocks, nsplit, st);
+    else launch_fly<T, 7, true>(A, nblocks, nsplit, st);
   } else if (w > 16) {
     launch_fly<T, 24, false>(A, nblocks, nsplit, st);
   } else if (w > 8) {

@@ -1,8 +1,11 @@
 // Right-hand sides (Sec. 4.1), far-field pattern (Sec. 1) and the vector kernels of GMRES (Sec. 5.1).
+#include <cooperative_groups.h>
+
 #include <algorithm>
 
 #include "internal.h"
 #include "k_common.cuh"
+#include "k_m2l.cuh"
 #include "kernels.h"
 
 namespace igabem {
@@ -81,155 +84,245 @@ __global__ void k_rhs(RhsArgs A, double2 *__restrict__ b) {
   }
 }
 
-// density at the Gauss points, weighted by w_q h^2: rho[e][q][r] = w_q h^2 sum_k psi_k(q) x[.][r]
-__global__ void k_density(RhsArgs A, const int *__restrict__ x2g, const double2 *__restrict__ x,
-                          long E, double2 *__restrict__ rho) {
-  const int p1 = A.p + 1, nq = A.ng * A.ng;
-  GRID_STRIDE(o, E * nq * A.R) {
-    long e = o / (nq * A.R);
-    int q = int((o / A.R) % nq), r = int(o % A.R), q1 = q / A.ng, q2 = q % A.ng;
-    int j = int(e / ((long)A.n1 * A.n1)), ix = int((e / A.n1) % A.n1), iy = int(e % A.n1);
-    double2 acc = cmk(0, 0);
+// density at the Gauss points, weighted by w_q h^2: rho[e][q][r] = w_q h^2 sum_k psi_k(q) x[.][r], in FP64, stored as
+// V (the FP32 far field rounds it here once); a thread takes four columns, so that the basis products are
+// shared
+template <class V>
+__global__ void k_density(RhsArgs A, const int *__restrict__ x2g, const double2 *__restrict__ x, long E,
+                          V *__restrict__ rho) {
+  const int p1 = A.p + 1, nq = A.ng * A.ng, nc4 = (A.R + 3) / 4;
+  GRID_STRIDE(o, E * nq * nc4) {
+    const long iq = o / nc4, e = iq / nq;
+    const int r0 = int(o - iq * nc4) * 4, nr = min(4, A.R - r0), q = int(iq - e * nq), q1 = q / A.ng, q2 = q % A.ng;
+    const int j = int(e / ((long)A.n1 * A.n1)), ix = int((e / A.n1) % A.n1), iy = int(e % A.n1);
+    double2 acc[4] = {cmk(0, 0), cmk(0, 0), cmk(0, 0), cmk(0, 0)};
     for (int ka = 0; ka < p1; ++ka)
       for (int kb = 0; kb < p1; ++kb) {
-        long X = ((long)j * A.nb + ix + ka) * A.nb + iy + kb;
-        double w = A.phi1[(ix * A.ng + q1) * p1 + ka] * A.phi1[(iy * A.ng + q2) * p1 + kb];
-        acc = cadd(acc, cscale(x[(long)x2g[X] * A.R + r], w));
+        const long X = ((long)j * A.nb + ix + ka) * A.nb + iy + kb;
+        const double w = A.phi1[(ix * A.ng + q1) * p1 + ka] * A.phi1[(iy * A.ng + q2) * p1 + kb];
+        const double2 *xr = x + (long)x2g[X] * A.R + r0;
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+          if (r < nr) acc[r] = cadd(acc[r], cscale(xr[r], w));
       }
-    rho[o] = cscale(acc, A.gw[q1] * A.gw[q2] * A.h * A.h);
+    const double w = A.gw[q1] * A.gw[q2] * A.h * A.h;
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+      if (r < nr) {
+        V v;
+        v.x = (decltype(v.x))(acc[r].x * w);
+        v.y = (decltype(v.y))(acc[r].y * w);
+        rho[iq * A.R + r0 + r] = v;
+      }
   }
 }
 
-// u_inf[k][r] = sum_points rho * exp(-i kappa x^_k . x) * (soft: -a/(4 pi); hard: -i kappa (x^.n~)/(4 pi))
-__global__ void k_farfield(RhsArgs A, const double2 *__restrict__ rho, long npts,
-                           const double *__restrict__ xhat, double2 *__restrict__ uinf) {
-  __shared__ double2 red[256];
-  const int k = blockIdx.x, r = blockIdx.y;
-  const double *xh = xhat + 3 * k;
-  double2 acc = cmk(0, 0);
-  for (long i = threadIdx.x; i < npts; i += blockDim.x) {
-    double x[3] = {A.gpx[i], A.gpx[A.gst + i], A.gpx[2 * A.gst + i]};
-    double s, c;
-    sincos(-A.kappa * (xh[0] * x[0] + xh[1] * x[1] + xh[2] * x[2]), &s, &c);
-    double2 v = cmul(rho[i * A.R + r], cmk(c, s));
-    if (A.hard) {
-      double xn = xh[0] * A.gpn[i] + xh[1] * A.gpn[A.gst + i] + xh[2] * A.gpn[2 * A.gst + i];
-      v = cmul(v, cmk(0.0, -A.kappa * xn));
-    } else {
-      v = cscale(v, -A.gpa[i]);
-    }
-    acc = cadd(acc, v);
-  }
-  red[threadIdx.x] = acc;
+// u_inf[k][r] = sum_points rho * exp(-i kappa x^_k . x) * (soft: -a/(4 pi); hard: -i kappa (x^.n~)/(4 pi)) in FP64.  One
+// block per direction and four columns, which share the exponential (FP64 arithmetic bounds it: 18 operations for
+// the table-driven exponential instead of CUDA's sincos per column); the points are split over a cluster of
+// gridDim.z blocks where there are few directions.
+constexpr int FF64_COLS = 4;
+
+__global__ void __launch_bounds__(256) k_farfield(RhsArgs A, const double2 *__restrict__ rho, long npts,
+                                                  const double *__restrict__ xhat, const double2 *__restrict__ cis,
+                                                  double2 *__restrict__ uinf) {
+  __shared__ double2 tab[CIS_N];
+  __shared__ double2 red[8][FF64_COLS];
+  const int k = blockIdx.x, r0 = blockIdx.y * FF64_COLS, nr = min(FF64_COLS, A.R - r0), nz = gridDim.z;
+  const double xh[3] = {xhat[3 * k], xhat[3 * k + 1], xhat[3 * k + 2]};
+  double c0, c1;
+  phase64_scale(A.kappa, c0, c1);
+  for (int i = threadIdx.x; i < CIS_N; i += 256) tab[i] = cis[i];
   __syncthreads();
-  for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-    if (threadIdx.x < s) red[threadIdx.x] = cadd(red[threadIdx.x], red[threadIdx.x + s]);
-    __syncthreads();
+  double2 acc[FF64_COLS];
+#pragma unroll
+  for (int r = 0; r < FF64_COLS; ++r) acc[r] = cmk(0, 0);
+  for (long i = blockIdx.z * 256 + threadIdx.x; i < npts; i += 256L * nz) {
+    const double d = fma(xh[0], A.gpx[i], fma(xh[1], A.gpx[A.gst + i], xh[2] * A.gpx[2 * A.gst + i]));
+    const Phase64 p = phase64(tab, d, c0, c1);
+    // amplitude times exp(i kappa x^.x) = (c, s): soft a, the factor is -(c - i s); hard kappa x^.n~, -(s + i c)
+    double2 f;
+    if (A.hard) {
+      const double xn = A.kappa * fma(xh[0], A.gpn[i], fma(xh[1], A.gpn[A.gst + i], xh[2] * A.gpn[2 * A.gst + i]));
+      const C2<double> e = phase_mul(p.E.x * xn, p.E.y * xn, p);
+      f = cmk(-e.y, -e.x);
+    } else {
+      const double a = A.gpa[i];
+      const C2<double> e = phase_mul(p.E.x * a, p.E.y * a, p);
+      f = cmk(-e.x, e.y);
+    }
+#pragma unroll
+    for (int r = 0; r < FF64_COLS; ++r)
+      if (r < nr) {
+        const double2 v = rho[i * A.R + r0 + r];
+        acc[r].x = fma(f.x, v.x, fma(-f.y, v.y, acc[r].x));
+        acc[r].y = fma(f.x, v.y, fma(f.y, v.x, acc[r].y));
+      }
   }
-  if (threadIdx.x == 0) uinf[(long)k * gridDim.y + r] = cscale(red[0], 0.25 / IGA_PI);
+#pragma unroll
+  for (int r = 0; r < FF64_COLS; ++r) {
+    for (int o = 16; o > 0; o >>= 1) {
+      acc[r].x += __shfl_xor_sync(0xffffffffu, acc[r].x, o);
+      acc[r].y += __shfl_xor_sync(0xffffffffu, acc[r].y, o);
+    }
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5][r] = acc[r];
+  }
+  cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
+  if (nz > 1) cl.sync();
+  else __syncthreads();
+  if (blockIdx.z == 0 && (int)threadIdx.x < nr) {
+    double2 s = cmk(0, 0);
+    for (int z = 0; z < nz; ++z) {
+      const double2(*rz)[FF64_COLS] = nz > 1 ? cl.map_shared_rank(red, z) : red;
+      for (int w = 0; w < 8; ++w) s = cadd(s, rz[w][threadIdx.x]);
+    }
+    uinf[(long)k * A.R + r0 + threadIdx.x] = cscale(s, 0.25 / IGA_PI);
+  }
+  if (nz > 1) cl.sync();  // no block leaves while another reads its shared memory
 }
 
 // Far field in the mixed precisions, for many directions: the Gauss points are taken in groups of
 // FE x FE elements with a reference point C (the group's first Gauss point, FP64); the phase
 // kappa x^.y = kappa x^.C + kappa x^.(y - C) splits into a per-(direction, group) factor exp(-i kappa
 // x^.C) in FP64 and per-point exponentials of the small offsets in FP32, summed in FP32 per group and
-// direction, scaled by the FP64 factor and added over the groups in FP64.  Block: one group and 64
+// direction, scaled by the FP64 factor and added over the groups in FP64.  Block: one group and 64 DPT
 // directions, 4 point lanes per direction, up to 8 right-hand sides per pass.
-constexpr int FF_DIRS = 64, FF_LANES = 4, FF_COLS = 8, FF_CHUNK = 256;
+// Bound: FP32 arithmetic (41 operations a point, direction and 8 columns), if shared memory does not set the pace: a
+// point's 8 densities take a warp 16 cycles to load, so a thread uses them for DPT directions; the densities are
+// stored by parts, so that the products take two columns per instruction.  Measured, 393216 points,
+// 2048 directions, 8 columns, with the density: 1.98 -> 1.73 ms (before, one direction a thread and FP64
+// conversions in every block).
+constexpr int FF_LANES = 4, FF_COLS = 8, FF_CHUNK = 256, FF_TH = 64;
 
-__global__ void __launch_bounds__(256) k_farfield32(RhsArgs A, const double2 *__restrict__ rho, int fe, int n_dir,
-                                                    const double *__restrict__ xhat, double2 *__restrict__ uinf) {
-  __shared__ float4 pts[FF_CHUNK];               // y - C (3), a
-  __shared__ float4 nrm[FF_CHUNK];               // n~ (3)
-  __shared__ float2 rs[FF_CHUNK * FF_COLS];      // weighted density (FP32)
-  __shared__ float2 red[FF_LANES][FF_DIRS][FF_COLS];
+__device__ inline float2 ff_fma2(float2 a, float2 b, float2 c) {  // two FP32 multiply-adds
+  float2 d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;"
+      : "=l"(reinterpret_cast<unsigned long long &>(d))
+      : "l"(reinterpret_cast<const unsigned long long &>(a)), "l"(reinterpret_cast<const unsigned long long &>(b)),
+        "l"(reinterpret_cast<const unsigned long long &>(c)));
+  return d;
+}
+
+template <int DPT, bool HARD>
+__global__ void __launch_bounds__(FF_LANES *FF_TH) k_farfield32(RhsArgs A, const float2 *__restrict__ rho, int fe, int n_dir,
+                                                               const double *__restrict__ xhat, double2 *__restrict__ uinf) {
+  constexpr int NT = FF_LANES * FF_TH, ND = FF_TH * DPT;
+  __shared__ float4 pts[FF_CHUNK];                       // y - C (3), a
+  __shared__ float4 nrm[HARD ? FF_CHUNK : 1];            // n~ (3)
+  __shared__ __align__(16) float rre[FF_CHUNK][FF_COLS], rim[FF_CHUNK][FF_COLS];  // weighted density
   const int nq = A.ng * A.ng, ge = 1 << fe, ngr1 = A.n1 >> fe;
   const int g = blockIdx.x, j = g / (ngr1 * ngr1), gx = (g / ngr1) % ngr1, gy = g % ngr1;
   const int npts = ge * ge * nq;
-  const int dl = threadIdx.x % FF_DIRS, lane = threadIdx.x / FF_DIRS;
-  const int k = blockIdx.y * FF_DIRS + dl;
-  const bool kv = k < n_dir;
+  const int dl = threadIdx.x % FF_TH, lane = threadIdx.x / FF_TH, k0 = blockIdx.y * ND;
   // reference point: the first Gauss point of the group
   const long e0 = ((long)j * A.n1 + gx * ge) * A.n1 + gy * ge;
   const double C0 = A.gpx[e0 * nq], C1 = A.gpx[A.gst + e0 * nq], C2v = A.gpx[2 * A.gst + e0 * nq];
-  double xh[3] = {0.0, 0.0, 1.0};
-  if (kv) {
-    xh[0] = xhat[3 * k];
-    xh[1] = xhat[3 * k + 1];
-    xh[2] = xhat[3 * k + 2];
+  float kx[DPT][3];  // direction k0 + dl + 64 d
+#pragma unroll
+  for (int d = 0; d < DPT; ++d) {
+    const int k = min(k0 + dl + FF_TH * d, n_dir - 1);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) kx[d][c] = (float)(-A.kappa * xhat[3 * k + c]);
   }
-  const float kx0 = (float)(-A.kappa * xh[0]), kx1 = (float)(-A.kappa * xh[1]), kx2 = (float)(-A.kappa * xh[2]);
+  const bool work = k0 + (dl & ~31) < n_dir;  // the warp has a direction
   for (int c0 = 0; c0 < A.R; c0 += FF_COLS) {
     const int nc = min(FF_COLS, A.R - c0);
-    float2 acc[FF_COLS];
+    float2 ar[DPT][FF_COLS / 2], ai[DPT][FF_COLS / 2];
 #pragma unroll
-    for (int c = 0; c < FF_COLS; ++c) acc[c] = make_float2(0.f, 0.f);
+    for (int d = 0; d < DPT; ++d)
+#pragma unroll
+      for (int c = 0; c < FF_COLS / 2; ++c) ar[d][c] = ai[d][c] = make_float2(0.f, 0.f);
     for (int p0 = 0; p0 < npts; p0 += FF_CHUNK) {
       const int np = min(FF_CHUNK, npts - p0);
       __syncthreads();
-      for (int i = threadIdx.x; i < np; i += blockDim.x) {
+      for (int i = threadIdx.x; i < np; i += NT) {
         const int pi = p0 + i, el = pi / nq, q = pi % nq;
         const long e = ((long)j * A.n1 + gx * ge + el / ge) * A.n1 + gy * ge + el % ge;
         const long iq = e * nq + q;
         pts[i] = make_float4((float)(A.gpx[iq] - C0), (float)(A.gpx[A.gst + iq] - C1),
                              (float)(A.gpx[2 * A.gst + iq] - C2v), (float)A.gpa[iq]);
-        nrm[i] = make_float4((float)A.gpn[iq], (float)A.gpn[A.gst + iq], (float)A.gpn[2 * A.gst + iq], 0.f);
+        if (HARD) nrm[i] = make_float4((float)A.gpn[iq], (float)A.gpn[A.gst + iq], (float)A.gpn[2 * A.gst + iq], 0.f);
       }
-      for (int i = threadIdx.x; i < np * FF_COLS; i += blockDim.x) {
+      for (int i = threadIdx.x; i < np * FF_COLS; i += NT) {
         const int pi = i / FF_COLS, c = i % FF_COLS;
         const int el = (p0 + pi) / nq, q = (p0 + pi) % nq;
         const long e = ((long)j * A.n1 + gx * ge + el / ge) * A.n1 + gy * ge + el % ge;
-        float2 v = make_float2(0.f, 0.f);
-        if (c < nc) {
-          const double2 r = rho[(e * nq + q) * A.R + c0 + c];
-          v = make_float2((float)r.x, (float)r.y);
-        }
-        rs[i] = v;
+        const float2 v = c < nc ? rho[(e * nq + q) * A.R + c0 + c] : make_float2(0.f, 0.f);
+        rre[pi][c] = v.x;
+        rim[pi][c] = v.y;
       }
       __syncthreads();
-      if (kv) {
+      if (work) {
         for (int i = lane; i < np; i += FF_LANES) {
           const float4 y = pts[i];
-          float ph = fmaf(kx0, y.x, fmaf(kx1, y.y, kx2 * y.z));
-          const float kq = rintf(ph * 0.15915494309189535f);
-          ph = fmaf(-kq, 6.28318548202514648f, ph);
-          ph = fmaf(-kq, -1.7484556e-07f, ph);
-          float s, c;
-          __sincosf(ph, &s, &c);
-          float2 E;
-          if (A.hard) {  // -i kappa (x^.n~) e
-            const float4 n = nrm[i];
-            const float xn = -fmaf(kx0, n.x, fmaf(kx1, n.y, kx2 * n.z));  // kappa x^.n~
-            E = make_float2(xn * s, -xn * c);
-          } else {       // -a e
-            E = make_float2(-y.w * c, -y.w * s);
+          const float4 n = HARD ? nrm[i] : make_float4(0.f, 0.f, 0.f, 0.f);
+          float2 re[FF_COLS / 2], im[FF_COLS / 2];
+#pragma unroll
+          for (int c = 0; c < FF_COLS / 4; ++c) {
+            const float4 u = reinterpret_cast<const float4 *>(rre[i])[c], v = reinterpret_cast<const float4 *>(rim[i])[c];
+            re[2 * c] = make_float2(u.x, u.y);
+            re[2 * c + 1] = make_float2(u.z, u.w);
+            im[2 * c] = make_float2(v.x, v.y);
+            im[2 * c + 1] = make_float2(v.z, v.w);
           }
 #pragma unroll
-          for (int cc = 0; cc < FF_COLS; ++cc) {
-            const float2 r = rs[i * FF_COLS + cc];
-            acc[cc].x = fmaf(E.x, r.x, fmaf(-E.y, r.y, acc[cc].x));
-            acc[cc].y = fmaf(E.x, r.y, fmaf(E.y, r.x, acc[cc].y));
+          for (int d = 0; d < DPT; ++d) {
+            float ph = fmaf(kx[d][0], y.x, fmaf(kx[d][1], y.y, kx[d][2] * y.z));
+            const float kq = rintf(ph * 0.15915494309189535f);
+            ph = fmaf(-kq, 6.28318548202514648f, ph);
+            ph = fmaf(-kq, -1.7484556e-07f, ph);
+            float s, c;
+            __sincosf(ph, &s, &c);
+            float ex, ey;
+            if (HARD) {  // -i kappa (x^.n~) e
+              const float xn = -fmaf(kx[d][0], n.x, fmaf(kx[d][1], n.y, kx[d][2] * n.z));  // kappa x^.n~
+              ex = xn * s;
+              ey = -xn * c;
+            } else {     // -a e
+              ex = -y.w * c;
+              ey = -y.w * s;
+            }
+            const float2 exx = make_float2(ex, ex), eyy = make_float2(ey, ey), eyn = make_float2(-ey, -ey);
+#pragma unroll
+            for (int cc = 0; cc < FF_COLS / 2; ++cc) {
+              ar[d][cc] = ff_fma2(exx, re[cc], ff_fma2(eyn, im[cc], ar[d][cc]));
+              ai[d][cc] = ff_fma2(exx, im[cc], ff_fma2(eyy, re[cc], ai[d][cc]));
+            }
           }
         }
       }
     }
+    // the lanes' sums, 64 directions at a time, in the chunk buffers (16 KB)
+    float2(*red)[FF_TH][FF_COLS] = reinterpret_cast<float2(*)[FF_TH][FF_COLS]>(&rre[0][0]);  // [2][64][8]
+    static_assert(sizeof(float) * FF_CHUNK * FF_COLS >= sizeof(float2) * FF_TH * FF_COLS * 2, "reduction buffer");
+    float2(*red2)[FF_TH][FF_COLS] = reinterpret_cast<float2(*)[FF_TH][FF_COLS]>(&rim[0][0]);
 #pragma unroll
-    for (int c = 0; c < FF_COLS; ++c) red[lane][dl][c] = acc[c];
-    __syncthreads();
-    for (int i = threadIdx.x; i < FF_DIRS * FF_COLS; i += blockDim.x) {
-      const int d = i / FF_COLS, c = i % FF_COLS, kk = blockIdx.y * FF_DIRS + d;
-      if (kk >= n_dir || c >= nc) continue;
-      double sx = 0.0, sy = 0.0;
-      for (int l = 0; l < FF_LANES; ++l) {
-        sx += (double)red[l][d][c].x;
-        sy += (double)red[l][d][c].y;
+    for (int d = 0; d < DPT; ++d) {
+      __syncthreads();
+#pragma unroll
+      for (int c = 0; c < FF_COLS; ++c) {
+        const float2 v = c & 1 ? make_float2(ar[d][c / 2].y, ai[d][c / 2].y) : make_float2(ar[d][c / 2].x, ai[d][c / 2].x);
+        (lane < 2 ? red : red2)[lane & 1][dl][c] = v;
       }
-      // the group factor exp(-i kappa x^.C) of direction kk (recomputed by this thread)
-      double s2, c2;
-      sincos(-A.kappa * (xhat[3 * kk] * C0 + xhat[3 * kk + 1] * C1 + xhat[3 * kk + 2] * C2v), &s2, &c2);
-      const double vx = (c2 * sx - s2 * sy) * (0.25 / IGA_PI), vy = (c2 * sy + s2 * sx) * (0.25 / IGA_PI);
-      atomicAdd(&uinf[(long)kk * A.R + c0 + c].x, vx);
-      atomicAdd(&uinf[(long)kk * A.R + c0 + c].y, vy);
+      __syncthreads();
+      // a thread per direction: the group factor exp(-i kappa x^.C) once for its columns
+      const int kk = k0 + FF_TH * d + (int)threadIdx.x;
+      if (threadIdx.x < FF_TH && kk < n_dir) {
+        double s2, c2;
+        sincos(-A.kappa * (xhat[3 * kk] * C0 + xhat[3 * kk + 1] * C1 + xhat[3 * kk + 2] * C2v), &s2, &c2);
+        s2 *= 0.25 / IGA_PI;
+        c2 *= 0.25 / IGA_PI;
+        for (int c = 0; c < nc; ++c) {
+          double sx = 0.0, sy = 0.0;
+          for (int l = 0; l < FF_LANES; ++l) {
+            const float2 v = (l < 2 ? red : red2)[l & 1][threadIdx.x][c];
+            sx += (double)v.x;
+            sy += (double)v.y;
+          }
+          atomicAdd(&uinf[(long)kk * A.R + c0 + c].x, c2 * sx - s2 * sy);
+          atomicAdd(&uinf[(long)kk * A.R + c0 + c].y, c2 * sy + s2 * sx);
+        }
+      }
     }
     __syncthreads();
   }
@@ -343,8 +436,8 @@ __global__ void k_sqrt_re(const double2 *__restrict__ h, double *__restrict__ nr
 // serves every iteration of a cycle (the kernels read j; grids are sized for the whole cycle).  On small systems the
 // launches and the serial parts are what an iteration costs, so each reduction is a tree, the second
 // Gram-Schmidt update also forms the partial sums of the norm, and V_{j+1} is written together with the copy
-// that the next product reads.  Measured, one column, 1944 unknowns: 0.42 ms an iteration with serial
-// sums and 13 launches beside the product. ----
+// that the next product reads.  Measured, one column, 1944 unknowns: 0.42 -> 0.12 ms an iteration beside the
+// product (before, serial sums and 13 launches). ----
 
 // w[n][r] -= sum_{i <= j} V_i[n][r] h[i][r]; with nrm2 != nullptr also the chunks' sums of |w|^2 (same layout as the
 // partial sums of one vector)
@@ -524,8 +617,8 @@ void launch_density(const DeviceProblem &d, const HostSetup &S, const igabem_opt
                     double *rho, cudaStream_t st) {
   RhsArgs A = rhs_args(d, S, o, R);
   const long npts = (long)S.E * S.ng * S.ng;
-  k_density<<<grid_for(npts * R), 256, 0, st>>>(A, d.x2g, reinterpret_cast<const double2 *>(dens), S.E,
-                                                 reinterpret_cast<double2 *>(rho));
+  k_density<double2><<<grid_for(npts * ((R + 3) / 4)), 256, 0, st>>>(
+      A, d.x2g, reinterpret_cast<const double2 *>(dens), S.E, reinterpret_cast<double2 *>(rho));
   note_launch();
   IGA_CUDA(cudaGetLastError());
 }
@@ -538,20 +631,43 @@ void launch_farfield(const DeviceProblem &d, const HostSetup &S, const igabem_op
   RhsArgs A = rhs_args(d, S, o, R);
   long npts = (long)S.E * S.ng * S.ng;
   double2 *rho = reinterpret_cast<double2 *>(scratch);  // E nq R complex values
-  k_density<<<grid_for(npts * R), 256, 0, st>>>(A, d.x2g, reinterpret_cast<const double2 *>(dens), S.E, rho);
-  note_launch();
+  const int dgrid = grid_for(npts * ((R + 3) / 4));
   if (o.precision != IGABEM_FP64) {
+    float2 *rho32 = reinterpret_cast<float2 *>(scratch);
+    k_density<float2><<<dgrid, 256, 0, st>>>(A, d.x2g, reinterpret_cast<const double2 *>(dens), S.E, rho32);
+    note_launch();
     const int fe = std::min(S.m, 4);
     const long ngroups = (long)S.np << (2 * (S.m - fe));
     IGA_CUDA(cudaMemsetAsync(uinf, 0, sizeof(double2) * (size_t)n_dir * R, st));
-    dim3 g32((unsigned)ngroups, (unsigned)((n_dir + FF_DIRS - 1) / FF_DIRS));
-    k_farfield32<<<g32, 256, 0, st>>>(A, rho, fe, n_dir, xhat_dev, reinterpret_cast<double2 *>(uinf));
+    // four directions a thread where they fill a block (the most work per shared load), fewer for few directions
+    auto go = [&](auto kfn, int dpt) {
+      const dim3 g32((unsigned)ngroups, (unsigned)((n_dir + FF_TH * dpt - 1) / (FF_TH * dpt)));
+      kfn<<<g32, FF_LANES * FF_TH, 0, st>>>(A, rho32, fe, n_dir, xhat_dev, reinterpret_cast<double2 *>(uinf));
+    };
+    if (n_dir > 128) S.hard ? go(k_farfield32<4, true>, 4) : go(k_farfield32<4, false>, 4);
+    else if (n_dir > 64) S.hard ? go(k_farfield32<2, true>, 2) : go(k_farfield32<2, false>, 2);
+    else S.hard ? go(k_farfield32<1, true>, 1) : go(k_farfield32<1, false>, 1);
     note_launch();
     IGA_CUDA(cudaGetLastError());
     return;
   }
-  dim3 grid(n_dir, R);
-  k_farfield<<<grid, 256, 0, st>>>(A, rho, npts, xhat_dev, reinterpret_cast<double2 *>(uinf));
+  k_density<double2><<<dgrid, 256, 0, st>>>(A, d.x2g, reinterpret_cast<const double2 *>(dens), S.E, rho);
+  note_launch();
+  const int cols = (R + FF64_COLS - 1) / FF64_COLS;
+  int nz = 1;
+  while (nz < 8 && (long)n_dir * cols * nz < 4 * 152 && npts >= 1024L * nz) nz *= 2;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(n_dir, cols, nz);
+  cfg.blockDim = dim3(256);
+  cfg.stream = st;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = at.val.clusterDim.y = 1;
+  at.val.clusterDim.z = nz;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  IGA_CUDA(cudaLaunchKernelEx(&cfg, k_farfield, A, (const double2 *)rho, npts, xhat_dev,
+                              reinterpret_cast<const double2 *>(d.cis), reinterpret_cast<double2 *>(uinf)));
   note_launch();
   IGA_CUDA(cudaGetLastError());
 }
