@@ -18,17 +18,24 @@
 // goes into a fresh tensor-memory buffer (two buffers, used alternately), which the CUDA cores scale
 // back (by the exact inverse powers of two) and add into FP32 registers, rounded to nearest.
 //
-// Work split: one CTA per (target cluster, column group); a group is up to four slices of at most 64
-// columns of one kernel type (hard: channel 0 is K, channels 1..6 are G), so each thread keeps at most
-// 128 accumulators.  Warps 1..7 generate the coupling block (FP32, with the phase split of the FP32
-// path, the pair factor exp(i kappa |D|) and the pair's scale folded in) straight into A; A is
-// double-buffered, so the block of pair p + 1 is generated, and pair p - 1 is added up, while the
-// tensor core multiplies pair p.  The B operands (X_s scaled and split, already in operand layout) are
-// packed once per matrix-vector product by k_m2l_tc_pack and streamed slice by slice by the bulk-copy
-// engine into three buffers, two slices loading while one multiplies.  One thread of warp 0 issues the
-// MMAs and copies; mbarriers track their completion with waits bounded in time: a wait that runs out
-// sets the status word, the CTA waits (bounded) for its copies and MMAs in flight, frees its tensor
-// memory and returns without writing.
+// Work split: one CTA per (target cluster, column group); a group is the slices of one kernel type (hard: channel 0
+// is K, channels 1..6 are G) whose accumulators fit (128 a thread).  Warps 1..7 generate the coupling block
+// (FP32, with the phase split of the FP32 path, the pair factor exp(i kappa |D|) and the pair's scale folded in)
+// straight into A; A is double-buffered, so the block of pair p + 1 is generated, and pair p - 1 is added
+// up, while the tensor core multiplies pair p.  The B operands (X_s scaled and split, already in operand
+// layout) are packed once per matrix-vector product by k_m2l_tc_pack and streamed part by part (hi, then lo) by
+// the bulk-copy engine into two buffers.  Warp 0 issues the MMAs and copies together (one elected lane): the
+// descriptors stay in uniform registers.  The interaction list with the scales is read once, and the nodes
+// and constants of a pair three pairs ahead, so that no step of a pair waits on memory.  mbarriers
+// track completion with waits bounded in time: a wait that runs out sets the status word, the CTA waits
+// (bounded) for its copies and MMAs in flight, frees its tensor memory and returns without writing.
+//
+// Bound and slice width: an MMA of 128 rows takes about 82 + N / 2 cycles here (the A operand is read from shared
+// memory for every instruction), so slices are as wide as two buffers of one part allow, 192 columns: a pair of
+// the 64-direction sound-hard product is then 3 x 21 instructions instead of 7 x 21.  Measured, 24576 elements,
+// 64 directions: 41.7 -> 22.8 ms (64 columns a slice with descriptors built by one thread, list and node
+// reads in the pair's critical path -> 33.0 ms with uniform descriptors and read-ahead -> 27.6 ms at 96
+// columns -> 22.8 ms at 192).
 //
 // Operand layout (no swizzle, K-major): core matrices of 8 rows x 16 bytes (8 FP16); element (row r, k)
 // at byte ((r / 8) * KC + k / 8) * 128 + (r % 8) * 16 + (k % 8) * 2, KC = K / 8.  Descriptor: leading
@@ -50,10 +57,11 @@ namespace {
 constexpr int TC_THREADS = 256;                            // 8 warps: warp 0 issues, 7 generate
 constexpr int TC_NQW = TC_THREADS / 128;                   // warps per tensor-memory lane quadrant
 constexpr int TC_MAXC = 16 / TC_NQW;                       // 16-column accumulator chunks per thread
-constexpr int TC_NS = 64;                                  // columns of a slice (MMA N <= 64)
+constexpr int TC_NS = 192;                                 // most columns of a slice (MMA N)
 constexpr int TC_MAX_SLOTS = 8;
-constexpr int TC_GROUP = 4;                                // slices per CTA (256 accumulator columns)
-constexpr int TC_NBUF = 3;                                 // B buffers (two copies in flight)
+constexpr int TC_GROUP = 256;                              // accumulator columns of a CTA
+constexpr int TC_NBUF = 2;                                 // buffers of B parts
+constexpr int TC_LIST = 1024;                              // pairs whose sources and scales fit in shared memory
 
 struct TCLevel {
   const int *far_ptr, *far_src;
@@ -91,24 +99,28 @@ __device__ inline void split2(float v0, float v1, uint32_t &hi, uint32_t &lo) {
   lo = *reinterpret_cast<const uint32_t *>(&l);
 }
 
-// byte offset of (r, k) (k even: a pair of FP16 values) in a K-major no-swizzle operand with KC core
-// matrices (8 rows x 8 FP16) along K
-__device__ inline uint32_t op_off(int r, int k, int KC) {
-  return (uint32_t)((((r >> 3) * KC + (k >> 3)) * 8 + (r & 7)) * 16 + (k & 7) * 2);
-}
-
 __device__ inline uint64_t smem_desc(uint32_t addr, int KC) {
   const uint64_t lbo = 128, sbo = (uint64_t)KC * 128;
   return (uint64_t)((addr >> 4) & 0x3FFF) | (((lbo >> 4) & 0x3FFF) << 16) | (((sbo >> 4) & 0x3FFF) << 32) |
          (1ull << 46);
 }
 
-__device__ inline void mma_f16(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
+// issued by the lane with el != 0 of a warp that runs this together: the operands are the same in every lane, so
+// they stay in uniform registers (computed by one thread alone, they were moved there per instruction, which
+// took longer than the products)
+__device__ inline void mma_f16(uint32_t el, uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
   asm volatile(
-      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d),
-      "l"(a), "l"(b), "r"(idesc), "r"(acc)
+      "{\n\t.reg .pred p, q;\n\tsetp.ne.b32 p, %4, 0;\n\tsetp.ne.b32 q, %5, 0;\n\t"
+      "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d),
+      "l"(a), "l"(b), "r"(idesc), "r"(acc), "r"(el)
       : "memory");
+}
+
+__device__ inline void cp_async4(void *dst, const void *src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
+__device__ inline void cp_async16(void *dst, const void *src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
 }
 
 __device__ inline void mma_commit(uint32_t bar) {
@@ -119,27 +131,29 @@ __device__ inline void mma_commit(uint32_t bar) {
 // Constants of one pair for the generation of its coupling block.
 struct TCPair {
   float D0, D1, D2, Dn, DD;  // D = c_t - c_s, |D|, |D|^2
-  float phi0;                // kappa |D| reduced to (-pi, pi]
+  float phi0;                // kappa |D| / (2 pi) reduced to [-1/2, 1/2]
   float fs;                  // the pair's power-of-two scale / (4 pi)
 };
 
 // Kernel sample of type TYPE (0: soft K' - i eta V; 1: hard K; 2: hard G, as node_sample) times the
 // pair factor exp(i kappa |D|) and the pair's scale.  Nodes in shared memory as three float4:
-// [x - c, n~_x][n~_y, n~_z, a, 0][D.(x - c), D.n~, 0, 0] (the last one for sources only; for the
-// target, Dx = D.(x - c) and Dnx = D.n~ are passed in).  The phase is kappa |D| + kappa (r - |D|)
-// with r - |D| = (2 D.d + |d|^2) / (r + |D|), d the difference of the node offsets.
+// [x - c, D.(x - c)][n~, D.n~][a] (D.(x - c) and D.n~ for sources; for the target, Dx and Dnx are passed in).  The
+// phase in turns is kappa / (2 pi) (|D| + (r - |D|)) with r - |D| = (2 D.d + |d|^2) / (r + |D|), d the difference
+// of the node offsets; k2pi = kappa / (2 pi).
 template <int TYPE>
-__device__ inline float2 tc_sample(const TCPair &g, float kappa, float eta, const float4 &x0, const float4 &x1,
-                                   float Dx, float Dnx, const float4 &y0, const float4 &y1, const float4 &y2) {
+__device__ inline float2 tc_sample(const TCPair &g, float kappa, float k2pi, float eta, const float4 &x0, const float4 &x1,
+                                   float ax, float Dx, float Dnx, const float4 *__restrict__ y) {
+  constexpr float M = 12582912.f;  // 1.5 2^23: adding it rounds to an integer
+  const float4 y0 = y[0];
   const float d0 = x0.x - y0.x, d1 = x0.y - y0.y, d2 = x0.z - y0.z;
   const float dd = fmaf(d0, d0, fmaf(d1, d1, d2 * d2));
-  const float num = fmaf(2.f, Dx - y2.x, dd);
+  const float num = fmaf(2.f, Dx - y0.w, dd);
   const float r2 = g.DD + num;
-  const float ir = rsqrtf(r2), r = r2 * ir;
-  float ph = fmaf(kappa, __fdividef(num, r + g.Dn), g.phi0);
-  const float kq = rintf(ph * 0.15915494309189535f);
-  ph = fmaf(-kq, 6.28318548202514648f, ph);
-  ph = fmaf(-kq, -1.7484556e-07f, ph);
+  float ir;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(ir) : "f"(r2));
+  const float r = r2 * ir;
+  const float tn = fmaf(k2pi, __fdividef(num, r + g.Dn), g.phi0);
+  const float ph = (tn - ((tn + M) - M)) * 6.28318530717958647692f;
   float sph, cph;
   __sincosf(ph, &sph, &cph);
   const float f = ir * g.fs;
@@ -147,81 +161,58 @@ __device__ inline float2 tc_sample(const TCPair &g, float kappa, float eta, cons
   const float kr = kappa * r, g2 = f * ir * ir;
   const float dGx = (-cph - sph * kr) * g2, dGy = (-sph + cph * kr) * g2;
   if (TYPE == 1) {  // -a_x ((x - y).n~_y) dG
-    const float dn = y2.y + fmaf(d0, y0.w, fmaf(d1, y1.x, d2 * y1.y));
-    const float w1 = -x1.z * dn;
+    const float4 y1 = y[1];
+    const float dn = y1.w + fmaf(d0, y1.x, fmaf(d1, y1.y, d2 * y1.z));
+    const float w1 = -ax * dn;
     return make_float2(dGx * w1, dGy * w1);
   }
   // a_y ((x - y).n~_x) dG - i eta a_x a_y G
-  const float dn = Dnx + fmaf(d0, x0.w, fmaf(d1, x1.x, d2 * x1.y));
-  const float w1 = y1.z * dn, w2 = x1.z * y1.z * eta;
+  const float ay = y[2].x;
+  const float dn = Dnx + fmaf(d0, x1.x, fmaf(d1, x1.y, d2 * x1.z));
+  const float w1 = ay * dn, w2 = ax * ay * eta;
   return make_float2(fmaf(dGx, w1, sph * f * w2), fmaf(dGy, w1, -cph * f * w2));
 }
 
-// The coupling block of one pair into A (hi at Ahi, lo at Alo) by warps 1..7: 8 x 8 tiles (row
-// a % 8 = lane % 8, column pair b, b + 1 with b % 8 = 2 (lane / 8)), two tiles per step for four
-// independent samples in flight, stored as packed FP16 pairs (conflict-free within a core matrix).
+// The coupling block of one pair into A (hi at Ahi, lo at Alo) by warps 1..7.  A task is 8 consecutive columns of
+// one row: eight independent samples in flight, the source nodes broadcast to the lanes (which take consecutive
+// rows), and one 16-byte store per operand part, quadrant and task (a row of a core matrix; 8 lanes fill one).
 template <int TYPE>
 __device__ void tc_generate(const TCPair &g, float kappa, float eta, const float4 *__restrict__ tn4,
                             const float4 *__restrict__ sn4, uint8_t *__restrict__ Ahi, uint8_t *__restrict__ Alo,
                             int Q, int KH, int KC, int warp, int lane) {
-  const int nb8 = (Q + 7) >> 3, ntile = nb8 * nb8, nw = TC_THREADS / 32 - 1;
-  int it = warp - 1;
-  int ag = it / nb8, bg = it % nb8;
-  auto next = [&](int &ag_, int &bg_) {
-    bg_ += nw;
-    while (bg_ >= nb8) {
-      bg_ -= nb8;
-      ++ag_;
-    }
-  };
-  while (it < ntile) {
-    int ag2 = ag, bg2 = bg;
-    next(ag2, bg2);
-    const bool two = it + nw < ntile;
-    float2 v[2][2];
-    int aa[2], bb[2];
+  const int ntask = (KH >> 3) * Q;
+  const float k2pi = kappa * 0.15915494309189533577f;
+  const uint32_t im = (uint32_t)(KH >> 3) * 128, lower = (uint32_t)KC * 8 * 128;  // -Im / Re half along K; rows 64..
+  for (int task = (warp - 1) * 32 + lane; task < ntask; task += TC_THREADS - 32) {
+    const int g8 = task / Q, a = task - g8 * Q;
+    const float4 x0 = tn4[3 * a], x1 = tn4[3 * a + 1];
+    const float ax = TYPE == 2 ? 0.f : tn4[3 * a + 2].x;
+    const float Dx = fmaf(g.D0, x0.x, fmaf(g.D1, x0.y, g.D2 * x0.z));
+    const float Dnx = TYPE == 0 ? fmaf(g.D0, x1.x, fmaf(g.D1, x1.y, g.D2 * x1.z)) : 0.f;
+    uint32_t rh[4], rl[4], ih[4], il[4];
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int a = (h ? ag2 : ag) * 8 + (lane & 7), b0 = (h ? bg2 : bg) * 8 + 2 * (lane >> 3);
-      aa[h] = a;
-      bb[h] = b0;
-      v[h][0] = v[h][1] = make_float2(0.f, 0.f);
-      if ((h == 0 || two) && a < Q && b0 < Q) {
-        const float4 x0 = tn4[3 * a], x1 = tn4[3 * a + 1];
-        const float Dx = fmaf(g.D0, x0.x, fmaf(g.D1, x0.y, g.D2 * x0.z));
-        const float Dnx = TYPE == 0 ? fmaf(g.D0, x0.w, fmaf(g.D1, x1.x, g.D2 * x1.y)) : 0.f;
+    for (int u = 0; u < 8; u += 2) {
+      float2 v[2];
 #pragma unroll
-        for (int u = 0; u < 2; ++u) {
-          const int b = min(b0 + u, Q - 1);
-          const float4 y0 = sn4[3 * b], y1 = sn4[3 * b + 1], y2 = sn4[3 * b + 2];
-          const float2 w = tc_sample<TYPE>(g, kappa, eta, x0, x1, Dx, Dnx, y0, y1, y2);
-          v[h][u] = b0 + u < Q ? w : make_float2(0.f, 0.f);
-        }
+      for (int h = 0; h < 2; ++h) {
+        const int b = g8 * 8 + u + h;
+        v[h] = tc_sample<TYPE>(g, kappa, k2pi, eta, x0, x1, ax, Dx, Dnx, sn4 + 3 * min(b, Q - 1));
+        if (b >= Q) v[h] = make_float2(0.f, 0.f);
       }
+      split2(v[0].x, v[1].x, rh[u / 2], rl[u / 2]);
+      split2(v[0].y, v[1].y, ih[u / 2], il[u / 2]);
     }
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int a = aa[h], b0 = bb[h];
-      if ((h == 0 || two) && a < Q && b0 < Q) {
-        uint32_t rh, rl, ih, il;
-        split2(v[h][0].x, v[h][1].x, rh, rl);
-        split2(v[h][0].y, v[h][1].y, ih, il);
-        const uint32_t o00 = op_off(a, b0, KC), o01 = op_off(a, KH + b0, KC);
-        const uint32_t o10 = op_off(64 + a, b0, KC), o11 = op_off(64 + a, KH + b0, KC);
-        *reinterpret_cast<uint32_t *>(Ahi + o00) = rh;                // Re S
-        *reinterpret_cast<uint32_t *>(Ahi + o01) = ih ^ 0x80008000u;  // -Im S
-        *reinterpret_cast<uint32_t *>(Ahi + o10) = ih;                // Im S
-        *reinterpret_cast<uint32_t *>(Ahi + o11) = rh;                // Re S
-        *reinterpret_cast<uint32_t *>(Alo + o00) = rl;
-        *reinterpret_cast<uint32_t *>(Alo + o01) = il ^ 0x80008000u;
-        *reinterpret_cast<uint32_t *>(Alo + o10) = il;
-        *reinterpret_cast<uint32_t *>(Alo + o11) = rl;
-      }
-    }
-    it += 2 * nw;
-    ag = ag2;
-    bg = bg2;
-    next(ag, bg);
+    const uint32_t o = (uint32_t)(((a >> 3) * KC + g8) * 128 + (a & 7) * 16);
+    auto put = [&](uint8_t *A, const uint32_t *re, const uint32_t *imv) {
+      const uint4 R = make_uint4(re[0], re[1], re[2], re[3]), I = make_uint4(imv[0], imv[1], imv[2], imv[3]);
+      *reinterpret_cast<uint4 *>(A + o) = R;                  // Re S
+      *reinterpret_cast<uint4 *>(A + o + im) =                // -Im S
+          make_uint4(I.x ^ 0x80008000u, I.y ^ 0x80008000u, I.z ^ 0x80008000u, I.w ^ 0x80008000u);
+      *reinterpret_cast<uint4 *>(A + o + lower) = I;          // Im S
+      *reinterpret_cast<uint4 *>(A + o + lower + im) = R;     // Re S
+    };
+    put(Ahi, rh, ih);
+    put(Alo, rl, il);
   }
 }
 
@@ -229,7 +220,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_m2l_tc(const TCArgs A) {
   extern __shared__ __align__(128) uint8_t smt[];
   __shared__ __align__(8) uint64_t bar_load[TC_NBUF], bar_free[TC_NBUF];
   __shared__ uint32_t tmem_base;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
   int li = 0;
   while (li + 1 < A.nlev && (int)blockIdx.x >= A.lev[li + 1].first) ++li;
   const TCLevel &L = A.lev[li];
@@ -242,16 +233,21 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_m2l_tc(const TCArgs A) {
   for (int jj = 0; jj < nsl; ++jj) W += A.sl.slot_ns[sl0 + jj];
   const uint32_t AB = 128u * K * 2, BB = (uint32_t)TC_NS * K * 2;
   uint8_t *Abuf = smt;            // A buffer u: hi at 2 u AB, lo at (2 u + 1) AB
-  uint8_t *Bbuf = smt + 4 * AB;   // B buffer b: hi at 2 b BB, lo at (2 b + 1) BB
-  float *tn = reinterpret_cast<float *>(smt + 4 * AB + 2 * TC_NBUF * BB);  // target nodes [64][12]
+  uint8_t *Bbuf = smt + 4 * AB;   // B buffer b at b BB
+  float *tn = reinterpret_cast<float *>(smt + 4 * AB + TC_NBUF * BB);  // target nodes [64][12]
   float *snb = tn + 64 * 12;                                               // source nodes [2][64][12]
+  // what the pairs' steps read from memory is brought in ahead of its use: the interaction list with the inverse
+  // scales at the start, the raw nodes and pair constants of the pairs to come by asynchronous copies
+  int *slist = reinterpret_cast<int *>(snb + 2 * 64 * 12);                 // [TC_LIST]
+  float *sinv = reinterpret_cast<float *>(slist + TC_LIST);                // [TC_LIST]
+  float *raw = sinv + TC_LIST;                                             // [4][7][64]
+  float *pcs = raw + 4 * 7 * 64;                                           // [4][8]: D, |D|, |D|^2, phi0, -, fs
   const long NQ = (long)L.n * Q;
   const int k0 = L.far_ptr[t], npairs = L.far_ptr[t + 1] - k0;
 
   // both A buffers are zeroed once: the padding rows and columns are never written
   for (uint32_t i = tid; i < 4 * AB / 16; i += TC_THREADS) reinterpret_cast<uint4 *>(smt)[i] = make_uint4(0, 0, 0, 0);
-  // nodes of cluster cl as [x - c, n~_x][n~_y, n~_z, a, 0][D.(x - c), D.n~, 0, 0] (D of pair kk) by the
-  // threads lo .. lo + nt - 1
+  // nodes of cluster cl as [x - c, D.(x - c)][n~, D.n~][a, 0, 0, 0] (D of pair kk) by the threads lo .. lo + nt - 1
   auto stage_nodes = [&](float *dst, int cl, int kk, int lo, int nt) {
     float Dv[3] = {0.f, 0.f, 0.f};
     if (kk >= 0) {
@@ -265,14 +261,55 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_m2l_tc(const TCArgs A) {
       float v[7];
       for (int c = 0; c < 7; ++c) v[c] = L.nodes32[c * NQ + ia];
       float4 *o = reinterpret_cast<float4 *>(dst + 12 * a);
-      o[0] = make_float4(v[0], v[1], v[2], v[3]);
-      o[1] = make_float4(v[4], v[5], v[6], 0.f);
-      o[2] = make_float4(Dv[0] * v[0] + Dv[1] * v[1] + Dv[2] * v[2], Dv[0] * v[3] + Dv[1] * v[4] + Dv[2] * v[5], 0.f,
-                         0.f);
+      o[0] = make_float4(v[0], v[1], v[2], Dv[0] * v[0] + Dv[1] * v[1] + Dv[2] * v[2]);
+      o[1] = make_float4(v[3], v[4], v[5], Dv[0] * v[3] + Dv[1] * v[4] + Dv[2] * v[5]);
+      o[2] = make_float4(v[6], 0.f, 0.f, 0.f);
     }
   };
   stage_nodes(tn, t, -1, 0, TC_THREADS);
   for (int p = 0; p < 2 && p < npairs; ++p) stage_nodes(snb + p * 768, L.far_src[k0 + p], k0 + p, 0, TC_THREADS);
+  for (int p = tid; p < min(npairs, TC_LIST); p += TC_THREADS) {
+    const int src = L.far_src[k0 + p];
+    slist[p] = src;
+    sinv[p] = 1.0f / (L.pc[8L * (k0 + p) + 7] * L.bscale[src]);
+  }
+  auto src_of = [&](int p) { return p < TC_LIST ? slist[p] : L.far_src[k0 + p]; };
+  // the constants the generation uses: the phase of exp(i kappa |D|) in turns, the scale over 4 pi
+  auto finish_consts = [&](float *c) {
+    c[5] = atan2f(c[6], c[5]) * 0.15915494309189533577f;
+    c[7] *= 0.0795774715459476679f;
+  };
+  if (tid < 2 && tid < npairs) {
+    for (int i = 0; i < 8; ++i) pcs[8 * tid + i] = L.pc[8L * (k0 + tid) + i];
+    finish_consts(pcs + 8 * tid);
+  }
+  auto fetch_raw = [&](int p) {  // warp 1: the raw nodes and constants of pair p into ring slot p & 3
+    const int src = src_of(p);
+    float *r = raw + (p & 3) * 7 * 64;
+    for (int a = lane; a < Q; a += 32)
+#pragma unroll
+      for (int c = 0; c < 7; ++c) cp_async4(r + c * 64 + a, L.nodes32 + c * NQ + (long)src * Q + a);
+    if (lane < 2) cp_async16(pcs + 8 * (p & 3) + 4 * lane, L.pc + 8L * (k0 + p) + 4 * lane);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  auto finish_raw = [&](int p) {  // warp 1: pair p's nodes from the ring into the buffer the generation reads
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncwarp();
+    const float *r = raw + (p & 3) * 7 * 64;
+    float *c = pcs + 8 * (p & 3);
+    const float D0 = c[0], D1 = c[1], D2 = c[2];
+    __syncwarp();
+    if (lane == 0) finish_consts(c);
+    for (int a = lane; a < Q; a += 32) {
+      float v[7];
+#pragma unroll
+      for (int i = 0; i < 7; ++i) v[i] = r[i * 64 + a];
+      float4 *o = reinterpret_cast<float4 *>(snb + (p & 1) * 768 + 12 * a);
+      o[0] = make_float4(v[0], v[1], v[2], D0 * v[0] + D1 * v[1] + D2 * v[2]);
+      o[1] = make_float4(v[3], v[4], v[5], D0 * v[3] + D1 * v[4] + D2 * v[5]);
+      o[2] = make_float4(v[6], 0.f, 0.f, 0.f);
+    }
+  };
   if (tid == 0) {
     for (int b = 0; b < TC_NBUF; ++b) {
       asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&bar_load[b])));
@@ -293,34 +330,35 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_m2l_tc(const TCArgs A) {
   const uint32_t idesc0 = (1u << 4) | ((uint32_t)(128 >> 4) << 24);  // FP32 accumulator, FP16 A and B, K-major
   const uint32_t a_base = smem_u32(Abuf), b_base = smem_u32(Bbuf);
 
-  const long total = (long)npairs * nsl;
+  // items: pair by pair, slice by slice, the hi and the lo part of its B operand
+  const long total = (long)npairs * nsl * 2;
   const size_t img_half = (size_t)CR * K * 2;
-  // issuing thread state
+  // state of the issuing warp
   bool ok = true;
   long n_loaded = 0, n_mma = 0;
   auto issue_load = [&](long j) {
-    const int p = (int)(j / nsl), sl = sl0 + (int)(j % nsl);
-    const int s = L.far_src[k0 + p];
-    const uint8_t *img = L.bimg + (size_t)s * 2 * img_half + (size_t)A.sl.slot_r0[sl] * K * 2;
+    const int p = (int)(j / (2 * nsl)), rest = (int)(j - (long)p * 2 * nsl), sl = sl0 + (rest >> 1);
+    const uint8_t *img = L.bimg + ((size_t)src_of(p) * 2 + (rest & 1)) * img_half + (size_t)A.sl.slot_r0[sl] * K * 2;
     const uint32_t bytes = (uint32_t)A.sl.slot_ns[sl] * K * 2;
     const uint32_t b = (uint32_t)(j % TC_NBUF), bar = smem_u32(&bar_load[b]);
-    mbar_expect(bar, 2 * bytes);
-    bulk_load(b_base + 2 * b * BB, img, bytes, bar);
-    bulk_load(b_base + (2 * b + 1) * BB, img + img_half, bytes, bar);
-    n_loaded = j + 1;
+    mbar_expect(bar, bytes);
+    bulk_load(b_base + b * BB, img, bytes, bar);
   };
-  if (tid == 0)
-    for (long j = 0; j < TC_NBUF - 1 && j < total; ++j) issue_load(j);
+  if (warp == 0)
+    for (long j = 0; j < TC_NBUF - 1 && j < total; ++j) {
+      if (lane == 0) issue_load(j);
+      n_loaded = j + 1;
+    }
+  __syncwarp();
+  if (warp == 1 && npairs > 2) fetch_raw(2);
 
   // coupling block of pair p into A buffer p & 1 (source nodes in snb[p & 1]) by warps 1..7; warp 0
   // issues the MMAs
   const float kappa = A.kappa, eta = A.eta;
   auto generate = [&](int p) {
     if (warp > 0) {
-      const int kk = k0 + p;
-      const float4 p0 = reinterpret_cast<const float4 *>(L.pc)[2 * kk];
-      const float4 p1 = reinterpret_cast<const float4 *>(L.pc)[2 * kk + 1];
-      const TCPair g{p0.x, p0.y, p0.z, p0.w, p1.x, atan2f(p1.z, p1.y), p1.w * 0.0795774715459476679f};
+      const float *c = pcs + 8 * (p & 3);
+      const TCPair g{c[0], c[1], c[2], c[3], c[4], c[5], c[7]};
       uint8_t *Ahi = Abuf + 2 * (p & 1) * AB, *Alo = Ahi + AB;
       const float4 *tn4 = reinterpret_cast<const float4 *>(tn);
       const float4 *sn4 = reinterpret_cast<const float4 *>(snb + (p & 1) * 768);
@@ -343,8 +381,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_m2l_tc(const TCArgs A) {
     for (int i = 0; i < 16; ++i) acc[c][i] = 0.f;
   const int cq = warp >> 2, nch = (W / 16 - cq + TC_NQW - 1) / TC_NQW;
   auto drain = [&](int p) {  // adds pair p's buffer, scaled back, to the accumulators
-    const int kk = k0 + p;
-    const float inv = 1.0f / (L.pc[8L * kk + 7] * L.bscale[L.far_src[kk]]);
+    const float inv = p < TC_LIST ? sinv[p] : 1.0f / (L.pc[8L * (k0 + p) + 7] * L.bscale[L.far_src[k0 + p]]);
     const uint32_t base = tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)((p & 1) * A.wmax + 16 * cq);
 #pragma unroll
     for (int c = 0; c < TC_MAXC; ++c) {
@@ -364,57 +401,72 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_m2l_tc(const TCArgs A) {
   };
 
   if (npairs > 0) generate(0);
-  // completion of item j (slice j % nsl of pair j / nsl): its buffer and the parity of its phase
+  // completion of item j: its buffer and the parity of its phase
   auto wait_free = [&](long j) { return mbar_wait(smem_u32(&bar_free[j % TC_NBUF]), (uint32_t)(j / TC_NBUF) & 1); };
   for (int p = 0; p < npairs; ++p) {
     // the MMAs of pair p - 1 have finished: its tensor-memory buffer is final and its A buffer (the one
     // pair p + 1 is generated into) is free
-    if (tid == 0 && ok && p > 0) ok = wait_free((long)p * nsl - 1);
-    if (__syncthreads_or(tid == 0 && !ok)) break;
+    if (warp == 0 && ok && p > 0) ok = __all_sync(0xffffffffu, wait_free((long)p * nsl * 2 - 1));
+    if (__syncthreads_or(!ok)) break;
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    if (tid == 0) {
-      const uint32_t ah = a_base + 2 * (p & 1) * AB, al = ah + AB;
+    if (warp == 0) {
+      const uint32_t el = lane == 0;
+      const uint32_t ah = a_base + 2 * (p & 1) * AB;
+      const uint64_t dah = smem_desc(ah, KC), dal = smem_desc(ah + AB, KC);
       uint32_t off = (uint32_t)((p & 1) * A.wmax);
-      for (int jj = 0; jj < nsl && ok; ++jj) {
+      for (int jj = 0; jj < 2 * nsl && ok; ++jj) {
         const long j = n_mma;
         const uint32_t b = (uint32_t)(j % TC_NBUF);
-        ok = mbar_wait(smem_u32(&bar_load[b]), (uint32_t)(j / TC_NBUF) & 1);
+        ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bar_load[b]), (uint32_t)(j / TC_NBUF) & 1));
         if (!ok) break;
-        const int ns = A.sl.slot_ns[sl0 + jj];
-        const uint32_t idesc = idesc0 | ((uint32_t)(ns >> 3) << 17);
-        const uint32_t bh = b_base + 2 * b * BB, bl = bh + BB;
-        for (int ks = 0; ks < K / 16; ++ks) {
-          const uint32_t o = (uint32_t)ks * 256;
-          mma_f16(tmem + off, smem_desc(ah + o, KC), smem_desc(bh + o, KC), idesc, ks > 0 ? 1u : 0u);
-          mma_f16(tmem + off, smem_desc(ah + o, KC), smem_desc(bl + o, KC), idesc, 1u);
-          mma_f16(tmem + off, smem_desc(al + o, KC), smem_desc(bh + o, KC), idesc, 1u);
+        const int ns = A.sl.slot_ns[sl0 + (jj >> 1)];
+        const uint32_t idesc = idesc0 | ((uint32_t)(ns >> 3) << 17), d = tmem + off;
+        // the operands' descriptors advance by 256 bytes (16 units of 16 bytes) per K step of 16
+        const uint64_t db = smem_desc(b_base + b * BB, KC);
+        if ((jj & 1) == 0) {  // hi part: hi hi + lo hi
+          mma_f16(el, d, dah, db, idesc, 0u);
+          mma_f16(el, d, dal, db, idesc, 1u);
+#pragma unroll 4
+          for (uint32_t ks = 16; ks < (uint32_t)K; ks += 16) {
+            mma_f16(el, d, dah + ks, db + ks, idesc, 1u);
+            mma_f16(el, d, dal + ks, db + ks, idesc, 1u);
+          }
+        } else {              // lo part: hi lo
+#pragma unroll 4
+          for (uint32_t ks = 0; ks < (uint32_t)K; ks += 16) mma_f16(el, d, dah + ks, db + ks, idesc, 1u);
+          off += ns;
         }
-        mma_commit(smem_u32(&bar_free[b]));
+        if (el) mma_commit(smem_u32(&bar_free[b]));
         n_mma = j + 1;
-        off += ns;
-        // slice j + NBUF - 1 goes into the buffer of item j - 1 once its MMAs have read it
+        // item j + NBUF - 1 goes into the buffer of item j - 1 once its MMAs have read it
         const long jn = j + TC_NBUF - 1;
         if (jn < total && jn >= n_loaded) {
-          if (j >= 1) ok = wait_free(j - 1);
-          if (ok) issue_load(jn);
+          if (j >= 1) ok = __all_sync(0xffffffffu, wait_free(j - 1));
+          if (ok && el) issue_load(jn);
+          if (ok) n_loaded = jn + 1;
+          __syncwarp();
         }
       }
     }
-    // while the tensor core multiplies pair p: add up pair p - 1, generate pair p + 1, stage the nodes
-    // of pair p + 2 (into the buffer pair p used)
+    // while the tensor core multiplies pair p: add up pair p - 1, generate pair p + 1, put the nodes of
+    // pair p + 2 into the buffer pair p used and request those of pair p + 3
+    if (warp == 1) {
+      if (p + 2 < npairs) finish_raw(p + 2);
+      if (p + 3 < npairs) fetch_raw(p + 3);
+    }
     if (p > 0) drain(p - 1);
     if (p + 1 < npairs) generate(p + 1);
-    if (p + 2 < npairs && warp == 0) stage_nodes(snb + (p & 1) * 768, L.far_src[k0 + p + 2], k0 + p + 2, 0, 32);
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   }
   // every MMA and copy issued by this CTA completes before its memory is released
-  if (tid == 0) {
+  asm volatile("cp.async.wait_all;" ::: "memory");
+  if (warp == 0) {
     if (n_mma > 0) ok = wait_free(n_mma - 1) && ok;
     for (long j = n_mma; j < n_loaded; ++j)
       ok = mbar_wait(smem_u32(&bar_load[j % TC_NBUF]), (uint32_t)(j / TC_NBUF) & 1) && ok;
     if (!ok) atomicExch(A.status, 1);
   }
-  const bool failed = __syncthreads_or(tid == 0 && !ok);
+  const bool failed = __syncthreads_or(!ok);
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   if (!failed) {
     if (npairs > 0) drain(npairs - 1);
@@ -509,24 +561,29 @@ __global__ void __launch_bounds__(256) k_m2l_tc_pack(const double2 *__restrict__
 int tc_kh(int Q) { return (Q + 7) / 8 * 8; }
 
 size_t tc_smem_bytes(int KH) {
-  return (size_t)4 * 128 * (2 * KH) * 2 + (size_t)2 * TC_NBUF * TC_NS * (2 * KH) * 2 + (64 * 12 + 2 * 64 * 12) * 4;
+  return (size_t)4 * 128 * (2 * KH) * 2 + (size_t)TC_NBUF * TC_NS * (2 * KH) * 2 + (64 * 12 + 2 * 64 * 12) * 4 +
+         (2 * TC_LIST + 4 * 7 * 64 + 4 * 8) * 4;
 }
 
-// slices of at most 64 columns within one kernel type, grouped up to four at a time
+// slices of at most TC_NS columns within one kernel type, of even widths (multiples of 16), grouped while their
+// accumulators fit
 TCSlices tc_slices(const HostSetup &S, int R) {
   TCSlices T{};
   const int CR = (S.hard ? 7 : 1) * R;
   auto add_type = [&](int r0, int r1, int type) {
-    int first = T.nslot;
-    for (int r = r0; r < r1; r += TC_NS) {
+    const int first = T.nslot, n = (r1 - r0 + TC_NS - 1) / TC_NS, w = ((r1 - r0 + n - 1) / n + 15) / 16 * 16;
+    for (int r = r0; r < r1; r += w) {
       T.slot_r0[T.nslot] = r;
-      T.slot_ns[T.nslot] = std::min(TC_NS, r1 - r);
+      T.slot_ns[T.nslot] = std::min(w, r1 - r);
       T.slot_type[T.nslot] = type;
       ++T.nslot;
     }
-    for (int f = first; f < T.nslot; f += TC_GROUP) {
+    // as many groups as the accumulators need, with equal numbers of slices
+    const int per = std::max(1, TC_GROUP / w), slots = T.nslot - first, groups = (slots + per - 1) / per,
+              each = (slots + groups - 1) / groups;
+    for (int f = first; f < T.nslot; f += each) {
       T.group_first[T.ngroup] = f;
-      T.group_n[T.ngroup] = std::min(TC_GROUP, T.nslot - f);
+      T.group_n[T.ngroup] = std::min(each, T.nslot - f);
       ++T.ngroup;
     }
   };
@@ -551,8 +608,8 @@ bool m2l_tc_supported(const HostSetup &S, int R) {
   if (Q > 64 || R % 16 != 0 || S.L - S.lmin + 1 > 16) return false;
   for (int l = S.lmin; l <= S.L; ++l)
     if (S.lev[l].q != S.q) return false;  // one operand layout per launch: the same q on every level
-  // slice count: hard R <= 64 gives 1 + 6, soft CR <= 512 gives 8
-  if ((S.hard && R > TC_NS) || (!S.hard && CR > TC_MAX_SLOTS * TC_NS)) return false;
+  // slices of the widest problems: hard R = 64 gives 1 + 2, soft CR = 512 gives 3
+  if ((S.hard && R > 64) || (!S.hard && CR > 512)) return false;
   return tc_smem_bytes(tc_kh(Q)) <= (size_t)max_optin_smem();
 }
 
