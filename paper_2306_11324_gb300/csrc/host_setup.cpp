@@ -361,22 +361,6 @@ static void csr_of_pairs(const std::vector<std::pair<int, int>> &pairs, int n, s
   for (int i : by_col) col[fill[pairs[i].first]++] = pairs[i].second;
 }
 
-// body(i) for i in [0, n) on up to 16 host threads (independent iterations writing disjoint data)
-template <class F>
-static void parallel_for(long n, const F &body) {
-  const long nt = std::min<long>(std::min<long>(16, std::max(1u, std::thread::hardware_concurrency())), n);
-  if (nt <= 1) {
-    for (long i = 0; i < n; ++i) body(i);
-    return;
-  }
-  std::vector<std::thread> th;
-  for (long k = 0; k < nt; ++k)
-    th.emplace_back([&, k] {
-      for (long i = k; i < n; i += nt) body(i);
-    });
-  for (auto &t : th) t.join();
-}
-
 static double dist3(const double *a, const double *b) {
   return std::sqrt((a[0] - b[0]) * (a[0] - b[0]) + (a[1] - b[1]) * (a[1] - b[1]) +
                    (a[2] - b[2]) * (a[2] - b[2]));

@@ -3,12 +3,14 @@
 
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstddef>
 #include <cstdint>
 #include <functional>
 #include <memory>
 #include <mutex>
 #include <string>
+#include <thread>
 #include <vector>
 
 #include "../../include/igabem.h"
@@ -189,6 +191,22 @@ struct GeoCache {
 // call's products when hit does not apply (or nullptr)
 void build_setup(const std::vector<Patch> &patches, const igabem_options &opt, HostSetup &S,
                  const GeoCache *hit = nullptr, GeoCache *fill = nullptr);
+
+// body(i) for i in [0, n) on up to 16 host threads (independent iterations writing disjoint data)
+template <class F>
+void parallel_for(long n, const F &body) {
+  const long nt = std::min<long>(std::min<long>(16, std::max(1u, std::thread::hardware_concurrency())), n);
+  if (nt <= 1) {
+    for (long i = 0; i < n; ++i) body(i);
+    return;
+  }
+  std::vector<std::thread> th;
+  for (long k = 0; k < nt; ++k)
+    th.emplace_back([&, k] {
+      for (long i = k; i < n; i += nt) body(i);
+    });
+  for (auto &t : th) t.join();
+}
 
 // Gauss-Legendre rule on [0,1] (Newton iteration on P_n).
 void gauss_legendre01(int n, std::vector<double> &x, std::vector<double> &w);

@@ -161,7 +161,7 @@ __global__ void __launch_bounds__(128) k_pot_m2m(PotArgs P, PotLevel Lp, PotLeve
 // node with its columns' sums in registers.  In FP32 the phase is split about the box centres
 // (kappa |D| in FP64 plus kappa (r - |D|), r - |D| = (2 D.d + |d|^2) / (r + |D|)) and the products take two
 // columns per instruction; the sums of 64 source nodes, then of their groups, are added to Z in FP64.
-// Measured on 4001 points around 6144 Gauss points, q = 7, 372,000 pairs (FP32): 1520 -> 28 ms a call, host
+// Measured on 4001 points around 6144 Gauss points, q = 7, 372,000 pairs (FP32): 1520 -> 22 ms a call, host
 // tree included (before: a sample per pair with FP64 differences and sums, and per-node Lagrange values in
 // P2M).
 constexpr int POT_COLS = 16, POT_ROWS = 128, POT_STEP = 64;
@@ -433,12 +433,25 @@ extern "C" int igabem_potential(igabem_problem *P, int n_rhs, const void *densit
       return std::min(n - 1, std::max(0, (int)((v - lo[c]) / side * n)));
     };
     if (!o.no_fmm) {
+      // a point's cell on level l is its cell on level 10 shifted: Morton codes sorted once give every level's counts
+      auto spread = [](unsigned v) {  // 10 bits, two zeros between neighbours
+        v = (v | v << 16) & 0x030000FFu;
+        v = (v | v << 8) & 0x0300F00Fu;
+        v = (v | v << 4) & 0x030C30C3u;
+        return (v | v << 2) & 0x09249249u;
+      };
+      std::vector<unsigned> code(G);
+      for (long i = 0; i < G; ++i)
+        code[i] = spread(cell(gx[i], 0, 10)) << 2 | spread(cell(gx[G + i], 1, 10)) << 1 | spread(cell(gx[2 * G + i], 2, 10));
+      std::sort(code.begin(), code.end());
       for (D = 1; D < 10; ++D) {
-        std::unordered_map<Key, int, KeyHash> cnt;
-        int mx = 0;
-        for (long i = 0; i < G; ++i) {
-          const int v = ++cnt[Key{pack(cell(gx[i], 0, D), cell(gx[G + i], 1, D), cell(gx[2 * G + i], 2, D))}];
-          mx = std::max(mx, v);
+        const int sh = 3 * (10 - D);
+        long mx = 0;
+        for (long i = 0; i < G;) {
+          long e = i;
+          while (e < G && code[e] >> sh == code[i] >> sh) ++e;
+          mx = std::max(mx, e - i);
+          i = e;
         }
         if (mx <= 64) break;
       }
@@ -537,30 +550,71 @@ extern "C" int igabem_potential(igabem_problem *P, int n_rhs, const void *densit
         ht[l - 1][p] |= ht[l][b];
       }
     }
-    // dual traversal: admissible pairs per level (CSR by target), near leaf pairs
+    // dual traversal: admissible pairs per level with their box offsets, near leaf pairs.  The candidates of a level go
+    // over host threads in chunks, whose lists are joined in order (as one thread would form them).
+    struct Box {
+      int i, j, k;
+    };
+    std::vector<std::vector<Box>> box(D + 1);
+    for (int l = 0; l <= D; ++l) {
+      box[l].reserve(keys[l].size());
+      for (long long v : keys[l]) box[l].push_back({int(v >> 42), int((v >> 21) & 0x1FFFFF), int(v & 0x1FFFFF)});
+    }
     const double cap = o.kappa_cap > 0 ? o.kappa_cap : INFINITY;
-    std::vector<std::vector<std::pair<int, int>>> far(D + 1);
+    struct FarPair {
+      int t, s;
+      short dx, dy, dz;  // box offset, below 2^10 in size
+    };
+    std::vector<std::vector<FarPair>> far(D + 1);
     std::vector<std::pair<int, int>> near, cand{{0, 0}}, nxt;
     if (!(ht[0][0] && hs[0][0])) cand.clear();
     for (int l = 0; l <= D; ++l) {
-      nxt.clear();
       const double rad = side / (1 << l) * std::sqrt(3.0) / 2;
-      for (auto [t, s] : cand) {
-        const double *ct = &cen[l][3 * t], *cs = &cen[l][3 * s];
-        const double dist = std::sqrt((ct[0] - cs[0]) * (ct[0] - cs[0]) + (ct[1] - cs[1]) * (ct[1] - cs[1]) +
-                                      (ct[2] - cs[2]) * (ct[2] - cs[2])) - 2 * rad;
-        const bool adm = !o.no_fmm && dist > 0 && 2 * rad <= o.eta_adm * dist && o.kappa * 2 * rad <= cap;
-        if (adm) {
-          far[l].push_back({t, s});
-        } else if (l == D) {
-          near.push_back({t, s});
-        } else {
-          for (int a = 0; a < 8; ++a)
+      const long n = (long)cand.size(), nch = std::min<long>(64, (n + 8191) / 8192);
+      struct Part {
+        std::vector<FarPair> far;
+        std::vector<std::pair<int, int>> near, next;
+      };
+      std::vector<Part> part(nch);
+      parallel_for(nch, [&](long c) {
+        Part &q_ = part[c];
+        for (long i = n * c / nch; i < n * (c + 1) / nch; ++i) {
+          const int t = cand[i].first, s = cand[i].second;
+          const double *ct = &cen[l][3 * t], *cs = &cen[l][3 * s];
+          const double dist = std::sqrt((ct[0] - cs[0]) * (ct[0] - cs[0]) + (ct[1] - cs[1]) * (ct[1] - cs[1]) +
+                                        (ct[2] - cs[2]) * (ct[2] - cs[2])) - 2 * rad;
+          const bool adm = !o.no_fmm && dist > 0 && 2 * rad <= o.eta_adm * dist && o.kappa * 2 * rad <= cap;
+          if (adm) {
+            const Box &bt = box[l][t], &bs = box[l][s];
+            q_.far.push_back({t, s, short(bt.i - bs.i), short(bt.j - bs.j), short(bt.k - bs.k)});
+          } else if (l == D) {
+            q_.near.push_back({t, s});
+          } else {
+            int sb[8], ns = 0;  // the source box's children with sources
             for (int b = 0; b < 8; ++b) {
-              const int ta = child[l][8 * t + a], sb = child[l][8 * s + b];
-              if (ta >= 0 && sb >= 0 && ht[l + 1][ta] && hs[l + 1][sb]) nxt.push_back({ta, sb});
+              const int ch = child[l][8 * s + b];
+              if (ch >= 0 && hs[l + 1][ch]) sb[ns++] = ch;
             }
+            for (int a = 0; a < 8; ++a) {
+              const int ta = child[l][8 * t + a];
+              if (ta < 0 || !ht[l + 1][ta]) continue;
+              for (int b = 0; b < ns; ++b) q_.next.push_back({ta, sb[b]});
+            }
+          }
         }
+      });
+      size_t nf = 0, nn = 0;
+      for (const Part &q_ : part) {
+        nf += q_.far.size();
+        nn += q_.next.size();
+      }
+      far[l].reserve(nf);
+      nxt.clear();
+      nxt.reserve(nn);
+      for (const Part &q_ : part) {
+        far[l].insert(far[l].end(), q_.far.begin(), q_.far.end());
+        near.insert(near.end(), q_.near.begin(), q_.near.end());
+        nxt.insert(nxt.end(), q_.next.begin(), q_.next.end());
       }
       cand.swap(nxt);
     }
@@ -581,44 +635,34 @@ extern "C" int igabem_potential(igabem_problem *P, int n_rhs, const void *densit
     for (int l = 0; l <= D; ++l) {
       const size_t n = far[l].size();
       if (n == 0) continue;
-      auto box = [&](int b, int &i, int &j, int &k) {
-        const long long v = keys[l][b];
-        i = int(v >> 42);
-        j = int((v >> 21) & 0x1FFFFF);
-        k = int(v & 0x1FFFFF);
-      };
-      std::vector<long long> off(n);  // the offset packed (each component below 2^11 in size, made positive)
       int most = 0;
-      for (size_t i = 0; i < n; ++i) {
-        int a0, a1, a2, b0, b1, b2;
-        box(far[l][i].first, a0, a1, a2);
-        box(far[l][i].second, b0, b1, b2);
-        most = std::max({most, std::abs(a0 - b0), std::abs(a1 - b1), std::abs(a2 - b2)});
-        off[i] = pack(a0 - b0 + 2048, a1 - b1 + 2048, a2 - b2 + 2048);
-      }
-      std::vector<int> order(n);
+      for (const FarPair &f : far[l]) most = std::max({most, std::abs((int)f.dx), std::abs((int)f.dy), std::abs((int)f.dz)});
       const long w = 2L * most + 1;
-      if (w * w * w <= 1 << 20) {  // counting sort over the offsets' cube
-        auto id = [&](long long v) {
-          return ((long(v >> 42) - 2048 + most) * w + (long((v >> 21) & 0x1FFFFF) - 2048 + most)) * w +
-                 (long(v & 0x1FFFFF) - 2048 + most);
-        };
-        std::vector<int> cnt(w * w * w + 1, 0);
-        for (size_t i = 0; i < n; ++i) cnt[id(off[i]) + 1]++;
-        for (long i = 0; i < w * w * w; ++i) cnt[i + 1] += cnt[i];
-        for (size_t i = 0; i < n; ++i) order[cnt[id(off[i])]++] = (int)i;
-      } else {
-        for (size_t i = 0; i < n; ++i) order[i] = (int)i;
-        std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return off[x] < off[y]; });
-      }
+      auto id = [&](const FarPair &f) { return ((f.dx + most) * w + f.dy + most) * w + f.dz + most; };
       fpair[l].resize(n);
-      for (size_t i = 0; i < n; ++i) {
-        const int o = order[i];
-        fpair[l][i] = make_int2(far[l][o].first, far[l][o].second);
-        if (i == 0 || off[o] != off[order[i - 1]] || chunk[l].back().count == per)
-          chunk[l].push_back({(int)i, 0, int(off[o] >> 42) - 2048, int((off[o] >> 21) & 0x1FFFFF) - 2048,
-                              int(off[o] & 0x1FFFFF) - 2048});
-        chunk[l].back().count++;
+      auto add_chunks = [&](size_t first, size_t count, const FarPair &f) {
+        for (size_t i = 0; i < count; i += per)
+          chunk[l].push_back({(int)(first + i), (int)std::min<size_t>(per, count - i), f.dx, f.dy, f.dz});
+      };
+      if (w * w * w <= 1 << 20) {  // counting sort over the offsets' cube
+        std::vector<int> first(w * w * w + 1, 0);
+        for (const FarPair &f : far[l]) first[id(f) + 1]++;
+        for (long i = 0; i < w * w * w; ++i) {
+          const int c = first[i + 1];
+          if (c)
+            add_chunks(first[i], c,
+                       {0, 0, short(i / (w * w) - most), short(i / w % w - most), short(i % w - most)});
+          first[i + 1] += first[i];
+        }
+        for (const FarPair &f : far[l]) fpair[l][first[id(f)]++] = make_int2(f.t, f.s);
+      } else {
+        std::stable_sort(far[l].begin(), far[l].end(), [&](const FarPair &x, const FarPair &y) { return id(x) < id(y); });
+        for (size_t i = 0; i < n;) {
+          size_t e = i;
+          for (; e < n && id(far[l][e]) == id(far[l][i]); ++e) fpair[l][e] = make_int2(far[l][e].t, far[l][e].s);
+          add_chunks(i, e - i, far[l][i]);
+          i = e;
+        }
       }
     }
     int lmin = D + 1;
