@@ -1,5 +1,6 @@
 // Leaf-level kernels of the matrix-vector product, one thread block per leaf cluster:
-//   * near-field SpMV over the leaf's near blocks (HBM-bound);
+//   * products with dense leaf blocks: the preconditioner, and near fields with blocks of more than 256 rows (the
+//     others: k_stream.cu);
 //   * P2M: channel fields of u = sum x_l psi_l at the leaf's Gauss points, projected onto the
 //     leaf's tensor Chebyshev basis (Sec. 4.4);
 //   * L2P: local expansions evaluated at the Gauss points and tested against the leaf's B-splines.
@@ -106,21 +107,18 @@ __global__ void k_near_spmv2(LeafArgs A, const int *__restrict__ near_ptr, const
   }
 }
 
-// Near-field SpMV for many columns: one thread block per (target leaf, chunk of 64 columns).  Each
-// near block and the source leaf's coefficients (converted to the block's precision) are staged in
-// shared memory; each thread owns a 4 x 4 tile of (local function, column) outputs.  One block's sum
-// is formed in the storage precision, the blocks are summed in FP64, as in k_near_spmv2.
+// Products with dense FP64 leaf blocks for many columns (the preconditioner's, one block per leaf): one thread block
+// per (target leaf, chunk of 64 columns).  Each block and the source leaf's coefficients are staged in shared
+// memory; each thread owns a 4 x 4 tile of (local function, column) outputs.
 constexpr int NM_COLS = 64;
 
-template <class BT>
 __global__ void __launch_bounds__(256) k_near_mrhs(LeafArgs A, const int *__restrict__ near_ptr,
-                                                   const int *__restrict__ near_src, const BT *__restrict__ blk,
+                                                   const int *__restrict__ near_src, const double2 *__restrict__ blk,
                                                    const double2 *__restrict__ xX, double2 *__restrict__ yleaf,
                                                    int nL) {
-  using RT = decltype(BT::x);
   extern __shared__ __align__(16) unsigned char smn[];
-  BT *Bs = reinterpret_cast<BT *>(smn);  // [nL (source)][nL (target)]
-  BT *Xs = Bs + nL * nL;                 // [nL][NM_COLS]
+  double2 *Bs = reinterpret_cast<double2 *>(smn);  // [nL (source)][nL (target)]
+  double2 *Xs = Bs + nL * nL;                 // [nL][NM_COLS]
   const int t = blockIdx.x, r0 = blockIdx.y * NM_COLS, Rc = min(NM_COLS, A.R - r0);
   const int nlL = 1 << A.L, e1 = 1 << A.b;
   const int ti = threadIdx.x >> 4, tr = threadIdx.x & 15;
@@ -132,26 +130,26 @@ __global__ void __launch_bounds__(256) k_near_mrhs(LeafArgs A, const int *__rest
     const int js = s / (nlL * nlL), cx = (s / nlL) % nlL, cy = s % nlL;
     const long base = ((long)js * A.nb + cx * e1) * A.nb + cy * e1;
     __syncthreads();  // the previous block's products are done
-    const BT *Bk = blk + (size_t)k * nL * nL;
+    const double2 *Bk = blk + (size_t)k * nL * nL;
     for (int e = threadIdx.x; e < nL * nL; e += blockDim.x) Bs[e] = Bk[e];
     for (int e = threadIdx.x; e < nL * NM_COLS; e += blockDim.x) {
       const int jj = e / NM_COLS, c = e % NM_COLS, al = jj / A.nL1, be = jj % A.nL1;
-      BT v;
+      double2 v;
       v.x = 0;
       v.y = 0;
       if (c < Rc) {
         const double2 xd = xX[(base + (long)al * A.nb + be) * A.R + r0 + c];
-        v.x = (RT)xd.x;
-        v.y = (RT)xd.y;
+        v.x = xd.x;
+        v.y = xd.y;
       }
       Xs[e] = v;
     }
     __syncthreads();
-    RT px[4][4], py[4][4];
+    double px[4][4], py[4][4];
     for (int m = 0; m < 4; ++m)
       for (int n = 0; n < 4; ++n) px[m][n] = py[m][n] = 0;
     for (int jj = 0; jj < nL; ++jj) {
-      BT bv[4], xv[4];
+      double2 bv[4], xv[4];
 #pragma unroll
       for (int m = 0; m < 4; ++m) {
         const int i = ti + 16 * m;
@@ -185,12 +183,11 @@ __global__ void __launch_bounds__(256) k_near_mrhs(LeafArgs A, const int *__rest
     }
 }
 
-// Near-field SpMV for up to 16 columns per block: one thread block per (target leaf, column chunk),
-// one thread per (local function i, CPT adjacent columns).  The near blocks of the target's list are
-// staged in shared memory by asynchronous copies (cp.async), double buffered: block k + 1 is in flight
-// while block k is multiplied, one barrier per block; the source coefficients (converted to the block
-// precision) go through registers.  One block's sum is formed in the storage precision, the blocks
-// are summed in FP64 (as in k_near_spmv2).
+// Products with dense FP64 leaf blocks for up to 16 columns per block (the preconditioner's): one thread block per
+// (target leaf, column chunk), one thread per (local function i, CPT adjacent columns).  The blocks of the
+// target's list are staged in shared memory by asynchronous copies (cp.async), double buffered: block k + 1
+// is in flight while block k is multiplied, one barrier per block; the source coefficients go through
+// registers.
 template <int BYTES>
 __device__ inline void cp_async(void *dst, const void *src) {
   const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
@@ -199,26 +196,25 @@ __device__ inline void cp_async(void *dst, const void *src) {
 __device__ inline void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 __device__ inline void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
 
-template <class BT, int CPT>
+template <int CPT>
 __global__ void __launch_bounds__(576) k_near_cols(LeafArgs A, const int *__restrict__ near_ptr,
-                                                   const int *__restrict__ near_src, const BT *__restrict__ blk,
-                                                   const double2 *__restrict__ xX, const float2 *__restrict__ x32,
-                                                   double2 *__restrict__ yleaf, int nL, int Rc) {
-  using RT = decltype(BT::x);
+                                                   const int *__restrict__ near_src, const double2 *__restrict__ blk,
+                                                   const double2 *__restrict__ xX, double2 *__restrict__ yleaf, int nL,
+                                                   int Rc) {
   extern __shared__ __align__(16) unsigned char smk[];
-  BT *Bs = reinterpret_cast<BT *>(smk);              // [2][nL * nL] (block column-major: [j][i])
-  BT *Xs = Bs + 2 * nL * nL;                         // [2][nL][Rc]
+  double2 *Bs = reinterpret_cast<double2 *>(smk);              // [2][nL * nL] (block column-major: [j][i])
+  double2 *Xs = Bs + 2 * nL * nL;                         // [2][nL][Rc]
   const int t = blockIdx.x, r0 = blockIdx.y * Rc, rc = min(Rc, A.R - r0);
   const int nlL = 1 << A.L, e1 = 1 << A.b;
   const int nthr = blockDim.x, nB = nL * nL, nX = nL * Rc;
   const int i = threadIdx.x % nL, cg = threadIdx.x / nL, c0 = cg * CPT;
   const bool active = cg * CPT < Rc;
   const int kb = near_ptr[t], ke = near_ptr[t + 1];
-  BT rx[2];
+  double2 rx[2];
   auto issue_block = [&](int k, int buf) {  // asynchronous copy of near block k into buffer buf
-    const BT *Bk = blk + (size_t)k * nB;
-    BT *dst = Bs + buf * nB;
-    for (int e = threadIdx.x; e < nB; e += nthr) cp_async<sizeof(BT)>(dst + e, Bk + e);
+    const double2 *Bk = blk + (size_t)k * nB;
+    double2 *dst = Bs + buf * nB;
+    for (int e = threadIdx.x; e < nB; e += nthr) cp_async<sizeof(double2)>(dst + e, Bk + e);
     cp_async_commit();
   };
   auto fetch_x = [&](int k) {  // this thread's share of block k's source coefficients
@@ -234,15 +230,7 @@ __global__ void __launch_bounds__(576) k_near_cols(LeafArgs A, const int *__rest
         const int jj = e / Rc, c = e % Rc, al = jj / A.nL1, be = jj % A.nL1;
         if (c < rc) {
           const long ix = (base + (long)al * A.nb + be) * A.R + r0 + c;
-          if constexpr (sizeof(RT) == 4) {  // FP32 blocks: the FP32 copy of the input
-            const float2 xf = x32[ix];
-            rx[u].x = xf.x;
-            rx[u].y = xf.y;
-          } else {
-            const double2 xd = xX[ix];
-            rx[u].x = xd.x;
-            rx[u].y = xd.y;
-          }
+          rx[u] = xX[ix];
         }
       }
     }
@@ -254,20 +242,9 @@ __global__ void __launch_bounds__(576) k_near_cols(LeafArgs A, const int *__rest
       if (e < nX) Xs[buf * nX + e] = rx[u];
     }
   };
-  // the blocks' sums: FP64 for FP64 blocks; for FP32 blocks an FP32 sum with a compensation term
-  // (Neumaier), as accurate as an FP64 sum here without FP64 arithmetic
   double2 acc[CPT];
-  float2 sh[CPT], sl[CPT];
 #pragma unroll
-  for (int c = 0; c < CPT; ++c) {
-    acc[c] = make_double2(0.0, 0.0);
-    sh[c] = sl[c] = make_float2(0.f, 0.f);
-  }
-  auto nsum = [](float &hi, float &lo, float v) {
-    const float t = hi + v;
-    lo += fabsf(hi) >= fabsf(v) ? (hi - t) + v : (v - t) + hi;
-    hi = t;
-  };
+  for (int c = 0; c < CPT; ++c) acc[c] = make_double2(0.0, 0.0);
   if (kb < ke) {
     issue_block(kb, 0);
     fetch_x(kb);
@@ -282,30 +259,25 @@ __global__ void __launch_bounds__(576) k_near_cols(LeafArgs A, const int *__rest
   for (int k = kb; k < ke; ++k) {
     const int cur = (k - kb) & 1;
     if (active) {
-      RT px[CPT], py[CPT];
+      double px[CPT], py[CPT];
 #pragma unroll
       for (int c = 0; c < CPT; ++c) px[c] = py[c] = 0;
-      const BT *B = Bs + cur * nB + i;
-      const BT *X = Xs + cur * nX + c0;
+      const double2 *B = Bs + cur * nB + i;
+      const double2 *X = Xs + cur * nX + c0;
       for (int jj = 0; jj < nL; ++jj) {
-        const BT bv = B[jj * nL];
+        const double2 bv = B[jj * nL];
 #pragma unroll
         for (int c = 0; c < CPT; ++c) {
           if (c0 + c >= Rc) break;  // odd chunk width: the last thread of a row has one column
-          const BT xv = X[jj * Rc + c];
+          const double2 xv = X[jj * Rc + c];
           px[c] += bv.x * xv.x - bv.y * xv.y;
           py[c] += bv.x * xv.y + bv.y * xv.x;
         }
       }
 #pragma unroll
       for (int c = 0; c < CPT; ++c) {
-        if constexpr (sizeof(RT) == 4) {
-          nsum(sh[c].x, sl[c].x, (float)px[c]);
-          nsum(sh[c].y, sl[c].y, (float)py[c]);
-        } else {
-          acc[c].x += (double)px[c];
-          acc[c].y += (double)py[c];
-        }
+        acc[c].x += px[c];
+        acc[c].y += py[c];
       }
     }
     if (k + 1 < ke) store_x(cur ^ 1);  // coefficients of block k + 1
@@ -319,27 +291,25 @@ __global__ void __launch_bounds__(576) k_near_cols(LeafArgs A, const int *__rest
   if (active) {
 #pragma unroll
     for (int c = 0; c < CPT; ++c) {
-      if (sizeof(RT) == 4) acc[c] = make_double2((double)sh[c].x + (double)sl[c].x, (double)sh[c].y + (double)sl[c].y);
       if (c0 + c < rc) yleaf[((size_t)t * nL + i) * A.R + r0 + c0 + c] = acc[c];
     }
   }
 }
 
 // launch of k_near_cols: columns per thread 2 (1 for a single column), chunks of up to 16 columns
-template <class BT>
-bool launch_near_cols(const LeafArgs &A, const int *near_ptr, const int *near_src, const BT *blk, const double2 *xX,
-                      const float2 *x32, double2 *yleaf, int nleaf, int nL, int R, cudaStream_t st) {
+bool launch_near_cols(const LeafArgs &A, const int *near_ptr, const int *near_src, const double2 *blk, const double2 *xX,
+                      double2 *yleaf, int nleaf, int nL, int R, cudaStream_t st) {
   const int Rc = std::min(R, 16), cpt = Rc >= 2 ? 2 : 1;
   const int threads = ((nL * ((Rc + cpt - 1) / cpt) + 31) / 32) * 32;
   if (threads > 576 || (size_t)nL * Rc > 2 * (size_t)threads) return false;
-  const size_t smem = sizeof(BT) * 2 * ((size_t)nL * nL + (size_t)nL * Rc);
+  const size_t smem = sizeof(double2) * 2 * ((size_t)nL * nL + (size_t)nL * Rc);
   dim3 grid(nleaf, (R + Rc - 1) / Rc);
   if (cpt == 2) {
-    IGA_CUDA(set_max_dynamic_smem(k_near_cols<BT, 2>, smem));
-    k_near_cols<BT, 2><<<grid, threads, smem, st>>>(A, near_ptr, near_src, blk, xX, x32, yleaf, nL, Rc);
+    IGA_CUDA(set_max_dynamic_smem(k_near_cols<2>, smem));
+    k_near_cols<2><<<grid, threads, smem, st>>>(A, near_ptr, near_src, blk, xX, yleaf, nL, Rc);
   } else {
-    IGA_CUDA(set_max_dynamic_smem(k_near_cols<BT, 1>, smem));
-    k_near_cols<BT, 1><<<grid, threads, smem, st>>>(A, near_ptr, near_src, blk, xX, x32, yleaf, nL, Rc);
+    IGA_CUDA(set_max_dynamic_smem(k_near_cols<1>, smem));
+    k_near_cols<1><<<grid, threads, smem, st>>>(A, near_ptr, near_src, blk, xX, yleaf, nL, Rc);
   }
   note_launch();
   return true;
@@ -931,8 +901,8 @@ void launch_block_apply(const DeviceProblem &d, const HostSetup &S, const igabem
                         cudaStream_t st) {
   LeafArgs A = leaf_args(d, S, o, R);
   const int nleaf = S.lev[S.L].n, nout = S.nL * R, threads = 256;
-  if (R <= 16 && launch_near_cols<double2>(A, d.ident_ptr, d.ident_src, reinterpret_cast<const double2 *>(d.binv),
-                                           reinterpret_cast<const double2 *>(d.xX), nullptr,
+  if (R <= 16 && launch_near_cols(A, d.ident_ptr, d.ident_src, reinterpret_cast<const double2 *>(d.binv),
+                                           reinterpret_cast<const double2 *>(d.xX),
                                            reinterpret_cast<double2 *>(d.yleaf), nleaf, S.nL, R, st)) {
     IGA_CUDA(cudaGetLastError());
     return;
@@ -940,8 +910,8 @@ void launch_block_apply(const DeviceProblem &d, const HostSetup &S, const igabem
   if (R >= 8 && S.nL <= 64) {
     dim3 grid(nleaf, (R + NM_COLS - 1) / NM_COLS);
     const size_t smem = sizeof(double2) * ((size_t)S.nL * S.nL + (size_t)S.nL * NM_COLS);
-    IGA_CUDA(set_max_dynamic_smem(k_near_mrhs<double2>, smem));
-    k_near_mrhs<double2><<<grid, threads, smem, st>>>(A, d.ident_ptr, d.ident_src,
+    IGA_CUDA(set_max_dynamic_smem(k_near_mrhs, smem));
+    k_near_mrhs<<<grid, threads, smem, st>>>(A, d.ident_ptr, d.ident_src,
                                                       reinterpret_cast<const double2 *>(d.binv),
                                                       reinterpret_cast<const double2 *>(d.xX),
                                                       reinterpret_cast<double2 *>(d.yleaf), S.nL);
