@@ -4,6 +4,7 @@
 
 #include "internal.h"
 #include "k_common.cuh"
+#include "k_m2l.cuh"
 #include "kernels.h"
 
 namespace igabem {
@@ -561,6 +562,285 @@ __global__ void k_near_regular_f(NearArgs A, int smem_block) {
   }
 }
 
+// Regular element pairs with 4 x 4 Gauss points and leaves of 1, 2 or 4 elements per direction (E1): the leaf pair
+// as a whole.  The Gauss points of a leaf form a tensor grid, so the block
+//   B[k][l] = sum_{x, y} phi_k(x) ks(x, y) phi_l(y) + gc(x, y) c_k(x) . c_l(y)
+// is contracted one direction at a time instead of per element pair.  A thread owns one target point x and sums
+// over the source points along the second direction, then along the first (a window of P1 rows of functions); a
+// finished row goes to shared memory, where the target points are contracted the same way.  With the curl
+// c_l = phi1' phi2 F_t - phi1 phi2' F_s the sound-hard part is three sums per target point: ks against phi_l, and
+// gc F_t(x), gc F_s(x) against c_l.  Touching element pairs are left out by a mask.  256 threads hold 256 target
+// points: one leaf pair, or 4 or 16 of the smaller ones; each entry is written by one thread (the singular
+// quadrature adds to it later).  Bound: the kernel samples (FP32 issue, FP64 arithmetic).  Measured against
+// k_near_regular_f, p = 2, element tables included: leaves of 4 x 4, 97752 pairs sound-soft FP32 59.6 -> 23.4 ms,
+// 24804 sound-hard FP32 29.6 -> 12.7 ms; leaves of 2 x 2, 29152 pairs sound-soft FP64 19.7 -> 11.0 ms.
+template <class T, int P1, int E1, bool HARD> struct NearTensor {
+  using V = typename std::conditional<sizeof(T) == 4, float2, double2>::type;
+  static constexpr int ND = 4 * E1, NX = ND * ND, NP = 256 / NX, F = E1 + P1 - 1, NL = F * F;
+  static constexpr int PT = HARD ? 12 : 4;   // source point: y, a; sound-hard y, n~, F_t, F_s
+  static constexpr int NB = HARD ? 8 : 4;    // target 1, 2, source 1, 2: values; then derivatives
+  static constexpr int CH = HARD ? 3 : 1, CV = HARD ? 2 : 1;
+  static constexpr size_t pts = (size_t)256 * PT * sizeof(T);
+  static constexpr size_t bas = (size_t)NP * NB * ND * P1 * sizeof(T);     // [NP][NB][ND][P1]
+  static constexpr size_t t = (size_t)NP * CH * F * NX * sizeof(V);        // [NP][CH][F][NX]
+  static constexpr size_t v = (size_t)NP * ND * CV * F * F * sizeof(V);    // [NP][ND][CV][F target][F source]
+  static constexpr size_t total = pts + bas + t + v;
+};
+
+template <class T, int P1, int E1, bool HARD>
+__global__ void __launch_bounds__(256) k_near_tensor(NearArgs A, int n_pairs, const double2 *__restrict__ cis) {
+  using K = NearTensor<T, P1, E1, HARD>;
+  using V = typename K::V;
+  constexpr int ND = K::ND, NX = K::NX, NP = K::NP, F = K::F, NL = K::NL, PT = K::PT, NB = K::NB, CH = K::CH,
+                CV = K::CV;
+  static_assert(!HARD || sizeof(T) == 4, "the sound-hard form keeps 3 P1 F sums in registers: FP32");
+  extern __shared__ __align__(16) unsigned char smn[];
+  T *ys = reinterpret_cast<T *>(smn), *bas = reinterpret_cast<T *>(smn + K::pts);
+  V *ts = reinterpret_cast<V *>(smn + K::pts + K::bas), *vs = reinterpret_cast<V *>(smn + K::pts + K::bas + K::t);
+  const int tid = threadIdx.x, z = tid / NX, xi = tid % NX, x1 = xi / ND, x2 = xi % ND;
+  const int bid = min((int)blockIdx.x * NP + z, n_pairs - 1);
+  const int tgt = A.near_tgt[bid], src = A.near_src[bid], nlL = 1 << A.L;
+  const int jt = tgt / (nlL * nlL), ixt = (tgt / nlL) % nlL * E1, iyt = tgt % nlL * E1;
+  const int js = src / (nlL * nlL), ixs = (src / nlL) % nlL * E1, iys = src % nlL * E1;
+  // this thread's target point and the source point with its index
+  const int e = (jt * A.n1 + ixt + x1 / 4) * A.n1 + iyt + x2 / 4, q = (x1 % 4) * 4 + x2 % 4;
+  const int es = (js * A.n1 + ixs + x1 / 4) * A.n1 + iys + x2 / 4;
+  const T *tp = static_cast<const T *>(A.tab_pts);
+  T X[7], Ft[HARD ? 3 : 1], Fs[HARD ? 3 : 1];
+#pragma unroll
+  for (int c = 0; c < 7; ++c) X[c] = tp[((long)e * 16 + q) * 7 + c];
+  {
+    const T *Y = tp + ((long)es * 16 + q) * 7;
+    T *o = ys + (size_t)tid * PT;
+    for (int c = 0; c < 3; ++c) {
+      o[c] = Y[c];
+      if constexpr (HARD) {
+        o[3 + c] = Y[3 + c];
+        o[6 + c] = (T)A.gft[c * A.gstride + (long)es * 16 + q];
+        o[9 + c] = (T)A.gfs[c * A.gstride + (long)es * 16 + q];
+        Ft[c] = (T)A.gft[c * A.gstride + (long)e * 16 + q];
+        Fs[c] = (T)A.gfs[c * A.gstride + (long)e * 16 + q];
+      }
+    }
+    if constexpr (!HARD) o[3] = Y[6];
+  }
+  // univariate basis values (and derivatives) times the Gauss weights (target: times h^4 in the first direction)
+  for (int w = xi; w < NB * ND * P1; w += NX) {
+    const int side = w / (ND * P1) % 4, g = w / P1 % ND, f = w % P1;
+    const int col = (side == 0 ? ixt : side == 1 ? iyt : side == 2 ? ixs : iys) + g / 4;
+    const double *b = w < 4 * ND * P1 ? A.phi1 : A.dphi1;
+    double v = b[(col * 4 + g % 4) * P1 + f] * A.gw[g % 4];
+    if (side == 0) v *= A.h * A.h * A.h * A.h;
+    bas[(size_t)z * NB * ND * P1 + w] = (T)v;
+  }
+  // source elements (ex, ey) that touch this point's element
+  unsigned touch = 0;
+  {
+    auto mark = [&](int f) {
+      const int jf = f / (A.n1 * A.n1), fx = (f / A.n1) % A.n1 - ixs, fy = f % A.n1 - iys;
+      if (f >= 0 && jf == js && fx >= 0 && fx < E1 && fy >= 0 && fy < E1) touch |= 1u << (fx * E1 + fy);
+    };
+    mark(e);
+    for (int c = 0; c < A.nbr_w; ++c) mark(A.nbr[(long)e * A.nbr_w + c]);
+  }
+  __syncthreads();
+  const T *bs = bas + (size_t)z * NB * ND * P1;
+  const T kappa = (T)A.kappa, eta = (T)A.eta;
+  double c0 = 0, c1 = 0;
+  if constexpr (sizeof(T) == 8) phase64_scale(A.kappa, c0, c1);
+  auto sample = [&](const T *y) {  // sound-soft, K' - i eta V at (x, y): cfie_kernel_t without the normal of y
+    V k;
+    const T d0 = X[0] - y[0], d1 = X[1] - y[1], d2 = X[2] - y[2];
+    const T r2 = d0 * d0 + d1 * d1 + d2 * d2, dn = d0 * X[3] + d1 * X[4] + d2 * X[5];
+    if constexpr (sizeof(T) == 4) {
+      const T ir = rsqrtf(r2), r = r2 * ir, f = ir * (T)(0.25 / IGA_PI), kr = kappa * r, g2 = f * ir * ir;
+      T sn, cs;
+      sincosf(kr, &sn, &cs);
+      const T w1 = y[3] * dn, w2 = X[6] * y[3] * eta * f;
+      k.x = (-cs - sn * kr) * g2 * w1 + sn * w2;
+      k.y = (-sn + cs * kr) * g2 * w1 - cs * w2;
+    } else {
+      const T ir = rsqrt64(r2), w = y[3] * (0.25 / IGA_PI) * ir, gw = dn * ir * w;
+      const Phase64 ph = phase64(cis, r2 * ir, c0, c1);
+      const T Ar = -gw * ir, Br = fma(kappa, gw, -(X[6] * eta) * w);
+      const C2<double> v = phase_mul(ph.E.x * Ar - ph.E.y * Br, ph.E.x * Br + ph.E.y * Ar, ph);
+      k.x = v.x;
+      k.y = v.y;
+    }
+    return k;
+  };
+  auto add = [](V &s, T w, V k) {
+    s.x += w * k.x;
+    s.y += w * k.y;
+  };
+  // window of P1 rows of functions along the first source direction
+  V acc[CH][P1][F];
+#pragma unroll
+  for (int c = 0; c < CH; ++c)
+#pragma unroll
+    for (int f = 0; f < P1; ++f)
+#pragma unroll
+      for (int g = 0; g < F; ++g) acc[c][f][g].x = acc[c][f][g].y = (T)0;
+  for (int ex = 0; ex < F; ++ex) {
+    if (ex < E1) {
+      for (int q1 = 0; q1 < 4; ++q1) {
+        const T *b1 = bs + (2 * ND + ex * 4 + q1) * P1;
+        if constexpr (!HARD) {
+          V u[F];
+#pragma unroll
+          for (int g = 0; g < F; ++g) u[g].x = u[g].y = (T)0;
+#pragma unroll
+          for (int ey = 0; ey < E1; ++ey) {
+            if (touch >> (ex * E1 + ey) & 1) continue;
+#pragma unroll
+            for (int q2 = 0; q2 < 4; ++q2) {
+              const V k = sample(ys + ((size_t)z * NX + (ex * 4 + q1) * ND + ey * 4 + q2) * PT);
+              const T *b = bs + (3 * ND + ey * 4 + q2) * P1;
+#pragma unroll
+              for (int f = 0; f < P1; ++f) add(u[ey + f], b[f], k);
+            }
+          }
+#pragma unroll
+          for (int f = 0; f < P1; ++f)
+#pragma unroll
+            for (int g = 0; g < F; ++g) add(acc[0][f][g], b1[f], u[g]);
+        } else {
+          const T *d1 = b1 + 4 * ND * P1;
+#pragma unroll
+          for (int ey = 0; ey < E1; ++ey) {
+            if (touch >> (ex * E1 + ey) & 1) continue;
+            // sums against phi2 of ks, gc F_t(x).F_t(y), gc F_s(x).F_t(y); against phi2' of gc F_t(x).F_s(y),
+            // gc F_s(x).F_s(y)
+            V u[5][P1];
+#pragma unroll
+            for (int c = 0; c < 5; ++c)
+#pragma unroll
+              for (int f = 0; f < P1; ++f) u[c][f].x = u[c][f].y = (T)0;
+#pragma unroll
+            for (int q2 = 0; q2 < 4; ++q2) {
+              const T *y = ys + ((size_t)z * NX + (ex * 4 + q1) * ND + ey * 4 + q2) * PT;
+              const T *b = bs + (3 * ND + ey * 4 + q2) * P1, *d = b + 4 * ND * P1;
+              const PK<T> pk = cfie_kernel_t<T>(true, kappa, eta, X, X + 3, X[6], y, y + 3, (T)0);
+              auto scaled = [&](const T *a, const T *c) {
+                const T m = a[0] * c[0] + a[1] * c[1] + a[2] * c[2];
+                V k;
+                k.x = pk.gcx * m;
+                k.y = pk.gcy * m;
+                return k;
+              };
+              V k;
+              k.x = pk.ksx;
+              k.y = pk.ksy;
+              const V tt = scaled(Ft, y + 6), st = scaled(Fs, y + 6), t_s = scaled(Ft, y + 9), ss = scaled(Fs, y + 9);
+#pragma unroll
+              for (int f = 0; f < P1; ++f) {
+                add(u[0][f], b[f], k);
+                add(u[1][f], b[f], tt);
+                add(u[2][f], b[f], st);
+                add(u[3][f], d[f], t_s);
+                add(u[4][f], d[f], ss);
+              }
+            }
+#pragma unroll
+            for (int f = 0; f < P1; ++f)
+#pragma unroll
+              for (int g = 0; g < P1; ++g) {
+                add(acc[0][f][ey + g], b1[f], u[0][g]);
+                add(acc[CH - 2][f][ey + g], d1[f], u[1][g]);
+                add(acc[CH - 2][f][ey + g], -b1[f], u[3][g]);
+                add(acc[CH - 1][f][ey + g], d1[f], u[2][g]);
+                add(acc[CH - 1][f][ey + g], -b1[f], u[4][g]);
+              }
+          }
+        }
+      }
+    }
+    // function row ex is complete: to shared memory, and the target points contracted
+#pragma unroll
+    for (int c = 0; c < CH; ++c)
+#pragma unroll
+      for (int g = 0; g < F; ++g) {
+        ts[((size_t)(z * CH + c) * F + g) * NX + xi] = acc[c][0][g];
+#pragma unroll
+        for (int f = 0; f + 1 < P1; ++f) acc[c][f][g] = acc[c][f + 1][g];
+        acc[c][P1 - 1][g].x = acc[c][P1 - 1][g].y = (T)0;
+      }
+    __syncthreads();
+    // second direction: sum_x2 phi_k2(x2) T[x1, x2] (sound-hard: phi_k2 T_K - phi_k2' T_s, and phi_k2 T_t)
+    for (int w = tid; w < NP * ND * CV * F; w += 256) {
+      const int l = w % F, c = w / F % CV, r = w / (F * CV) % ND, pz = w / (F * CV * ND);
+      const T *b = bas + (size_t)pz * NB * ND * P1 + ND * P1;
+      V u[F];
+#pragma unroll
+      for (int g = 0; g < F; ++g) u[g].x = u[g].y = (T)0;
+      const V *t = ts + ((size_t)(pz * CH + c) * F + l) * NX + r * ND;
+#pragma unroll
+      for (int g2 = 0; g2 < ND; ++g2)
+#pragma unroll
+        for (int f = 0; f < P1; ++f) add(u[g2 / 4 + f], b[g2 * P1 + f], t[g2]);
+      if (HARD && c == 0) {
+        const V *t2 = t + (size_t)2 * F * NX;
+        const T *d = b + 4 * ND * P1;
+#pragma unroll
+        for (int g2 = 0; g2 < ND; ++g2)
+#pragma unroll
+          for (int f = 0; f < P1; ++f) add(u[g2 / 4 + f], -d[g2 * P1 + f], t2[g2]);
+      }
+#pragma unroll
+      for (int g = 0; g < F; ++g) vs[((((size_t)pz * ND + r) * CV + c) * F + g) * F + l] = u[g];
+    }
+    __syncthreads();
+    // first direction: the entries (k1 F + k2, ex F + l)
+    for (int w = tid; w < NP * F * F; w += 256) {
+      const int k2 = w % F, l = w / F % F, pz = w / (F * F);
+      if (blockIdx.x * NP + pz >= n_pairs) break;
+      V u[F];
+#pragma unroll
+      for (int g = 0; g < F; ++g) u[g].x = u[g].y = (T)0;
+#pragma unroll
+      for (int c = 0; c < CV; ++c) {
+        const V *v = vs + (((size_t)pz * ND * CV + c) * F + k2) * F + l;
+        const T *b = bas + (size_t)pz * NB * ND * P1 + (c ? 4 * ND * P1 : 0);
+#pragma unroll
+        for (int g1 = 0; g1 < ND; ++g1)
+#pragma unroll
+          for (int f = 0; f < P1; ++f) add(u[g1 / 4 + f], b[g1 * P1 + f], v[(size_t)g1 * CV * F * F]);
+      }
+      double2 *o = A.blk + ((size_t)blockIdx.x * NP + pz) * NL * NL + (size_t)(ex * F + l) * NL + k2;
+#pragma unroll
+      for (int g = 0; g < F; ++g) o[g * F] = cmk((double)u[g].x, (double)u[g].y);
+    }
+  }
+}
+
+// launches k_near_tensor where it takes the problem: 4 Gauss points, p <= 2, leaves of up to 4 x 4 elements, sound-hard
+// in FP32 alone (in FP64 its sums don't fit the registers; k_near_regular_f stays).  Larger leaves would need
+// more sums than registers too.  Milliseconds before -> now on 6 patches of 8 x 8 (leaves of 1), 16 x 16 (2 x 2), 32 x 32
+// (4 x 4): soft FP32 p = 2 0.32 -> 0.07, 1.04 -> 0.38, 14.3 -> 5.1; p = 0 0.26 -> 0.05, 1.18 -> 0.27, 18.1 -> 3.4; soft
+// FP64 p = 2 2.09 -> 0.65, 16.1 -> 9.1, 264 -> 145; hard FP32 p = 2 0.59 -> 0.17, 2.12 -> 1.08, 29.1 -> 12.5.
+template <class T, bool HARD>
+bool launch_near_tensor(const NearArgs &A, int n_pairs, const double2 *cis, cudaStream_t st) {
+  if (A.ng != 4 || A.p > 2 || A.b > 2) return false;
+  auto go = [&](auto p1, auto e1) {
+    constexpr int P1 = decltype(p1)::value, E1 = decltype(e1)::value;
+    using K = NearTensor<T, P1, E1, HARD>;
+    IGA_CUDA(set_max_dynamic_smem(k_near_tensor<T, P1, E1, HARD>, K::total));
+    k_near_tensor<T, P1, E1, HARD><<<(n_pairs + K::NP - 1) / K::NP, 256, K::total, st>>>(A, n_pairs, cis);
+    note_launch();
+  };
+  auto by_leaf = [&](auto p1) {
+    if (A.b == 0) go(p1, std::integral_constant<int, 1>{});
+    else if (A.b == 1) go(p1, std::integral_constant<int, 2>{});
+    else go(p1, std::integral_constant<int, 4>{});
+  };
+  if (A.p == 1) by_leaf(std::integral_constant<int, 2>{});
+  else if (A.p == 2) by_leaf(std::integral_constant<int, 3>{});
+  else if constexpr (!HARD) by_leaf(std::integral_constant<int, 1>{});
+  else return false;
+  IGA_CUDA(cudaGetLastError());
+  return true;
+}
+
 // ----------------------------------------------------------------------------------------------
 // touching element pairs: regularising transforms (identical 8, common edge 6, common vertex 4
 // regions) with the canonical position given by the square symmetries (Te, Tf) found on the host.
@@ -1021,6 +1301,10 @@ void launch_near_field(const DeviceProblem &d, const HostSetup &S, const igabem_
                                                     (double *)A.tab_cuw);
       note_launch();
     }
+    const double2 *cis = reinterpret_cast<const double2 *>(d.cis);
+    const bool whole = S.hard ? f32 && launch_near_tensor<float, true>(A, nblk, cis, st)
+                       : f32  ? launch_near_tensor<float, false>(A, nblk, cis, st)
+                              : launch_near_tensor<double, false>(A, nblk, cis, st);
     // the fused kernel keeps Tm (and Tc) in registers: p <= 2, and p = 3 for sound-soft
     const bool fused = nloc == 4 || nloc == 9 || (nloc == 16 && !S.hard);
     const size_t per = (size_t)(fused ? near_fused_scratch(nq, nloc, S.hard) : near_regular_scratch(nq, nloc, S.hard)) * tsz;
@@ -1033,7 +1317,9 @@ void launch_near_field(const DeviceProblem &d, const HostSetup &S, const igabem_
       IGA_CUDA(set_max_dynamic_smem(kfn, smem));
       kfn<<<nblk, 32 * warps, smem, st>>>(A, smem_block);
     };
-    if (fused) {
+    if (whole) {
+      // done
+    } else if (fused) {
       const bool h = S.hard;
       if (f32) {
         if (nloc == 4) h ? go(k_near_regular_f<float, 4, true>) : go(k_near_regular_f<float, 4, false>);
@@ -1051,7 +1337,7 @@ void launch_near_field(const DeviceProblem &d, const HostSetup &S, const igabem_
       IGA_CUDA(set_max_dynamic_smem(k_near_regular_t<double>, smem));
       k_near_regular_t<double><<<nblk, 32 * warps, smem, st>>>(A, smem_block);
     }
-    note_launch();
+    if (!whole) note_launch();
     IGA_CUDA(cudaGetLastError());
   }
   Phase ph(d.prof, IGABEM_PH_SETUP_SINGULAR, st);
