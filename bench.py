@@ -90,10 +90,10 @@ DEFAULT = "deformed_soft_6x256x256_p2_k50-60_8dirs"
 PRECISIONS = {}                              # name -> igabem_precision (filled once the binding is loaded)
 FLOPS_PER_SAMPLE = {False: 40, True: 52}     # FP32 M2L kernel-sample arithmetic: soft 40 flops, hard 52 per pair of samples
 FLOPS_PER_MAC = 8                            # one complex multiply-add
-# DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) of one k_near_singular launch per 4-D point,
-# from one ncu capture of the small sweep case (29.6 + 22.7 MB for 92,130,000 points); the traffic of a
-# launch grows with its points (block writes per pair, rule and net reads per chunk)
-SINGULAR_DRAM_BYTES_PER_POINT = 52.274424e6 / 92130000
+# DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) of one k_sing_tensor launch per 4-D point,
+# from one ncu capture at 1536 elements (10.06 + 30.09 MB for 23,010,000 points); the traffic of a
+# launch grows with its points (block writes, nets and tables per pair)
+SINGULAR_DRAM_BYTES_PER_POINT = 40.141984e6 / 23010000
 
 
 def hbm_peak_gbs():
@@ -105,33 +105,24 @@ def hbm_peak_gbs():
 
 
 def singular_flops(info, p, hard, pg=4):
-    """FP64 operations of the touching pairs' quadrature (the model behind the roofline of
-    k_near_singular), from the counts the library reports.  Per element net contracted along its second
-    coordinate (once per distinct value in a chunk of the rule): the homogeneous rows of the rational
-    Bezier net of degree pg with their derivatives, 2 (pg+1)^2 4 2 flops.  Per distinct element point:
-    the columns with value, d/du, d/dv ((pg+1) 4 3 2), the rational quotient, normal and Jacobian (30).
-    Per 4-D point: the kernel (distance, sincos, G, G'/r, the two orientations and the weight, 60), the
-    (p+1)^2 B-splines of the side that is not grouped by Bernstein extraction (5 per function; the surface
-    curls 6 more for sound-hard) and the group sums (the kernel value of each orientation times each
-    function, 8 per function; sound-hard adds w gc times the curls, 12).  Per group of points sharing an
-    element point: that side's B-splines (and curls) and the accumulation of the (p+1)^2 x (p+1)^2 entries
-    of both blocks (8 per entry; sound-hard 16 more for the curl products).  Identical sound-soft pairs
-    summed in factorised form (groups of ns^2 points, ns = 5): per point the kernel alone; per group the
-    univariate basis values (4 ns of them, 5 (p+1) each), the inner sums (ns (p+1)^2 ns, 10 flops each:
-    the product of two basis values and two complex-by-real multiply-adds) and the outer sums
-    ((p+1)^4 ns, 10 each)."""
-    n = (p + 1) ** 2
-    ns = 5
-    per_column = 2 * (pg + 1) ** 2 * 4 * 2
-    per_geo_point = (pg + 1) * 4 * 3 * 2 + 30
-    basis = 5 * n + (6 * n if hard else 0)
-    per_point = 60 + basis + 8 * n + (12 * n if hard else 0)
-    per_group = basis + n * n * (8 + (16 if hard else 0))
-    fact = info.get("n_singular_factored_points", 0)
-    per_fact_group = 4 * ns * 5 * (p + 1) + ns * n * ns * 10 + n * n * ns * 10
-    return (info["n_singular_geo_columns"] * per_column + info["n_singular_geo_points"] * per_geo_point
-            + (info["n_singular_points"] - fact) * per_point + fact * 60
-            + info["n_singular_groups"] * per_group + fact / ns ** 2 * per_fact_group)
+    """FP64 operations of the touching pairs' quadrature (the model behind the roofline of k_sing_tensor; p <= 3,
+    five Gauss points), from the mesh: on a closed quadrilateral mesh of E elements there are E identical pairs
+    (20 slabs of 125 points each, half of the rule), 2 E common-edge pairs (30 slabs) and the common-vertex
+    pairs (20 slabs).  Per slab: the elements' nets contracted along the coordinate with fewer values (values x
+    (pg+1)^2 x 8 x 2), the distinct element points (columns with value, d/du, d/dv, (pg+1) 4 3 2, and 40 for the
+    quotient, normal and Jacobian), the kernel in both orientations (100 a point, sound-hard 150 with the four
+    curl kernels), and the contractions of the G = 2 (sound-hard 6) complex kernel groups, one index or index pair
+    at a time, with univariate values (2 flops a real multiply-add)."""
+    n, G, E = p + 1, (6 if hard else 2), info["n_elements"]
+    pairs = {"id": E, "edge": 2 * E, "vertex": (info["n_touching_pairs"] - E) // 2 - 2 * E}
+    kernel = 125 * (150 if hard else 100)
+    point, net = (pg + 1) * 4 * 3 * 2 + 40, (pg + 1) ** 2 * 8 * 2
+    first, last = 5 * 25 * n * G * 4, n ** 4 * G * 4
+    edge01 = kernel + 150 * point + 6 * net + first + 25 * n ** 3 * G * 4 + last
+    edge2 = kernel + 50 * point + 10 * net + first + 25 * n ** 2 * G * 4 + 5 * last
+    vertex = kernel + 30 * point + 6 * net + first + 25 * n ** 2 * G * 4 + 5 * last
+    ident = kernel + 250 * point + 10 * net + 125 * n ** 2 * G * 4 + 5 * last
+    return pairs["id"] * 20 * ident + pairs["edge"] * (20 * edge01 + 10 * edge2) + pairs["vertex"] * 20 * vertex
 
 
 def mie_soft_far_field(kappa, xhat, d=(0.0, 0.0, 1.0)):
@@ -573,7 +564,7 @@ def run_matvec_steps(args, wl, B, inputs, geom, options, stream, flush, local, w
             if tc and os.path.exists(os.path.join(ROOT, "MEASURED_PEAKS.json")) else peaks["fp32_tflops"])
     kh = (Q + 7) // 8 * 8
     executed = far * 3 * 2 * 128 * (2 * kh) * C * R                  # tensor-core flops issued (split, padding)
-    roofline = {"bound": "tensor" if tc else "alu", "kernel": "k_m2l_tc" if tc else "k_m2l_gemm<float>",
+    roofline = {"bound": "tensor" if tc else "alu", "kernel": "k_m2l_tc" if tc else "k_m2l_fly<float> / k_m2l_gemm<float>",
                 "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak, "traffic": None,
                 "peak_source": ("measured dense BF16 burst (FP16 has the same tensor rate), MEASURED_PEAKS.json"
                                 if tc else "measured FP32 FMA rate (igabem_measure_peaks, this run)"),
@@ -799,30 +790,26 @@ def run_sweep_steps(args, wl, B, inputs, geom, patches, stream, flush, local, wo
         m2l_bytes = sum(f * q ** 4 for f, q in zip(far_by_level, qs)) * (2 if hard else 1) * ebytes
         hbm = hbm_peak_gbs()
         m2l_gbs = m2l_bytes / (m2l_ms / 1e3) / 1e9 if m2l_ms > 0 else 0.0
-        m2l_roof = {"kernel": "k_m2l_stored<float>", "bound": "hbm", "achieved": m2l_gbs, "unit": "GB/s",
+        m2l_roof = {"kernel": "k_stream32", "bound": "hbm", "achieved": m2l_gbs, "unit": "GB/s",
                     "peak": hbm, "frac": m2l_gbs / hbm if hbm else None,
                     "algorithmic_bytes_per_matvec": m2l_bytes, "avg_ms_per_matvec": m2l_ms,
                     "peak_source": "measured copy bandwidth, MEASURED_PEAKS.json"}
     else:
-        m2l_roof = {"kernel": "k_m2l_rows<float> / k_m2l_gemm<float>", "achieved": m2l_ach, "unit": "TFLOP/s",
+        m2l_roof = {"kernel": "k_m2l_fly<float> / k_m2l_gemm<float>", "achieved": m2l_ach, "unit": "TFLOP/s",
                     "peak": peaks["fp32_tflops"], "frac": m2l_ach / peaks["fp32_tflops"],
                     "xu_frac": (m2l_samples / (peaks["sincosf_gops"] * 1e9) + m2l_samples / (peaks["rsqrtf_gops"] * 1e9))
                     / (m2l_ms / 1e3) if m2l_ms > 0 else None,
                     "algorithmic_flops_per_matvec": m2l_flops, "avg_ms_per_matvec": m2l_ms,
                     "node_pairs_per_matvec": m2l_samples,
                     "peak_source": "measured FP32 FMA rate (igabem_measure_peaks, this run)"}
-    roofline = {"bound": "alu", "kernel": "k_near_singular (FP64)", "achieved": sing_ach,
+    roofline = {"bound": "alu", "kernel": "k_sing_tensor (FP64)", "achieved": sing_ach,
                 "peak": peaks["fp64_tflops"], "unit": "TFLOP/s", "frac": sing_ach / peaks["fp64_tflops"],
                 "traffic": SINGULAR_DRAM_BYTES_PER_POINT * info["n_singular_points"],
-                "traffic_source": "DRAM bytes per 4-D point of one ncu capture of the small sweep case, "
+                "traffic_source": "DRAM bytes per 4-D point of one ncu capture at 1536 elements, "
                                   "times this launch's points",
                 "peak_source": "measured FP64 FMA rate (igabem_measure_peaks, this run; 2 flops per FMA)",
                 "algorithmic_flops_per_setup": sing_flops, "avg_ms_per_setup": sing_ms,
                 "singular_points": info["n_singular_points"],
-                "singular_geometry_points": info["n_singular_geo_points"],
-                "singular_geometry_columns": info["n_singular_geo_columns"],
-                "singular_groups": info["n_singular_groups"],
-                "singular_factored_points": info["n_singular_factored_points"],
                 "m2l": m2l_roof}
     lat = sorted(step_ms)
     value = R * args.steps * world / (total_ms / 1e3)
@@ -1017,7 +1004,7 @@ def main():
     d2h = int(info["n_dofs"] * 16 * len(dirs) + len(xhat) * 16 * len(dirs))
 
     # ---- roofline of the dominant kernel of a solve step from the timed region's CUDA events: the FP64
-    # singular quadrature of the touching element pairs (k_near_singular); the M2L beside it ----
+    # singular quadrature of the touching element pairs (k_sing_tensor); the M2L beside it ----
     far = info["n_far_pairs"]
     Q = wl["cheb_q"] ** 2
     hard = bool(wl["bc"])
@@ -1028,17 +1015,13 @@ def main():
     sing_achieved = sing_flops / (sing_ms / 1e3) / 1e12 if sing_ms > 0 else 0.0
     m2l = main_form["prof"].get("m2l", {"ms": 0.0, "calls": 0})
     m2l_ms = m2l["ms"] / max(1, m2l["calls"])
-    roofline = {"bound": "alu", "kernel": "k_near_singular (FP64)", "achieved": sing_achieved,
+    roofline = {"bound": "alu", "kernel": "k_sing_tensor (FP64)", "achieved": sing_achieved,
                 "peak": peaks["fp64_tflops"], "unit": "TFLOP/s", "frac": sing_achieved / peaks["fp64_tflops"],
                 "traffic": None,
                 "peak_source": "measured FP64 FMA rate (igabem_measure_peaks, this run; 2 flops per FMA)",
                 "algorithmic_flops_per_setup": sing_flops, "avg_ms_per_setup": sing_ms,
                 "singular_points": info["n_singular_points"],
-                "singular_geometry_points": info["n_singular_geo_points"],
-                "singular_geometry_columns": info["n_singular_geo_columns"],
-                "singular_groups": info["n_singular_groups"],
-                "singular_factored_points": info["n_singular_factored_points"],
-                "m2l": m2l_alu_roofline("k_m2l_rows<double>" if fp64 else "k_m2l_rows<float>", far, Q, hard,
+                "m2l": m2l_alu_roofline("k_m2l_fly<double>" if fp64 else "k_m2l_fly<float>", far, Q, hard,
                                         len(dirs), m2l_ms, peaks, fp64)}
 
     def summary(f):
