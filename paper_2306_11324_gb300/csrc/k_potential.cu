@@ -160,11 +160,14 @@ __global__ void __launch_bounds__(128) k_pot_m2m(PotArgs P, PotLevel Lp, PotLeve
 // nodes, and generates each sample once for all of them instead of once per pair; a thread owns one target
 // node with its columns' sums in registers.  In FP32 the phase is split about the box centres
 // (kappa |D| in FP64 plus kappa (r - |D|), r - |D| = (2 D.d + |d|^2) / (r + |D|)) and the products take two
-// columns per instruction; the sums of 64 source nodes, then of their groups, are added to Z in FP64.
-// Measured on 4001 points around 6144 Gauss points, q = 7, 372,000 pairs (FP32): 1520 -> 22 ms a call, host
+// columns per instruction; the sums of 4 source nodes are added up with their rounding errors, then to Z in FP64.
+// The sine and cosine are rounded to FP32: at small kappa all samples have nearly one phase, and the errors of the
+// fast ones (4e-7) add up.  Difference to the FP64 form at kappa = 1, 3, 12, 20: 5, 5, 12, 20e-8 (rms; 17 to 28e-8 with
+// the fast ones and sums of 64, at 22 ms a call).
+// Measured on 4001 points around 6144 Gauss points, q = 7, 372,000 pairs (FP32): 1520 -> 36 ms a call, host
 // tree included (before: a sample per pair with FP64 differences and sums, and per-node Lagrange values in
 // P2M).
-constexpr int POT_COLS = 16, POT_ROWS = 128, POT_STEP = 64;
+constexpr int POT_COLS = 16, POT_ROWS = 128, POT_STEP = 64, POT_GROUP = 4;
 
 __device__ inline float2 fma2x(float2 a, float2 b, float2 c) {  // two FP32 multiply-adds
   float2 d;
@@ -173,6 +176,26 @@ __device__ inline float2 fma2x(float2 a, float2 b, float2 c) {  // two FP32 mult
       : "l"(reinterpret_cast<const unsigned long long &>(a)), "l"(reinterpret_cast<const unsigned long long &>(b)),
         "l"(reinterpret_cast<const unsigned long long &>(c)));
   return d;
+}
+
+// sine and cosine of x + xl, |x| < 1e6, xl tiny: reduced to |y| <= pi/4 about a multiple of pi/2, there the Taylor series
+// (first terms left out: 2e-9 and 3e-8 at pi/4)
+__device__ inline void sincos_series(float x, float xl, float &sn, float &cs) {
+  const float m = fmaf(x, 0.636619772f, 12582912.f), k = m - 12582912.f;  // 1.5 2^23: rounds to an integer
+  const int n = __float_as_int(m);
+  const float y = fmaf(-k, -4.37113883e-8f, fmaf(-k, 1.57079637f, x)) + xl, z = y * y;
+  const float s = fmaf(y * z, fmaf(z, fmaf(z, fmaf(z, 1.f / 362880, -1.f / 5040), 1.f / 120), -1.f / 6), y);
+  const float c = fmaf(z, fmaf(z, fmaf(z, fmaf(z, 1.f / 40320, -1.f / 720), 1.f / 24), -0.5f), 1.f);
+  const float a = n & 1 ? c : s, b = n & 1 ? s : c;
+  sn = n & 2 ? -a : a;
+  cs = (n + 1) & 2 ? -b : b;
+}
+
+// s + l += v, l the rounding errors of s (Knuth's two-sum)
+__device__ inline void two_sum(float &s, float &l, float v) {
+  const float t = s + v, b = t - s;
+  l += (s - (t - b)) + (v - b);
+  s = t;
 }
 
 template <class T>
@@ -190,10 +213,12 @@ __global__ void __launch_bounds__(POT_ROWS) k_pot_m2l(PotArgs P, PotLevel L, con
   const double Dd[3] = {ck.dx * side, ck.dy * side, ck.dz * side};
   const double D2d = Dd[0] * Dd[0] + Dd[1] * Dd[1] + Dd[2] * Dd[2], Dnd = sqrt(D2d);
   double c0 = 0, c1 = 0;
-  float phi0 = 0;
+  float phi0 = 0, phi0l = 0;  // kappa |D| in two floats
   if constexpr (F32) {
     const double x = P.kappa * Dnd, k = rint(x / TWO_PI);  // reduced to (-pi, pi]
-    phi0 = (float)fma(-k, 2.4492935982947064e-16, fma(-k, TWO_PI, x));
+    const double ph = fma(-k, 2.4492935982947064e-16, fma(-k, TWO_PI, x));
+    phi0 = (float)ph;
+    phi0l = (float)(ph - (double)phi0);
   } else {
     phase64_scale(P.kappa, c0, c1);
     for (int i = tid; i < CIS_N; i += POT_ROWS) tab[i] = P.cis[i];
@@ -212,8 +237,12 @@ __global__ void __launch_bounds__(POT_ROWS) k_pot_m2l(PotArgs P, PotLevel L, con
     for (int c = 0; c < 3; ++c) xa[c] += D[c];
   }
   T tr[POT_COLS], ti[POT_COLS];
+  float lr[F32 ? POT_COLS : 1], li[F32 ? POT_COLS : 1];  // FP32: what the sums over the groups round off
 #pragma unroll
-  for (int c = 0; c < POT_COLS; ++c) tr[c] = ti[c] = 0;
+  for (int c = 0; c < POT_COLS; ++c) {
+    tr[c] = ti[c] = 0;
+    if constexpr (F32) lr[c] = li[c] = 0;
+  }
   for (int b0 = 0; b0 < Q; b0 += POT_STEP) {
     const int nb = min(POT_STEP, Q - b0);
     __syncthreads();
@@ -232,21 +261,18 @@ __global__ void __launch_bounds__(POT_ROWS) k_pot_m2l(PotArgs P, PotLevel L, con
     }
     __syncthreads();
     if (a >= Q) continue;
-    if constexpr (F32) {
+    if constexpr (F32) for (int g0 = 0; g0 < nb; g0 += POT_GROUP) {
       float2 pr[POT_COLS / 2], pi[POT_COLS / 2];
 #pragma unroll
       for (int c = 0; c < POT_COLS / 2; ++c) pr[c] = pi[c] = make_float2(0.f, 0.f);
-      for (int b = 0; b < nb; ++b) {
+      for (int b = g0; b < min(nb, g0 + POT_GROUP); ++b) {
         const float4 y = *reinterpret_cast<const float4 *>(ys[b]);
         const float d0 = xa[0] - y.x, d1 = xa[1] - y.y, d2 = xa[2] - y.z;
         const float num = fmaf(2.f, Dx - y.w, fmaf(d0, d0, fmaf(d1, d1, d2 * d2)));
-        const float r2 = D2 + num, ir = rsqrtf(r2), r = r2 * ir;
-        float ph = fmaf(kappa, __fdividef(num, r + Dn), phi0);
-        const float kq = rintf(ph * 0.15915494309189535f);
-        ph = fmaf(-kq, 6.28318548202514648f, ph);
-        ph = fmaf(-kq, -1.7484556e-07f, ph);
+        const float r2 = D2 + num, i0 = rsqrtf(r2), ir = fmaf(0.5f * i0, fmaf(-r2 * i0, i0, 1.f), i0), r = r2 * ir;
+        const float ph = fmaf(kappa, __fdividef(num, r + Dn), phi0);
         float sn, cs;
-        __sincosf(ph, &sn, &cs);
+        sincos_series(ph, phi0l, sn, cs);
         const float f = ir * 0.0795774715459476679f, gx = cs * f, gy = sn * f;
         const float2 gxx = make_float2(gx, gx), gyy = make_float2(gy, gy), gyn = make_float2(-gy, -gy);
         const float4 *wr = reinterpret_cast<const float4 *>(wre[b]), *wi = reinterpret_cast<const float4 *>(wim[b]);
@@ -263,8 +289,8 @@ __global__ void __launch_bounds__(POT_ROWS) k_pot_m2l(PotArgs P, PotLevel L, con
       }
 #pragma unroll
       for (int c = 0; c < POT_COLS / 2; ++c) {
-        tr[2 * c] += pr[c].x; tr[2 * c + 1] += pr[c].y;
-        ti[2 * c] += pi[c].x; ti[2 * c + 1] += pi[c].y;
+        two_sum(tr[2 * c], lr[2 * c], pr[c].x); two_sum(tr[2 * c + 1], lr[2 * c + 1], pr[c].y);
+        two_sum(ti[2 * c], li[2 * c], pi[c].x); two_sum(ti[2 * c + 1], li[2 * c + 1], pi[c].y);
       }
     } else {
       for (int b = 0; b < nb; ++b) {
@@ -286,8 +312,13 @@ __global__ void __launch_bounds__(POT_ROWS) k_pot_m2l(PotArgs P, PotLevel L, con
     for (int c = 0; c < POT_COLS; ++c) {
       if (c >= ncol) break;
       double2 *z = L.Z + ((long)pairs[ck.first + c / R].x * Q + a) * R + c % R;
-      atomicAdd(&z->x, (double)tr[c]);
-      atomicAdd(&z->y, (double)ti[c]);
+      if constexpr (F32) {
+        atomicAdd(&z->x, (double)tr[c] + (double)lr[c]);
+        atomicAdd(&z->y, (double)ti[c] + (double)li[c]);
+      } else {
+        atomicAdd(&z->x, tr[c]);
+        atomicAdd(&z->y, ti[c]);
+      }
     }
 }
 
