@@ -1062,16 +1062,19 @@ int igabem_farfield(igabem_problem *P, int n_rhs, const void *density, int n_dir
     bool dd = is_device_ptr(density), du = is_device_ptr(uinf);
     const double *dens = dd ? static_cast<const double *>(density) : W.xin;
     if (!dd) IGA_CUDA(cudaMemcpyAsync(W.xin, density, db, cudaMemcpyHostToDevice, st));
-    // the directions (and, for a host result, the pattern) in a buffer kept with the problem
+    // the directions in a buffer kept with the problem, and the pattern too where the kernels cannot write it in
+    // place: a host result, or a device result off the 16-byte boundary that their complex stores need
+    const bool direct = du && reinterpret_cast<uintptr_t>(uinf) % 16 == 0;
+    const size_t ub = 2 * sizeof(double) * (size_t)n_dir * n_rhs;
     const size_t xb = (3 * sizeof(double) * (size_t)n_dir + 255) & ~size_t(255);
-    const size_t need = xb + (du ? 0 : 2 * sizeof(double) * (size_t)n_dir * n_rhs);
+    const size_t need = xb + (direct ? 0 : ub);
     if (W.ff.cap < need) W.ff.reserve(need);
     double *dx = reinterpret_cast<double *>(W.ff.base);
-    double *du_ = du ? static_cast<double *>(uinf) : reinterpret_cast<double *>(W.ff.base + xb);
+    double *du_ = direct ? static_cast<double *>(uinf) : reinterpret_cast<double *>(W.ff.base + xb);
     IGA_CUDA(cudaMemcpyAsync(dx, xhat, 3 * sizeof(double) * n_dir, cudaMemcpyHostToDevice, st));
     launch_farfield(P->d, P->S, P->opt, n_rhs, dens, n_dir, dx, du_, P->d.gq, st);
-    if (!du)
-      IGA_CUDA(cudaMemcpyAsync(uinf, du_, 2 * sizeof(double) * n_dir * n_rhs, cudaMemcpyDeviceToHost, st));
+    if (!direct)
+      IGA_CUDA(cudaMemcpyAsync(uinf, du_, ub, du ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, st));
     IGA_CUDA(cudaStreamSynchronize(st));
     P->prof.flush();
   });
