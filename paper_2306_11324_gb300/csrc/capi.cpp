@@ -150,11 +150,15 @@ struct IterGraph {
   }
 };
 
+// far-field buffer kept with a problem between calls (2048 directions with 8 columns take 0.3 MiB); a larger one is
+// given back at the end of its call
+constexpr size_t FF_KEEP = size_t(32) << 20;
+
 struct ProblemWork {
   int R = 0;
   int gmres_m = 0;
   Arena arena;
-  Arena ff;                          // far-field directions (and a host caller's result), grown as needed
+  Arena ff;                          // far-field directions and results that are copied, at most FF_KEEP after a call
   double *xX, *yleaf, *gq, *xin, *yout, *red;
   std::vector<void *> xhat, yhat;
   std::vector<uint8_t *> tc_bimg;
@@ -623,6 +627,12 @@ void problem_release(igabem_problem *P) {
   delete P;
 }
 
+size_t problem_work_held(const igabem_problem *P) {
+  std::lock_guard<std::mutex> lk(g_ext_mu);
+  auto it = g_ext.find(P);
+  return it != g_ext.end() ? it->second->work.arena.cap : 0;
+}
+
 }  // namespace igabem
 
 extern "C" {
@@ -748,7 +758,7 @@ int igabem_problem_info(const igabem_problem *prob, igabem_info *out) {
     *out = prob->info;
     std::lock_guard<std::mutex> lk(g_ext_mu);
     auto it = g_ext.find(prob);
-    if (it != g_ext.end()) out->device_bytes += it->second->work.arena.cap;
+    if (it != g_ext.end()) out->device_bytes += it->second->work.arena.cap + it->second->work.ff.cap;
   });
 }
 
@@ -1076,6 +1086,7 @@ int igabem_farfield(igabem_problem *P, int n_rhs, const void *density, int n_dir
     if (!direct)
       IGA_CUDA(cudaMemcpyAsync(uinf, du_, ub, du ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, st));
     IGA_CUDA(cudaStreamSynchronize(st));
+    if (W.ff.cap > FF_KEEP) W.ff.release();
     P->prof.flush();
   });
 }

@@ -331,6 +331,7 @@ igabem_problem *problem_plan(igabem_geom *geom, const igabem_options *opt);
 void problem_materialize(igabem_problem *P, cudaStream_t st);
 void problem_release(igabem_problem *P);
 size_t problem_work_bytes(const HostSetup &S, int R, int gmres_m, int precision);
+size_t problem_work_held(const igabem_problem *P);  // what it holds of these now
 double now_ms();
 }  // namespace igabem
 

@@ -119,7 +119,6 @@ void worker_loop(igabem_server *S) {
   for (;;) {
     std::vector<igabem_request *> batch;
     igabem_problem *P = nullptr;
-    size_t held = 0;          // bytes of a cached problem taken by this worker
     bool from_cache = false;
     {
       std::unique_lock<std::mutex> lk(S->mu);
@@ -143,7 +142,6 @@ void worker_loop(igabem_server *S) {
         if (!c.busy && same_problem(c.geom, c.opt, batch[0]->geom, batch[0]->opt)) {
           c.busy = true;
           P = c.P;
-          held = c.bytes;
           from_cache = true;
           S->cache_hits += 1;
           break;
@@ -159,7 +157,8 @@ void worker_loop(igabem_server *S) {
     try {
       if (!P) P = problem_plan(r->geom, &r->opt);
       const size_t work = problem_work_bytes(P->S, R, std::max(1, r->opt.gmres_restart), r->opt.precision);
-      need = from_cache ? (work > held - P->arena.cap ? work - (held - P->arena.cap) : 0) + (size_t(64) << 20)
+      const size_t held = from_cache ? problem_work_held(P) : 0;
+      need = from_cache ? (work > held ? work - held : 0) + (size_t(64) << 20)
                         : P->arena_bytes + P->temp_bytes + work + (size_t(64) << 20);
       for (auto *q : batch) q->bytes = need;
       if (need > S->budget) {

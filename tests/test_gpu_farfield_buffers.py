@@ -32,3 +32,20 @@ def test_result_at_an_8_byte_boundary(precision, n_dir, columns):
     assert G.rel(got, aligned) <= tol and G.rel(host, aligned) <= tol
     assert torch.isnan(buf[0]) and torch.isnan(buf[-1])
     B.igabem_problem_destroy(prob)
+
+
+def test_memory_of_the_call_is_counted_and_given_back():
+    """The problem's device_bytes follow the buffer it keeps, and a call of 88 MB leaves no more than that behind (to the
+    2 MB of cudaMalloc's granularity on either side)."""
+    import torch
+    prob, info = G.problem(level_m=1, degree_p=1, kappa=2.0, eta_cfie=1.0, no_fmm=1)
+    x = inputs.random_complex(info["n_dofs"], seed=1, cols=4)
+    B.igabem_farfield(prob, x, inputs.fibonacci_directions(40))    # work buffers and kernels are there
+    held = B.igabem_problem_info(prob)["device_bytes"]
+    free = torch.cuda.mem_get_info()[0]
+    for n_dir in (200_000, 1_000_000, 40):
+        B.igabem_farfield(prob, x, inputs.fibonacci_directions(n_dir))
+        more = B.igabem_problem_info(prob)["device_bytes"] - held
+        assert free - torch.cuda.mem_get_info()[0] <= more + (4 << 20)
+        assert more <= 32 << 20
+    B.igabem_problem_destroy(prob)
