@@ -6,6 +6,7 @@
 #include <algorithm>
 #include <cstddef>
 #include <cstdint>
+#include <exception>
 #include <functional>
 #include <memory>
 #include <mutex>
@@ -192,20 +193,33 @@ struct GeoCache {
 void build_setup(const std::vector<Patch> &patches, const igabem_options &opt, HostSetup &S,
                  const GeoCache *hit = nullptr, GeoCache *fill = nullptr);
 
-// body(i) for i in [0, n) on up to 16 host threads (independent iterations writing disjoint data)
+// body(i) for i in [0, n) on up to 16 host threads (independent iterations writing disjoint data).  The first exception
+// of a body is thrown again here, after every thread has ended (one that left a thread would end the process, and
+// bodies that grow lists can run out of memory); shares whose thread does not start run on the caller.
 template <class F>
 void parallel_for(long n, const F &body) {
   const long nt = std::min<long>(std::min<long>(16, std::max(1u, std::thread::hardware_concurrency())), n);
-  if (nt <= 1) {
-    for (long i = 0; i < n; ++i) body(i);
-    return;
-  }
-  std::vector<std::thread> th;
-  for (long k = 0; k < nt; ++k)
-    th.emplace_back([&, k] {
+  std::mutex mu;
+  std::exception_ptr error;
+  auto share = [&](long k) {
+    try {
       for (long i = k; i < n; i += nt) body(i);
-    });
+    } catch (...) {
+      std::lock_guard<std::mutex> lk(mu);
+      if (!error) error = std::current_exception();
+    }
+  };
+  std::vector<std::thread> th;
+  long k = 1;
+  try {
+    th.reserve(std::max(0L, nt - 1));
+    for (; k < nt; ++k) th.emplace_back([&share, k] { share(k); });
+  } catch (...) {
+  }
+  if (nt > 0) share(0);
+  for (; k < nt; ++k) share(k);
   for (auto &t : th) t.join();
+  if (error) std::rethrow_exception(error);
 }
 
 // Gauss-Legendre rule on [0,1] (Newton iteration on P_n).
