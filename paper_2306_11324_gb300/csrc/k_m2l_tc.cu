@@ -134,19 +134,18 @@ __device__ inline void mma_commit(uint32_t bar) {
 // Constants of one pair for the generation of its coupling block.
 struct TCPair {
   float D0, D1, D2, Dn, DD;  // D = c_t - c_s, |D|, |D|^2
-  float phi0;                // kappa |D| / (2 pi) reduced to [-1/2, 1/2]
+  float phi0;                // kappa |D| reduced to [-pi, pi]
   float fs;                  // the pair's power-of-two scale / (4 pi)
 };
 
 // Kernel sample of type TYPE (0: soft K' - i eta V; 1: hard K; 2: hard G, as node_sample) times the
 // pair factor exp(i kappa |D|) and the pair's scale.  Nodes in shared memory as three float4:
 // [x - c, D.(x - c)][n~, D.n~][a] (D.(x - c) and D.n~ for sources; for the target, Dx and Dnx are passed in).  The
-// phase in turns is kappa / (2 pi) (|D| + (r - |D|)) with r - |D| = (2 D.d + |d|^2) / (r + |D|), d the difference
-// of the node offsets; k2pi = kappa / (2 pi).
+// phase is kappa |D| + kappa (r - |D|) with r - |D| = (2 D.d + |d|^2) / (r + |D|), d the difference of the node
+// offsets.
 template <int TYPE>
-__device__ inline float2 tc_sample(const TCPair &g, float kappa, float k2pi, float eta, const float4 &x0, const float4 &x1,
-                                   float ax, float Dx, float Dnx, const float4 *__restrict__ y) {
-  constexpr float M = 12582912.f;  // 1.5 2^23: adding it rounds to an integer
+__device__ inline float2 tc_sample(const TCPair &g, float kappa, float eta, const float4 &x0, const float4 &x1, float ax,
+                                   float Dx, float Dnx, const float4 *__restrict__ y) {
   const float4 y0 = y[0];
   const float d0 = x0.x - y0.x, d1 = x0.y - y0.y, d2 = x0.z - y0.z;
   const float dd = fmaf(d0, d0, fmaf(d1, d1, d2 * d2));
@@ -155,8 +154,7 @@ __device__ inline float2 tc_sample(const TCPair &g, float kappa, float k2pi, flo
   float ir;
   asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(ir) : "f"(r2));
   const float r = r2 * ir;
-  const float tn = fmaf(k2pi, __fdividef(num, r + g.Dn), g.phi0);
-  const float ph = (tn - ((tn + M) - M)) * 6.28318530717958647692f;
+  const float ph = phase32(kappa, __fdividef(num, r + g.Dn), g.phi0);
   float sph, cph;
   __sincosf(ph, &sph, &cph);
   const float f = ir * g.fs;
@@ -184,7 +182,6 @@ __device__ void tc_generate(const TCPair &g, float kappa, float eta, const float
                             const float4 *__restrict__ sn4, uint8_t *__restrict__ Ahi, uint8_t *__restrict__ Alo,
                             int Q, int KH, int KC, int warp, int lane) {
   const int ntask = (KH >> 3) * Q;
-  const float k2pi = kappa * 0.15915494309189533577f;
   const uint32_t im = (uint32_t)(KH >> 3) * 128, lower = (uint32_t)KC * 8 * 128;  // -Im / Re half along K; rows 64..
   for (int task = (warp - 1) * 32 + lane; task < ntask; task += TC_THREADS - 32) {
     const int g8 = task / Q, a = task - g8 * Q;
@@ -199,7 +196,7 @@ __device__ void tc_generate(const TCPair &g, float kappa, float eta, const float
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
         const int b = g8 * 8 + u + h;
-        v[h] = tc_sample<TYPE>(g, kappa, k2pi, eta, x0, x1, ax, Dx, Dnx, sn4 + 3 * min(b, Q - 1));
+        v[h] = tc_sample<TYPE>(g, kappa, eta, x0, x1, ax, Dx, Dnx, sn4 + 3 * min(b, Q - 1));
         if (b >= Q) v[h] = make_float2(0.f, 0.f);
       }
       split2(v[0].x, v[1].x, rh[u / 2], rl[u / 2]);
@@ -277,9 +274,9 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_m2l_tc(const TCArgs A) {
     sinv[p] = 1.0f / (L.pc[8L * (k0 + p) + 7] * L.bscale[src]);
   }
   auto src_of = [&](int p) { return p < TC_LIST ? slist[p] : L.far_src[k0 + p]; };
-  // the constants the generation uses: the phase of exp(i kappa |D|) in turns, the scale over 4 pi
+  // the constants the generation uses: the phase of exp(i kappa |D|), the scale over 4 pi
   auto finish_consts = [&](float *c) {
-    c[5] = atan2f(c[6], c[5]) * 0.15915494309189533577f;
+    c[5] = atan2f(c[6], c[5]);
     c[7] *= 0.0795774715459476679f;
   };
   if (tid < 2 && tid < npairs) {
