@@ -61,17 +61,31 @@ template <> struct __align__(16) FlyNode<float, true> { float y[3], Dy, n[3], Dn
 // per pair with two rows a lane used 49 of 64).  It generates its row of the pair's coupling block in
 // registers, reading the source nodes from shared memory, and multiplies it into NC columns: for
 // sound-hard one sample gives K and G, which serve the columns of all seven channels.  Sums: the pair's in
-// registers, then over the thread's pairs, then over the P threads of a node and over the blocks
+// registers, then over the thread's pairs (FP32: see FLY_BLOCK), then over the P threads of a node and over the blocks
 // of a cluster, in that fixed order (FP64).  A target's interaction list is split over a cluster of
 // gridDim.y blocks, which add their sums through distributed shared memory, where a level has too few
 // targets to fill the device.  Measured on GB300, FP64 products (before: one warp per pair, 72 FP64
 // instructions a sample and CUDA's sincos, or for several columns the tile of k_m2l_gemm mostly padding): 6936
 // unknowns, one column, 175 M samples 32.2 -> 17.1 ms; 150 unknowns, 8 M samples 2.20 -> 1.08 ms; sound-hard,
 // 1736 unknowns, 3 columns of 7 channels 41 -> 4 ms.
+// FP32 sums: FLY_BLOCK source nodes at a time within a pair.  Over the pairs: forms of up to 16 columns keep the sum and
+// its rounding errors in shared memory (their registers would cost them a second block on the SM); wider ones, which
+// run one block anyway, add FLY_PAIRS pairs at a time in registers (shared memory costs them 6 %, by the L1 it takes).
+// Far rows against FP64 (rms; one chain of q^2 products and of all pairs -> this): q = 12 1.06 -> 1.04e-7, q = 16, short
+// lists 6.8 -> 5.2e-8; 6144 elements, q = 7, lists of 256 pairs 9.4 -> 8.8e-8.  1 to 16 columns within 2 % of the single
+// chain's time, 24 columns 2.25 -> 2.10 ms, 21 (sound-hard) 2.34 -> 2.39 ms (1536 elements).
+constexpr int FLY_BLOCK = 16, FLY_PAIRS = 8;
+template <class T, int NC> constexpr bool fly_sums = std::is_same<T, float>::value && NC <= 16;
+
+// bytes in front of the nodes: the table of phase64, or the sums of the FP32 form
+template <class T, int NC> __host__ __device__ constexpr size_t fly_head() {
+  return fly_sums<T, NC> ? (size_t)NC * 256 * sizeof(float4) : std::is_same<T, float>::value ? 0 : CIS_N * sizeof(double2);
+}
+
 template <class T, int NC, bool HARD>
 __global__ void __launch_bounds__(256) k_m2l_fly(const __grid_constant__ M2LArgs A) {
   extern __shared__ __align__(16) unsigned char smf[];
-  constexpr bool F32 = std::is_same<T, float>::value;
+  constexpr bool F32 = std::is_same<T, float>::value, SUMS = fly_sums<T, NC>;
   using Node = FlyNode<T, HARD>;
   const int tid = threadIdx.x, nsplit = gridDim.y, rank = blockIdx.y, cr0 = blockIdx.z * NC;
   int li = 0;
@@ -81,11 +95,16 @@ __global__ void __launch_bounds__(256) k_m2l_fly(const __grid_constant__ M2LArgs
   const long NQ = (long)L.n * Q;
   const int ncr = min(NC, A.CR - cr0);
   double2 *tab = reinterpret_cast<double2 *>(smf);                       // FP64: the table of phase64
-  Node *src = reinterpret_cast<Node *>(smf + (F32 ? 0 : CIS_N * sizeof(double2)));  // [P Q]
+  float4 *sums = reinterpret_cast<float4 *>(smf);                        // SUMS: [NC][256], sum and its rounding errors
+  Node *src = reinterpret_cast<Node *>(smf + fly_head<T, NC>());         // [P Q]
   C2<T> *xs = reinterpret_cast<C2<T> *>(src + A.rows_most);              // [P Q][NC]
   C2<T> *red = xs;
-  if constexpr (!F32)
+  if constexpr (SUMS) {
+#pragma unroll
+    for (int c = 0; c < NC; ++c) sums[c * 256 + tid] = make_float4(0.f, 0.f, 0.f, 0.f);
+  } else if constexpr (!F32) {
     for (int i = tid; i < CIS_N; i += 256) tab[i] = A.cis[i];
+  }
   double c0, c1;
   phase64_scale(A.kappa, c0, c1);
   const T kappa = (T)A.kappa, eta = (T)A.eta;
@@ -101,9 +120,16 @@ __global__ void __launch_bounds__(256) k_m2l_fly(const __grid_constant__ M2LArgs
     ta = F32 ? (T)L.nodes32[6 * NQ + ia] : (T)L.nodes[6 * NQ + ia];
     if (!HARD) ta *= eta;
   }
-  C2<T> tot[NC];
+  C2<T> tot[SUMS ? 1 : NC], few[F32 && !SUMS ? NC : 1];  // few: of the last FLY_PAIRS pairs at most
+  int kept = 0;
+  if constexpr (!SUMS) {
 #pragma unroll
-  for (int c = 0; c < NC; ++c) tot[c] = c2((T)0, (T)0);
+    for (int c = 0; c < NC; ++c) tot[c] = c2((T)0, (T)0);
+    if constexpr (F32) {
+#pragma unroll
+      for (int c = 0; c < NC; ++c) few[c] = c2((T)0, (T)0);
+    }
+  }
   const int k0 = L.far_ptr[t], np = L.far_ptr[t + 1] - k0;
   for (int p0 = rank * P; p0 < np; p0 += nsplit * P) {
     const bool work = on && p0 + slot < np;
@@ -161,7 +187,7 @@ __global__ void __launch_bounds__(256) k_m2l_fly(const __grid_constant__ M2LArgs
     const C2<T> *xp = xs + slot * Q * NC;
     const T Ddx = D[0] * tx[0] + D[1] * tx[1] + D[2] * tx[2];
     const T Dnx = D[0] * tn[0] + D[1] * tn[1] + D[2] * tn[2];
-    for (int b = 0; b < Q; ++b) {
+    auto add_node = [&](int b, C2<T> (&sum)[NC]) {
       const Node y = sp[b];
       const T d0 = tx[0] - y.y[0], d1 = tx[1] - y.y[1], d2 = tx[2] - y.y[2];
       C2<T> S0, S1 = c2((T)0, (T)0);  // soft: S0; hard: S0 = K, S1 = G
@@ -204,17 +230,58 @@ __global__ void __launch_bounds__(256) k_m2l_fly(const __grid_constant__ M2LArgs
 #pragma unroll
       for (int c = 0; c < NC; ++c) {
         const bool k = !HARD || cr0 + c < A.R;  // the first R columns are channel 0
-        part[c] = fma2(k ? S0 : S1, xp[b * NC + c], part[c]);
+        sum[c] = fma2(k ? S0 : S1, xp[b * NC + c], sum[c]);
       }
-    }
+    };
+    if constexpr (F32) {
+      int b = 0;
+      for (; b + FLY_BLOCK <= Q; b += FLY_BLOCK) {
+        C2<T> sum[NC];
 #pragma unroll
-    for (int c = 0; c < NC; ++c) tot[c] = F32 ? fma2(e0, part[c], tot[c]) : add(tot[c], part[c]);
+        for (int c = 0; c < NC; ++c) sum[c] = c2((T)0, (T)0);
+#pragma unroll
+        for (int u = 0; u < FLY_BLOCK; ++u) add_node(b + u, sum);
+#pragma unroll
+        for (int c = 0; c < NC; ++c) part[c] = add(part[c], sum[c]);
+      }
+      for (; b < Q; ++b) add_node(b, part);
+      if constexpr (SUMS) {
+#pragma unroll
+        for (int c = 0; c < NC; ++c) {
+          const C2<T> v = mul(e0, part[c]);
+          float4 w = sums[c * 256 + tid];
+          two_sum(w.x, w.z, v.x);
+          two_sum(w.y, w.w, v.y);
+          sums[c * 256 + tid] = w;
+        }
+      } else {
+#pragma unroll
+        for (int c = 0; c < NC; ++c) few[c] = fma2(e0, part[c], few[c]);
+        if (++kept == FLY_PAIRS) {
+          kept = 0;
+#pragma unroll
+          for (int c = 0; c < NC; ++c) {
+            tot[c] = add(tot[c], few[c]);
+            few[c] = c2((T)0, (T)0);
+          }
+        }
+      }
+    } else {
+      for (int b = 0; b < Q; ++b) add_node(b, part);
+#pragma unroll
+      for (int c = 0; c < NC; ++c) tot[c] = add(tot[c], part[c]);
+    }
   }
   // sums over the P threads of a node and the blocks of the cluster
-  __syncthreads();
-  if (on)
+  if constexpr (!SUMS) {
+    __syncthreads();
+    if (on)
 #pragma unroll
-    for (int c = 0; c < NC; ++c) red[tid * NC + c] = tot[c];
+      for (int c = 0; c < NC; ++c) {
+        if constexpr (F32) tot[c] = add(tot[c], few[c]);
+        red[tid * NC + c] = tot[c];
+      }
+  }
   cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
   if (nsplit > 1) cl.sync();
   else __syncthreads();
@@ -223,11 +290,20 @@ __global__ void __launch_bounds__(256) k_m2l_fly(const __grid_constant__ M2LArgs
     const int aa = o / ncr, c = o - aa * ncr;
     double2 sum = make_double2(0, 0);
     for (int z = 0; z < nsplit; ++z) {
-      const C2<T> *rz = nsplit > 1 ? cl.map_shared_rank(red, z) : red;
-      for (int p = 0; p < P; ++p) {
-        const C2<T> v = rz[(p * Q + aa) * NC + c];
-        sum.x += (double)v.x;
-        sum.y += (double)v.y;
+      if constexpr (SUMS) {
+        const float4 *sz = nsplit > 1 ? cl.map_shared_rank(sums, z) : sums;
+        for (int p = 0; p < P; ++p) {
+          const float4 v = sz[c * 256 + p * Q + aa];
+          sum.x += (double)v.x + (double)v.z;
+          sum.y += (double)v.y + (double)v.w;
+        }
+      } else {
+        const C2<T> *rz = nsplit > 1 ? cl.map_shared_rank(red, z) : red;
+        for (int p = 0; p < P; ++p) {
+          const C2<T> v = rz[(p * Q + aa) * NC + c];
+          sum.x += (double)v.x;
+          sum.y += (double)v.y;
+        }
       }
     }
     L.yhat[((long)t * Q + aa) * A.CR + cr0 + c] = sum;
@@ -422,8 +498,7 @@ __global__ void k_pair_consts(const int *__restrict__ far_ptr, const int *__rest
 
 template <class T, int NC, bool HARD>
 void launch_fly(const M2LArgs &A, int nblocks, int nsplit, cudaStream_t st) {
-  const size_t smem = (std::is_same<T, float>::value ? 0 : CIS_N * sizeof(double2)) +
-                      (size_t)A.rows_most * (sizeof(FlyNode<T, HARD>) + NC * sizeof(C2<T>));
+  const size_t smem = fly_head<T, NC>() + (size_t)A.rows_most * (sizeof(FlyNode<T, HARD>) + NC * sizeof(C2<T>));
   auto kfn = k_m2l_fly<T, NC, HARD>;
   IGA_CUDA(set_max_dynamic_smem(kfn, smem));
   cudaLaunchConfig_t cfg{};

@@ -83,6 +83,13 @@ __device__ inline float phase32(float kappa, float d, float phi0) {
   return fmaf(-turns, -1.7484556e-07f, fmaf(-turns, 6.28318548202514648f, ph));
 }
 
+// s + l += v, l the rounding errors of s (Knuth's two-sum)
+__device__ inline void two_sum(float &s, float &l, float v) {
+  const float t = s + v, b = t - s;
+  l += (s - (t - b)) + (v - b);
+  s = t;
+}
+
 // Sample of one node pair in precision T: returns the kernel value of the requested type.
 //   type 0: soft  a_y G'(r)/r (x-y).n~x - i eta a_x a_y G
 //   type 1: hard  a_x G'(r)/r (y-x).n~y

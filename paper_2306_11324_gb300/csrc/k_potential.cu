@@ -191,13 +191,6 @@ __device__ inline void sincos_series(float x, float xl, float &sn, float &cs) {
   cs = (n + 1) & 2 ? -b : b;
 }
 
-// s + l += v, l the rounding errors of s (Knuth's two-sum)
-__device__ inline void two_sum(float &s, float &l, float v) {
-  const float t = s + v, b = t - s;
-  l += (s - (t - b)) + (v - b);
-  s = t;
-}
-
 template <class T>
 __global__ void __launch_bounds__(POT_ROWS) k_pot_m2l(PotArgs P, PotLevel L, const PotChunk *__restrict__ chunks,
                                                       const int2 *__restrict__ pairs) {
