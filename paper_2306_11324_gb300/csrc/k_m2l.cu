@@ -634,9 +634,16 @@ void launch_m2l_rows(const DeviceProblem &d, const HostSetup &S, const igabem_op
       Wc = w;
       break;
     }
-  if (Wc >= 48 && A.QS <= 64) {
-    // Its tile has room for 64 columns: below 48 the padding costs more than k_m2l_fly's regenerated samples
-    // (FP64 operations per sample and 7 x 5 columns: 7 (72 + 256) here, 2 x 43 + 140 there).
+  // Its tile has room for 64 columns: below 48 the padding costs more than k_m2l_fly's regenerated samples
+  // (FP64 operations per sample and 7 x 5 columns: 7 (72 + 256) here, 2 x 43 + 140 there).  Sound-hard in FP32, where
+  // k_m2l_fly takes three of these columns a pass, they meet earlier, its time being that of the columns and of q^2, the
+  // tile's of neither: 480 clusters, here and there in ms at q = 8, 32 columns 34.2 and 36.4; q = 7, 34: 25.7 and 25.6,
+  // 36: 25.8 and 25.9, 40: 26.2 and 30.6; q = 6, 40: 18.8 and 18.0, 47: 19.3 and 20.0; q = 5, 47: 13.4 and 12.6.  Lists
+  // of few clusters leave its blocks few pairs each: 120 clusters, q = 5 and 7, 24 columns 0.82 and 0.72, 1.47 and 1.36;
+  // 28: 0.84 and 0.84, 1.52 and 1.59; 40: 0.92 and 1.15, 1.62 and 2.21.
+  const bool filled =
+      Wc >= 48 || (S.hard && fp32 && (nblocks < 2 * 152 ? Wc >= 28 : Wc >= 32 && Wc * A.QS >= 1750));
+  if (filled && A.QS <= 64) {
     const size_t tsz = fp32 ? sizeof(float) : sizeof(double);
     size_t smem = (size_t)A.QS * A.QS * 2 * tsz + (size_t)A.QS * Wc * 2 * tsz + (size_t)A.QS * 16 * tsz;
     dim3 grid(nblocks, A.CR / Wc);
