@@ -158,7 +158,8 @@ __global__ void __launch_bounds__(128) k_pot_m2m(PotArgs P, PotLevel Lp, PotLeve
 // M2L on one level.  G(x_a, y_b) depends on the box offset c_t - c_s alone, so the pairs of a level are
 // grouped by it: one block takes up to POT_COLS columns (pairs of one offset times densities) and 128 target
 // nodes, and generates each sample once for all of them instead of once per pair; a thread owns one target
-// node with its columns' sums in registers.  In FP32 the phase is split about the box centres
+// node with its columns' sums in registers.  The pairs' results go through a buffer of POT_BUFFER bytes, some pairs at a
+// time, and are added per target in the order of the pairs (k_pot_add), so that a call repeats bit for bit.  In FP32 the phase is split about the box centres
 // (kappa |D| in FP64 plus kappa (r - |D|), r - |D| = (2 D.d + |d|^2) / (r + |D|)) and the products take two
 // columns per instruction; the sums of 4 source nodes are added up with their rounding errors, then to Z in FP64.
 // The sine and cosine are rounded to FP32: at small kappa all samples have nearly one phase, and the errors of the
@@ -168,6 +169,10 @@ __global__ void __launch_bounds__(128) k_pot_m2m(PotArgs P, PotLevel Lp, PotLeve
 // tree included (before: a sample per pair with FP64 differences and sums, and per-node Lagrange values in
 // P2M).
 constexpr int POT_COLS = 16, POT_ROWS = 128, POT_STEP = 64, POT_GROUP = 4;
+// Results of the pairs at a time.  Each part ends with a wave of blocks that does not fill the device: 4001 points, q = 7,
+// 2 GB in all, FP32: 32 MiB 36.1, 128 MiB 35.5, 512 MiB 33.1, 2 GiB 33.2 ms (32.6 with atomics in no fixed order);
+// 20000 points, 8 densities: 860, 738, 699, 689 ms (674).
+constexpr size_t POT_BUFFER = size_t(512) << 20;
 
 __device__ inline float2 fma2x(float2 a, float2 b, float2 c) {  // two FP32 multiply-adds
   float2 d;
@@ -193,7 +198,7 @@ __device__ inline void sincos_series(float x, float xl, float &sn, float &cs) {
 
 template <class T>
 __global__ void __launch_bounds__(POT_ROWS) k_pot_m2l(PotArgs P, PotLevel L, const PotChunk *__restrict__ chunks,
-                                                      const int2 *__restrict__ pairs) {
+                                                      const int2 *__restrict__ pairs, int p0, double2 *__restrict__ out) {
   constexpr bool F32 = sizeof(T) == 4;
   __shared__ __align__(16) T wre[POT_STEP][POT_COLS];
   __shared__ __align__(16) T wim[POT_STEP][POT_COLS];
@@ -304,15 +309,32 @@ __global__ void __launch_bounds__(POT_ROWS) k_pot_m2l(PotArgs P, PotLevel L, con
 #pragma unroll
     for (int c = 0; c < POT_COLS; ++c) {
       if (c >= ncol) break;
-      double2 *z = L.Z + ((long)pairs[ck.first + c / R].x * Q + a) * R + c % R;
-      if constexpr (F32) {
-        atomicAdd(&z->x, (double)tr[c] + (double)lr[c]);
-        atomicAdd(&z->y, (double)ti[c] + (double)li[c]);
-      } else {
-        atomicAdd(&z->x, tr[c]);
-        atomicAdd(&z->y, ti[c]);
-      }
+      double2 *z = out + ((long)(ck.first - p0 + c / R) * Q + a) * R + c % R;
+      if constexpr (F32) *z = cmk((double)tr[c] + (double)lr[c], (double)ti[c] + (double)li[c]);
+      else *z = cmk(tr[c], ti[c]);
     }
+}
+
+// Z_t += the results of the pairs p0 .. p1 with target t, in the order of the pairs (list: each target's pairs, ascending)
+__global__ void __launch_bounds__(128) k_pot_add(PotLevel L, int QR, const int *__restrict__ ptr, const int *__restrict__ list,
+                                                 int p0, int p1, const double2 *__restrict__ out) {
+  const int t = blockIdx.x;
+  auto first = [&](int p) {  // first entry of target t that is not below p
+    int lo = ptr[t], hi = ptr[t + 1];
+    while (lo < hi) {
+      const int mid = (lo + hi) >> 1;
+      if (list[mid] < p) lo = mid + 1;
+      else hi = mid;
+    }
+    return lo;
+  };
+  const int k0 = first(p0), k1 = first(p1);
+  if (k0 == k1) return;
+  for (int o = blockIdx.y * 128 + threadIdx.x; o < QR; o += gridDim.y * 128) {
+    double2 z = L.Z[(long)t * QR + o];
+    for (int k = k0; k < k1; ++k) z = cadd(z, out[(long)(list[k] - p0) * QR + o]);
+    L.Z[(long)t * QR + o] = z;
+  }
 }
 
 // L2L from level l into level l + 1: Z_c[b] += sum_a T_c(a, b) Z_p[a], direction by direction; one block per
@@ -656,6 +678,7 @@ extern "C" int igabem_potential(igabem_problem *P, int n_rhs, const void *densit
     const int per = std::max(1, POT_COLS / R);
     std::vector<std::vector<int2>> fpair(D + 1);
     std::vector<std::vector<PotChunk>> chunk(D + 1);
+    std::vector<std::vector<int>> tptr_far(D + 1), tlist(D + 1);  // each target's pairs, ascending
     for (int l = 0; l <= D; ++l) {
       const size_t n = far[l].size();
       if (n == 0) continue;
@@ -688,6 +711,13 @@ extern "C" int igabem_potential(igabem_problem *P, int n_rhs, const void *densit
           i = e;
         }
       }
+      std::vector<int> &tp_ = tptr_far[l];
+      tp_.assign(keys[l].size() + 1, 0);
+      for (const int2 &f : fpair[l]) tp_[f.x + 1]++;
+      for (size_t t = 0; t + 1 < tp_.size(); ++t) tp_[t + 1] += tp_[t];
+      tlist[l].resize(n);
+      std::vector<int> fill(tp_.begin(), tp_.end() - 1);
+      for (size_t i = 0; i < n; ++i) tlist[l][fill[fpair[l][i].x]++] = (int)i;
     }
     int lmin = D + 1;
     for (int l = 0; l <= D; ++l)
@@ -722,6 +752,8 @@ extern "C" int igabem_potential(igabem_problem *P, int n_rhs, const void *densit
       add(sizeof(double) * 3 * n); add(sizeof(int) * 8 * n); add(sizeof(int) * n); add(sizeof(int) * n);
       add(sizeof(int2) * std::max<size_t>(fpair[l].size(), 1));
       add(sizeof(PotChunk) * std::max<size_t>(chunk[l].size(), 1));
+      add(sizeof(int) * std::max<size_t>(tptr_far[l].size(), 1));
+      add(sizeof(int) * std::max<size_t>(tlist[l].size(), 1));
       if (l >= lmin) {
         add(sizeof(double2) * n * Q * R);
         add(sizeof(double2) * n * Q * R);
@@ -735,7 +767,24 @@ extern "C" int igabem_potential(igabem_problem *P, int n_rhs, const void *densit
       if (!v.empty()) IGA_CUDA(cudaMemcpyAsync(p, v.data(), v.size() * sizeof(T), cudaMemcpyHostToDevice, st));
       return p;
     };
+    struct Buffer {
+      double2 *p = nullptr;
+      ~Buffer() { cudaFree(p); }
+    } out;
     try {
+      // the buffer of the pairs' results: smaller where the memory for it is not there (the results do not depend on it)
+      const size_t QR = (size_t)Q * R;
+      size_t most_pairs = 0, room = 0;  // pairs of a level; pairs that the buffer holds
+      for (int l = 0; l <= D; ++l) most_pairs = std::max(most_pairs, fpair[l].size());
+      if (most_pairs) {
+        room = std::min(most_pairs, std::max<size_t>(per, POT_BUFFER / (QR * sizeof(double2))));
+        while (cudaMalloc(&out.p, room * QR * sizeof(double2)) != cudaSuccess) {
+          cudaGetLastError();
+          out.p = nullptr;
+          if (room <= (size_t)per) fail(IGABEM_ENOMEM, "no device memory for the potential's buffer");
+          room = std::max<size_t>(per, room / 2);
+        }
+      }
       PotArgs PA{};
       PA.q = q;
       PA.Q = Q;
@@ -763,6 +812,7 @@ extern "C" int igabem_potential(igabem_problem *P, int n_rhs, const void *densit
       std::vector<int *> par_d(D + 1), slot_d(D + 1);
       std::vector<int2 *> pair_d(D + 1);
       std::vector<PotChunk *> chunk_d(D + 1);
+      std::vector<int *> tptr_d(D + 1), tlist_d(D + 1);
       for (int l = 0; l <= D; ++l) {
         PotLevel &L = LV[l];
         L.n = (int)keys[l].size();
@@ -775,6 +825,8 @@ extern "C" int igabem_potential(igabem_problem *P, int n_rhs, const void *densit
         L.child = up(with_src);
         pair_d[l] = up(fpair[l]);
         chunk_d[l] = up(chunk[l]);
+        tptr_d[l] = up(tptr_far[l]);
+        tlist_d[l] = up(tlist[l]);
         par_d[l] = up(parent[l].empty() ? std::vector<int>(1, 0) : parent[l]);
         slot_d[l] = up(slot[l].empty() ? std::vector<int>(1, 0) : slot[l]);
         L.W = L.Z = nullptr;
@@ -796,11 +848,20 @@ extern "C" int igabem_potential(igabem_problem *P, int n_rhs, const void *densit
           note_launch();
         }
         for (int l = lmin; l <= D; ++l) {
-          if (far[l].empty()) continue;
-          const dim3 grid((unsigned)chunk[l].size(), (Q + POT_ROWS - 1) / POT_ROWS);
-          if (fp32) k_pot_m2l<float><<<grid, POT_ROWS, 0, st>>>(PA, LV[l], chunk_d[l], pair_d[l]);
-          else k_pot_m2l<double><<<grid, POT_ROWS, 0, st>>>(PA, LV[l], chunk_d[l], pair_d[l]);
-          note_launch();
+          for (size_t i = 0; i < chunk[l].size();) {
+            const int p0 = chunk[l][i].first;
+            size_t e = i;
+            int p1 = p0;
+            for (; e < chunk[l].size() && (size_t)(p1 - p0 + chunk[l][e].count) <= room; ++e) p1 += chunk[l][e].count;
+            const dim3 grid((unsigned)(e - i), (Q + POT_ROWS - 1) / POT_ROWS);
+            if (fp32) k_pot_m2l<float><<<grid, POT_ROWS, 0, st>>>(PA, LV[l], chunk_d[l] + i, pair_d[l], p0, out.p);
+            else k_pot_m2l<double><<<grid, POT_ROWS, 0, st>>>(PA, LV[l], chunk_d[l] + i, pair_d[l], p0, out.p);
+            note_launch();
+            k_pot_add<<<dim3(LV[l].n, (unsigned)((QR + 511) / 512)), 128, 0, st>>>(LV[l], (int)QR, tptr_d[l], tlist_d[l], p0, p1,
+                                                                                  out.p);
+            note_launch();
+            i = e;
+          }
         }
         for (int l = lmin; l < D; ++l) {
           k_pot_l2l<<<dim3(LV[l + 1].n, R), 128, smt, st>>>(PA, LV[l], LV[l + 1], par_d[l + 1], slot_d[l + 1]);
