@@ -239,9 +239,10 @@ int igabem_rhs_sources(igabem_problem *prob, int n_rhs, const double *z, void *b
    (the representations of Sec. 2), summed over the regular Gauss rule of every element, by an
    interpolation fast multipole method in physical space (Sec. 4.4, last part, and Sec. 5.3): an octree
    over the sources and points (leaves of at most 64 Gauss points), min(cheb_q, 10)^3 Chebyshev nodes
-   per box, eta_adm and kappa_cap as for the surface tree, kernel samples generated on the fly (FP32 in
-   the mixed precisions, FP64 otherwise), the near field summed directly; no_fmm = 1 sums everything
-   directly.  u = [n_pts][n_rhs] complex (host or device).  Allocates its octree and expansions for the
+   per box, eta_adm and kappa_cap as for the surface tree, kernel samples generated on the fly and
+   multiplied with the expansions (FP32 in the mixed precisions: differences of 1e-9 to 3e-7 from the
+   FP64 form up to kappa = 20; FP64 otherwise), the near field summed directly in FP64; no_fmm = 1 sums everything directly.  Calls with
+   the same inputs give the same bits.  u = [n_pts][n_rhs] complex (host or device).  Allocates its octree and expansions for the
    duration of the call. */
 int igabem_potential(igabem_problem *prob, int n_rhs, const void *density, int n_pts, const double *pts,
                      void *u);

@@ -36,6 +36,8 @@ struct PotLevel {
   double half;              // half side
   const int *child;         // [n][8] child box on level l + 1 with sources, or -1
   double2 *W, *Z;           // multipole / local expansions [n][q^3][R]
+  double2 *M;               // FP32: sum of a box's expansion [n][R], and the power of two that scales its entries to
+  double *scale;            // at most 1
 };
 
 struct PotArgs {
@@ -155,20 +157,49 @@ __global__ void __launch_bounds__(128) k_pot_m2m(PotArgs P, PotLevel Lp, PotLeve
     for (int o = threadIdx.x; o < Q; o += blockDim.x) Lp.W[((long)t * Q + o) * R + r] = S[o];
 }
 
+// M and scale of one level's boxes, one warp per (box, column); a box without sources gets M = 0 (never read)
+__global__ void __launch_bounds__(128) k_pot_sums(PotLevel L, int Q, int R, const double2 *__restrict__ W) {
+  const long o = blockIdx.x * 4L + (threadIdx.x >> 5);
+  if (o >= (long)L.n * R) return;
+  const long b = o / R, r = o - b * R;
+  double2 sum = cmk(0, 0);
+  double most = 0;
+  for (int a = threadIdx.x & 31; a < Q; a += 32) {
+    const double2 w = W[(b * Q + a) * R + r];
+    sum = cadd(sum, w);
+    most = fmax(most, fmax(fabs(w.x), fabs(w.y)));
+  }
+  for (int k = 16; k > 0; k >>= 1) {
+    sum.x += __shfl_xor_sync(0xffffffffu, sum.x, k);
+    sum.y += __shfl_xor_sync(0xffffffffu, sum.y, k);
+    most = fmax(most, __shfl_xor_sync(0xffffffffu, most, k));
+  }
+  if ((threadIdx.x & 31) == 0) {
+    int e = 0;
+    if (most > 0 && isfinite(most)) frexp(most, &e);
+    L.M[o] = sum;
+    L.scale[o] = scalbn(1.0, -max(-1000, min(1000, e)));
+  }
+}
+
 // M2L on one level.  G(x_a, y_b) depends on the box offset c_t - c_s alone, so the pairs of a level are
 // grouped by it: one block takes up to POT_COLS columns (pairs of one offset times densities) and 128 target
 // nodes, and generates each sample once for all of them instead of once per pair; a thread owns one target
 // node with its columns' sums in registers.  The pairs' results go through a buffer of POT_BUFFER bytes, some pairs at a
-// time, and are added per target in the order of the pairs (k_pot_add), so that a call repeats bit for bit.  In FP32 the phase is split about the box centres
-// (kappa |D| in FP64 plus kappa (r - |D|), r - |D| = (2 D.d + |d|^2) / (r + |D|)) and the products take two
-// columns per instruction; the sums of 4 source nodes are added up with their rounding errors, then to Z in FP64.
-// The sine and cosine are rounded to FP32: at small kappa all samples have nearly one phase, and the errors of the
-// fast ones (4e-7) add up.  Difference to the FP64 form at kappa = 1, 3, 12, 20: 5, 5, 12, 20e-8 (rms; 17 to 28e-8 with
-// the fast ones and sums of 64, at 22 ms a call).
-// Measured on 4001 points around 6144 Gauss points, q = 7, 372,000 pairs (FP32): 1520 -> 36 ms a call, host
-// tree included (before: a sample per pair with FP64 differences and sums, and per-node Lagrange values in
-// P2M).
-constexpr int POT_COLS = 16, POT_ROWS = 128, POT_STEP = 64, POT_GROUP = 4;
+// time, and are added per target in the order of the pairs (k_pot_add), so that a call repeats bit for bit.  In FP32,
+// in units of the half side and about the source box's centre (distance r0 from the target node), a sample is
+//   G = exp(i kappa r0) / (4 pi half) (1 / r0 + h),  h = (exp(i kappa (r - r0)) - 1) / r + (1 / r - 1 / r0),
+// whose first part times the sum of the expansion is formed in FP64 and whose second, small unless the phase turns within
+// the box, from r^2 - r0^2 = |y|^2 - 2 X.y without cancellation: what FP32 rounds off samples, expansions (scaled by a
+// power of two per box) and products is a part of h, not of G.  The products take two columns per instruction, the
+// sums of 16 source nodes are added up with their rounding errors.  Difference to the FP64 form (rms, random densities,
+// sound-soft kappa = 0.3, 3, 12, 20): 0.25, 1.4, 8.0, 11e-8; sound-hard 0.5: 20e-8.  (A sample at a time with FP64
+// differences, expansions and sums 4.3, 7.9, 50, 90, 128e-8; FP32 products of G, split about the box centres, 4.5, 4.4,
+// 10, 14, 185e-8.)
+// Measured on 4001 points around 6144 Gauss points, q = 7, 372,000 pairs, host tree included: FP32 1516 -> 29.9 ms a
+// call (before: a sample per pair with FP64 differences and sums, and per-node Lagrange values in P2M), FP64 451 ms.
+// Groups of 4, 8, 16, 32 nodes: 35.4, 32.6, 29.9, 28.8 ms at 1.03, 1.13, 1.38, 1.87e-8 (kappa = 3).
+constexpr int POT_COLS = 16, POT_ROWS = 128, POT_STEP = 64, POT_GROUP = 16;
 // Results of the pairs at a time.  Each part ends with a wave of blocks that does not fill the device: 4001 points, q = 7,
 // 2 GB in all, FP32: 32 MiB 36.1, 128 MiB 35.5, 512 MiB 33.1, 2 GiB 33.2 ms (32.6 with atomics in no fixed order);
 // 20000 points, 8 densities: 860, 738, 699, 689 ms (674).
@@ -183,17 +214,18 @@ __device__ inline float2 fma2x(float2 a, float2 b, float2 c) {  // two FP32 mult
   return d;
 }
 
-// sine and cosine of x + xl, |x| < 1e6, xl tiny: reduced to |y| <= pi/4 about a multiple of pi/2, there the Taylor series
-// (first terms left out: 2e-9 and 3e-8 at pi/4)
-__device__ inline void sincos_series(float x, float xl, float &sn, float &cs) {
+// sin(x) and cos(x) - 1, |x| < 1e6: reduced to |y| <= pi/4 about a multiple of pi/2, there the Taylor series (first terms
+// left out: 2e-9 and 2e-10 at pi/4); for |x| < pi/4 both are accurate relative to themselves
+__device__ inline void sin_cosm1(float x, float &sn, float &cm) {
   const float m = fmaf(x, 0.636619772f, 12582912.f), k = m - 12582912.f;  // 1.5 2^23: rounds to an integer
   const int n = __float_as_int(m);
-  const float y = fmaf(-k, -4.37113883e-8f, fmaf(-k, 1.57079637f, x)) + xl, z = y * y;
+  const float y = fmaf(-k, -4.37113883e-8f, fmaf(-k, 1.57079637f, x)), z = y * y;
   const float s = fmaf(y * z, fmaf(z, fmaf(z, fmaf(z, 1.f / 362880, -1.f / 5040), 1.f / 120), -1.f / 6), y);
-  const float c = fmaf(z, fmaf(z, fmaf(z, fmaf(z, 1.f / 40320, -1.f / 720), 1.f / 24), -0.5f), 1.f);
-  const float a = n & 1 ? c : s, b = n & 1 ? s : c;
+  const float c = z * fmaf(z, fmaf(z, fmaf(z, fmaf(z, -1.f / 3628800, 1.f / 40320), -1.f / 720), 1.f / 24), -0.5f),
+              c1 = 1.f + c;
+  const float a = n & 1 ? c1 : s, b = n & 1 ? s : c1;
   sn = n & 2 ? -a : a;
-  cs = (n + 1) & 2 ? -b : b;
+  cm = n & 3 ? ((n + 1) & 2 ? -b : b) - 1.f : c;
 }
 
 template <class T>
@@ -204,36 +236,26 @@ __global__ void __launch_bounds__(POT_ROWS) k_pot_m2l(PotArgs P, PotLevel L, con
   __shared__ __align__(16) T wim[POT_STEP][POT_COLS];
   __shared__ __align__(16) T ys[POT_STEP][4];
   __shared__ double2 tab[F32 ? 1 : CIS_N];
+  __shared__ long wcol[POT_COLS];           // a column's first entry in W
+  __shared__ double scale[F32 ? POT_COLS : 1];
   const int Q = P.Q, q = P.q, R = P.R, tid = threadIdx.x;
   const PotChunk ck = chunks[blockIdx.x];
   const int ncol = ck.count * R, a = blockIdx.y * POT_ROWS + tid;
-  const double side = 2.0 * L.half;
-  const double Dd[3] = {ck.dx * side, ck.dy * side, ck.dz * side};
-  const double D2d = Dd[0] * Dd[0] + Dd[1] * Dd[1] + Dd[2] * Dd[2], Dnd = sqrt(D2d);
-  double c0 = 0, c1 = 0;
-  float phi0 = 0, phi0l = 0;  // kappa |D| in two floats
-  if constexpr (F32) {
-    const double x = P.kappa * Dnd, k = rint(x / TWO_PI);  // reduced to (-pi, pi]
-    const double ph = fma(-k, 2.4492935982947064e-16, fma(-k, TWO_PI, x));
-    phi0 = (float)ph;
-    phi0l = (float)(ph - (double)phi0);
-  } else {
-    phase64_scale(P.kappa, c0, c1);
-    for (int i = tid; i < CIS_N; i += POT_ROWS) tab[i] = P.cis[i];
+  if (tid < ncol) {
+    const long s = pairs[ck.first + tid / R].y;
+    wcol[tid] = s * Q * R + tid % R;
+    if constexpr (F32) scale[tid] = L.scale[s * R + tid % R];
   }
-  const T D[3] = {(T)Dd[0], (T)Dd[1], (T)Dd[2]}, D2 = (T)D2d, Dn = (T)Dnd, kappa = (T)P.kappa;
-  T xa[3] = {0, 0, 0};
+  // FP32: positions in units of the half side about the source centre; FP64: lengths
+  const double unit = F32 ? 1.0 : L.half;
+  double X[3] = {2.0 * unit * ck.dx, 2.0 * unit * ck.dy, 2.0 * unit * ck.dz};
   if (a < Q) {
-    xa[0] = (T)(P.cheb[a / (q * q)] * L.half);
-    xa[1] = (T)(P.cheb[(a / q) % q] * L.half);
-    xa[2] = (T)(P.cheb[a % q] * L.half);
+    X[0] += P.cheb[a / (q * q)] * unit;
+    X[1] += P.cheb[(a / q) % q] * unit;
+    X[2] += P.cheb[a % q] * unit;
   }
-  T Dx = 0;
-  if constexpr (F32) {
-    Dx = D[0] * xa[0] + D[1] * xa[1] + D[2] * xa[2];
-  } else {  // absolute positions about the source centre
-    for (int c = 0; c < 3; ++c) xa[c] += D[c];
-  }
+  double c0, c1;
+  phase64_scale(F32 ? P.kappa * L.half : P.kappa, c0, c1);
   T tr[POT_COLS], ti[POT_COLS];
   float lr[F32 ? POT_COLS : 1], li[F32 ? POT_COLS : 1];  // FP32: what the sums over the groups round off
 #pragma unroll
@@ -241,21 +263,36 @@ __global__ void __launch_bounds__(POT_ROWS) k_pot_m2l(PotArgs P, PotLevel L, con
     tr[c] = ti[c] = 0;
     if constexpr (F32) lr[c] = li[c] = 0;
   }
+  T x2[3] = {0, 0, 0}, r02 = 1, r0 = 1, ir0 = 1;  // FP32: -2 X, |X|^2, |X|, 1 / |X|
+  const T kappa = (T)(P.kappa * L.half);
+  if constexpr (F32) {
+    const double d2 = X[0] * X[0] + X[1] * X[1] + X[2] * X[2], id = rsqrt64(d2);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) x2[c] = (T)(-2.0 * X[c]);
+    r02 = (T)d2;
+    r0 = (T)(d2 * id);
+    ir0 = (T)id;
+  } else {
+    for (int i = tid; i < CIS_N; i += POT_ROWS) tab[i] = P.cis[i];
+  }
   for (int b0 = 0; b0 < Q; b0 += POT_STEP) {
     const int nb = min(POT_STEP, Q - b0);
     __syncthreads();
     for (int o = tid; o < nb * POT_COLS; o += POT_ROWS) {
       const int b = o / POT_COLS, c = o % POT_COLS;
       double2 v = cmk(0, 0);
-      if (c < ncol) v = L.W[((long)pairs[ck.first + c / R].y * Q + b0 + b) * R + c % R];
+      if (c < ncol) {
+        v = L.W[wcol[c] + (long)(b0 + b) * R];
+        if constexpr (F32) v = cscale(v, scale[c]);
+      }
       wre[b][c] = (T)v.x;
       wim[b][c] = (T)v.y;
     }
     for (int b = tid; b < nb; b += POT_ROWS) {
       const int bb = b0 + b;
-      const double y[3] = {P.cheb[bb / (q * q)] * L.half, P.cheb[(bb / q) % q] * L.half, P.cheb[bb % q] * L.half};
+      const double y[3] = {P.cheb[bb / (q * q)] * unit, P.cheb[(bb / q) % q] * unit, P.cheb[bb % q] * unit};
       for (int c = 0; c < 3; ++c) ys[b][c] = (T)y[c];
-      ys[b][3] = (T)(Dd[0] * y[0] + Dd[1] * y[1] + Dd[2] * y[2]);
+      ys[b][3] = (T)(y[0] * y[0] + y[1] * y[1] + y[2] * y[2]);
     }
     __syncthreads();
     if (a >= Q) continue;
@@ -265,13 +302,12 @@ __global__ void __launch_bounds__(POT_ROWS) k_pot_m2l(PotArgs P, PotLevel L, con
       for (int c = 0; c < POT_COLS / 2; ++c) pr[c] = pi[c] = make_float2(0.f, 0.f);
       for (int b = g0; b < min(nb, g0 + POT_GROUP); ++b) {
         const float4 y = *reinterpret_cast<const float4 *>(ys[b]);
-        const float d0 = xa[0] - y.x, d1 = xa[1] - y.y, d2 = xa[2] - y.z;
-        const float num = fmaf(2.f, Dx - y.w, fmaf(d0, d0, fmaf(d1, d1, d2 * d2)));
-        const float r2 = D2 + num, i0 = rsqrtf(r2), ir = fmaf(0.5f * i0, fmaf(-r2 * i0, i0, 1.f), i0), r = r2 * ir;
-        const float ph = fmaf(kappa, __fdividef(num, r + Dn), phi0);
-        float sn, cs;
-        sincos_series(ph, phi0l, sn, cs);
-        const float f = ir * 0.0795774715459476679f, gx = cs * f, gy = sn * f;
+        const float num = fmaf(x2[0], y.x, fmaf(x2[1], y.y, fmaf(x2[2], y.z, y.w)));  // r^2 - r0^2
+        const float r2 = r02 + num, i0 = rsqrtf(r2), ir = fmaf(0.5f * i0, fmaf(-r2 * i0, i0, 1.f), i0);
+        const float del = __fdividef(num, fmaf(r2, ir, r0));                            // r - r0
+        float sn, cm;
+        sin_cosm1(kappa * del, sn, cm);
+        const float gx = fmaf(-del, ir0, cm) * ir, gy = sn * ir;
         const float2 gxx = make_float2(gx, gx), gyy = make_float2(gy, gy), gyn = make_float2(-gy, -gy);
         const float4 *wr = reinterpret_cast<const float4 *>(wre[b]), *wi = reinterpret_cast<const float4 *>(wim[b]);
 #pragma unroll
@@ -292,7 +328,7 @@ __global__ void __launch_bounds__(POT_ROWS) k_pot_m2l(PotArgs P, PotLevel L, con
       }
     } else {
       for (int b = 0; b < nb; ++b) {
-        const double d0 = xa[0] - ys[b][0], d1 = xa[1] - ys[b][1], d2 = xa[2] - ys[b][2];
+        const double d0 = X[0] - ys[b][0], d1 = X[1] - ys[b][1], d2 = X[2] - ys[b][2];
         const double r2 = d0 * d0 + d1 * d1 + d2 * d2, ir = rsqrt64(r2), f = ir * (0.25 / IGA_PI);
         const Phase64 p = phase64(tab, r2 * ir, c0, c1);
         const C2<double> G = phase_mul(p.E.x * f, p.E.y * f, p);
@@ -305,14 +341,31 @@ __global__ void __launch_bounds__(POT_ROWS) k_pot_m2l(PotArgs P, PotLevel L, con
       }
     }
   }
-  if (a < Q)
+  if (a >= Q) return;
+  double fx = 0, fy = 0, id = 0;  // FP32: exp(i kappa r0) / (4 pi half), 1 / r0
+  if constexpr (F32) {
+    const double d2 = X[0] * X[0] + X[1] * X[1] + X[2] * X[2];
+    id = rsqrt64(d2);
+    const Phase64 p = phase64(P.cis, d2 * id, c0, c1);
+    const double f = 0.25 / IGA_PI / L.half;
+    const C2<double> E = phase_mul(p.E.x * f, p.E.y * f, p);
+    fx = E.x;
+    fy = E.y;
+  }
 #pragma unroll
-    for (int c = 0; c < POT_COLS; ++c) {
-      if (c >= ncol) break;
-      double2 *z = out + ((long)(ck.first - p0 + c / R) * Q + a) * R + c % R;
-      if constexpr (F32) *z = cmk((double)tr[c] + (double)lr[c], (double)ti[c] + (double)li[c]);
-      else *z = cmk(tr[c], ti[c]);
+  for (int c = 0; c < POT_COLS; ++c) {
+    if (c >= ncol) break;
+    double2 *z = out + ((long)(ck.first - p0 + c / R) * Q + a) * R + c % R;
+    if constexpr (F32) {
+      const double is = 1.0 / scale[c];  // exact
+      const double2 M = L.M[(long)pairs[ck.first + c / R].y * R + c % R];
+      const double hx = fma(id, M.x, ((double)tr[c] + (double)lr[c]) * is);
+      const double hy = fma(id, M.y, ((double)ti[c] + (double)li[c]) * is);
+      *z = cmk(fma(fx, hx, -fy * hy), fma(fx, hy, fy * hx));
+    } else {
+      *z = cmk(tr[c], ti[c]);
     }
+  }
 }
 
 // Z_t += the results of the pairs p0 .. p1 with target t, in the order of the pairs (list: each target's pairs, ascending)
@@ -757,6 +810,8 @@ extern "C" int igabem_potential(igabem_problem *P, int n_rhs, const void *densit
       if (l >= lmin) {
         add(sizeof(double2) * n * Q * R);
         add(sizeof(double2) * n * Q * R);
+        add(sizeof(double2) * n * R);
+        add(sizeof(double) * n * R);
       }
     }
     Arena A;
@@ -829,10 +884,13 @@ extern "C" int igabem_potential(igabem_problem *P, int n_rhs, const void *densit
         tlist_d[l] = up(tlist[l]);
         par_d[l] = up(parent[l].empty() ? std::vector<int>(1, 0) : parent[l]);
         slot_d[l] = up(slot[l].empty() ? std::vector<int>(1, 0) : slot[l]);
-        L.W = L.Z = nullptr;
+        L.W = L.Z = L.M = nullptr;
+        L.scale = nullptr;
         if (l >= lmin) {
           L.W = A.get<double2>((size_t)L.n * Q * R);
           L.Z = A.get<double2>((size_t)L.n * Q * R);
+          L.M = A.get<double2>((size_t)L.n * R);
+          L.scale = A.get<double>((size_t)L.n * R);
           IGA_CUDA(cudaMemsetAsync(L.Z, 0, sizeof(double2) * (size_t)L.n * Q * R, st));
         }
       }
@@ -848,6 +906,10 @@ extern "C" int igabem_potential(igabem_problem *P, int n_rhs, const void *densit
           note_launch();
         }
         for (int l = lmin; l <= D; ++l) {
+          if (fp32 && !chunk[l].empty()) {
+            k_pot_sums<<<(unsigned)(((long)LV[l].n * R + 3) / 4), 128, 0, st>>>(LV[l], Q, R, LV[l].W);
+            note_launch();
+          }
           for (size_t i = 0; i < chunk[l].size();) {
             const int p0 = chunk[l][i].first;
             size_t e = i;
