@@ -650,7 +650,8 @@ extern "C" int igabem_potential(igabem_problem *P, int n_rhs, const void *densit
       }
     }
     // dual traversal: admissible pairs per level with their box offsets, near leaf pairs.  The candidates of a level go
-    // over host threads in chunks, whose lists are joined in order (as one thread would form them).
+    // over host threads in chunks, whose lists are taken in order (as one thread would form them); a level's admissible
+    // pairs are sorted at once, so that the lists of one level alone are in memory with their offsets.
     struct Box {
       int i, j, k;
     };
@@ -660,19 +661,19 @@ extern "C" int igabem_potential(igabem_problem *P, int n_rhs, const void *densit
       for (long long v : keys[l]) box[l].push_back({int(v >> 42), int((v >> 21) & 0x1FFFFF), int(v & 0x1FFFFF)});
     }
     const double cap = o.kappa_cap > 0 ? o.kappa_cap : INFINITY;
-    struct FarPair {
-      int t, s;
-      short dx, dy, dz;  // box offset, below 2^10 in size
-    };
-    std::vector<std::vector<FarPair>> far(D + 1);
+    // admissible pairs of every level sorted by box offset, in chunks of POT_COLS columns
+    const int per = std::max(1, POT_COLS / R);
+    std::vector<std::vector<int2>> fpair(D + 1);
+    std::vector<std::vector<PotChunk>> chunk(D + 1);
+    std::vector<std::vector<int>> tptr_far(D + 1), tlist(D + 1);  // each target's pairs, ascending
     std::vector<std::pair<int, int>> near, cand{{0, 0}}, nxt;
     if (!(ht[0][0] && hs[0][0])) cand.clear();
     for (int l = 0; l <= D; ++l) {
       const double rad = side / (1 << l) * std::sqrt(3.0) / 2;
       const long n = (long)cand.size(), nch = std::min<long>(64, (n + 8191) / 8192);
       struct Part {
-        std::vector<FarPair> far;
-        std::vector<std::pair<int, int>> near, next;
+        std::vector<std::pair<int, int>> far, near, next;
+        int most = 0;  // largest box offset in far
       };
       std::vector<Part> part(nch);
       parallel_for(nch, [&](long c) {
@@ -685,7 +686,8 @@ extern "C" int igabem_potential(igabem_problem *P, int n_rhs, const void *densit
           const bool adm = !o.no_fmm && dist > 0 && 2 * rad <= o.eta_adm * dist && o.kappa * 2 * rad <= cap;
           if (adm) {
             const Box &bt = box[l][t], &bs = box[l][s];
-            q_.far.push_back({t, s, short(bt.i - bs.i), short(bt.j - bs.j), short(bt.k - bs.k)});
+            q_.far.push_back({t, s});
+            q_.most = std::max({q_.most, std::abs(bt.i - bs.i), std::abs(bt.j - bs.j), std::abs(bt.k - bs.k)});
           } else if (l == D) {
             q_.near.push_back({t, s});
           } else {
@@ -702,20 +704,69 @@ extern "C" int igabem_potential(igabem_problem *P, int n_rhs, const void *densit
           }
         }
       });
-      size_t nf = 0, nn = 0;
-      for (const Part &q_ : part) {
-        nf += q_.far.size();
-        nn += q_.next.size();
-      }
-      far[l].reserve(nf);
+      size_t n_next = 0;
+      for (const Part &q_ : part) n_next += q_.next.size();
       nxt.clear();
-      nxt.reserve(nn);
-      for (const Part &q_ : part) {
-        far[l].insert(far[l].end(), q_.far.begin(), q_.far.end());
+      nxt.reserve(n_next);
+      for (Part &q_ : part) {
         near.insert(near.end(), q_.near.begin(), q_.near.end());
         nxt.insert(nxt.end(), q_.next.begin(), q_.next.end());
+        std::vector<std::pair<int, int>>().swap(q_.near);
+        std::vector<std::pair<int, int>>().swap(q_.next);
       }
       cand.swap(nxt);
+      size_t nf = 0;
+      int most = 0;
+      for (const Part &q_ : part) {
+        nf += q_.far.size();
+        most = std::max(most, q_.most);
+      }
+      if (nf == 0) continue;
+      const long w = 2L * most + 1;
+      auto id = [&](const std::pair<int, int> &f) {  // of the pair's box offset
+        const Box &t = box[l][f.first], &s = box[l][f.second];
+        return ((t.i - s.i + most) * w + t.j - s.j + most) * w + t.k - s.k + most;
+      };
+      fpair[l].resize(nf);
+      auto add_chunks = [&](size_t first, size_t count, long o) {
+        for (size_t i = 0; i < count; i += per)
+          chunk[l].push_back({(int)(first + i), (int)std::min<size_t>(per, count - i), int(o / (w * w) - most),
+                              int(o / w % w - most), int(o % w - most)});
+      };
+      if (w * w * w <= 1 << 20) {  // counting sort over the offsets' cube
+        std::vector<int> first(w * w * w + 1, 0);
+        for (const Part &q_ : part)
+          for (const auto &f : q_.far) first[id(f) + 1]++;
+        for (long o = 0; o < w * w * w; ++o) {
+          if (first[o + 1]) add_chunks(first[o], first[o + 1], o);
+          first[o + 1] += first[o];
+        }
+        for (Part &q_ : part) {
+          for (const auto &f : q_.far) fpair[l][first[id(f)]++] = make_int2(f.first, f.second);
+          std::vector<std::pair<int, int>>().swap(q_.far);
+        }
+      } else {
+        size_t i = 0;
+        for (Part &q_ : part) {
+          for (const auto &f : q_.far) fpair[l][i++] = make_int2(f.first, f.second);
+          std::vector<std::pair<int, int>>().swap(q_.far);
+        }
+        auto key = [&](const int2 &f) { return id({f.x, f.y}); };
+        std::stable_sort(fpair[l].begin(), fpair[l].end(), [&](const int2 &x, const int2 &y) { return key(x) < key(y); });
+        for (i = 0; i < nf;) {
+          size_t e = i;
+          while (e < nf && key(fpair[l][e]) == key(fpair[l][i])) ++e;
+          add_chunks(i, e - i, key(fpair[l][i]));
+          i = e;
+        }
+      }
+      std::vector<int> &tp_ = tptr_far[l];
+      tp_.assign(keys[l].size() + 1, 0);
+      for (const int2 &f : fpair[l]) tp_[f.x + 1]++;
+      for (size_t t = 0; t + 1 < tp_.size(); ++t) tp_[t + 1] += tp_[t];
+      tlist[l].resize(nf);
+      std::vector<int> fill(tp_.begin(), tp_.end() - 1);
+      for (size_t i = 0; i < nf; ++i) tlist[l][fill[fpair[l][i].x]++] = (int)i;
     }
     auto csr = [](const std::vector<std::pair<int, int>> &pairs, int n, std::vector<int> &ptr, std::vector<int> &src) {
       ptr.assign(n + 1, 0);
@@ -727,54 +778,9 @@ extern "C" int igabem_potential(igabem_problem *P, int n_rhs, const void *densit
     };
     std::vector<int> nptr, nsrc;
     csr(near, nleaf, nptr, nsrc);
-    // admissible pairs of every level sorted by box offset, in chunks of POT_COLS columns
-    const int per = std::max(1, POT_COLS / R);
-    std::vector<std::vector<int2>> fpair(D + 1);
-    std::vector<std::vector<PotChunk>> chunk(D + 1);
-    std::vector<std::vector<int>> tptr_far(D + 1), tlist(D + 1);  // each target's pairs, ascending
-    for (int l = 0; l <= D; ++l) {
-      const size_t n = far[l].size();
-      if (n == 0) continue;
-      int most = 0;
-      for (const FarPair &f : far[l]) most = std::max({most, std::abs((int)f.dx), std::abs((int)f.dy), std::abs((int)f.dz)});
-      const long w = 2L * most + 1;
-      auto id = [&](const FarPair &f) { return ((f.dx + most) * w + f.dy + most) * w + f.dz + most; };
-      fpair[l].resize(n);
-      auto add_chunks = [&](size_t first, size_t count, const FarPair &f) {
-        for (size_t i = 0; i < count; i += per)
-          chunk[l].push_back({(int)(first + i), (int)std::min<size_t>(per, count - i), f.dx, f.dy, f.dz});
-      };
-      if (w * w * w <= 1 << 20) {  // counting sort over the offsets' cube
-        std::vector<int> first(w * w * w + 1, 0);
-        for (const FarPair &f : far[l]) first[id(f) + 1]++;
-        for (long i = 0; i < w * w * w; ++i) {
-          const int c = first[i + 1];
-          if (c)
-            add_chunks(first[i], c,
-                       {0, 0, short(i / (w * w) - most), short(i / w % w - most), short(i % w - most)});
-          first[i + 1] += first[i];
-        }
-        for (const FarPair &f : far[l]) fpair[l][first[id(f)]++] = make_int2(f.t, f.s);
-      } else {
-        std::stable_sort(far[l].begin(), far[l].end(), [&](const FarPair &x, const FarPair &y) { return id(x) < id(y); });
-        for (size_t i = 0; i < n;) {
-          size_t e = i;
-          for (; e < n && id(far[l][e]) == id(far[l][i]); ++e) fpair[l][e] = make_int2(far[l][e].t, far[l][e].s);
-          add_chunks(i, e - i, far[l][i]);
-          i = e;
-        }
-      }
-      std::vector<int> &tp_ = tptr_far[l];
-      tp_.assign(keys[l].size() + 1, 0);
-      for (const int2 &f : fpair[l]) tp_[f.x + 1]++;
-      for (size_t t = 0; t + 1 < tp_.size(); ++t) tp_[t + 1] += tp_[t];
-      tlist[l].resize(n);
-      std::vector<int> fill(tp_.begin(), tp_.end() - 1);
-      for (size_t i = 0; i < n; ++i) tlist[l][fill[fpair[l][i].x]++] = (int)i;
-    }
     int lmin = D + 1;
     for (int l = 0; l <= D; ++l)
-      if (!far[l].empty()) lmin = std::min(lmin, l);
+      if (!fpair[l].empty()) lmin = std::min(lmin, l);
     // interpolation tables
     std::vector<double> cheb(q + (size_t)q * q, 0.0), T1(2L * q * q);
     for (int a = 0; a < q; ++a) cheb[a] = std::cos((2 * a + 1) * M_PI / (2 * q));
