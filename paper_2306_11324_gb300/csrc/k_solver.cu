@@ -487,7 +487,7 @@ __global__ void k_gm_init(GmDev G, const double *__restrict__ beta, const int *_
     G.s[o] = active[o] ? 1.0 / beta[o] : 0.0;
   }
   if (blockIdx.x == 0 && threadIdx.x == 0) {
-    *G.j = 0;
+    G.j[0] = G.j[1] = 0;
     G.flags[0] = 0;
     G.flags[1] = 0;
   }
@@ -496,24 +496,22 @@ __global__ void k_gm_init(GmDev G, const double *__restrict__ beta, const int *_
 // Arnoldi column j of every active right-hand side: h = hA + hB (the two Gram-Schmidt passes), the norm from its G
 // partial sums nrm2, the new column of H rotated by the previous Givens rotations, the new rotation, g updated, the
 // convergence test |g_{j+1}| <= tol ||b||; s = 1 / h_{j+1,j} for the next basis vector (0 for finished
-// columns); then j advances.  One block, a warp per column: its lanes load 32 entries and rotations at a time,
-// lane 0 runs the recurrence over them.  flags[0] = every column finished, flags[1] = non-finite met.
-constexpr int ARN_WARPS = 16;
+// columns); then j advances.  A warp per column: its lanes load 32 entries and rotations at a time, lane 0 runs the
+// recurrence over them, 16 FP64 instructions a rotation, which hold the FP64 pipe of a quarter of an SM for 0.6 us;
+// so four warps a block, and as many blocks as the columns need (the last one to finish advances j).  200 iterations on
+// 216 unknowns with 16, 64, 256 columns: 48, 51, 94 ms (all columns in one block of 16 warps 73, 181, 645 ms; a thread per
+// column 95, 134, 174 ms).
+// flags[0] = every column finished, flags[1] = non-finite met in the cycle; j[1] counts the blocks that are done.
+constexpr int ARN_WARPS = 4;
 
 __global__ void __launch_bounds__(32 * ARN_WARPS) k_gm_arnoldi(GmDev G, const double2 *__restrict__ nrm2, int chunks) {
   __shared__ double2 hs[ARN_WARPS][32], cv[ARN_WARPS][32], sv[ARN_WARPS][32];
-  __shared__ int all_done, bad;
+  __shared__ int last, all_done;
   const int R = G.R, m = G.m, j = *G.j, wp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (threadIdx.x == 0) {
-    all_done = 1;
-    bad = 0;
-  }
-  __syncthreads();
-  for (int r = wp; r < R; r += ARN_WARPS) {
-    if (G.done[r]) {
-      if (lane == 0) G.s[r] = 0.0;
-      continue;
-    }
+  const int r = blockIdx.x * ARN_WARPS + wp;
+  if (r < R && G.done[r]) {
+    if (lane == 0) G.s[r] = 0.0;
+  } else if (r < R) {
     double n2 = 0.0;
     for (int g = lane; g < chunks; g += 32) n2 += nrm2[(size_t)g * R + r].x;
     for (int k = 16; k > 0; k >>= 1) n2 += __shfl_xor_sync(0xffffffffu, n2, k);
@@ -544,32 +542,43 @@ __global__ void __launch_bounds__(32 * ARN_WARPS) k_gm_arnoldi(GmDev G, const do
       __syncwarp();
       if (lane < n - 1) Hc[((size_t)i * m + j) * R] = hs[wp][lane];
     }
-    if (lane) continue;
-    const double den = sqrt(a.x * a.x + a.y * a.y + hn * hn);
-    const double2 c = den > 0 ? cmk(a.x / den, -a.y / den) : cmk(1, 0);
-    const double2 q = den > 0 ? cmk(hn / den, 0.0) : cmk(0, 0);
-    G.cs[j * R + r] = c;
-    G.sn[j * R + r] = q;
-    Hc[((size_t)j * m + j) * R] = cmk(den, 0);
-    Hc[((size_t)(j + 1) * m + j) * R] = cmk(0, 0);
-    const double2 gj = G.g[j * R + r];
-    const double2 gn = cmul(cmk(-q.x, q.y), gj);
-    G.g[(j + 1) * R + r] = gn;
-    G.g[j * R + r] = cmul(c, gj);
-    G.k[r] = j + 1;
-    const int its = ++G.its[r];
-    const double res = sqrt(gn.x * gn.x + gn.y * gn.y);
-    if (!isfinite(res) || !isfinite(hn)) atomicExch(&bad, 1);
-    const bool done = res <= G.tol * G.bn[r] || its >= G.maxit || hn == 0.0 || j + 1 >= m;
-    G.done[r] = done ? 1 : 0;
-    G.s[r] = (!done && hn > 0) ? 1.0 / hn : 0.0;
-    if (!done) atomicExch(&all_done, 0);
+    if (lane == 0) {
+      const double den = sqrt(a.x * a.x + a.y * a.y + hn * hn);
+      const double2 c = den > 0 ? cmk(a.x / den, -a.y / den) : cmk(1, 0);
+      const double2 q = den > 0 ? cmk(hn / den, 0.0) : cmk(0, 0);
+      G.cs[j * R + r] = c;
+      G.sn[j * R + r] = q;
+      Hc[((size_t)j * m + j) * R] = cmk(den, 0);
+      Hc[((size_t)(j + 1) * m + j) * R] = cmk(0, 0);
+      const double2 gj = G.g[j * R + r];
+      const double2 gn = cmul(cmk(-q.x, q.y), gj);
+      G.g[(j + 1) * R + r] = gn;
+      G.g[j * R + r] = cmul(c, gj);
+      G.k[r] = j + 1;
+      const int its = ++G.its[r];
+      const double res = sqrt(gn.x * gn.x + gn.y * gn.y);
+      if (!isfinite(res) || !isfinite(hn)) atomicExch(&G.flags[1], 1);
+      const bool done = res <= G.tol * G.bn[r] || its >= G.maxit || hn == 0.0 || j + 1 >= m;
+      G.done[r] = done ? 1 : 0;
+      G.s[r] = (!done && hn > 0) ? 1.0 / hn : 0.0;
+    }
   }
   __syncthreads();
   if (threadIdx.x == 0) {
+    __threadfence();  // the block's done[] and its read of j come before its count
+    last = atomicAdd(&G.j[1], 1) == (int)gridDim.x - 1;
+    all_done = 1;
+  }
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  for (int c = threadIdx.x; c < R; c += 32 * ARN_WARPS)
+    if (!__ldcg(&G.done[c])) atomicExch(&all_done, 0);
+  __syncthreads();
+  if (threadIdx.x == 0) {
     G.flags[0] = all_done;
-    G.flags[1] = bad;
-    *G.j = j + 1;
+    G.j[0] = j + 1;
+    G.j[1] = 0;
   }
 }
 
@@ -706,7 +715,7 @@ void launch_gm_iteration_tail(const GmDev &G, double *red, long N, double *vj, c
                                                                       pass ? reinterpret_cast<double2 *>(red) : nullptr);
     note_launch();
     if (pass) {
-      k_gm_arnoldi<<<1, 32 * ARN_WARPS, 0, st>>>(G, reinterpret_cast<const double2 *>(red), blocks);
+      k_gm_arnoldi<<<(R + ARN_WARPS - 1) / ARN_WARPS, 32 * ARN_WARPS, 0, st>>>(G, reinterpret_cast<const double2 *>(red), blocks);
       note_launch();
     }
   }

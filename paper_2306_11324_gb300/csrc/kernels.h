@@ -84,7 +84,7 @@ void launch_sub(const double *b, const double *y, double *r, long n, cudaStream_
 struct GmDev {
   int m, R, maxit;
   double tol;
-  int *j;                     // Arnoldi index
+  int *j;                     // [0] Arnoldi index, [1] blocks of k_gm_arnoldi that are done
   int *k, *its, *done;        // [R]
   int *flags;                 // [2]: every column finished; non-finite value met
   double2 *H;                 // [(m+1)][m][R]
