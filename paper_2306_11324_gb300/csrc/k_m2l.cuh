@@ -43,6 +43,23 @@ __device__ inline double rsqrt64(double x) {
   return fma(y, e * fma(e, 0.375, 0.5), y);
 }
 
+// 1 / x, x a normal number: the single-precision estimate y, one step of Householder's third-order iteration
+// y (1 + r + r^2), r = 1 - x y (the relative error of the estimate 2^-23, cubed).
+__device__ inline double rcp64(double x) {
+  const int hi = __double2hiint(x), lo = __double2loint(x);
+  const int e = ((hi >> 20) & 0x7FF) - 1023;       // x = m 2^e, |m| in [1, 2)
+  const int hm = hi - (e << 20);
+  float f;
+  asm("rcp.approx.ftz.f32 %0, %1;"
+      : "=f"(f)
+      : "f"(__uint_as_float((hi & 0x80000000u) | ((unsigned)((hm & 0x7FFFFFFF) - (896 << 20)) << 3 | (unsigned)lo >> 29))));
+  const unsigned fb = __float_as_uint(f);
+  const double y = __hiloint2double((int)((fb & 0x80000000u) | (((fb & 0x7FFFFFFFu) >> 3) + (896u << 20))) - (e << 20),
+                                    (int)(fb << 29));
+  const double r = fma(-x, y, 1.0);
+  return fma(y, fma(r, r, r), y);
+}
+
 // Table-driven exp(i kappa r) (Tang's method): kappa r = 2 pi (k + u) / CIS_N, |u| <= 1/2, so
 // exp(i kappa r) = table[k] (1 + m1 + i s) with m1 + i s = exp(2 pi i u / CIS_N) - 1 by its series.  c0 + c1 is
 // kappa CIS_N / (2 pi) in two doubles, so that u is correct to the rounding of r.
@@ -81,6 +98,20 @@ __device__ inline float phase32(float kappa, float d, float phi0) {
   constexpr float M = 12582912.f;  // 1.5 2^23: adding it rounds to an integer
   const float ph = fmaf(kappa, d, phi0), turns = fmaf(ph, 0.15915494309189533577f, M) - M;
   return fmaf(-turns, -1.7484556e-07f, fmaf(-turns, 6.28318548202514648f, ph));
+}
+
+// sin(x) and cos(x) - 1, |x| < 1e6: reduced to |y| <= pi/4 about a multiple of pi/2, there the Taylor series (first terms
+// left out: 2e-9 and 2e-10 at pi/4); for |x| < pi/4 both are accurate relative to themselves
+__device__ inline void sin_cosm1(float x, float &sn, float &cm) {
+  const float m = fmaf(x, 0.636619772f, 12582912.f), k = m - 12582912.f;  // 1.5 2^23: rounds to an integer
+  const int n = __float_as_int(m);
+  const float y = fmaf(-k, -4.37113883e-8f, fmaf(-k, 1.57079637f, x)), z = y * y;
+  const float s = fmaf(y * z, fmaf(z, fmaf(z, fmaf(z, 1.f / 362880, -1.f / 5040), 1.f / 120), -1.f / 6), y);
+  const float c = z * fmaf(z, fmaf(z, fmaf(z, fmaf(z, -1.f / 3628800, 1.f / 40320), -1.f / 720), 1.f / 24), -0.5f),
+              c1 = 1.f + c;
+  const float a = n & 1 ? c1 : s, b = n & 1 ? s : c1;
+  sn = n & 2 ? -a : a;
+  cm = n & 3 ? ((n + 1) & 2 ? -b : b) - 1.f : c;
 }
 
 // s + l += v, l the rounding errors of s (Knuth's two-sum)

@@ -214,20 +214,6 @@ __device__ inline float2 fma2x(float2 a, float2 b, float2 c) {  // two FP32 mult
   return d;
 }
 
-// sin(x) and cos(x) - 1, |x| < 1e6: reduced to |y| <= pi/4 about a multiple of pi/2, there the Taylor series (first terms
-// left out: 2e-9 and 2e-10 at pi/4); for |x| < pi/4 both are accurate relative to themselves
-__device__ inline void sin_cosm1(float x, float &sn, float &cm) {
-  const float m = fmaf(x, 0.636619772f, 12582912.f), k = m - 12582912.f;  // 1.5 2^23: rounds to an integer
-  const int n = __float_as_int(m);
-  const float y = fmaf(-k, -4.37113883e-8f, fmaf(-k, 1.57079637f, x)), z = y * y;
-  const float s = fmaf(y * z, fmaf(z, fmaf(z, fmaf(z, 1.f / 362880, -1.f / 5040), 1.f / 120), -1.f / 6), y);
-  const float c = z * fmaf(z, fmaf(z, fmaf(z, fmaf(z, -1.f / 3628800, 1.f / 40320), -1.f / 720), 1.f / 24), -0.5f),
-              c1 = 1.f + c;
-  const float a = n & 1 ? c1 : s, b = n & 1 ? s : c1;
-  sn = n & 2 ? -a : a;
-  cm = n & 3 ? ((n + 1) & 2 ? -b : b) - 1.f : c;
-}
-
 template <class T>
 __global__ void __launch_bounds__(POT_ROWS) k_pot_m2l(PotArgs P, PotLevel L, const PotChunk *__restrict__ chunks,
                                                       const int2 *__restrict__ pairs, int p0, double2 *__restrict__ out) {

@@ -125,22 +125,6 @@ __device__ inline int point_of(int mask, int i) {
 __device__ inline bool d4_swaps(int k) { return (k & 1) != (k >= 4); }
 __device__ inline bool d4_flips(int k, int c) { return ((c == 0 ? 0x6C : 0xC6) >> k) & 1; }
 
-// 1 / x, x a normal number: the single-precision estimate, one third-order step
-__device__ inline double rcp64(double x) {
-  const int hi = __double2hiint(x), lo = __double2loint(x);
-  const int e = ((hi >> 20) & 0x7FF) - 1023;       // x = m 2^e, |m| in [1, 2)
-  const int hm = hi - (e << 20);
-  float f;
-  asm("rcp.approx.ftz.f32 %0, %1;"
-      : "=f"(f)
-      : "f"(__uint_as_float((hi & 0x80000000u) | ((unsigned)((hm & 0x7FFFFFFF) - (896 << 20)) << 3 | (unsigned)lo >> 29))));
-  const unsigned fb = __float_as_uint(f);
-  const double y = __hiloint2double((int)((fb & 0x80000000u) | (((fb & 0x7FFFFFFFu) >> 3) + (896u << 20))) - (e << 20),
-                                    (int)(fb << 29));
-  const double r = fma(-x, y, 1.0);
-  return fma(y, fma(r, r, r), y);
-}
-
 // shared-memory layout, offsets in doubles
 template <int P1, bool HARD> struct Lay {
   static constexpr int G = HARD ? 6 : 2;              // kernel groups: xy, yx, and the four curl terms
