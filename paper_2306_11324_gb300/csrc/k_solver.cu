@@ -194,15 +194,6 @@ __global__ void __launch_bounds__(256) k_farfield(RhsArgs A, const double2 *__re
 // conversions in every block).
 constexpr int FF_LANES = 4, FF_COLS = 8, FF_CHUNK = 256, FF_TH = 64;
 
-__device__ inline float2 ff_fma2(float2 a, float2 b, float2 c) {  // two FP32 multiply-adds
-  float2 d;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;"
-      : "=l"(reinterpret_cast<unsigned long long &>(d))
-      : "l"(reinterpret_cast<const unsigned long long &>(a)), "l"(reinterpret_cast<const unsigned long long &>(b)),
-        "l"(reinterpret_cast<const unsigned long long &>(c)));
-  return d;
-}
-
 template <int DPT, bool HARD>
 __global__ void __launch_bounds__(FF_LANES *FF_TH) k_farfield32(RhsArgs A, const float2 *__restrict__ rho, int fe, int n_dir,
                                                                const double *__restrict__ xhat, double2 *__restrict__ uinf) {
@@ -285,8 +276,8 @@ __global__ void __launch_bounds__(FF_LANES *FF_TH) k_farfield32(RhsArgs A, const
             const float2 exx = make_float2(ex, ex), eyy = make_float2(ey, ey), eyn = make_float2(-ey, -ey);
 #pragma unroll
             for (int cc = 0; cc < FF_COLS / 2; ++cc) {
-              ar[d][cc] = ff_fma2(exx, re[cc], ff_fma2(eyn, im[cc], ar[d][cc]));
-              ai[d][cc] = ff_fma2(exx, im[cc], ff_fma2(eyy, re[cc], ai[d][cc]));
+              ar[d][cc] = fma2x(exx, re[cc], fma2x(eyn, im[cc], ar[d][cc]));
+              ai[d][cc] = fma2x(exx, im[cc], fma2x(eyy, re[cc], ai[d][cc]));
             }
           }
         }
@@ -401,14 +392,13 @@ __global__ void k_dot_final(const double2 *__restrict__ red, const int *__restri
 }
 
 __global__ void k_multiaxpy(const double2 *__restrict__ V, int nv, const double2 *__restrict__ h,
-                            double2 *__restrict__ w, long N, int R, double sign) {
+                            double2 *__restrict__ w, long N, int R) {
   GRID_STRIDE(o, N * R) {
     int r = int(o % R);
     double2 acc = w[o];
 #pragma unroll 4
     for (int i = 0; i < nv; ++i) {
-      double2 t = cmul(V[(size_t)i * N * R + o], h[i * R + r]);
-      acc = cmk(acc.x + sign * t.x, acc.y + sign * t.y);
+      acc = cadd(acc, cmul(V[(size_t)i * N * R + o], h[i * R + r]));
     }
     w[o] = acc;
   }
@@ -506,9 +496,10 @@ constexpr int ARN_WARPS = 4;
 
 __global__ void __launch_bounds__(32 * ARN_WARPS) k_gm_arnoldi(GmDev G, const double2 *__restrict__ nrm2, int chunks) {
   __shared__ double2 hs[ARN_WARPS][32], cv[ARN_WARPS][32], sv[ARN_WARPS][32];
-  __shared__ int last, all_done;
+  __shared__ int last, all_done, unfinished[ARN_WARPS];
   const int R = G.R, m = G.m, j = *G.j, wp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int r = blockIdx.x * ARN_WARPS + wp;
+  if (lane == 0) unfinished[wp] = 0;
   if (r < R && G.done[r]) {
     if (lane == 0) G.s[r] = 0.0;
   } else if (r < R) {
@@ -561,9 +552,19 @@ __global__ void __launch_bounds__(32 * ARN_WARPS) k_gm_arnoldi(GmDev G, const do
       const bool done = res <= G.tol * G.bn[r] || its >= G.maxit || hn == 0.0 || j + 1 >= m;
       G.done[r] = done ? 1 : 0;
       G.s[r] = (!done && hn > 0) ? 1.0 / hn : 0.0;
+      unfinished[wp] = !done;
     }
   }
   __syncthreads();
+  if (gridDim.x == 1) {  // no other block to wait for
+    if (threadIdx.x == 0) {
+      int any = 0;
+      for (int w = 0; w < ARN_WARPS; ++w) any |= unfinished[w];
+      G.flags[0] = !any;
+      G.j[0] = j + 1;
+    }
+    return;
+  }
   if (threadIdx.x == 0) {
     __threadfence();  // the block's done[] and its read of j come before its count
     last = atomicAdd(&G.j[1], 1) == (int)gridDim.x - 1;
@@ -739,7 +740,7 @@ void launch_gm_solve(const GmDev &G, cudaStream_t st) {
 void launch_update(const double *V, int nv, const double *y, double *x, long N, int R, cudaStream_t st) {
   k_multiaxpy<<<grid_for(N * R), 256, 0, st>>>(reinterpret_cast<const double2 *>(V), nv,
                                                 reinterpret_cast<const double2 *>(y),
-                                                reinterpret_cast<double2 *>(x), N, R, 1.0);
+                                                reinterpret_cast<double2 *>(x), N, R);
   note_launch();
 }
 
