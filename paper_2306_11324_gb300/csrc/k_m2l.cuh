@@ -21,6 +21,15 @@ template <class T> __device__ inline C2<T> fma2(C2<T> a, C2<T> b, C2<T> acc) {  
   return {acc.x + a.x * b.x - a.y * b.y, acc.y + a.x * b.y + a.y * b.x};
 }
 
+__device__ inline float2 fma2x(float2 a, float2 b, float2 c) {  // two FP32 multiply-adds, a b + c
+  float2 d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;"
+      : "=l"(reinterpret_cast<unsigned long long &>(d))
+      : "l"(reinterpret_cast<const unsigned long long &>(a)), "l"(reinterpret_cast<const unsigned long long &>(b)),
+        "l"(reinterpret_cast<const unsigned long long &>(c)));
+  return d;
+}
+
 constexpr double TWO_PI = 6.283185307179586476925286766559;
 
 // ---- FP64 arithmetic of the kernel samples -------------------------------------------------------

@@ -7,7 +7,7 @@
 //     [Re Y]   [Re S  -Im S] [Re X]
 //     [Im Y] = [Im S   Re S] [Im X],
 // so the MMA has M = 128 rows (Re rows 0..q^2-1, Im rows 64..64+q^2-1), K = 2 KH (Re X in k < q^2,
-// Im X in KH <= k < KH + q^2, KH = q^2 rounded up to 8) and N = up to 64 right-hand-side columns per
+// Im X in KH <= k < KH + q^2, KH = q^2 rounded up to 8) and N = up to 192 right-hand-side columns per
 // instruction.  FP32 accuracy from FP16 operands: every operand is first scaled by an exact power of two
 // (per pair for S, from a bound on the kernel over the two clusters; per source cluster for X, from its
 // largest entry) so that its entries lie well inside the FP16 range, then split v = hi + lo
@@ -247,8 +247,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_m2l_tc(const TCArgs A) {
 
   // both A buffers are zeroed once: the padding rows and columns are never written
   for (uint32_t i = tid; i < 4 * AB / 16; i += TC_THREADS) reinterpret_cast<uint4 *>(smt)[i] = make_uint4(0, 0, 0, 0);
-  // nodes of cluster cl as [x - c, D.(x - c)][n~, D.n~][a, 0, 0, 0] (D of pair kk) by the threads lo .. lo + nt - 1
-  auto stage_nodes = [&](float *dst, int cl, int kk, int lo, int nt) {
+  // nodes of cluster cl as [x - c, D.(x - c)][n~, D.n~][a, 0, 0, 0] (D of pair kk; 0 without one)
+  auto stage_nodes = [&](float *dst, int cl, int kk) {
     float Dv[3] = {0.f, 0.f, 0.f};
     if (kk >= 0) {
       const float4 p0 = reinterpret_cast<const float4 *>(L.pc)[2 * kk];
@@ -256,7 +256,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_m2l_tc(const TCArgs A) {
       Dv[1] = p0.y;
       Dv[2] = p0.z;
     }
-    for (int a = tid - lo; a < Q; a += nt) {
+    for (int a = tid; a < Q; a += TC_THREADS) {
       const long ia = (long)cl * Q + a;
       float v[7];
       for (int c = 0; c < 7; ++c) v[c] = L.nodes32[c * NQ + ia];
@@ -266,8 +266,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_m2l_tc(const TCArgs A) {
       o[2] = make_float4(v[6], 0.f, 0.f, 0.f);
     }
   };
-  stage_nodes(tn, t, -1, 0, TC_THREADS);
-  for (int p = 0; p < 2 && p < npairs; ++p) stage_nodes(snb + p * 768, L.far_src[k0 + p], k0 + p, 0, TC_THREADS);
+  stage_nodes(tn, t, -1);
+  for (int p = 0; p < 2 && p < npairs; ++p) stage_nodes(snb + p * 768, L.far_src[k0 + p], k0 + p);
   for (int p = tid; p < min(npairs, TC_LIST); p += TC_THREADS) {
     const int src = L.far_src[k0 + p];
     slist[p] = src;

@@ -66,8 +66,7 @@ extern "C" int igabem_farfield_noalloc(igabem_problem *P, int n_rhs, const void 
   return run_guarded([&] {
     if (!P || !density || !xhat || !uinf || n_rhs <= 0 || n_dir <= 0)
       fail(IGABEM_EINVAL, "invalid arguments to igabem_farfield_noalloc");
-    // the far-field kernel runs one thread block per (direction, right-hand side), the right-hand sides
-    // along the grid's y dimension
+    // the far-field kernels take the right-hand sides along the grid's y dimension; what fits stays as documented
     if (n_rhs > 65535) fail(IGABEM_EINVAL, "igabem_farfield_noalloc: at most 65535 right-hand sides per call");
     const HostSetup &S = P->S;
     const long gst = (long)S.E * S.ng * S.ng;

@@ -205,15 +205,6 @@ constexpr int POT_COLS = 16, POT_ROWS = 128, POT_STEP = 64, POT_GROUP = 16;
 // 20000 points, 8 densities: 860, 738, 699, 689 ms (674).
 constexpr size_t POT_BUFFER = size_t(512) << 20;
 
-__device__ inline float2 fma2x(float2 a, float2 b, float2 c) {  // two FP32 multiply-adds
-  float2 d;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;"
-      : "=l"(reinterpret_cast<unsigned long long &>(d))
-      : "l"(reinterpret_cast<const unsigned long long &>(a)), "l"(reinterpret_cast<const unsigned long long &>(b)),
-        "l"(reinterpret_cast<const unsigned long long &>(c)));
-  return d;
-}
-
 template <class T>
 __global__ void __launch_bounds__(POT_ROWS) k_pot_m2l(PotArgs P, PotLevel L, const PotChunk *__restrict__ chunks,
                                                       const int2 *__restrict__ pairs, int p0, double2 *__restrict__ out) {

@@ -47,15 +47,6 @@ __device__ inline void cp_async_zfill(void *dst, const void *src, int src_bytes)
                : "memory");
 }
 
-__device__ inline float2 fma2x(float2 a, float2 b, float2 c) {  // two FP32 multiply-adds
-  float2 d;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;"
-      : "=l"(reinterpret_cast<unsigned long long &>(d))
-      : "l"(reinterpret_cast<const unsigned long long &>(a)), "l"(reinterpret_cast<const unsigned long long &>(b)),
-        "l"(reinterpret_cast<const unsigned long long &>(c)));
-  return d;
-}
-
 // The sums over the pairs in FP32 carry a compensation term (Neumaier: hi, lo), as accurate as FP64 sums here
 // without FP64 arithmetic.
 __device__ inline void sum_add(float4 &t, float x, float y) {
@@ -124,7 +115,7 @@ template <int NC, bool NEAR, bool ONE>
 __global__ void __launch_bounds__(ONE ? 160 : 288, ONE ? 2 : 1) k_stream32(const __grid_constant__ StreamArgs A) {
   extern __shared__ __align__(16) unsigned char sms[];
   __shared__ __align__(8) uint64_t full[STREAM_STAGES], empty[STREAM_STAGES];
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, nsplit = gridDim.y, rank = blockIdx.y;
+  const int tid = threadIdx.x, lane = tid & 31, nsplit = gridDim.y, rank = blockIdx.y;
   const int ncons = blockDim.x - 32;  // threads that multiply; the last warp copies
   const int tg = blockIdx.x / A.npass, c_pass = A.c0 + (blockIdx.x - tg * A.npass) * A.w;
   int li = 0;
