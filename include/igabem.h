@@ -241,9 +241,10 @@ int igabem_rhs_sources(igabem_problem *prob, int n_rhs, const double *z, void *b
    over the sources and points (leaves of at most 64 Gauss points), min(cheb_q, 10)^3 Chebyshev nodes
    per box, eta_adm and kappa_cap as for the surface tree, kernel samples generated on the fly and
    multiplied with the expansions (FP32 in the mixed precisions: differences of 1e-9 to 3e-7 from the
-   FP64 form up to kappa = 20; FP64 otherwise), the near field summed directly in FP64; no_fmm = 1 sums everything directly.  Calls with
-   the same inputs give the same bits.  u = [n_pts][n_rhs] complex (host or device).  Allocates its octree and expansions for the
-   duration of the call. */
+   FP64 form up to kappa = 20; FP64 otherwise), the near field summed directly in FP64; no_fmm = 1 sums
+   everything directly.  Calls with the same inputs give the same bits.  u = [n_pts][n_rhs] complex (host
+   or device).  Allocates its octree and expansions, and up to 512 MiB for the results of box pairs, for
+   the duration of the call. */
 int igabem_potential(igabem_problem *prob, int n_rhs, const void *density, int n_pts, const double *pts,
                      void *u);
 
