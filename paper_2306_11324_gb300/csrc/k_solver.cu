@@ -649,14 +649,32 @@ void launch_farfield(const DeviceProblem &d, const HostSetup &S, const igabem_op
     const int fe = std::min(S.m, 4);
     const long ngroups = (long)S.np << (2 * (S.m - fe));
     IGA_CUDA(cudaMemsetAsync(uinf, 0, sizeof(double2) * (size_t)n_dir * R, st));
-    // four directions a thread where they fill a block (the most work per shared load), fewer for few directions
-    auto go = [&](auto kfn, int dpt) {
+    // Directions a thread: more of them share a load, fewer make more blocks.  A launch lasts as long as the SM with the
+    // most blocks; the measured milliseconds for k blocks on it (4096 points, 24 columns, sound-soft and sound-hard alike) with
+    // one direction a thread are 0.54, 0.67, -, 1.15 for k = 1, 2, 3, 4, with two 0.82, 1.09, 1.53, with four 1.07, 1.8, 2.6;
+    // the least of them is taken.  24 columns, one, two, four directions a thread: 6 groups, 3000 directions 0.67, 0.82, 1.07;
+    // 6000: 1.15, 1.09, 1.07; 16 groups, 6000: 2.6, 2.4, 2.6; 24 groups, 3000: 2.4, 2.2, 1.9; 96 groups, 1000: 3.2, 3.2, 3.0 ms.
+    struct Form {
+      int dpt;
+      double first, each;
+    };
+    int dpt = 1;
+    double least = 1e300;
+    for (const Form &f : {Form{1, 0.54, 0.29}, Form{2, 0.82, 0.51}, Form{4, 1.07, 0.88}}) {
+      const long blocks = ngroups * ((n_dir + FF_TH * f.dpt - 1) / (FF_TH * f.dpt));
+      const double t = std::max(f.first, f.each * ((blocks + 151) / 152));
+      if (t < least) {
+        least = t;
+        dpt = f.dpt;
+      }
+    }
+    auto go = [&](auto kfn) {
       const dim3 g32((unsigned)ngroups, (unsigned)((n_dir + FF_TH * dpt - 1) / (FF_TH * dpt)));
       kfn<<<g32, FF_LANES * FF_TH, 0, st>>>(A, rho32, fe, n_dir, xhat_dev, reinterpret_cast<double2 *>(uinf));
     };
-    if (n_dir > 128) S.hard ? go(k_farfield32<4, true>, 4) : go(k_farfield32<4, false>, 4);
-    else if (n_dir > 64) S.hard ? go(k_farfield32<2, true>, 2) : go(k_farfield32<2, false>, 2);
-    else S.hard ? go(k_farfield32<1, true>, 1) : go(k_farfield32<1, false>, 1);
+    if (dpt == 4) S.hard ? go(k_farfield32<4, true>) : go(k_farfield32<4, false>);
+    else if (dpt == 2) S.hard ? go(k_farfield32<2, true>) : go(k_farfield32<2, false>);
+    else S.hard ? go(k_farfield32<1, true>) : go(k_farfield32<1, false>);
     note_launch();
     IGA_CUDA(cudaGetLastError());
     return;
