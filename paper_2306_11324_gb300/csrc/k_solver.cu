@@ -120,23 +120,26 @@ __global__ void k_density(RhsArgs A, const int *__restrict__ x2g, const double2 
 // u_inf[k][r] = sum_points rho * exp(-i kappa x^_k . x) * (soft: -a/(4 pi); hard: -i kappa (x^.n~)/(4 pi)) in FP64.  One
 // block per direction and four columns, which share the exponential (FP64 arithmetic bounds it: 18 operations for
 // the table-driven exponential instead of CUDA's sincos per column); the points are split over a cluster of
-// gridDim.z blocks where there are few directions.
+// gridDim.z blocks where there are few directions.  A single column has a form of its own: columns that are not there cost
+// the wider one as much as the others.  98304 points, 3000 directions, 1 and 4 columns: 12.1 and 17.9 ms (one column in the wide form
+// 19.1, CUDA's sincos per column 18.4 and 72).
 constexpr int FF64_COLS = 4;
 
-__global__ void __launch_bounds__(256) k_farfield(RhsArgs A, const double2 *__restrict__ rho, long npts,
+template <int NC>
+__global__ void __launch_bounds__(256, NC == 1 ? 4 : 3) k_farfield(RhsArgs A, const double2 *__restrict__ rho, long npts,
                                                   const double *__restrict__ xhat, const double2 *__restrict__ cis,
                                                   double2 *__restrict__ uinf) {
   __shared__ double2 tab[CIS_N];
-  __shared__ double2 red[8][FF64_COLS];
-  const int k = blockIdx.x, r0 = blockIdx.y * FF64_COLS, nr = min(FF64_COLS, A.R - r0), nz = gridDim.z;
+  __shared__ double2 red[8][NC];
+  const int k = blockIdx.x, r0 = blockIdx.y * NC, nr = min(NC, A.R - r0), nz = gridDim.z;
   const double xh[3] = {xhat[3 * k], xhat[3 * k + 1], xhat[3 * k + 2]};
   double c0, c1;
   phase64_scale(A.kappa, c0, c1);
   for (int i = threadIdx.x; i < CIS_N; i += 256) tab[i] = cis[i];
   __syncthreads();
-  double2 acc[FF64_COLS];
+  double2 acc[NC];
 #pragma unroll
-  for (int r = 0; r < FF64_COLS; ++r) acc[r] = cmk(0, 0);
+  for (int r = 0; r < NC; ++r) acc[r] = cmk(0, 0);
   for (long i = blockIdx.z * 256 + threadIdx.x; i < npts; i += 256L * nz) {
     const double d = fma(xh[0], A.gpx[i], fma(xh[1], A.gpx[A.gst + i], xh[2] * A.gpx[2 * A.gst + i]));
     const Phase64 p = phase64(tab, d, c0, c1);
@@ -152,7 +155,7 @@ __global__ void __launch_bounds__(256) k_farfield(RhsArgs A, const double2 *__re
       f = cmk(-e.x, e.y);
     }
 #pragma unroll
-    for (int r = 0; r < FF64_COLS; ++r)
+    for (int r = 0; r < NC; ++r)
       if (r < nr) {
         const double2 v = rho[i * A.R + r0 + r];
         acc[r].x = fma(f.x, v.x, fma(-f.y, v.y, acc[r].x));
@@ -160,7 +163,7 @@ __global__ void __launch_bounds__(256) k_farfield(RhsArgs A, const double2 *__re
       }
   }
 #pragma unroll
-  for (int r = 0; r < FF64_COLS; ++r) {
+  for (int r = 0; r < NC; ++r) {
     for (int o = 16; o > 0; o >>= 1) {
       acc[r].x += __shfl_xor_sync(0xffffffffu, acc[r].x, o);
       acc[r].y += __shfl_xor_sync(0xffffffffu, acc[r].y, o);
@@ -173,7 +176,7 @@ __global__ void __launch_bounds__(256) k_farfield(RhsArgs A, const double2 *__re
   if (blockIdx.z == 0 && (int)threadIdx.x < nr) {
     double2 s = cmk(0, 0);
     for (int z = 0; z < nz; ++z) {
-      const double2(*rz)[FF64_COLS] = nz > 1 ? cl.map_shared_rank(red, z) : red;
+      const double2(*rz)[NC] = nz > 1 ? cl.map_shared_rank(red, z) : red;
       for (int w = 0; w < 8; ++w) s = cadd(s, rz[w][threadIdx.x]);
     }
     uinf[(long)k * A.R + r0 + threadIdx.x] = cscale(s, 0.25 / IGA_PI);
@@ -681,7 +684,7 @@ void launch_farfield(const DeviceProblem &d, const HostSetup &S, const igabem_op
   }
   k_density<double2><<<dgrid, 256, 0, st>>>(A, d.x2g, reinterpret_cast<const double2 *>(dens), S.E, rho);
   note_launch();
-  const int cols = (R + FF64_COLS - 1) / FF64_COLS;
+  const int per = R == 1 ? 1 : FF64_COLS, cols = (R + per - 1) / per;
   int nz = 1;
   while (nz < 8 && (long)n_dir * cols * nz < 4 * 152 && npts >= 1024L * nz) nz *= 2;
   cudaLaunchConfig_t cfg{};
@@ -694,7 +697,7 @@ void launch_farfield(const DeviceProblem &d, const HostSetup &S, const igabem_op
   at.val.clusterDim.z = nz;
   cfg.attrs = &at;
   cfg.numAttrs = 1;
-  IGA_CUDA(cudaLaunchKernelEx(&cfg, k_farfield, A, (const double2 *)rho, npts, xhat_dev,
+  IGA_CUDA(cudaLaunchKernelEx(&cfg, R == 1 ? k_farfield<1> : k_farfield<FF64_COLS>, A, (const double2 *)rho, npts, xhat_dev,
                               reinterpret_cast<const double2 *>(d.cis), reinterpret_cast<double2 *>(uinf)));
   note_launch();
   IGA_CUDA(cudaGetLastError());
