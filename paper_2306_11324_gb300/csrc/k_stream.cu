@@ -33,8 +33,8 @@ struct StreamArgs {
   int c0, cols;           // the launch's columns c0 .. c0 + cols
   int npass, w;           // in passes of w columns
   int types, type;        // blocks per pair, and the one that applies to these columns
-  int rows_most;          // most block rows in use by a thread group
-  int group;              // threads of a group
+  int rows_most;          // most block rows in use by a thread block
+  int group;              // threads that multiply
   int ring, stage;        // FP32: byte offset of the buffers of block entries; bytes of one
   int *status;            // device status word
   int L, b, nb, nL1;      // near field: leaf grid and patch-wise coefficient grid of x
@@ -98,12 +98,15 @@ __device__ inline void stream_reduce(const StreamArgs &A, const StreamLevel &L, 
 // memory: a 16-byte shared load delivers two columns' coefficients to a warp in 4 cycles, so a thread owns two rows
 // of a pair's block (a and a + ceil(NR / 2)) and uses each coefficient twice; products take two multiply-adds
 // per instruction (for the entry s and the coefficient (x, y) the sums of s.x (x, y) and of s.y (x, y)).  The row pairs of
-// P pairs lie side by side in a thread group (NR = 49: 125 of 128 threads), and up to two groups, of up to
-// 8 columns each, share the entries in shared memory.  These come by bulk copies of whole column ranges of the
-// blocks into STREAM_STAGES buffers, issued by a warp of its own as the multiplying warps release the buffers (a
-// copy starts at the 16-byte boundary below its first entry); the pairs' source coefficients are staged by
-// cp.async one round ahead.  Every wait is bounded (2 s): one that runs out sets the status word, no further
-// copy is issued, and the block leaves once its copies in flight have landed (waited for with the same bound).
+// P pairs lie side by side in a thread block (NR = 49: 125 of 128 threads), for up to 8 columns a pass; a second
+// thread group for 8 more columns on the same entries left one block an SM and cost more than reading the blocks
+// again: near field of 384 leaves, 12 columns 0.172 -> 0.067 ms without it (other loads that wait for every row: 0.147),
+// M2L of 6144 elements, 12 and 32 columns 0.65 -> 0.64 and 1.68 -> 1.59 ms, of 24576, 12 columns 2.53 -> 2.62 ms.
+// The entries come by bulk copies of whole column ranges of the blocks into STREAM_STAGES buffers, issued by a warp
+// of its own as the multiplying warps release the buffers (a copy starts at the 16-byte boundary below its first
+// entry); the pairs' source coefficients are staged by cp.async one round ahead.  Every wait is bounded (2 s): one
+// that runs out sets the status word, no further copy is issued, and the block leaves once its copies in flight have
+// landed (waited for with the same bound).
 // Measured on GB300, 8 columns, 98304 elements (34.6 GB of coupling blocks, 4.0 GB of near field): M2L 11.6 -> 7.9 ms
 // (4.4 TB/s), near field 2.2 -> 1.1 ms; 64 columns, 24576 elements: near field 7.6 -> 2.6 ms; sound-hard, 5 columns
 // of 7 channels, 3.9 GB: M2L 5.7 -> 2.7 ms (before, each lane waited on every row's copy and every 7 or 8 columns
@@ -111,21 +114,20 @@ __device__ inline void stream_reduce(const StreamArgs &A, const StreamLevel &L, 
 // products.
 constexpr int STREAM_STAGES = 3;
 
-template <int NC, bool NEAR, bool ONE>
-__global__ void __launch_bounds__(ONE ? 160 : 288, ONE ? 2 : 1) k_stream32(const __grid_constant__ StreamArgs A) {
+template <int NC, bool NEAR>
+__global__ void __launch_bounds__(160, 2) k_stream32(const __grid_constant__ StreamArgs A) {
   extern __shared__ __align__(16) unsigned char sms[];
   __shared__ __align__(8) uint64_t full[STREAM_STAGES], empty[STREAM_STAGES];
   const int tid = threadIdx.x, lane = tid & 31, nsplit = gridDim.y, rank = blockIdx.y;
   const int ncons = blockDim.x - 32;  // threads that multiply; the last warp copies
-  const int tg = blockIdx.x / A.npass, c_pass = A.c0 + (blockIdx.x - tg * A.npass) * A.w;
+  const int tg = blockIdx.x / A.npass;
   int li = 0;
   while (li + 1 < A.nlev && tg >= A.lev[li + 1].first) ++li;
   const StreamLevel &L = A.lev[li];
   const int t = tg - L.first, NR = L.NR, HR = (NR + 1) >> 1, P = A.group / HR;
-  const int grp = tid / A.group, gt = tid - grp * A.group, slot = gt / HR, a = gt - slot * HR;
-  const int ncr_pass = min(A.w, A.c0 + A.cols - c_pass);
-  const int cr0 = c_pass + grp * NC, ncr = min(NC, ncr_pass - grp * NC);  // this group's columns
-  float2 *xs = reinterpret_cast<float2 *>(sms) + (size_t)grp * 2 * A.rows_most * NC;         // [2][P NR][NC]
+  const int slot = tid / HR, a = tid - slot * HR;
+  const int cr0 = A.c0 + (blockIdx.x - tg * A.npass) * A.w, ncr = min(A.w, A.c0 + A.cols - cr0);
+  float2 *xs = reinterpret_cast<float2 *>(sms);                                              // [2][P NR][NC]
   unsigned char *ring = sms + A.ring;                                                        // [STAGES][stage]
   const bool on = slot < P, two = a + HR < NR;
   const int k0 = L.ptr[t], np = L.ptr[t + 1] - k0, step = nsplit * P;
@@ -150,7 +152,7 @@ __global__ void __launch_bounds__(ONE ? 160 : 288, ONE ? 2 : 1) k_stream32(const
     __syncwarp();
     if (lane == 0) mbar_arrive(bar);
   };
-  auto stage_x = [&](int r) {  // this thread's two rows of its group's columns
+  auto stage_x = [&](int r) {  // this thread's two rows
     const int p0 = rank * P + r * step;
     if (on && p0 + slot < np) {
       const float2 *src0 = reinterpret_cast<const float2 *>(L.x) + source_base<NEAR>(A, NR, L.src[k0 + p0 + slot]) + cr0;
@@ -285,7 +287,7 @@ __global__ void __launch_bounds__(ONE ? 160 : 288, ONE ? 2 : 1) k_stream32(const
     asm volatile("cp.async.wait_group 0;\n" ::: "memory");
   }
   __syncthreads();
-  double2 *red = reinterpret_cast<double2 *>(ring);  // [groups NC][P NR]
+  double2 *red = reinterpret_cast<double2 *>(ring);  // [NC][P NR]
   if (on && tid < ncons)
 #pragma unroll
     for (int h = 0; h < 2; ++h)
@@ -293,10 +295,10 @@ __global__ void __launch_bounds__(ONE ? 160 : 288, ONE ? 2 : 1) k_stream32(const
 #pragma unroll
         for (int c = 0; c < NC; ++c) {
           const float4 v = tot[h][c];
-          red[(size_t)(grp * NC + c) * A.rows_most + slot * NR + a + h * HR] =
+          red[(size_t)c * A.rows_most + slot * NR + a + h * HR] =
               make_double2((double)v.x + (double)v.z, (double)v.y + (double)v.w);
         }
-  stream_reduce(A, L, red, A.rows_most, t, P, c_pass, ncr_pass);
+  stream_reduce(A, L, red, A.rows_most, t, P, cr0, ncr);
 }
 
 // FP64 blocks: FP64 arithmetic bounds them (four multiply-adds per entry and column).  A thread owns one row of one
@@ -384,21 +386,18 @@ void launch_one(StreamArgs &A, int targets, int threads, int nsplit, cudaStream_
   size_t smem;
   void (*kfn)(const StreamArgs);
   if constexpr (std::is_same<T, float>::value) {
-    // buffers for two thread blocks on an SM (one with several groups), at least one column of every pair and room
-    // for the final sums
-    const int groups = (threads - 32) / A.group;
-    A.ring = (int)(((size_t)groups * 2 * A.rows_most * NC * 8 + 15) & ~size_t(15));
-    const size_t avail = (groups == 1 ? 112 : 224) * 1024 - A.ring;
+    // buffers for two thread blocks on an SM, at least one column of every pair and room for the final sums
+    A.ring = (int)(((size_t)2 * A.rows_most * NC * 8 + 15) & ~size_t(15));
+    const size_t avail = 112 * 1024 - A.ring;
     size_t least = 0;
     for (int i = 0; i < A.nlev; ++i) {
       const int NR = A.lev[i].NR;
       least = std::max<size_t>(least, (size_t)(A.group / ((NR + 1) / 2)) * (NR * 8 + 32));
     }
-    least = std::max(least, (size_t)groups * NC * A.rows_most * 16 / STREAM_STAGES + 16);
+    least = std::max(least, (size_t)NC * A.rows_most * 16 / STREAM_STAGES + 16);
     A.stage = (int)(std::max(std::min<size_t>(avail / STREAM_STAGES, 48 * 1024) & ~size_t(127), (least + 127) & ~size_t(127)));
     smem = (size_t)A.ring + (size_t)STREAM_STAGES * A.stage;
-    if constexpr (NC >= 6) kfn = groups == 1 ? k_stream32<NC, NEAR, true> : k_stream32<NC, NEAR, false>;
-    else kfn = k_stream32<NC, NEAR, true>;  // more than 8 columns: groups of 6 or 8
+    kfn = k_stream32<NC, NEAR>;
   } else {
     smem = ((size_t)2 * A.rows_most + threads) * NC * 16;
     kfn = k_stream64<NC, NEAR>;
@@ -420,23 +419,19 @@ void launch_one(StreamArgs &A, int targets, int threads, int nsplit, cudaStream_
   note_launch();
 }
 
-// Columns c0 .. c0 + cols with the blocks of one type.  FP64: passes of at most 8 columns (their sums fill the
-// registers).  FP32: passes of up to two thread groups of at most 8 columns.
+// Columns c0 .. c0 + cols with the blocks of one type, in passes of at most 8 columns (their sums fill the registers).
 template <class T, bool NEAR>
 void launch_columns(StreamArgs &A, int c0, int cols, int type, int targets, double mean_pairs, cudaStream_t st) {
   constexpr bool F32 = std::is_same<T, float>::value;
-  const int per_pass = F32 ? 16 : 8;
   A.c0 = c0;
   A.cols = cols;
   A.type = type;
-  A.npass = (cols + per_pass - 1) / per_pass;
+  A.npass = (cols + 7) / 8;
   A.w = (cols + A.npass - 1) / A.npass;
-  const int groups = (A.w + 7) / 8;
-  int nc = (A.w + groups - 1) / groups;  // columns of a group
-  nc = nc <= 2 ? nc : (nc + 1) & ~1;     // 1, 2, 4, 6 or 8
-  if (A.npass > 1) A.w = groups * nc;
+  const int nc = A.w <= 2 ? A.w : (A.w + 1) & ~1;  // 1, 2, 4, 6 or 8
+  if (A.npass > 1) A.w = nc;
   A.npass = (cols + A.w - 1) / A.w;
-  // threads of a group (whole warps) that the levels' rows (FP32: row pairs) fill best, weighted by the levels' entries;
+  // threads that multiply (whole warps) that the levels' rows (FP32: row pairs) fill best, weighted by the levels' entries;
   // the larger of two equally good ones
   const int lo = F32 ? 96 : 128, hi = F32 ? 128 : 256;
   int group = hi;
@@ -461,11 +456,14 @@ void launch_columns(StreamArgs &A, int c0, int cols, int type, int targets, doub
     A.rows_most = std::max(A.rows_most, group / k * NR);
   }
   // targets split over clusters of blocks while the device is not filled several times and every block keeps
-  // pairs for all its threads
+  // pairs for all its threads, in FP32 for four rounds of them (its copies run three buffers ahead; near field of 384 leaves
+  // of 36 rows, one column, split in 1, 2, 4, 8: 0.024, 0.021, 0.031, 0.046 ms; M2L of 120 targets of 49 rows 0.022, 0.018,
+  // 0.024, 0.035 ms, of 144 rows 0.154, 0.098, 0.113, 0.102 ms)
   const int NRl = A.lev[A.nlev - 1].NR, P = std::max(1, group / (F32 ? (NRl + 1) / 2 : NRl));
   int nsplit = 1;
-  while (nsplit < 8 && (long)targets * A.npass * nsplit < 4 * 152 && 2.0 * nsplit * P <= mean_pairs + P) nsplit *= 2;
-  const int threads = F32 ? groups * group + 32 : group;
+  const int rounds = F32 ? 4 : 1;
+  while (nsplit < 8 && (long)targets * A.npass * nsplit < 4 * 152 && 2.0 * nsplit * P * rounds <= mean_pairs + P) nsplit *= 2;
+  const int threads = F32 ? group + 32 : group;
   auto go = [&](auto n) { launch_one<T, decltype(n)::value, NEAR>(A, targets, threads, nsplit, st); };
   if (nc == 1) go(std::integral_constant<int, 1>{});
   else if (nc == 2) go(std::integral_constant<int, 2>{});
