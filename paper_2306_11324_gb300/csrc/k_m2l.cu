@@ -68,14 +68,15 @@ template <> struct __align__(16) FlyNode<float, true> { float y[3], Dy, n[3], Dn
 // instructions a sample and CUDA's sincos, or for several columns the tile of k_m2l_gemm mostly padding): 6936
 // unknowns, one column, 175 M samples 32.2 -> 17.1 ms; 150 unknowns, 8 M samples 2.20 -> 1.08 ms; sound-hard,
 // 1736 unknowns, 3 columns of 7 channels 41 -> 4 ms.
-// FP32 sums: FLY_BLOCK source nodes at a time within a pair.  Over the pairs: forms of up to 16 columns keep the sum and
-// its rounding errors in shared memory (their registers would cost them a second block on the SM); wider ones, which
-// run one block anyway, add FLY_PAIRS pairs at a time in registers (shared memory costs them 6 %, by the L1 it takes).
+// FP32 sums: FLY_BLOCK source nodes at a time within a pair.  Over the pairs: the sum and its rounding errors, in registers
+// for up to 4 columns, in shared memory for up to 16 (their registers would cost them a second block on the SM); wider
+// forms, which run one block anyway, add FLY_PAIRS pairs at a time in registers (shared memory costs them 6 %, by the L1
+// it takes).
 // Far rows against FP64 (rms; one chain of q^2 products and of all pairs -> this): q = 12 1.06 -> 1.04e-7, q = 16, short
 // lists 6.8 -> 5.2e-8; 6144 elements, q = 7, lists of 256 pairs 9.4 -> 8.8e-8.  1 to 16 columns within 2 % of the single
 // chain's time, 24 columns 2.25 -> 2.10 ms, 21 (sound-hard) 2.34 -> 2.39 ms (1536 elements).
 constexpr int FLY_BLOCK = 16, FLY_PAIRS = 8;
-template <class T, int NC> constexpr bool fly_sums = std::is_same<T, float>::value && NC <= 16;
+template <class T, int NC> constexpr bool fly_sums = std::is_same<T, float>::value && NC > 4 && NC <= 16;
 
 // bytes in front of the nodes: the table of phase64, or the sums of the FP32 form
 template <class T, int NC> __host__ __device__ constexpr size_t fly_head() {
@@ -120,7 +121,8 @@ __global__ void __launch_bounds__(256) k_m2l_fly(const __grid_constant__ M2LArgs
     ta = F32 ? (T)L.nodes32[6 * NQ + ia] : (T)L.nodes[6 * NQ + ia];
     if (!HARD) ta *= eta;
   }
-  C2<T> tot[SUMS ? 1 : NC], few[F32 && !SUMS ? NC : 1];  // few: of the last FLY_PAIRS pairs at most
+  // FP32: few has the rounding errors of tot (up to 4 columns), or the last FLY_PAIRS pairs at most (above 16)
+  C2<T> tot[SUMS ? 1 : NC], few[F32 && !SUMS ? NC : 1];
   int kept = 0;
   if constexpr (!SUMS) {
 #pragma unroll
@@ -254,6 +256,13 @@ __global__ void __launch_bounds__(256) k_m2l_fly(const __grid_constant__ M2LArgs
           two_sum(w.y, w.w, v.y);
           sums[c * 256 + tid] = w;
         }
+      } else if constexpr (NC <= 4) {
+#pragma unroll
+        for (int c = 0; c < NC; ++c) {
+          const C2<T> v = mul(e0, part[c]);
+          two_sum(tot[c].x, few[c].x, v.x);
+          two_sum(tot[c].y, few[c].y, v.y);
+        }
       } else {
 #pragma unroll
         for (int c = 0; c < NC; ++c) few[c] = fma2(e0, part[c], few[c]);
@@ -267,7 +276,17 @@ __global__ void __launch_bounds__(256) k_m2l_fly(const __grid_constant__ M2LArgs
         }
       }
     } else {
-      for (int b = 0; b < Q; ++b) add_node(b, part);
+      // nodes at a time: 4 columns, 175 M samples 22.3 -> 21.1 ms with four; sound-hard, one column of 7 channels, 8 M
+      // samples 1.43 -> 1.37 ms with two
+      if constexpr (NC == 4) {
+#pragma unroll 4
+        for (int b = 0; b < Q; ++b) add_node(b, part);
+      } else if constexpr (NC == 7) {
+#pragma unroll 2
+        for (int b = 0; b < Q; ++b) add_node(b, part);
+      } else {
+        for (int b = 0; b < Q; ++b) add_node(b, part);
+      }
 #pragma unroll
       for (int c = 0; c < NC; ++c) tot[c] = add(tot[c], part[c]);
     }
