@@ -66,15 +66,17 @@ template <> struct __align__(16) FlyNode<float, true> { float y[3], Dy, n[3], Dn
 // gridDim.y blocks, which add their sums through distributed shared memory, where a level has too few
 // targets to fill the device.  Measured on GB300, FP64 products (before: one warp per pair, 72 FP64
 // instructions a sample and CUDA's sincos, or for several columns the tile of k_m2l_gemm mostly padding): 6936
-// unknowns, one column, 175 M samples 32.2 -> 17.1 ms; 150 unknowns, 8 M samples 2.20 -> 1.08 ms; sound-hard,
+// unknowns, one column, 175 M samples 32.2 -> 16.3 ms; 150 unknowns, 8 M samples 2.20 -> 0.89 ms; sound-hard,
 // 1736 unknowns, 3 columns of 7 channels 41 -> 4 ms.
 // FP32 sums: FLY_BLOCK source nodes at a time within a pair.  Over the pairs: the sum and its rounding errors, in registers
 // for up to 4 columns, in shared memory for up to 16 (their registers would cost them a second block on the SM); wider
 // forms, which run one block anyway, add FLY_PAIRS pairs at a time in registers (shared memory costs them 6 %, by the L1
 // it takes).
 // Far rows against FP64 (rms; one chain of q^2 products and of all pairs -> this): q = 12 1.06 -> 1.04e-7, q = 16, short
-// lists 6.8 -> 5.2e-8; 6144 elements, q = 7, lists of 256 pairs 9.4 -> 8.8e-8.  1 to 16 columns within 2 % of the single
-// chain's time, 24 columns 2.25 -> 2.10 ms, 21 (sound-hard) 2.34 -> 2.39 ms (1536 elements).
+// lists 6.8 -> 5.2e-8; 6144 elements, q = 7, lists of 256 pairs 9.4 -> 8.8e-8.  Time against the single chain, 1536
+// elements: 1 to 4 columns 0.41 -> 0.38 (one), 0.54 -> 0.48 ms (four), 8 and 16 within 2 %, 24 2.25 -> 2.10 ms, 21
+// (sound-hard) 2.34 -> 2.39 ms; where a target has few pairs the sums in shared memory show (1024 elements of a torus,
+// 8 columns 0.26 -> 0.29 ms).
 constexpr int FLY_BLOCK = 16, FLY_PAIRS = 8;
 template <class T, int NC> constexpr bool fly_sums = std::is_same<T, float>::value && NC > 4 && NC <= 16;
 

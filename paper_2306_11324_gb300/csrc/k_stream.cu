@@ -107,9 +107,9 @@ __device__ inline void stream_reduce(const StreamArgs &A, const StreamLevel &L, 
 // entry); the pairs' source coefficients are staged by cp.async one round ahead.  Every wait is bounded (2 s): one
 // that runs out sets the status word, no further copy is issued, and the block leaves once its copies in flight have
 // landed (waited for with the same bound).
-// Measured on GB300, 8 columns, 98304 elements (34.6 GB of coupling blocks, 4.0 GB of near field): M2L 11.6 -> 7.9 ms
-// (4.4 TB/s), near field 2.2 -> 1.1 ms; 64 columns, 24576 elements: near field 7.6 -> 2.6 ms; sound-hard, 5 columns
-// of 7 channels, 3.9 GB: M2L 5.7 -> 2.7 ms (before, each lane waited on every row's copy and every 7 or 8 columns
+// Measured on GB300, 8 columns, 98304 elements (34.6 GB of coupling blocks, 4.0 GB of near field): M2L 11.4 -> 7.7 ms
+// (4.5 TB/s), near field 2.2 -> 1.1 ms; 64 columns, 24576 elements: M2L 36.7 -> 21.7, near field 7.5 -> 2.3 ms;
+// sound-hard, 6144 elements, 5 columns of 7 channels: M2L 4.6 -> 2.1 ms (before, each lane waited on every row's copy and every 7 or 8 columns
 // read the blocks again).  What bounds it now: two blocks of four multiplying warps an SM, latency between the
 // products.
 constexpr int STREAM_STAGES = 3;
